@@ -467,7 +467,7 @@ fftpl_status fftpl_server_set_clock(fftpl_server_t s, double now_s);
  * cudaStream_t (NULL: legacy default stream).
  *
  * Memory: the intermediate transforms live in one fixed array in the
- * library's device image (about 20 MiB), which every GPU that loads the
+ * library's device image (about 12 MiB), which every GPU that loads the
  * library keeps until the process exits; the call allocates nothing (no
  * cudaMalloc, cudaFree or allocating library routine).  The first call on a
  * device looks up that array's device address and sets up the kernels for

@@ -771,8 +771,6 @@ static fftpl_status create_impl(Ctx& c, const fftpl_region* R, int32_t n, const 
     spec_maps_init(c);
     TRY(dalloc(c, &c.psi, nn));
     TRY(dalloc(c, &c.E2, nn));
-    TRY(dalloc(c, &c.tw, n));
-    TRY(dalloc(c, &c.ph, n + 1));
     TRY(dalloc(c, &c.acc, kAccDoubles));
     TRY(dalloc(c, &c.err, 1));
     TRY(dalloc(c, &c.gN, 2 * (size_t)c.m_mov));
@@ -790,19 +788,6 @@ static fftpl_status create_impl(Ctx& c, const fftpl_region* R, int32_t n, const 
         CK(cudaMemcpyAsync(c.fix_x, cells->fix_x, c.m_fix * sizeof(float), cudaMemcpyHostToDevice, s));
         CK(cudaMemcpyAsync(c.fix_y, cells->fix_y, c.m_fix * sizeof(float), cudaMemcpyHostToDevice, s));
     }
-    // transform tables (FP64 on the host, rounded once): FFT twiddles
-    // exp(-2 pi i k / n) and cosine-transform twiddles exp(-i pi u / 2n)
-    std::vector<float2> tw(n), ph(n + 1);
-    for (int k = 0; k < n; ++k) {
-        double a = 2.0 * M_PI * k / n;
-        tw[k] = make_float2((float)cos(a), (float)-sin(a));
-    }
-    for (int u = 0; u <= n; ++u) {
-        double a = M_PI * u / (2.0 * n);
-        ph[u] = make_float2((float)cos(a), (float)-sin(a));
-    }
-    CK(cudaMemcpyAsync(c.tw, tw.data(), n * sizeof(float2), cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(c.ph, ph.data(), (n + 1) * sizeof(float2), cudaMemcpyHostToDevice, s));
     TRY(build_slabs(c, nets, pins));
     if (c.opt.deterministic) {
         // capacity in blocks of every kernel that reduces on each stream
@@ -850,6 +835,22 @@ static fftpl_status create_impl(Ctx& c, const fftpl_region* R, int32_t n, const 
         float2* zv = nullptr;
         TRY(dalloc(c, &block, tcr_elems(n)));
         TRY(dalloc(c, &zv, 2 * nn));
+        // its transform tables (FP64 on the host, rounded once): twiddles
+        // exp(-2 pi i k / n) and exp(-i pi u / 2n)
+        TRY(dalloc(c, &c.tw, n));
+        TRY(dalloc(c, &c.ph, n + 1));
+        std::vector<float2> tw(n), ph(n + 1);
+        for (int k = 0; k < n; ++k) {
+            double a = 2.0 * M_PI * k / n;
+            tw[k] = make_float2((float)cos(a), (float)-sin(a));
+        }
+        for (int u = 0; u <= n; ++u) {
+            double a = M_PI * u / (2.0 * n);
+            ph[u] = make_float2((float)cos(a), (float)-sin(a));
+        }
+        CK(cudaMemcpyAsync(c.tw, tw.data(), n * sizeof(float2), cudaMemcpyHostToDevice, s));
+        CK(cudaMemcpyAsync(c.ph, ph.data(), (n + 1) * sizeof(float2), cudaMemcpyHostToDevice, s));
+        CK(cudaStreamSynchronize(s));
         cudaError_t e = tcr_setup(c, block, zv, s);
         if (e == cudaErrorInvalidValue)
             return set_err(c, FFTPL_ECUDA, "cuTensorMapEncodeTiled unavailable or failed");

@@ -5,8 +5,9 @@
 //   movable cells   w, h                       (m_mov)
 //   fixed cells     fix_x, fix_y (m_fix)       macro map M = rho_t F  [n][n]
 //   density         D (movable overlap area, float) or Dq (int64, 2^-32 units)
-//   spectral        T1 [u][y]  (rows transformed along x, stored transposed)
-//                   PT [y][u], RT [y][u]  (columns transformed and inverted)
+//   spectral        T1 [u/2][y] of (u even, u odd)  (rows transformed along x,
+//                   stored transposed), PT, RT [y/2][u] of (y even, y odd)
+//                   (columns transformed and inverted)
 //                   psi, ex, ey [y][x], rho [y][x] (formed on demand)
 //   nets/pins       slabs of nets of equal degree; pin_cell, pin_dx, pin_dy,
 //                   pin_slot in slab order (slot base + 32 k + lane);
@@ -28,8 +29,6 @@
 namespace fftpl {
 
 // ------------------------------------------------------------------ sizes
-constexpr int kSpecThreads = 256;   // threads of the transform kernels
-constexpr int kSpecBuffers = 4;     // complex length-n buffers per CTA
 constexpr int kCellThreads = 256;
 constexpr int kWaThreads = 256;
 // Nets of degree kBigMin..kBigMax go to the WA kernel with several lanes per
@@ -410,15 +409,15 @@ struct Ctx {
     float *M = nullptr, *D = nullptr;
     long long* Dq = nullptr;
     float *T1 = nullptr, *PT = nullptr, *RT = nullptr;
-    // tensor maps of T1 (boxes of 8 columns), PT and RT (boxes of 4 columns),
-    // 256 rows (n if smaller): the transposed tiles of the row and column
+    // tensor maps of T1, PT and RT (n/2 rows of n pairs; boxes of 4 pairs by
+    // 256 rows, n/2 if smaller): the transposed tiles of the row and column
     // passes leave shared memory through the tensor-memory-access unit
     CUtensorMap map_t1{}, map_pt{}, map_rt{};
     bool spec_tma = false;      // the transposed stores go through the maps
     bool spec_maps_ok = false;  // the maps could be encoded
     float *psi = nullptr, *ex = nullptr, *ey = nullptr, *rho = nullptr;
     float2* E2 = nullptr;       // interleaved field (E_x, E_y) [n][n]
-    float2 *tw = nullptr, *ph = nullptr;
+    float2 *tw = nullptr, *ph = nullptr;   // tables of the radix tensor-core path
     // pins re-laid into degree slabs (see k_wire.cu): slot base + 32 k + lane
     int4* slabs = nullptr;      // {base slot, degree, net count, lanes per net (0: one
                                 // net per lane)}
@@ -520,8 +519,10 @@ cudaError_t launch_bin_ranges(Ctx& c, const float* x, const float* y, int32_t* r
 cudaError_t launch_rows_fwd(Ctx& c, cudaStream_t s);
 cudaError_t launch_cols_spectral(Ctx& c, cudaStream_t s);
 cudaError_t launch_rows_inv(Ctx& c, cudaStream_t s);
-// psi rows from PT (transform path; formed on demand, not in the evaluation)
+// psi rows from PT (transform path; formed on demand, not in the evaluation);
+// launch_rows_maps: psi, E_x and E_y into their separate maps
 cudaError_t launch_rows_psi(Ctx& c, cudaStream_t s);
+cudaError_t launch_rows_maps(Ctx& c, cudaStream_t s);
 // Tensor maps for the transposed stores of the transform passes (host only,
 // no allocation); clears c.spec_tma if the driver cannot encode them.
 void spec_maps_init(Ctx& c);

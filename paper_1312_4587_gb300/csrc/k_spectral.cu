@@ -8,39 +8,45 @@
 //   E_x[y][x] = sum_u w_u S(u,x) P[u][y]
 //   E_y[y][x] = sum_u C(u,x) R[u][y],        R[u][y] = sum_v w_v Psi[v][u] S(v,y)
 //
-// Three passes, each over whole rows held in shared memory:
-//   rows_fwd  : rho rows -> DCT-II along x -> T1[u][y] (written transposed)
+// Three passes:
+//   rows_fwd  : rho rows -> DCT-II along x -> T1 (written transposed)
 //   cols      : T1 rows  -> DCT-II along y -> divide -> inverse along y for P
-//               and R -> PT[y][u], RT[y][u] (written transposed); the energy
+//               and R -> PT, RT (written transposed); the energy
 //               N = 1/2 A_b sum B Psi (Parseval) is reduced here
 //   rows_inv  : PT, RT rows -> E_x, E_y rows (psi from PT on demand)
+// The transposed maps hold two neighbouring rows interleaved, as the complex
+// rows of the next pass's FFTs: T1[u/2][y] = (u even, u odd) and
+// PT[y/2][u], RT[y/2][u] = (y even, y odd).
 //
 // Each 1-D cosine transform of length n is one complex FFT of length n
 // (Makhoul's reordering: v[k] = r[2k], v[n-1-k] = r[2k+1]; A[u] =
 // Re(exp(-i pi u / 2n) V[u])), two real rows packed into one complex FFT.
 // The inverse cosine sum y[x] = sum_u c[u] C(u,x) is the inverse of that map;
 // a sine sum is a cosine sum of the reversed coefficients times (-1)^x.
-// The FFTs are radix-4 Stockham (plus one radix-2 stage for odd log2 n) in
-// shared memory with twiddles from a float32 table computed in FP64: a
-// radix-R butterfly loads W^(b st) for b = 1, 2, 4, 8 and forms the other
-// R - 1 - log2 R by products, at most three deep (about 3 ulp; each table
-// load costs more than the multiplies: 4 instead of 15 loads per radix-16
-// butterfly took the three passes from 124 to 114 us).
+//
+// The FFT lives in registers: n/E threads per FFT hold E elements each.  A
+// Stockham FFT of radices n / E^k, E, .., E reads in every stage and leaves
+// at the end, in thread t, the elements t + (n/E) q, q < E, whatever the
+// radix, so that the work around the FFTs needs no shared memory either:
+// Makhoul's order (elements p and n-1-p), the split of two packed spectra
+// (u and n-u) and the unshuffle pair element q of thread t with element
+// E-1-q of thread n/E-1-t or n/E-t, and the threads are numbered so that this
+// is another lane of the same warp (lane_rev, lane_neg): one shuffle.  Only
+// the exchanges between stages go through shared memory (two at n = 2048).
+// What bounds it: latency and the FP32 pipe.  Against the same transforms
+// with every stage, the packing and the unshuffle through shared buffers
+// (bound by the shared-memory pipe at 22 % warps active), launch times under
+// ncu, cold caches: n = 2048 rows_fwd 19.9 -> 15.2, cols 39.3 -> 24.5,
+// rows_inv 26.6 -> 15.8 us; n = 4096 96 -> 58, 187 -> 99, 111 -> 52 us.
 #include "fftpl_internal.cuh"
 
 namespace fftpl {
 
-// ------------------------------------------------------------ FFT core
-// Buffers are padded by one element every 16 (index i lives at i + i/16) so
-// that the strided Stockham writes spread over the shared-memory banks.
-__host__ __device__ constexpr int padded(int n) { return n + n / 16; }
-__device__ __forceinline__ int pidx(int i) { return i + (i >> 4); }
-
 // ------------------------------------- stores through the TMA unit
 // A pass that writes its output transposed first lays the tile out in shared
 // memory in the output's order, then one thread stores it box by box with
-// cp.async.bulk.tensor: the tile leaves the SM as whole rows of the box
-// instead of one 16- or 32-byte piece per thread and store instruction.
+// cp.async.bulk.tensor: the tile leaves the SM as whole 32-byte rows of the
+// box instead of one piece per thread and store instruction.
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
@@ -70,6 +76,85 @@ __device__ __forceinline__ void tma_store_drain() {
     asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
+// ------------------------------------------------------- transform tables
+// Constants of the build (Taylor series in FP64, rounded once), the same for
+// every handle.  w: for a radix-16 stage after Ns points (Ns = 2 .. 256) and
+// k < Ns, the twiddles W^bk, W = exp(-2 pi i / 16 Ns), b = 2, 4, 6, 8, 1, 3,
+// 12 at [8 (Ns - 2 + k)]; the others are one product of two of them (loads
+// cost more than the multiplies).  A radix-8 stage's W, W^2, W^3 and W^4 are
+// the first four (two 16-byte loads).  ph: exp(-i pi u / 2n) for u < n at
+// [n - 16 + u].  Fewer loads and more products (W, W^2, W^4, W^8 only; ph
+// from one load and constants) saved 1 to 2 % of the passes and raised the
+// relative error of psi, E_x and E_y from 2.1-2.9 to 2.8-3.2 1e-7 at n = 2048
+// and 4096 (shared-memory form: 2.3-3.0).
+constexpr double kPi = 3.14159265358979323846;
+
+struct UnitD {
+    double c, s;
+};
+
+// sine and cosine series on [-pi/4, pi/4] (terms to a^23)
+constexpr UnitD unit_small(double a) {
+    double c = 1.0, s = a, tc = 1.0, ts = a;
+    for (int k = 1; k < 12; ++k) {
+        tc *= -a * a / ((2 * k - 1) * (2 * k));
+        ts *= -a * a / ((2 * k) * (2 * k + 1));
+        c += tc;
+        s += ts;
+    }
+    return {c, s};
+}
+
+// cos and sin of 2 pi num / den (num >= 0)
+constexpr UnitD unit_root(long num, long den) {
+    num %= den;
+    const long quad = (4 * num + den / 2) / den;   // nearest multiple of pi/2
+    const UnitD u = unit_small(0.5 * kPi * (double)(4 * num - quad * den) / (double)den);
+    switch (quad & 3) {
+        case 0: return {u.c, u.s};
+        case 1: return {-u.s, u.c};
+        case 2: return {-u.c, -u.s};
+        default: return {u.s, -u.c};
+    }
+}
+
+struct Pair {
+    float x, y;
+};
+
+constexpr int kMaxNs = FFTPL_MAX_N / 16;
+
+struct alignas(16) SpecTables {
+    Pair w[8 * (2 * kMaxNs - 2)];
+    Pair ph[2 * FFTPL_MAX_N - 16];
+};
+
+constexpr SpecTables make_tables() {
+    SpecTables t{};
+    for (int ns = 2; ns <= kMaxNs; ns *= 2)
+        for (int k = 0; k < ns; ++k)
+            for (int b = 0; b < 7; ++b) {
+                const int e[7] = {2, 4, 6, 8, 1, 3, 12};
+                const UnitD u = unit_root((long)k * e[b], 16L * ns);
+                t.w[8 * (ns - 2 + k) + b] = {(float)u.c, (float)-u.s};
+            }
+    for (int n = 16; n <= FFTPL_MAX_N; n *= 2)
+        for (int k = 0; k < n; ++k) {
+            const UnitD u = unit_root(k, 4L * n);
+            t.ph[n - 16 + k] = {(float)u.c, (float)-u.s};
+        }
+    return t;
+}
+
+static __device__ const SpecTables g_tab = make_tables();
+
+// exp(-i pi u / 2N)
+template <int N>
+__device__ __forceinline__ float2 phase(int u) {
+    return __ldg(reinterpret_cast<const float2*>(g_tab.ph) + (N - 16 + u));
+}
+
+// ------------------------------------------------------------ FFT core
 // Twiddle exp(-+2 pi i k / 16) for the small exponents a radix-16 butterfly
 // uses (cos and sin of multiples of pi/8).
 __device__ __forceinline__ float2 w16(int e, bool inv) {
@@ -110,34 +195,25 @@ __device__ __forceinline__ void dft4(float2& a0, float2& a1, float2& a2, float2&
     a3 = csub(d02, d13);
 }
 
-// R-point DFT in registers, natural order in and out.
-template <int R>
-__device__ __forceinline__ void dft(float2 (&v)[R], bool inv);
-
-template <>
-__device__ __forceinline__ void dft<2>(float2 (&v)[2], bool) { dft2(v[0], v[1]); }
-
-template <>
-__device__ __forceinline__ void dft<4>(float2 (&v)[4], bool inv) { dft4(v[0], v[1], v[2], v[3], inv); }
-
-template <>
-__device__ __forceinline__ void dft<8>(float2 (&v)[8], bool inv) {
+// 8-point DFT of v[0], v[S], .., v[7 S] in place, natural order
+template <int S>
+__device__ __forceinline__ void dft8(float2* v, bool inv) {
     // 8 = 2 x 4: DFT4 of even and odd samples, twiddle W8^k, combine
-    float2 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6];
-    float2 o0 = v[1], o1 = v[3], o2 = v[5], o3 = v[7];
+    float2 e0 = v[0], e1 = v[2 * S], e2 = v[4 * S], e3 = v[6 * S];
+    float2 o0 = v[S], o1 = v[3 * S], o2 = v[5 * S], o3 = v[7 * S];
     dft4(e0, e1, e2, e3, inv);
     dft4(o0, o1, o2, o3, inv);
     o1 = cmul(o1, w16(2, inv));
     o2 = cmul(o2, w16(4, inv));
     o3 = cmul(o3, w16(6, inv));
-    v[0] = cadd(e0, o0); v[4] = csub(e0, o0);
-    v[1] = cadd(e1, o1); v[5] = csub(e1, o1);
-    v[2] = cadd(e2, o2); v[6] = csub(e2, o2);
-    v[3] = cadd(e3, o3); v[7] = csub(e3, o3);
+    v[0] = cadd(e0, o0); v[4 * S] = csub(e0, o0);
+    v[S] = cadd(e1, o1); v[5 * S] = csub(e1, o1);
+    v[2 * S] = cadd(e2, o2); v[6 * S] = csub(e2, o2);
+    v[3 * S] = cadd(e3, o3); v[7 * S] = csub(e3, o3);
 }
 
-template <>
-__device__ __forceinline__ void dft<16>(float2 (&v)[16], bool inv) {
+// 16-point DFT in place, natural order
+__device__ __forceinline__ void dft16(float2* v, bool inv) {
     // 16 = 4 x 4: X[k1 + 4 k2] = sum_n2 W4^(n2 k2) W16^(n2 k1) sum_n1 x[4 n1 + n2] W4^(n1 k1)
     float2 y[4][4];
 #pragma unroll
@@ -156,89 +232,238 @@ __device__ __forceinline__ void dft<16>(float2 (&v)[16], bool inv) {
     }
 }
 
-// One Stockham stage of radix R over NB padded buffers of length N, with Ns
-// the product of the radices already applied.  Reads everything it needs
-// into registers, synchronises, then writes.
-template <int LOGN, int NB, int R>
-__device__ __forceinline__ void stockham_stage(float2* __restrict__ buf, const float2* __restrict__ tw,
-                                               int Ns, bool inv) {
-    constexpr int N = 1 << LOGN;
-    constexpr int NP = padded(N);
-    constexpr int T = kSpecThreads;
-    constexpr int NR = N / R;
-    constexpr int ITEMS = NB * NR;
-    constexpr int PER = (ITEMS + T - 1) / T;
-    float2 v[PER][R];
-    int dst[PER];
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-        int gi = threadIdx.x + i * T;
-        dst[i] = -1;
-        if (ITEMS % T == 0 || gi < ITEMS) {
-            int f = gi / NR, j = gi % NR;
-            int k = j & (Ns - 1);
-            const float2* src = buf + f * NP;
-            int st = (N / (R * Ns)) * k;   // twiddle index step: W_N^(r st)
-            v[i][0] = src[pidx(j)];
-            if (Ns == 1) {
-                // first stage: every twiddle is exp(0) = 1
-#pragma unroll
-                for (int r = 1; r < R; ++r) v[i][r] = src[pidx(j + r * NR)];
-            } else {
-                // W^(r st) for r < R from the table's W^(st), W^(2 st),
-                // W^(4 st), W^(8 st) by products (at most three deep)
-                float2 w[R];
-                w[0] = make_float2(1.0f, 0.0f);
-#pragma unroll
-                for (int b = 1; b < R; b <<= 1) w[b] = tw[b * st];
-#pragma unroll
-                for (int r = 3; r < R; ++r)
-                    if (r & (r - 1)) w[r] = cmul(w[r & (r - 1)], w[r & -r]);
-#pragma unroll
-                for (int r = 1; r < R; ++r) {
-                    float2 ww = w[r];
-                    if (inv) ww.y = -ww.y;
-                    v[i][r] = cmul(src[pidx(j + r * NR)], ww);
-                }
-            }
-            dst[i] = (f << 24) | ((j - k) * R + k);   // buffer and element index
+// Elements per thread: 8 up to n = 1024, where a pass has fewer warps than
+// the GPU has room for and the length of a thread's own chain decides, 16
+// above, where fewer exchanges win.  A graph-replayed evaluation without nets
+// (two memsets, scatter, the passes, cell kernel) of 1,000 cells, E = 8
+// against E = 16: n = 64 17.8 / 22.5 us, 512 20.6 / 26.1, 1024 28.8 / 30.4,
+// 2048 82.1 / 65.7, 4096 284 / 231.
+constexpr int spec_elems(int logn) { return logn <= 10 ? 8 : 16; }
+// Blocks of t threads per SM the registers are budgeted for: 16 warps of up
+// to 128, or 24 of up to 80.
+constexpr int spec_blocks(int logn, int t) {
+    const int b = (spec_elems(logn) == 16 ? 512 : 768) / t;
+    return b > 32 ? 32 : b;
+}
+
+// Layout of a pass: NF FFTs of length n side by side per group of
+// NF n / E threads (FFT f = thread % NF, so that shared memory holds the NF
+// elements of one index together), as many groups as fill a warp per block.
+template <int LOGN, int NF>
+struct Lay {
+    static constexpr int N = 1 << LOGN;
+    static constexpr int E = spec_elems(LOGN);   // elements per thread
+    static constexpr int LOGE = E == 16 ? 4 : 3;
+    static constexpr int Q = N / E;              // threads per FFT
+    static constexpr int LT = NF * Q;            // threads per group
+    static constexpr int GB = LT >= 32 ? 1 : 32 / LT;   // groups per block
+    static constexpr int T = LT >= 32 ? LT : 32;        // threads per block
+    static constexpr int R0 = 1 << (LOGN % LOGE);   // radix of the first stage (1: E)
+    static constexpr int LQ = NF == 1 ? 4 : 3;      // log2(16 / NF)
+    // elements of one padded buffer
+    static constexpr int PADN = N + (R0 == 1 || (N >> LQ) < N / E ? N / E : (N >> LQ));
+    // shared bytes of one group holding V buffers per FFT (128-byte multiple)
+    static constexpr int group_bytes(int v) { return (v * NF * PADN * 8 + 127) / 128 * 128; }
+};
+
+// Thread's element offset t (elements t + Q q) such that thread Q - 1 - t of
+// the same FFT is lane *partner of the same warp.
+template <int LOGN, int NF>
+__device__ __forceinline__ int lane_rev(int lt, int* partner) {
+    using L = Lay<LOGN, NF>;
+    const int lane = threadIdx.x & 31;
+    if constexpr (L::LT <= 32) {
+        const int t = lt / NF;
+        *partner = lane + (L::Q - 1 - 2 * t) * NF;
+        return t;
+    } else {
+        constexpr int half = 16 / NF;
+        const int i = (lt >> 5) * half + (lane & 15) / NF;
+        *partner = lane ^ 16;
+        return lane < 16 ? i : L::Q - 1 - i;
+    }
+}
+
+// The same with thread (Q - t) mod Q as the partner.
+template <int LOGN, int NF>
+__device__ __forceinline__ int lane_neg(int lt, int* partner) {
+    using L = Lay<LOGN, NF>;
+    const int lane = threadIdx.x & 31;
+    if constexpr (L::LT <= 32) {
+        const int t = lt / NF;
+        *partner = lane + (((L::Q - t) & (L::Q - 1)) - t) * NF;
+        return t;
+    } else {
+        constexpr int half = 16 / NF;
+        const int i = (lt >> 5) * half + (lane & 15) / NF;
+        *partner = i == 0 ? lane : lane ^ 16;
+        return lane < 16 ? i : (i == 0 ? L::Q / 2 : L::Q - i);
+    }
+}
+
+// Padding of the exchange after a stage, so that its strided writes spread
+// over the banks: after the first small radix, and after a radix-E stage that
+// followed Ns points.
+template <int LQ>
+__device__ __forceinline__ int pad_first(int i) { return i + (i >> LQ); }
+template <int E, int Ns>
+__device__ __forceinline__ int pad_stage(int i) {
+    if constexpr (Ns < 16) return i + Ns * (i / (E * Ns));
+    else return i;
+}
+
+template <int LOGN, int NF>
+__device__ __forceinline__ void group_sync() {
+    if constexpr (Lay<LOGN, NF>::T == 32) __syncwarp();
+    else __syncthreads();
+}
+
+__device__ __forceinline__ float2 shfl2(float2 v, int src) {
+    return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
+}
+
+// Twiddles W^r, r < E, of a radix-E stage from the table's entry.
+template <int E>
+struct Tw {
+    float4 a, b, c;
+    float2 d;
+    __device__ __forceinline__ void load(int Ns, int k) {
+        const float4* tb = reinterpret_cast<const float4*>(g_tab.w) + 4 * (Ns - 2 + k);
+        a = __ldg(tb);
+        b = __ldg(tb + 1);
+        if (E == 16) {
+            c = __ldg(tb + 2);
+            d = __ldg(reinterpret_cast<const float2*>(tb + 3));
         }
     }
-    __syncthreads();
+    template <int NV>
+    __device__ __forceinline__ void apply(float2 (&v)[NV][E], bool inv) const {
+        const float s = inv ? -1.0f : 1.0f;
+        float2 w[E];
+        if constexpr (E == 16) {
+            w[2] = make_float2(a.x, s * a.y);
+            w[4] = make_float2(a.z, s * a.w);
+            w[6] = make_float2(b.x, s * b.y);
+            w[8] = make_float2(b.z, s * b.w);
+            w[1] = make_float2(c.x, s * c.y);
+            w[3] = make_float2(c.z, s * c.w);
+            w[12] = make_float2(d.x, s * d.y);
+            w[5] = cmul(w[4], w[1]);
+            w[7] = cmul(w[4], w[3]);
+            w[9] = cmul(w[8], w[1]);
+            w[10] = cmul(w[8], w[2]);
+            w[11] = cmul(w[8], w[3]);
+            w[13] = cmul(w[12], w[1]);
+            w[14] = cmul(w[12], w[2]);
+            w[15] = cmul(w[12], w[3]);
+        } else {
+            w[1] = make_float2(a.x, s * a.y);
+            w[2] = make_float2(a.z, s * a.w);
+            w[3] = make_float2(b.x, s * b.y);
+            w[4] = make_float2(b.z, s * b.w);
+            w[5] = cmul(w[4], w[1]);
+            w[6] = cmul(w[4], w[2]);
+            w[7] = cmul(w[4], w[3]);
+        }
 #pragma unroll
-    for (int i = 0; i < PER; ++i) {
-        if (dst[i] < 0) continue;
-        dft<R>(v[i], inv);
-        float2* out = buf + (dst[i] >> 24) * NP;
-        int o = dst[i] & 0xffffff;
+        for (int i = 0; i < NV; ++i)
 #pragma unroll
-        for (int r = 0; r < R; ++r) out[pidx(o + r * Ns)] = v[i][r];
+            for (int r = 1; r < E; ++r) v[i][r] = cmul(v[i][r], w[r]);
     }
-    __syncthreads();
+};
+
+template <int E>
+__device__ __forceinline__ void dft_full(float2* v, bool inv) {
+    if constexpr (E == 16) dft16(v, inv);
+    else dft8<1>(v, inv);
 }
 
-// NB complex FFTs of length N = 2^LOGN in the padded buffers.  Forward:
-// X[k] = sum x[j] exp(-2 pi i jk / N); inverse: + sign, no 1/N.  Radix-16
-// stages first, then one radix-2/4/8 stage for the remaining factor.
-template <int LOGN, int NB>
-__device__ __forceinline__ void fft_block(float2* __restrict__ buf, const float2* __restrict__ tw,
-                                          bool inv) {
-    int Ns = 1;
+// The radix-E stages from Ns points on; the elements of index i of FFT f are
+// in buf[PAD(i) NF + f] (PNs > 0: padded by a radix-E stage after PNs points,
+// 0: by the first small radix).
+template <int LOGN, int NF, int NV, int Ns, int PNs, int E>
+__device__ __forceinline__ void fft_stages(float2 (&v)[NV][E], float2* buf, int lt, int tl, int f,
+                                           bool inv) {
+    using L = Lay<LOGN, NF>;
+    if constexpr (Ns < L::N) {
+        constexpr bool last = E * Ns == L::N;
+        const int t = last ? tl : lt / NF;
+        const int k = t & (Ns - 1);
+        Tw<E> tw;
+        tw.load(Ns, k);
+        group_sync<LOGN, NF>();
 #pragma unroll
-    for (int s = 0; s + 4 <= LOGN; s += 4) {
-        stockham_stage<LOGN, NB, 16>(buf, tw, Ns, inv);
-        Ns <<= 4;
+        for (int a = 0; a < NV; ++a)
+#pragma unroll
+            for (int q = 0; q < E; ++q) {
+                const int i = t + L::Q * q;
+                const int p = PNs == 0 ? pad_first<L::LQ>(i) : pad_stage<E, (PNs ? PNs : 1)>(i);
+                v[a][q] = buf[a * (NF * L::PADN) + p * NF + f];
+            }
+        tw.apply(v, inv);
+#pragma unroll
+        for (int a = 0; a < NV; ++a) dft_full<E>(v[a], inv);
+        if constexpr (!last) {
+            group_sync<LOGN, NF>();
+            const int o = (t - k) * E + k;
+#pragma unroll
+            for (int a = 0; a < NV; ++a)
+#pragma unroll
+                for (int r = 0; r < E; ++r)
+                    buf[a * (NF * L::PADN) + pad_stage<E, Ns>(o + r * Ns) * NF + f] = v[a][r];
+            fft_stages<LOGN, NF, NV, E * Ns, Ns>(v, buf, lt, tl, f, inv);
+        }
     }
-    constexpr int REM = LOGN & 3;
-    if (REM == 1) stockham_stage<LOGN, NB, 2>(buf, tw, Ns, inv);
-    if (REM == 2) stockham_stage<LOGN, NB, 4>(buf, tw, Ns, inv);
-    if (REM == 3) stockham_stage<LOGN, NB, 8>(buf, tw, Ns, inv);
 }
 
-// Position of sample x in Makhoul's reordering.
-__device__ __forceinline__ int mk_pos(int x, int N) { return (x & 1) ? (N - 1 - (x >> 1)) : (x >> 1); }
-// Sample of the natural order held at position k of the reordering.
-__device__ __forceinline__ int mk_src(int y, int N) { return (y & 1) ? (N - 1 - (y >> 1)) : (y >> 1); }
+// NV complex FFTs of length N per thread group and f: thread element offset
+// t0 on input, tl on output (elements t + Q q in natural order).  Forward:
+// X[k] = sum x[j] exp(-2 pi i jk / N); inverse: + sign, no 1/N.  buf (NV
+// buffers of NF PADN elements) must be free on entry; the caller
+// synchronises before it uses buf again.
+template <int LOGN, int NF, int NV, int E>
+__device__ __forceinline__ void fft_regs(float2 (&v)[NV][E], float2* buf, int lt, int t0, int tl,
+                                         int f, bool inv) {
+    using L = Lay<LOGN, NF>;
+    constexpr int R0 = L::R0;
+    if constexpr (R0 == 1) {
+#pragma unroll
+        for (int a = 0; a < NV; ++a) dft_full<E>(v[a], inv);
+        if constexpr (L::N > E) {
+#pragma unroll
+            for (int a = 0; a < NV; ++a)
+#pragma unroll
+                for (int r = 0; r < E; ++r)
+                    buf[a * (NF * L::PADN) + pad_stage<E, 1>(E * t0 + r) * NF + f] = v[a][r];
+            fft_stages<LOGN, NF, NV, E, 1>(v, buf, lt, tl, f, inv);
+        }
+    } else {
+        constexpr int C = E / R0;   // butterflies per thread: j = t0 + Q i, inputs v[i + C r]
+#pragma unroll
+        for (int a = 0; a < NV; ++a) {
+#pragma unroll
+            for (int i = 0; i < C; ++i) {
+                float2* x = v[a] + i;
+                if constexpr (R0 == 2) dft2(x[0], x[C]);
+                else if constexpr (R0 == 4) dft4(x[0], x[C], x[2 * C], x[3 * C], inv);
+                else dft8<C>(x, inv);
+            }
+#pragma unroll
+            for (int q = 0; q < E; ++q) {
+                const int o = (t0 + L::Q * (q % C)) * R0 + q / C;
+                buf[a * (NF * L::PADN) + pad_first<L::LQ>(o) * NF + f] = v[a][q];
+            }
+        }
+        fft_stages<LOGN, NF, NV, R0, 0>(v, buf, lt, tl, f, inv);
+    }
+}
+
+// The two real spectra of a packed pair at u, from Z[u] and Z[n-u], times 2:
+// V_1 = Z[u] + conj Z[n-u], V_2 = (Z[u] - conj Z[n-u]) / i.
+__device__ __forceinline__ void split_pair(float2 zu, float2 zn, float2* v1, float2* v2) {
+    *v1 = make_float2(zu.x + zn.x, zu.y - zn.y);
+    *v2 = make_float2(zu.y + zn.y, zn.x - zu.x);
+}
 
 // Spectrum of an inverse-cosine pair packed for one complex IFFT.  For the
 // sums y1 = sum c1[u] C(u,.), y2 = sum c2[u] C(u,.), with ct[0] = c[0],
@@ -251,54 +476,68 @@ __device__ __forceinline__ float2 pack_inv(float c1u, float c1nu, float c2u, flo
     return make_float2(re * ph.x + im * ph.y, im * ph.x - re * ph.y);
 }
 
+// Position of sample x in Makhoul's reordering.
+__device__ __forceinline__ int mk_pos(int x, int N) { return (x & 1) ? (N - 1 - (x >> 1)) : (x >> 1); }
+// Sample of the natural order held at position k of the reordering.
+__device__ __forceinline__ int mk_src(int y, int N) { return (y & 1) ? (N - 1 - (y >> 1)) : (y >> 1); }
+
+// A group's finished tile [N/2][8 floats] to columns c0 .. c0+7 of a
+// transposed map of N/2 rows of 2N floats: one thread through the TMA unit,
+// or every thread of the group with plain stores.
+template <int LOGN>
+__device__ __forceinline__ void store_tile(const float4* tile, float* dst, const CUtensorMap* map,
+                                           int c0, int lt, int nthreads, bool tma) {
+    constexpr int N = 1 << LOGN, ROWS = N / 2, BOX = ROWS < 256 ? ROWS : 256;
+    if (tma) {
+        if (lt == 0)
+            for (int b = 0; b < ROWS / BOX; ++b) tma_store_2d(map, tile + 2 * b * BOX, c0, b * BOX);
+    } else {
+        for (int i = lt; i < 2 * ROWS; i += nthreads)
+            *reinterpret_cast<float4*>(dst + (size_t)(i >> 1) * (2 * N) + c0 + 4 * (i & 1)) = tile[i];
+    }
+}
+
 // -------------------------------------------------------- pass 1: rows
-// CTA: 8 rows of rho (2 per complex buffer).  Writes T1[u][y0..y0+7].
-// At most 96 registers below n = 4096 (it needs no more): two blocks leave
-// room on the SM for a block of the concurrent WA kernel (measured 2 %
-// faster steps than with 128).  At n = 4096 the four buffers (139 KB) allow
-// one block per SM in every pass, which may then use all its registers
-// instead of spilling.
+// Group: 4 rows y0 .. y0+3 of rho (2 per complex FFT) -> T1[u/2][y0..y0+3].
 template <int LOGN, bool QUANT>
-__global__ void __maxnreg__(LOGN >= 12 ? 255 : 96)
+__global__ void __launch_bounds__(Lay<LOGN, 2>::T, spec_blocks(LOGN, Lay<LOGN, 2>::T))
 k_rows_fwd(const float* __restrict__ D, const long long* __restrict__ Dq,
            const float* __restrict__ M, float inv_ab, float cap, float* __restrict__ T1,
-           const float2* __restrict__ tw, const float2* __restrict__ ph, double* __restrict__ acc,
-           DetRed dr, const __grid_constant__ CUtensorMap mT1, int tma) {
-    constexpr int N = 1 << LOGN;
-    constexpr int NB = kSpecBuffers;
-    constexpr int ROWS = 2 * NB;
-    constexpr int T = kSpecThreads;
-    constexpr int NP = padded(N);
-    extern __shared__ __align__(128) float2 sm[];
-    const int y0 = blockIdx.x * ROWS;
-    // per-thread sums of at most 8 n / 256 non-negative terms in float32
+           double* __restrict__ acc, DetRed dr, const __grid_constant__ CUtensorMap mT1, int tma) {
+    using L = Lay<LOGN, 2>;
+    constexpr int N = L::N, Q = L::Q, E = L::E;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int g = L::GB == 1 ? 0 : threadIdx.x / L::LT;
+    const int lt = L::GB == 1 ? threadIdx.x : threadIdx.x % L::LT;
+    const int gi = blockIdx.x * L::GB + g, f = lt & 1;
+    const bool live = gi < N / 4;
+    const int y0 = 4 * (live ? gi : N / 4 - 1);
+    float2* buf = reinterpret_cast<float2*>(smem + g * L::group_bytes(1));
+    if (smem_addr(smem) & 127u) tma = 0;   // the TMA unit's source alignment
+    int pa, pb;
+    const int ta = lane_rev<LOGN, 2>(lt, &pa);
+    // per-thread sums of 2 E non-negative terms in float32
     float tau = 0.0f, charge = 0.0f;
-    // Buffer f packs rows 2f (real part) and 2f+1 (imaginary part) in
-    // Makhoul's order: item p reads samples 2p and 2p+1 of both rows
-    // (8-byte loads, a warp reads 256 contiguous bytes of each row) and
-    // writes positions p and N-1-p (consecutive across the warp: no bank
-    // conflicts)
-    constexpr int ITEMS_IN = NB * (N / 2);
-#pragma unroll 4
-    for (int it = 0; it < (ITEMS_IN + T - 1) / T; ++it) {
-        const int q = threadIdx.x + it * T;
-        if (ITEMS_IN % T != 0 && q >= ITEMS_IN) break;
-        const int f = q / (N / 2), pp = q % (N / 2);
-        const size_t b0 = (size_t)(y0 + 2 * f) * N + 2 * pp, b1 = b0 + N;
+    float2 v[1][E];
+#pragma unroll
+    for (int q = 0; q < E / 2; ++q) {
+        // samples 2p and 2p+1 of both rows: elements p and N-1-p
+        const int p = ta + Q * q;
+        const size_t b0 = (size_t)(y0 + 2 * f) * N + 2 * p, b1 = b0 + N;
         float d[4], mm[4];
-        const float2 m0 = *reinterpret_cast<const float2*>(M + b0);
-        const float2 m1 = *reinterpret_cast<const float2*>(M + b1);
+        const float2 m0 = __ldg(reinterpret_cast<const float2*>(M + b0));
+        const float2 m1 = __ldg(reinterpret_cast<const float2*>(M + b1));
         mm[0] = m0.x; mm[1] = m0.y; mm[2] = m1.x; mm[3] = m1.y;
         if (QUANT) {
-            const longlong2 q0 = *reinterpret_cast<const longlong2*>(Dq + b0);
-            const longlong2 q1 = *reinterpret_cast<const longlong2*>(Dq + b1);
+            const longlong2 q0 = __ldg(reinterpret_cast<const longlong2*>(Dq + b0));
+            const longlong2 q1 = __ldg(reinterpret_cast<const longlong2*>(Dq + b1));
             d[0] = (float)q0.x * 2.3283064365386963e-10f;
             d[1] = (float)q0.y * 2.3283064365386963e-10f;
             d[2] = (float)q1.x * 2.3283064365386963e-10f;
             d[3] = (float)q1.y * 2.3283064365386963e-10f;
         } else {
-            const float2 v0 = *reinterpret_cast<const float2*>(D + b0);
-            const float2 v1 = *reinterpret_cast<const float2*>(D + b1);
+            const float2 v0 = __ldg(reinterpret_cast<const float2*>(D + b0));
+            const float2 v1 = __ldg(reinterpret_cast<const float2*>(D + b1));
             d[0] = v0.x; d[1] = v0.y; d[2] = v1.x; d[3] = v1.y;
         }
         float rv[4];
@@ -308,368 +547,264 @@ k_rows_fwd(const float* __restrict__ D, const long long* __restrict__ Dq,
             charge += d[t] + mm[t];
             rv[t] = (d[t] + mm[t]) * inv_ab;
         }
-        float2* buf = sm + f * NP;
-        buf[pidx(pp)] = make_float2(rv[0], rv[2]);
-        buf[pidx(N - 1 - pp)] = make_float2(rv[1], rv[3]);
+        v[0][q] = make_float2(rv[0], rv[2]);
+        v[0][E - 1 - q] = shfl2(make_float2(rv[1], rv[3]), pa);
     }
-    reduce2(tau, charge, acc, ACC_TAU, ACC_CHARGE, dr);
-    __syncthreads();
-    fft_block<LOGN, NB>(sm, tw, false);
-    // split the packed spectra and apply the post-twiddle:
-    // A_j[u] = Re(ph[u] V_j[u]), V_1 = (Z[u] + conj Z[N-u]) / 2,
-    // V_2 = (Z[u] - conj Z[N-u]) / 2i.
-    constexpr int HALF = N / 2 + 1;
-    constexpr int ITEMS = NB * HALF;
-    constexpr int PI = (ITEMS + T - 1) / T;
-    float out[PI][4];
-    int where[PI];
+    const int k = lane_neg<LOGN, 2>(lt, &pb);
+    fft_regs<LOGN, 2, 1>(v, buf, lt, ta, k, f, false);
+    group_sync<LOGN, 2>();   // the tile replaces the exchange buffer
+    // split the packed spectra and apply the post-twiddle: A_j[u] = Re(ph[u] V_j[u])
+    float* tile = reinterpret_cast<float*>(buf);
 #pragma unroll
-    for (int i = 0; i < PI; ++i) {
-        int gi = threadIdx.x + i * T;
-        where[i] = -1;
-        if (gi < ITEMS) {
-            int f = gi / HALF, u = gi % HALF;
-            float2 zu = sm[f * NP + pidx(u)];
-            float2 zn = sm[f * NP + pidx((N - u) & (N - 1))];
-            float2 v1 = make_float2(0.5f * (zu.x + zn.x), 0.5f * (zu.y - zn.y));
-            float2 v2 = make_float2(0.5f * (zu.y + zn.y), 0.5f * (zn.x - zu.x));
-            float2 p = ph[u];
-            out[i][0] = v1.x * p.x - v1.y * p.y;   // A1[u]
-            out[i][1] = v2.x * p.x - v2.y * p.y;   // A2[u]
-            // at N-u the spectra are conjugated
-            float2 q = ph[N - u];
-            out[i][2] = v1.x * q.x + v1.y * q.y;   // A1[N-u]
-            out[i][3] = v2.x * q.x + v2.y * q.y;   // A2[N-u]
-            where[i] = f * HALF + u;
-        }
+    for (int r = 0; r < E; ++r) {
+        float2 zn = shfl2(v[0][E - 1 - r], pb), v1, v2;
+        if (k == 0) zn = v[0][(E - r) & (E - 1)];
+        split_pair(v[0][r], zn, &v1, &v2);
+        const float2 p = phase<N>(k + Q * r);
+        const int u = k + Q * r;
+        float* dst = tile + (u >> 1) * 8 + 4 * f + (u & 1);
+        dst[0] = 0.5f * (v1.x * p.x - v1.y * p.y);
+        dst[2] = 0.5f * (v2.x * p.x - v2.y * p.y);
     }
-    __syncthreads();
-    float* sf = reinterpret_cast<float*>(sm);
-#pragma unroll
-    for (int i = 0; i < PI; ++i) {
-        if (where[i] < 0) continue;
-        int f = where[i] / HALF, u = where[i] % HALF;
-        float* r1 = sf + (2 * f) * N;
-        float* r2 = sf + (2 * f + 1) * N;
-        r1[u & (N - 1)] = out[i][0];
-        r2[u & (N - 1)] = out[i][1];
-        if (u > 0 && u < N / 2) {
-            r1[N - u] = out[i][2];
-            r2[N - u] = out[i][3];
-        }
-    }
-    __syncthreads();
-    // transposed write: T1[u][y0 .. y0+7]
-    if (tma && (smem_addr(sm) & 127u) == 0) {
-        // the eight values of each u go through registers into the tile
-        // [u][8] (which replaces the rows), stored in boxes of BOX values of u
-        constexpr int CNT = (N + T - 1) / T;
-        constexpr int BOX = N < 256 ? N : 256;
-        float4 va[CNT], vb[CNT];
-#pragma unroll
-        for (int k = 0; k < CNT; ++k) {
-            const int u = threadIdx.x + k * T;
-            if (N % T == 0 || u < N) {
-                va[k] = make_float4(sf[0 * N + u], sf[1 * N + u], sf[2 * N + u], sf[3 * N + u]);
-                vb[k] = make_float4(sf[4 * N + u], sf[5 * N + u], sf[6 * N + u], sf[7 * N + u]);
-            }
-        }
-        __syncthreads();
-        float4* tile = reinterpret_cast<float4*>(sm);
-#pragma unroll
-        for (int k = 0; k < CNT; ++k) {
-            const int u = threadIdx.x + k * T;
-            if (N % T == 0 || u < N) {
-                tile[2 * u] = va[k];
-                tile[2 * u + 1] = vb[k];
-            }
-        }
-        fence_async_smem();
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int b = 0; b < N / BOX; ++b) tma_store_2d(&mT1, tile + 2 * b * BOX, y0, b * BOX);
-            tma_store_drain();
-        }
-        return;
-    }
-    for (int u = threadIdx.x; u < N; u += T) {
-        float4 a = make_float4(sf[0 * N + u], sf[1 * N + u], sf[2 * N + u], sf[3 * N + u]);
-        float4 b = make_float4(sf[4 * N + u], sf[5 * N + u], sf[6 * N + u], sf[7 * N + u]);
-        float4* dst = reinterpret_cast<float4*>(T1 + (size_t)u * N + y0);
-        dst[0] = a;
-        dst[1] = b;
-    }
+    if (tma) fence_async_smem();
+    group_sync<LOGN, 2>();
+    if (live) store_tile<LOGN>(reinterpret_cast<const float4*>(tile), T1, &mT1, 2 * y0, lt, L::LT, tma);
+    reduce2(live ? tau : 0.0f, live ? charge : 0.0f, acc, ACC_TAU, ACC_CHARGE, dr);
+    if (tma && live && lt == 0) tma_store_drain();
 }
 
 // ------------------------------------------------- pass 2: columns
-// CTA: 4 rows u of T1.  Forward DCT-II along y, spectral divide, energy,
-// then the inverse sums along y: P (cosine sum of Psi) and R (sine sum of
-// w_v Psi, via reversed coefficients).  Each complex IFFT carries the same
+// One spectral element of two rows (u, u+1) at v: from Z[v] and Z[n-v] the
+// DCT-II values, the divide, the energy terms and the packed inputs of the
+// inverse sums P (cosine sum of Psi) and R (sine sum of w_v Psi as a cosine
+// sum of c2[v'] = s[N-v'], s[v] = w_v Psi[v], c2[0] = 0).
+struct SpecRow {
+    float w2a, w2b;   // w_u^2 + eps of the two rows
+    float ha, hb;     // eps_u / 2n^2
+    bool drop;        // row u = 0 without the Helmholtz term: the (0,0) mode dropped
+};
+
+__device__ __forceinline__ void spectral_elem(float2 zu, float2 zn, float2 p, float wv, float wn,
+                                              bool v0, const SpecRow& s, float2* zp, float2* zr,
+                                              dfloat* energy) {
+    float2 v1, v2;
+    split_pair(zu, zn, &v1, &v2);
+    // ph[n-v] = -i conj(ph[v]): both values of a pair from one product
+    const float2 wa = cmul(p, v1), wb = cmul(p, v2);
+    const float ba = wa.x, bna = -wa.y, bb = wb.x, bnb = -wb.y;   // twice B
+    // the divisors are at least (pi/L)^2 > 0 (or eps): the fast divide (2 ulp)
+    // stays far inside the transform's bound
+    const float wv2 = wv * wv, wn2 = wn * wn;
+    float ca = __fdividef(s.ha * ba, wv2 + s.w2a);
+    const float cb = __fdividef(s.hb * bb, wv2 + s.w2b);
+    float na = __fdividef(s.ha * bna, wn2 + s.w2a);
+    float nb = __fdividef(s.hb * bnb, wn2 + s.w2b);
+    if (v0) {
+        if (s.drop) ca = 0.0f;   // Poisson: no (0,0) mode
+        na = 0.0f;
+        nb = 0.0f;
+    }
+    // B Psi: Psi = 2 ct but at v = 0 (ct = Psi); B is half of ba
+    const float e = fmaf(ba, ca, bb * cb);
+    *energy = df_add(*energy, v0 ? 0.5f * e : e);
+    *zp = pack_inv(ca, na, cb, nb, p);
+    *zr = pack_inv(wn * na, wv * ca, wn * nb, wv * cb, p);
+}
+
+// Group: 4 rows u0 .. u0+3 of T1.  Forward DCT-II along y, spectral divide,
+// energy, then the inverse sums along y.  Each complex IFFT carries the same
 // quantity for two rows (P with P, R with R), so both parts share a scale.
+// The forward FFT ends in each thread with the elements its inverse FFTs
+// begin with, so the spectrum never leaves the registers.
 template <int LOGN>
-__global__ void __launch_bounds__(kSpecThreads, LOGN >= 12 ? 1 : 2)
-k_cols(const float* __restrict__ T1, float* __restrict__ PT, float* __restrict__ RT,
-       const float2* __restrict__ tw, const float2* __restrict__ ph, float pi_lx, float pi_ly,
-       float eps, double* __restrict__ acc, DetRed dr, const __grid_constant__ CUtensorMap mPT,
-       const __grid_constant__ CUtensorMap mRT, int tma) {
-    constexpr int N = 1 << LOGN;
-    constexpr int NB = kSpecBuffers;
-    constexpr int ROWS = NB;
-    constexpr int T = kSpecThreads;
-    constexpr int NP = padded(N);
-    extern __shared__ __align__(128) float2 sm[];
-    const int u0 = blockIdx.x * ROWS;
-    // buffer f packs rows 2f, 2f+1 in Makhoul's order (as in k_rows_fwd)
-    constexpr int ITEMS_IN = (ROWS / 2) * (N / 2);
-#pragma unroll 4
-    for (int it = 0; it < (ITEMS_IN + T - 1) / T; ++it) {
-        const int q = threadIdx.x + it * T;
-        if (ITEMS_IN % T != 0 && q >= ITEMS_IN) break;
-        const int f = q / (N / 2), pp = q % (N / 2);
-        const size_t b0 = (size_t)(u0 + 2 * f) * N + 2 * pp;
-        const float2 a = *reinterpret_cast<const float2*>(T1 + b0);
-        const float2 c = *reinterpret_cast<const float2*>(T1 + b0 + N);
-        float2* buf = sm + f * NP;
-        buf[pidx(pp)] = make_float2(a.x, c.x);
-        buf[pidx(N - 1 - pp)] = make_float2(a.y, c.y);
-    }
-    __syncthreads();
-    fft_block<LOGN, NB / 2>(sm, tw, false);
-    constexpr int HALF = N / 2 + 1;
-    constexpr int ITEMS = (NB / 2) * HALF;
-    constexpr int PI = (ITEMS + T - 1) / T;
-    float2 zo[PI][4];   // [P at v, P at N-v, R at v, R at N-v], rows packed re/im
-    int where[PI];
-    const float invn2 = 1.0f / ((float)N * (float)N);
+__global__ void __launch_bounds__(Lay<LOGN, 2>::T, spec_blocks(LOGN, Lay<LOGN, 2>::T))
+k_cols(const float* __restrict__ T1, float* __restrict__ PT, float* __restrict__ RT, float pi_lx,
+       float pi_ly, float eps, double* __restrict__ acc, DetRed dr,
+       const __grid_constant__ CUtensorMap mPT, const __grid_constant__ CUtensorMap mRT, int tma) {
+    using L = Lay<LOGN, 2>;
+    constexpr int N = L::N, Q = L::Q, E = L::E;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int g = L::GB == 1 ? 0 : threadIdx.x / L::LT;
+    const int lt = L::GB == 1 ? threadIdx.x : threadIdx.x % L::LT;
+    const int gi = blockIdx.x * L::GB + g, f = lt & 1;
+    const bool live = gi < N / 4;
+    const int u0 = 4 * (live ? gi : N / 4 - 1);
+    float2* buf = reinterpret_cast<float2*>(smem + g * L::group_bytes(2));
+    if (smem_addr(smem) & 127u) tma = 0;
+    int pa, pb;
+    const int ta = lane_rev<LOGN, 2>(lt, &pa);
+    float2 z[2][E];
     dfloat energy = df_zero();
+    int k;
+    {
+        float2 v[1][E];
+        const float4* row = reinterpret_cast<const float4*>(T1 + (size_t)(u0 / 2 + f) * (2 * N));
 #pragma unroll
-    for (int i = 0; i < PI; ++i) {
-        int gi = threadIdx.x + i * T;
-        where[i] = -1;
-        if (gi < ITEMS) {
-            int f = gi / HALF, v = gi % HALF;
-            int vn = (N - v) & (N - 1);
-            float2 zu = sm[f * NP + pidx(v)];
-            float2 zn = sm[f * NP + pidx(vn)];
-            float2 v1 = make_float2(0.5f * (zu.x + zn.x), 0.5f * (zu.y - zn.y));
-            float2 v2 = make_float2(0.5f * (zu.y + zn.y), 0.5f * (zn.x - zu.x));
-            float2 p = ph[v], q = ph[N - v];
-            // B[row][v], B[row][N-v] (unnormalised DCT-II along y)
-            float B[2][2];
-            B[0][0] = v1.x * p.x - v1.y * p.y;
-            B[1][0] = v2.x * p.x - v2.y * p.y;
-            B[0][1] = v1.x * q.x + v1.y * q.y;
-            B[1][1] = v2.x * q.x + v2.y * q.y;
-            float wv = pi_ly * (float)v, wvn = pi_ly * (float)(N - v);
-            float ev = (v == 0) ? 1.0f : 2.0f;
-            bool has_n = (v > 0 && v < N / 2);
-            // halved inverse coefficients per row: c1 (P) and c2 (R) at v and N-v
-            float c1v[2], c1n[2], c2v[2], c2n[2];
+        for (int q = 0; q < E / 2; ++q) {
+            const float4 a = __ldg(row + ta + Q * q);   // samples 2p, 2p+1 of both rows
+            v[0][q] = make_float2(a.x, a.y);
+            v[0][E - 1 - q] = make_float2(a.z, a.w);
+        }
 #pragma unroll
-            for (int rr = 0; rr < 2; ++rr) {
-                int u = u0 + 2 * f + rr;
-                float wu = pi_lx * (float)u;
-                float eu = (u == 0) ? 1.0f : 2.0f;
-                float a0 = eu * ev * invn2 * B[rr][0];
-                // Poisson: (0,0) mode dropped; Helmholtz (eps > 0): divisor
-                // w^2 + eps and the (0,0) mode kept
-                // the divisor is at least (pi/L)^2 > 0 (or eps): the fast
-                // divide (2 ulp) stays far inside the transform's bound
-                float psi0 = (u == 0 && v == 0 && !(eps > 0.0f))
-                                 ? 0.0f
-                                 : __fdividef(a0, wu * wu + wv * wv + eps);
-                float psin = 0.0f;
-                if (has_n) {
-                    float an = eu * 2.0f * invn2 * B[rr][1];
-                    psin = __fdividef(an, wu * wu + wvn * wvn + eps);
-                    energy = df_add(energy, B[rr][1] * psin);
-                }
-                energy = df_add(energy, B[rr][0] * psi0);
-                // P: cosine sum of Psi.  R: cosine sum of c2[v'] = s[N-v'],
-                // s[v] = w_v Psi[v], c2[0] = 0; then R = (-1)^y * that.
-                c1v[rr] = (v == 0) ? psi0 : 0.5f * psi0;
-                c1n[rr] = 0.5f * psin;
-                c2v[rr] = (v == 0) ? 0.0f : 0.5f * wvn * psin;
-                c2n[rr] = (v == 0) ? 0.0f : 0.5f * wv * psi0;
-                if (v == N / 2) {
-                    c1n[rr] = c1v[rr];
-                    c2v[rr] = 0.5f * wv * psi0;
-                    c2n[rr] = c2v[rr];
-                }
+        for (int q = E / 2; q < E; ++q) v[0][q] = shfl2(v[0][q], pa);
+        k = lane_neg<LOGN, 2>(lt, &pb);
+        fft_regs<LOGN, 2, 1>(v, buf, lt, ta, k, f, false);
+        SpecRow s;
+        const int u = u0 + 2 * f;
+        const float wa = pi_lx * (float)u, wb = pi_lx * (float)(u + 1);
+        const float invn2 = 1.0f / ((float)N * (float)N);
+        s.w2a = fmaf(wa, wa, eps);
+        s.w2b = fmaf(wb, wb, eps);
+        s.ha = (u == 0 ? 0.5f : 1.0f) * invn2;
+        s.hb = invn2;
+        s.drop = u == 0 && !(eps > 0.0f);
+        const float kf = (float)k;
+        // pairs (r, E - 1 - r): each needs the other's element of the partner
+        // (element E - r of the own thread at k = 0)
+        float2 hi = v[0][0];
+#pragma unroll
+        for (int r = 0; r < E / 2; ++r) {
+            const float2 a = v[0][r], b = v[0][E - 1 - r];
+            float2 na = shfl2(b, pb), nb = shfl2(a, pb);
+            if (k == 0) {
+                na = hi;
+                nb = v[0][r + 1];
             }
-            zo[i][0] = pack_inv(c1v[0], c1n[0], c1v[1], c1n[1], p);
-            zo[i][1] = pack_inv(c1n[0], c1v[0], c1n[1], c1v[1], q);
-            zo[i][2] = pack_inv(c2v[0], c2n[0], c2v[1], c2n[1], p);
-            zo[i][3] = pack_inv(c2n[0], c2v[0], c2n[1], c2v[1], q);
-            where[i] = f * HALF + v;
+            hi = b;
+            const float va = kf + (float)(Q * r), vb = kf + (float)(Q * (E - 1 - r));
+            spectral_elem(a, na, phase<N>(k + Q * r), pi_ly * va, pi_ly * ((float)N - va),
+                          r == 0 && k == 0, s, &z[0][r], &z[1][r], &energy);
+            spectral_elem(b, nb, phase<N>(k + Q * (E - 1 - r)), pi_ly * vb, pi_ly * ((float)N - vb), false,
+                          s, &z[0][E - 1 - r], &z[1][E - 1 - r], &energy);
         }
     }
-    reduce2(df_val(energy), 0.0f, acc, ACC_N, -1, dr);
-    __syncthreads();
+    group_sync<LOGN, 2>();   // the forward exchange has been read
+    fft_regs<LOGN, 2, 2>(z, buf, lt, k, ta, f, true);
+    group_sync<LOGN, 2>();   // the tiles replace the exchange buffers
+    // unshuffle: y = 2o <- element o, y = 2o+1 <- element N-1-o; R times (-1)^y
+    float4* tP = reinterpret_cast<float4*>(buf);
+    float4* tR = tP + N;
 #pragma unroll
-    for (int i = 0; i < PI; ++i) {
-        if (where[i] < 0) continue;
-        int f = where[i] / HALF, v = where[i] % HALF;
-        float2* rowP = sm + (2 * f) * NP;
-        float2* rowR = sm + (2 * f + 1) * NP;
-        rowP[pidx(v & (N - 1))] = zo[i][0];
-        rowR[pidx(v & (N - 1))] = zo[i][2];
-        if (v > 0 && v < N / 2) {
-            rowP[pidx(N - v)] = zo[i][1];
-            rowR[pidx(N - v)] = zo[i][3];
-        }
+    for (int q = 0; q < E / 2; ++q) {
+        const int o = ta + Q * q;
+        const float2 p0 = z[0][q], p1 = shfl2(z[0][E - 1 - q], pa);
+        const float2 r0 = z[1][q], r1 = shfl2(z[1][E - 1 - q], pa);
+        tP[2 * o + f] = make_float4(p0.x, p1.x, p0.y, p1.y);
+        tR[2 * o + f] = make_float4(r0.x, -r1.x, r0.y, -r1.y);
     }
-    __syncthreads();
-    fft_block<LOGN, NB>(sm, tw, true);
-    // unshuffle: y even <- k = y/2, y odd <- k = N-1-(y-1)/2
-    if (tma && (smem_addr(sm) & 127u) == 0) {
-        // through registers into the tiles PT[y][u0..u0+3] and RT[y][...]
-        // (16 bytes per y, in place of the buffers), stored in boxes of BOX y
-        constexpr int CNT = (N + T - 1) / T;
-        constexpr int BOX = N < 256 ? N : 256;
-        float4 pv[CNT], rv[CNT];
-#pragma unroll
-        for (int k = 0; k < CNT; ++k) {
-            const int y = threadIdx.x + k * T;
-            if (N % T == 0 || y < N) {
-                const int q = pidx(mk_src(y, N));
-                const float sgn = (y & 1) ? -1.0f : 1.0f;
-                const float2 p0 = sm[0 * NP + q], r0 = sm[1 * NP + q];
-                const float2 p1 = sm[2 * NP + q], r1 = sm[3 * NP + q];
-                pv[k] = make_float4(p0.x, p0.y, p1.x, p1.y);
-                rv[k] = make_float4(sgn * r0.x, sgn * r0.y, sgn * r1.x, sgn * r1.y);
-            }
-        }
-        __syncthreads();
-        float4* tP = reinterpret_cast<float4*>(sm);
-        float4* tR = tP + N;
-#pragma unroll
-        for (int k = 0; k < CNT; ++k) {
-            const int y = threadIdx.x + k * T;
-            if (N % T == 0 || y < N) {
-                tP[y] = pv[k];
-                tR[y] = rv[k];
-            }
-        }
-        fence_async_smem();
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int b = 0; b < N / BOX; ++b) {
-                tma_store_2d(&mPT, tP + b * BOX, u0, b * BOX);
-                tma_store_2d(&mRT, tR + b * BOX, u0, b * BOX);
-            }
-            tma_store_drain();
-        }
-        return;
+    if (tma) fence_async_smem();
+    group_sync<LOGN, 2>();
+    if (live) {
+        store_tile<LOGN>(tP, PT, &mPT, 2 * u0, lt, L::LT, tma);
+        store_tile<LOGN>(tR, RT, &mRT, 2 * u0, lt, L::LT, tma);
     }
-    for (int y = threadIdx.x; y < N; y += T) {
-        int k = pidx(mk_src(y, N));
-        float sgn = (y & 1) ? -1.0f : 1.0f;
-        float2 p0 = sm[0 * NP + k], r0 = sm[1 * NP + k], p1 = sm[2 * NP + k], r1 = sm[3 * NP + k];
-        *reinterpret_cast<float4*>(PT + (size_t)y * N + u0) = make_float4(p0.x, p0.y, p1.x, p1.y);
-        *reinterpret_cast<float4*>(RT + (size_t)y * N + u0) =
-            make_float4(sgn * r0.x, sgn * r0.y, sgn * r1.x, sgn * r1.y);
-    }
+    reduce2(live ? df_val(energy) : 0.0f, 0.0f, acc, ACC_N, -1, dr);
+    if (tma && live && lt == 0) tma_store_drain();
 }
 
 // ------------------------------------------------- pass 3: inverse rows
-// CTA: 4 rows y, one round of four inverse FFTs: buffers 0 and 1 hold E_x
-// (the sine sum of w_u P, via reversed coefficients: c[u'] = s[N-u'],
-// u' >= 1, c[0] = 0, s[u] = w_u P[u]; E_x[x] = (-1)^x cosine-sum(c)[x]) for
-// rows (0, 1) and (2, 3); buffers 2 and 3 hold E_y (the cosine sum of R).
-// Written as the interleaved field map E2[y][x] = (E_x, E_y).  The potential
-// psi (the cosine sum of P) is not needed by the evaluation (the energy comes
-// from the column pass by Parseval) and is formed on demand by k_rows_psi.
-template <int LOGN>
-__global__ void __launch_bounds__(kSpecThreads, LOGN >= 12 ? 1 : 2)
-k_rows_inv(const float* __restrict__ PT, const float* __restrict__ RT, float2* __restrict__ E2,
-           const float2* __restrict__ tw, const float2* __restrict__ ph, float pi_lx) {
-    constexpr int N = 1 << LOGN;
-    constexpr int NB = kSpecBuffers;
-    constexpr int ROWS = NB;
-    constexpr int T = kSpecThreads;
-    constexpr int HALF = N / 2 + 1;
-    constexpr int NP = padded(N);
-    extern __shared__ __align__(128) float2 sm[];
-    const int y0 = blockIdx.x * ROWS;
-#pragma unroll 2
-    for (int idx = threadIdx.x; idx < (ROWS / 2) * HALF; idx += T) {
-        int f = idx / HALF, u = idx % HALF;
-        int un = (N - u) & (N - 1);
-        // E_y: cosine sums of the R rows (2f, 2f+1)
-        {
-            const float* A = RT + (size_t)(y0 + 2 * f) * N;
-            const float* Bq = A + N;
-            float au = A[u & (N - 1)], bu = Bq[u & (N - 1)];
-            float an = (u > 0) ? A[un] : 0.0f, bn = (u > 0) ? Bq[un] : 0.0f;
-            float cau = (u == 0) ? au : 0.5f * au, cbu = (u == 0) ? bu : 0.5f * bu;
-            float can = 0.5f * an, cbn = 0.5f * bn;
-            if (u == N / 2) { can = cau; cbn = cbu; }
-            float2* row = sm + (2 + f) * NP;
-            row[pidx(u & (N - 1))] = pack_inv(cau, can, cbu, cbn, ph[u]);
-            if (u > 0 && u < N / 2) row[pidx(N - u)] = pack_inv(can, cau, cbn, cbu, ph[N - u]);
+// Coefficients c[t + Q q] of two rows (re, im) and their partners, packed in
+// place for the inverse FFT: the cosine sum of c (SINE = false), or the
+// reversed coefficients w_u c of the sine sum (c'[u] = w_{N-u} c[N-u],
+// c'[0] = 0), whose cosine sum times (-1)^x is the sine sum.
+template <int LOGN, bool SINE>
+__device__ __forceinline__ void pack_rows(const float2 (&c)[spec_elems(LOGN)], float2* z, int k,
+                                          int pb, float pi_lx) {
+    constexpr int N = 1 << LOGN, E = spec_elems(LOGN), Q = N / E;
+    const float kf = (float)k;
+#pragma unroll
+    for (int r = 0; r < E; ++r) {
+        const float2 a = c[r];
+        float2 n = shfl2(c[E - 1 - r], pb);
+        if (k == 0) n = r == 0 ? make_float2(0.0f, 0.0f) : c[(E - r) & (E - 1)];
+        const float2 p = phase<N>(k + Q * r);
+        if (SINE) {
+            const float u = kf + (float)(Q * r);
+            const float wu = 0.5f * (pi_lx * u), wn = 0.5f * (pi_lx * ((float)N - u));
+            // u = 0: both coefficients vanish (n = 0 and w_0 = 0)
+            z[r] = pack_inv(wn * n.x, wu * a.x, wn * n.y, wu * a.y, p);
+        } else {
+            const float h = r == 0 && k == 0 ? 1.0f : 0.5f;   // c[0] is not halved
+            z[r] = pack_inv(h * a.x, 0.5f * n.x, h * a.y, 0.5f * n.y, p);
         }
-        // E_x: reversed sine coefficients of the P rows (2f, 2f+1)
-        {
-            const float* Pa = PT + (size_t)(y0 + 2 * f) * N;
-            const float* Pb = Pa + N;
-            float wu = pi_lx * (float)u, wn = pi_lx * (float)(N - u);
-            // c[u] = s[N-u] = w_{N-u} P[N-u]  (u >= 1);  c[N-u] = s[u] = w_u P[u]
-            float ca_u = (u == 0) ? 0.0f : 0.5f * wn * Pa[N - u];
-            float cb_u = (u == 0) ? 0.0f : 0.5f * wn * Pb[N - u];
-            float ca_n = (u == 0) ? 0.0f : 0.5f * wu * Pa[u];
-            float cb_n = (u == 0) ? 0.0f : 0.5f * wu * Pb[u];
-            if (u == N / 2) { ca_n = ca_u; cb_n = cb_u; }
-            float2* row = sm + f * NP;
-            row[pidx(u & (N - 1))] = pack_inv(ca_u, ca_n, cb_u, cb_n, ph[u]);
-            if (u > 0 && u < N / 2) row[pidx(N - u)] = pack_inv(ca_n, ca_u, cb_n, cb_u, ph[N - u]);
-        }
-    }
-    __syncthreads();
-    fft_block<LOGN, NB>(sm, tw, true);
-    for (int idx = threadIdx.x; idx < ROWS * N; idx += T) {
-        int r = idx >> LOGN, x = idx & (N - 1);
-        int k = pidx(mk_src(x, N));
-        float2 zx = sm[(r >> 1) * NP + k], zy = sm[(2 + (r >> 1)) * NP + k];
-        float vx = (r & 1) ? zx.y : zx.x, vy = (r & 1) ? zy.y : zy.x;
-        E2[(size_t)(y0 + r) * N + x] = make_float2((x & 1) ? -vx : vx, vy);
     }
 }
 
-// psi on demand: CTA of 4 rows y, the cosine sums of the P rows (2f, 2f+1)
-// in buffer f.
-template <int LOGN>
-__global__ void __launch_bounds__(kSpecThreads, LOGN >= 12 ? 1 : 2)
-k_rows_psi(const float* __restrict__ PT, float* __restrict__ psi, const float2* __restrict__ tw,
-           const float2* __restrict__ ph) {
-    constexpr int N = 1 << LOGN;
-    constexpr int ROWS = kSpecBuffers;
-    constexpr int NB = ROWS / 2;
-    constexpr int T = kSpecThreads;
-    constexpr int HALF = N / 2 + 1;
-    constexpr int NP = padded(N);
-    extern __shared__ __align__(128) float2 sm[];
-    const int y0 = blockIdx.x * ROWS;
-    for (int idx = threadIdx.x; idx < NB * HALF; idx += T) {
-        int f = idx / HALF, u = idx % HALF;
-        int un = (N - u) & (N - 1);
-        const float* A = PT + (size_t)(y0 + 2 * f) * N;
-        const float* Bq = A + N;
-        float au = A[u & (N - 1)], bu = Bq[u & (N - 1)];
-        float an = (u > 0) ? A[un] : 0.0f, bn = (u > 0) ? Bq[un] : 0.0f;
-        float cau = (u == 0) ? au : 0.5f * au, cbu = (u == 0) ? bu : 0.5f * bu;
-        float can = 0.5f * an, cbn = 0.5f * bn;
-        if (u == N / 2) { can = cau; cbn = cbu; }
-        float2* row = sm + f * NP;
-        row[pidx(u & (N - 1))] = pack_inv(cau, can, cbu, cbn, ph[u]);
-        if (u > 0 && u < N / 2) row[pidx(N - u)] = pack_inv(can, cau, cbn, cbu, ph[N - u]);
+// What an inverse-row pass writes: the interleaved field of the evaluation,
+// the potential alone (on demand), or the three separate maps of a solve.
+enum { INV_FIELD, INV_PSI, INV_MAPS };
+
+// Group: one pair of rows y, y+1.  E_x (the sine sum of w_u P) and E_y (the
+// cosine sum of R) in one round of two inverse FFTs; psi (the cosine sum of
+// P) is not needed by the evaluation (the energy comes from the column pass
+// by Parseval).
+template <int LOGN, int WHAT>
+__global__ void __launch_bounds__(Lay<LOGN, 1>::T, spec_blocks(LOGN, Lay<LOGN, 1>::T))
+k_rows_inv(const float* __restrict__ PT, const float* __restrict__ RT, float2* __restrict__ E2,
+           float* __restrict__ psi, float* __restrict__ ex, float* __restrict__ ey, float pi_lx) {
+    using L = Lay<LOGN, 1>;
+    constexpr int N = L::N, Q = L::Q, E = L::E;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int g = L::GB == 1 ? 0 : threadIdx.x / L::LT;
+    const int lt = L::GB == 1 ? threadIdx.x : threadIdx.x % L::LT;
+    const int gi = blockIdx.x * L::GB + g;
+    const bool live = gi < N / 2;
+    const int j = live ? gi : N / 2 - 1;
+    constexpr int NV = WHAT == INV_PSI ? 1 : 2;
+    float2* buf = reinterpret_cast<float2*>(smem + g * L::group_bytes(NV));
+    int pa, pb;
+    const int ta = lane_rev<LOGN, 1>(lt, &pa), k = lane_neg<LOGN, 1>(lt, &pb);
+    const float2* pr = reinterpret_cast<const float2*>(PT) + (size_t)j * N + k;
+    const float2* rr = reinterpret_cast<const float2*>(RT) + (size_t)j * N + k;
+    const size_t row0 = (size_t)(2 * j) * N, row1 = row0 + N;
+    if (WHAT != INV_PSI) {
+        float2 z[2][E];
+        {
+            float2 c[E], e[E];
+#pragma unroll
+            for (int q = 0; q < E; ++q) {
+                c[q] = __ldg(pr + Q * q);
+                e[q] = __ldg(rr + Q * q);
+            }
+            pack_rows<LOGN, true>(c, z[0], k, pb, pi_lx);
+            pack_rows<LOGN, false>(e, z[1], k, pb, pi_lx);
+        }
+        fft_regs<LOGN, 1, 2>(z, buf, lt, k, ta, 0, true);
+#pragma unroll
+        for (int q = 0; q < E / 2; ++q) {
+            const int o = ta + Q * q;   // samples 2o, 2o+1 of both rows
+            const float2 x0 = z[0][q], x1 = shfl2(z[0][E - 1 - q], pa);
+            const float2 e0 = z[1][q], e1 = shfl2(z[1][E - 1 - q], pa);
+            if (!live) continue;
+            if (WHAT == INV_FIELD) {
+                reinterpret_cast<float4*>(E2 + row0)[o] = make_float4(x0.x, e0.x, -x1.x, e1.x);
+                reinterpret_cast<float4*>(E2 + row1)[o] = make_float4(x0.y, e0.y, -x1.y, e1.y);
+            } else {
+                reinterpret_cast<float2*>(ex + row0)[o] = make_float2(x0.x, -x1.x);
+                reinterpret_cast<float2*>(ex + row1)[o] = make_float2(x0.y, -x1.y);
+                reinterpret_cast<float2*>(ey + row0)[o] = make_float2(e0.x, e1.x);
+                reinterpret_cast<float2*>(ey + row1)[o] = make_float2(e0.y, e1.y);
+            }
+        }
     }
-    __syncthreads();
-    fft_block<LOGN, NB>(sm, tw, true);
-    for (int idx = threadIdx.x; idx < ROWS * N; idx += T) {
-        int r = idx >> LOGN, x = idx & (N - 1);
-        float2 z = sm[(r >> 1) * NP + pidx(mk_src(x, N))];
-        psi[(size_t)(y0 + r) * N + x] = (r & 1) ? z.y : z.x;
+    if (WHAT != INV_FIELD) {
+        float2 z[1][E];
+        {
+            float2 c[E];
+#pragma unroll
+            for (int q = 0; q < E; ++q) c[q] = __ldg(pr + Q * q);
+            pack_rows<LOGN, false>(c, z[0], k, pb, pi_lx);
+        }
+        if (WHAT == INV_MAPS) group_sync<LOGN, 1>();   // the field's exchange has been read
+        fft_regs<LOGN, 1, 1>(z, buf, lt, k, ta, 0, true);
+#pragma unroll
+        for (int q = 0; q < E / 2; ++q) {
+            const int o = ta + Q * q;
+            const float2 s0 = z[0][q], s1 = shfl2(z[0][E - 1 - q], pa);
+            if (!live) continue;
+            reinterpret_cast<float2*>(psi + row0)[o] = make_float2(s0.x, s1.x);
+            reinterpret_cast<float2*>(psi + row1)[o] = make_float2(s0.y, s1.y);
+        }
     }
 }
 
@@ -841,31 +976,26 @@ k_tcr_spectral(int n, int rows2, const float2* __restrict__ V, const float2* __r
 }
 
 // Inverse outputs of the column pass: pair r of P (V[r]) and of R
-// (V[rows2 + r]) unshuffled (y <- position mk_src(y); R times (-1)^y) and
-// written transposed, PT[y][8 g .. 8 g + 7], RT likewise.
+// (V[rows2 + r]) unshuffled (y = 2j <- position j, y = 2j+1 <- n-1-j; R times
+// (-1)^y) and written transposed, PT[j][8 g .. 8 g + 7] (two rows y
+// interleaved), RT likewise.
 __global__ void __launch_bounds__(256)
 k_tcr_post_cols(int n, int rows2, const float2* __restrict__ V, float* __restrict__ PT,
                 float* __restrict__ RT) {
-    const int groups = rows2 / 4;
+    const int groups = rows2 / 4, half = n / 2;
     const long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (q >= (long long)groups * n) return;
-    const int g = (int)(q / n), y = (int)(q % n);
-    const int k = mk_src(y, n);
-    const float sgn = (y & 1) ? -1.0f : 1.0f;
-    float p[8], rr[8];
+    if (q >= (long long)groups * half) return;
+    const int g = (int)(q / half), j = (int)(q % half);
+    float4* dp = reinterpret_cast<float4*>(PT + (size_t)j * 2 * n + 16 * g);
+    float4* dr4 = reinterpret_cast<float4*>(RT + (size_t)j * 2 * n + 16 * g);
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
-        const float2 zp = V[(size_t)(4 * g + t) * n + k];
-        const float2 zr = V[(size_t)(rows2 + 4 * g + t) * n + k];
-        p[2 * t] = zp.x; p[2 * t + 1] = zp.y;
-        rr[2 * t] = sgn * zr.x; rr[2 * t + 1] = sgn * zr.y;
+        const float2* zp = V + (size_t)(4 * g + t) * n;
+        const float2* zr = V + (size_t)(rows2 + 4 * g + t) * n;
+        const float2 p0 = zp[j], p1 = zp[n - 1 - j], r0 = zr[j], r1 = zr[n - 1 - j];
+        dp[t] = make_float4(p0.x, p1.x, p0.y, p1.y);
+        dr4[t] = make_float4(r0.x, -r1.x, r0.y, -r1.y);
     }
-    float4* dp = reinterpret_cast<float4*>(PT + (size_t)y * n + 8 * g);
-    float4* dr4 = reinterpret_cast<float4*>(RT + (size_t)y * n + 8 * g);
-    dp[0] = make_float4(p[0], p[1], p[2], p[3]);
-    dp[1] = make_float4(p[4], p[5], p[6], p[7]);
-    dr4[0] = make_float4(rr[0], rr[1], rr[2], rr[3]);
-    dr4[1] = make_float4(rr[4], rr[5], rr[6], rr[7]);
 }
 
 // Inverse inputs of the row pass for y-row pairs r: Z[r] E_x (reversed sine
@@ -880,10 +1010,10 @@ k_tcr_pack_inv(int n, int rows2, const float* __restrict__ PT, const float* __re
     const int r = (int)(q / half), u = (int)(q % half);
     const int un = (n - u) & (n - 1);
     {
-        const float* A = RT + (size_t)(2 * r) * n;
-        const float* Bq = A + n;
-        const float au = A[u & (n - 1)], bu = Bq[u & (n - 1)];
-        const float an = (u > 0) ? A[un] : 0.0f, bn = (u > 0) ? Bq[un] : 0.0f;
+        const float2* A = reinterpret_cast<const float2*>(RT) + (size_t)r * n;
+        const float2 cu = A[u & (n - 1)], cn = A[un];
+        const float au = cu.x, bu = cu.y;
+        const float an = (u > 0) ? cn.x : 0.0f, bn = (u > 0) ? cn.y : 0.0f;
         const float cau = (u == 0) ? au : 0.5f * au, cbu = (u == 0) ? bu : 0.5f * bu;
         float can = 0.5f * an, cbn = 0.5f * bn;
         if (u == n / 2) { can = cau; cbn = cbu; }
@@ -892,13 +1022,13 @@ k_tcr_pack_inv(int n, int rows2, const float* __restrict__ PT, const float* __re
         if (u > 0 && u < n / 2) row[n - u] = pack_inv(can, cau, cbn, cbu, ph[n - u]);
     }
     {
-        const float* Pa = PT + (size_t)(2 * r) * n;
-        const float* Pb = Pa + n;
+        const float2* Pr = reinterpret_cast<const float2*>(PT) + (size_t)r * n;
+        const float2 cu = Pr[u & (n - 1)], cn = Pr[un];
         const float wu = pi_lx * (float)u, wn = pi_lx * (float)(n - u);
-        const float ca_u = (u == 0) ? 0.0f : 0.5f * wn * Pa[n - u];
-        const float cb_u = (u == 0) ? 0.0f : 0.5f * wn * Pb[n - u];
-        float ca_n = (u == 0) ? 0.0f : 0.5f * wu * Pa[u];
-        float cb_n = (u == 0) ? 0.0f : 0.5f * wu * Pb[u];
+        const float ca_u = (u == 0) ? 0.0f : 0.5f * wn * cn.x;
+        const float cb_u = (u == 0) ? 0.0f : 0.5f * wn * cn.y;
+        float ca_n = (u == 0) ? 0.0f : 0.5f * wu * cu.x;
+        float cb_n = (u == 0) ? 0.0f : 0.5f * wu * cu.y;
         if (u == n / 2) { ca_n = ca_u; cb_n = cb_u; }
         float2* row = Z + (size_t)r * n;
         row[u & (n - 1)] = pack_inv(ca_u, ca_n, cb_u, cb_n, ph[u]);
@@ -951,8 +1081,8 @@ cudaError_t launch_tcr_stage(Ctx& c, int which, const float2* V, float2* Z, cuda
                 det_red(c, 0));
             break;
         case 4:     // P, R sums -> PT, RT (transposed)
-            k_tcr_post_cols<<<tcr_blocks((long long)(rows2 / 4) * n), 256, 0, s>>>(n, rows2, V,
-                                                                                  c.PT, c.RT);
+            k_tcr_post_cols<<<tcr_blocks((long long)(rows2 / 4) * (n / 2)), 256, 0, s>>>(n, rows2, V,
+                                                                                        c.PT, c.RT);
             break;
         case 5:     // PT, RT rows -> Z (E_x rows, then E_y rows)
             k_tcr_pack_inv<<<tcr_blocks((long long)rows2 * (n / 2 + 1)), 256, 0, s>>>(
@@ -967,56 +1097,63 @@ cudaError_t launch_tcr_stage(Ctx& c, int which, const float2* V, float2* Z, cuda
 }
 
 // ------------------------------------------------------------ launch
+enum { PASS_FWD, PASS_COLS, PASS_FIELD, PASS_PSI, PASS_MAPS };
+
 template <int LOGN>
 static cudaError_t launch_all_logn(Ctx& c, int which, cudaStream_t s) {
+    using L2 = Lay<LOGN, 2>;
+    using L1 = Lay<LOGN, 1>;
     constexpr int N = 1 << LOGN;
-    size_t smem = (size_t)kSpecBuffers * padded(N) * sizeof(float2);
-    float inv_ab = (float)(1.0 / c.Ab);
-    float cap = (float)(c.opt.target_density * c.Ab);
-    float pi_lx = (float)(M_PI / c.Lx), pi_ly = (float)(M_PI / c.Ly);
-    cudaError_t e = cudaSuccess;
-    if (which == 0) {
-        if (c.opt.deterministic) {
-            auto kf = k_rows_fwd<LOGN, true>;
-            kf<<<N / (2 * kSpecBuffers), kSpecThreads, smem, s>>>(nullptr, c.Dq, c.M, inv_ab, cap,
-                                                                   c.T1, c.tw, c.ph, c.acc,
-                                                                   det_red(c, 0), c.map_t1,
-                                                                   c.spec_tma ? 1 : 0);
-        } else {
-            auto kf = k_rows_fwd<LOGN, false>;
-            kf<<<N / (2 * kSpecBuffers), kSpecThreads, smem, s>>>(c.D, nullptr, c.M, inv_ab, cap,
-                                                                   c.T1, c.tw, c.ph, c.acc,
-                                                                   det_red(c, 0), c.map_t1,
-                                                                   c.spec_tma ? 1 : 0);
+    constexpr int nb2 = (N / 4 + L2::GB - 1) / L2::GB, nb1 = (N / 2 + L1::GB - 1) / L1::GB;
+    const float inv_ab = (float)(1.0 / c.Ab);
+    const float cap = (float)(c.opt.target_density * c.Ab);
+    const float pi_lx = (float)(M_PI / c.Lx), pi_ly = (float)(M_PI / c.Ly);
+    const int tma = c.spec_tma ? 1 : 0;
+    auto inv = [&](auto kern, int nv) {
+        kern<<<nb1, L1::T, L1::GB * L1::group_bytes(nv), s>>>(c.PT, c.RT, c.E2, c.psi, c.ex, c.ey,
+                                                              pi_lx);
+    };
+    switch (which) {
+        case PASS_FWD: {
+            const int smem = L2::GB * L2::group_bytes(1);
+            if (c.opt.deterministic)
+                k_rows_fwd<LOGN, true><<<nb2, L2::T, smem, s>>>(nullptr, c.Dq, c.M, inv_ab, cap,
+                                                                c.T1, c.acc, det_red(c, 0),
+                                                                c.map_t1, tma);
+            else
+                k_rows_fwd<LOGN, false><<<nb2, L2::T, smem, s>>>(c.D, nullptr, c.M, inv_ab, cap,
+                                                                 c.T1, c.acc, det_red(c, 0),
+                                                                 c.map_t1, tma);
+            break;
         }
-    } else if (which == 1) {
-        auto kf = k_cols<LOGN>;
-        kf<<<N / kSpecBuffers, kSpecThreads, smem, s>>>(c.T1, c.PT, c.RT, c.tw, c.ph, pi_lx, pi_ly,
-                                                        (float)c.opt.helmholtz_eps, c.acc,
-                                                        det_red(c, 0), c.map_pt, c.map_rt,
-                                                        c.spec_tma ? 1 : 0);
-    } else if (which == 2) {
-        auto kf = k_rows_inv<LOGN>;
-        kf<<<N / kSpecBuffers, kSpecThreads, smem, s>>>(c.PT, c.RT, c.E2, c.tw, c.ph, pi_lx);
-    } else {
-        auto kf = k_rows_psi<LOGN>;
-        kf<<<N / kSpecBuffers, kSpecThreads, smem / 2, s>>>(c.PT, c.psi, c.tw, c.ph);
+        case PASS_COLS:
+            k_cols<LOGN><<<nb2, L2::T, L2::GB * L2::group_bytes(2), s>>>(
+                c.T1, c.PT, c.RT, pi_lx, pi_ly, (float)c.opt.helmholtz_eps, c.acc, det_red(c, 0),
+                c.map_pt, c.map_rt, tma);
+            break;
+        case PASS_FIELD: inv(k_rows_inv<LOGN, INV_FIELD>, 2); break;
+        case PASS_PSI: inv(k_rows_inv<LOGN, INV_PSI>, 1); break;
+        default: inv(k_rows_inv<LOGN, INV_MAPS>, 2); break;
     }
     c.launches++;
-    e = cudaGetLastError();
-    return e;
+    return cudaGetLastError();
 }
 
 // Shared-memory opt-in for every kernel of one transform size (done at create,
 // outside any stream capture).
 template <int LOGN>
 static void prepare_logn() {
-    int smem = (int)((size_t)kSpecBuffers * padded(1 << LOGN) * sizeof(float2));
-    cudaFuncSetAttribute(k_rows_fwd<LOGN, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaFuncSetAttribute(k_rows_fwd<LOGN, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaFuncSetAttribute(k_cols<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaFuncSetAttribute(k_rows_inv<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaFuncSetAttribute(k_rows_psi<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem / 2);
+    using L2 = Lay<LOGN, 2>;
+    using L1 = Lay<LOGN, 1>;
+    auto set = [](auto kern, int smem) {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    };
+    set(k_rows_fwd<LOGN, true>, L2::GB * L2::group_bytes(1));
+    set(k_rows_fwd<LOGN, false>, L2::GB * L2::group_bytes(1));
+    set(k_cols<LOGN>, L2::GB * L2::group_bytes(2));
+    set(k_rows_inv<LOGN, INV_FIELD>, L1::GB * L1::group_bytes(2));
+    set(k_rows_inv<LOGN, INV_PSI>, L1::GB * L1::group_bytes(1));
+    set(k_rows_inv<LOGN, INV_MAPS>, L1::GB * L1::group_bytes(2));
 }
 
 void prepare_spectral(int logn) {
@@ -1050,17 +1187,19 @@ static cudaError_t dispatch(Ctx& c, int which, cudaStream_t s) {
 }
 
 void spec_maps_init(Ctx& c) {
-    const int n = c.n, box = n < 256 ? n : 256;
+    // n/2 rows of n complex elements, boxes of four of them by up to 256 rows
+    const int n = c.n, rows = n / 2, box = rows < 256 ? rows : 256;
     c.spec_maps_ok = c.T1 && c.PT && c.RT && n >= 16 &&
-                     make_map_f32(&c.map_t1, c.T1, n, n, 8, box) &&
-                     make_map_f32(&c.map_pt, c.PT, n, n, 4, box) &&
-                     make_map_f32(&c.map_rt, c.RT, n, n, 4, box);
+                     make_map_f32(&c.map_t1, c.T1, rows, 2 * n, 8, box) &&
+                     make_map_f32(&c.map_pt, c.PT, rows, 2 * n, 8, box) &&
+                     make_map_f32(&c.map_rt, c.RT, rows, 2 * n, 8, box);
     c.spec_tma = c.spec_maps_ok;
 }
 
-cudaError_t launch_rows_fwd(Ctx& c, cudaStream_t s) { return dispatch(c, 0, s); }
-cudaError_t launch_cols_spectral(Ctx& c, cudaStream_t s) { return dispatch(c, 1, s); }
-cudaError_t launch_rows_inv(Ctx& c, cudaStream_t s) { return dispatch(c, 2, s); }
-cudaError_t launch_rows_psi(Ctx& c, cudaStream_t s) { return dispatch(c, 3, s); }
+cudaError_t launch_rows_fwd(Ctx& c, cudaStream_t s) { return dispatch(c, PASS_FWD, s); }
+cudaError_t launch_cols_spectral(Ctx& c, cudaStream_t s) { return dispatch(c, PASS_COLS, s); }
+cudaError_t launch_rows_inv(Ctx& c, cudaStream_t s) { return dispatch(c, PASS_FIELD, s); }
+cudaError_t launch_rows_psi(Ctx& c, cudaStream_t s) { return dispatch(c, PASS_PSI, s); }
+cudaError_t launch_rows_maps(Ctx& c, cudaStream_t s) { return dispatch(c, PASS_MAPS, s); }
 
 }  // namespace fftpl

@@ -1,9 +1,9 @@
 // fftpl_solve_noalloc: the spectral Poisson solve of a caller-supplied
 // density map without any device allocation, for callers that cannot
-// allocate (see include/fftpl.h).  The three transform passes and the field
-// split are the library's own kernels; their intermediates (the transposed
-// row transforms, the column results, the interleaved field), the transform
-// tables and the FP64 sums live in one file-scope device array.
+// allocate (see include/fftpl.h).  The three transform passes are the
+// library's own kernels, the last one writing psi, E_x and E_y straight into
+// the caller's maps; their intermediates (the transposed row transforms and
+// the column results) and the FP64 sums live in one file-scope device array.
 #include <math.h>
 
 #include <mutex>
@@ -20,10 +20,7 @@ constexpr size_t kMap = (size_t)kMaxN * kMaxN;   // floats per map
 constexpr size_t kOffT1 = 0;
 constexpr size_t kOffPT = kOffT1 + kMap * sizeof(float);
 constexpr size_t kOffRT = kOffPT + kMap * sizeof(float);
-constexpr size_t kOffE2 = kOffRT + kMap * sizeof(float);
-constexpr size_t kOffTw = kOffE2 + kMap * sizeof(float2);
-constexpr size_t kOffPh = kOffTw + (size_t)kMaxN * sizeof(float2);
-constexpr size_t kOffAcc = kOffPh + ((size_t)kMaxN + 256 / sizeof(float2)) * sizeof(float2);
+constexpr size_t kOffAcc = kOffRT + kMap * sizeof(float);
 constexpr size_t kScratchBytes = kOffAcc + (size_t)kAccDoubles * sizeof(double);
 static_assert(kOffAcc % 256 == 0, "scratch layout alignment");
 
@@ -34,22 +31,6 @@ static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 unsigned char* g_dev_ptr[kMaxDevices] = {};
-
-// FFT twiddles exp(-2 pi i k / n) and cosine-transform twiddles
-// exp(-i pi u / 2n), from sincospi in FP64.
-__global__ void k_tables(int n, float2* __restrict__ tw, float2* __restrict__ ph) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) {
-        double s, c;
-        sincospi(2.0 * i / n, &s, &c);
-        tw[i] = make_float2((float)c, (float)-s);
-    }
-    if (i <= n) {
-        double s, c;
-        sincospi((double)i / (2.0 * n), &s, &c);
-        ph[i] = make_float2((float)c, (float)-s);
-    }
-}
 
 // Per-device set-up: the array's device address (with the device current),
 // and the kernels' shared-memory limits for every grid size.
@@ -138,24 +119,15 @@ extern "C" fftpl_status fftpl_solve_noalloc(const float* rho, int32_t n, double 
     c.PT = reinterpret_cast<float*>(base + kOffPT);
     c.RT = reinterpret_cast<float*>(base + kOffRT);
     spec_maps_init(c);
-    c.E2 = reinterpret_cast<float2*>(base + kOffE2);
-    c.tw = reinterpret_cast<float2*>(base + kOffTw);
-    c.ph = reinterpret_cast<float2*>(base + kOffPh);
     c.acc = reinterpret_cast<double*>(base + kOffAcc);
     c.psi = psi;
     c.ex = ex;
     c.ey = ey;
 
     cudaError_t e = cudaMemsetAsync(c.acc, 0, (size_t)kAccDoubles * sizeof(double), s);
-    if (e == cudaSuccess) {
-        k_tables<<<(n + 1 + 255) / 256, 256, 0, s>>>(n, c.tw, c.ph);
-        e = cudaGetLastError();
-    }
     if (e == cudaSuccess) e = launch_rows_fwd(c, s);
     if (e == cudaSuccess) e = launch_cols_spectral(c, s);
-    if (e == cudaSuccess) e = launch_rows_inv(c, s);
-    if (e == cudaSuccess) e = launch_rows_psi(c, s);
-    if (e == cudaSuccess) e = launch_split_field(c, s);
+    if (e == cudaSuccess) e = launch_rows_maps(c, s);
     if (e == cudaSuccess && N) {
         double acc[kAccDoubles];
         e = cudaMemcpyAsync(acc, c.acc, sizeof(acc), cudaMemcpyDeviceToHost, s);
