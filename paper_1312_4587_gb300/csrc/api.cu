@@ -1210,6 +1210,7 @@ static fftpl_status loop_eval(Ctx& c, bool cells) {
             CK(cudaMemsetAsync(c.gW2, 0, (size_t)c.m_mov * sizeof(float2), c.side));
         CK(launch_wa_impl(c, vx, vy, 1.0f, ctrl_f(c.ctrl) + F_INV_G, ctrl_f(c.ctrl) + F_DONE,
                           false, c.side));
+        if (cells) CK(launch_ctrl_lambda(c, c.side));
     }
     CK(cudaEventRecord(c.ev_join, c.side));
     TRY(enqueue_solve(c, s));

@@ -18,8 +18,7 @@ struct LoopBufs {
     DetRed dr;
 };
 
-// gather + pin sums at v (like k_cells, 48 warps per SM); k_ctrl_lambda
-// then forms lambda_k.
+// gather + pin sums at v (like k_cells, 48 warps per SM).
 template <bool CSR>
 __global__ void __launch_bounds__(kCellThreads, 6)
 k_loop_cells(Grid gr, int m, LoopBufs b, const float2* __restrict__ E2,
@@ -55,11 +54,35 @@ k_loop_cells(Grid gr, int m, LoopBufs b, const float2* __restrict__ E2,
     reduce2(fabsf(nx) + fabsf(ny), fabsf(wx) + fabsf(wy), b.acc, ACC_GN_L1, ACC_GW_L1, b.dr);
 }
 
-// lambda_k from the cell kernel's sums (one thread, launched after it: a
-// ticket at the end of each of the cell kernel's 8.6K blocks cost more)
+// lambda_k and the momentum weight beside the density chain (one warp on the
+// wirelength stream, after its kernels); lambda_0 waits for the gradient
+// norms (loop_lambda).
 __global__ void k_ctrl_lambda(double* ctrl, const double* acc) {
     if (ctrl_f(ctrl)[F_DONE] != 0.0f) return;
-    ctrl_lambda(ctrl, acc);
+    if (threadIdx.x < 32) ctrl_lambda(ctrl, acc);
+    else if (threadIdx.x == 32) ctrl_momentum(ctrl);
+}
+
+// lambda for the combined gradient: from the control scalars, in the first
+// iteration (unless given) from the gradients' norms, which the first warp of
+// every block forms for the block (FP64 by every warp took the first iteration
+// from 11 to 23 us); the block that draws the last ticket stores it.
+__device__ __forceinline__ float loop_lambda(const LoopBufs& b) {
+    if (!lambda_from_norms(b.ctrl)) return ctrl_f(b.ctrl)[F_LAMBDA];
+    __shared__ float s_lam;
+    if (threadIdx.x < 32) {
+        const float lam = (float)lambda_start(b.acc);
+        if (threadIdx.x == 0) s_lam = lam;
+    }
+    __syncthreads();
+    return s_lam;
+}
+__device__ __forceinline__ void store_lambda(const LoopBufs& b) {
+    if (!lambda_from_norms(b.ctrl)) return;
+    const double lam = lambda_start(b.acc);
+    if (threadIdx.x != 0) return;
+    b.ctrl[C_LAMBDA] = lam;
+    ctrl_f(b.ctrl)[F_LAMBDA] = (float)lam;
 }
 
 // The vector kernels of the loop (2m coordinates) run on a fixed grid of
@@ -71,11 +94,11 @@ __global__ void k_ctrl_lambda(double* ctrl, const double* acc) {
 // coordinates paid 17K times per kernel at 2.2M cells.
 constexpr int kVecBlocksPerSm = 6;
 
-// g = gW + lambda gN; sums for alpha_k; last CTA: alpha_k and beta_k.
+// g = gW + lambda gN; sums for alpha_k; last CTA: alpha_k and gamma_{k+1}.
 __global__ void __launch_bounds__(kCellThreads, kVecBlocksPerSm) k_loop_g(int m2, LoopBufs b) {
     const float* cf = ctrl_f(b.ctrl);
     if (cf[F_DONE] != 0.0f) return;
-    const float lam = cf[F_LAMBDA];
+    const float lam = loop_lambda(b);
     const bool first = cf[F_FIRST] != 0.0f;
     dfloat dg = df_zero(), dv = df_zero();
     float gi = 0.0f;
@@ -117,7 +140,13 @@ __global__ void __launch_bounds__(kCellThreads, kVecBlocksPerSm) k_loop_g(int m2
     }
     reduce2(df_val(dg), df_val(dv), b.acc, ACC_DG2, ACC_DV2, b.dr);
     block_max(gi, b.acc, ACC_GINF);
-    if (last_cta(b.counters + 1) && threadIdx.x == 0) ctrl_alpha(b.ctrl, b.acc);
+    if (!last_cta(b.counters + 1)) return;
+    if (threadIdx.x < 32) {
+        store_lambda(b);
+        ctrl_alpha(b.ctrl, b.acc);
+    } else if (threadIdx.x < 64) {
+        ctrl_gamma_next(b.ctrl, b.acc);
+    }
 }
 
 // u_{k+1} = clamp(v_k - alpha g_k); v_{k+1} = clamp(u_{k+1} + beta (u_{k+1} - u_k));
@@ -166,7 +195,7 @@ k_loop_update(int m, Grid gr, float x1, float y1, LoopBufs b) {
     }
     block_max(step, b.acc, ACC_STEPMAX);
     reduce2(df_val(uphill), 0.0f, b.acc, ACC_GD, -1, b.dr);
-    if (last_cta(b.counters + 2) && threadIdx.x == 0) ctrl_record(b.ctrl, b.acc, b.recs);
+    if (last_cta(b.counters + 2) && threadIdx.x < 32) ctrl_record(b.ctrl, b.acc, b.recs);
 }
 
 // ------------------------------------------------ conjugate-gradient loop
@@ -178,7 +207,7 @@ k_loop_update(int m, Grid gr, float x1, float y1, LoopBufs b) {
 __global__ void __launch_bounds__(kCellThreads, kVecBlocksPerSm) k_cg_g(int m2, LoopBufs b) {
     const float* cf = ctrl_f(b.ctrl);
     if (cf[F_DONE] != 0.0f) return;
-    const float lam = cf[F_LAMBDA];
+    const float lam = loop_lambda(b);
     const bool first = cf[F_FIRST] != 0.0f;
     dfloat sq = df_zero(), gp = df_zero();
     float gi = 0.0f;
@@ -211,7 +240,13 @@ __global__ void __launch_bounds__(kCellThreads, kVecBlocksPerSm) k_cg_g(int m2, 
     }
     reduce2(df_val(sq), df_val(gp), b.acc, ACC_DG2, ACC_DV2, b.dr);
     block_max(gi, b.acc, ACC_GINF);
-    if (last_cta(b.counters + 3) && threadIdx.x == 0) ctrl_cg_g(b.ctrl, b.acc);
+    if (!last_cta(b.counters + 3)) return;
+    if (threadIdx.x < 32) {
+        store_lambda(b);
+        ctrl_cg_g(b.ctrl, b.acc);
+    } else if (threadIdx.x < 64) {
+        ctrl_gamma_next(b.ctrl, b.acc);
+    }
 }
 
 // d = -g + beta d; sum g . d and max |d|; last CTA: restart test, |d|_inf
@@ -249,7 +284,7 @@ __global__ void __launch_bounds__(kCellThreads, kVecBlocksPerSm) k_cg_dir(int m2
     }
     reduce2(df_val(gd), 0.0f, b.acc, ACC_GD, -1, b.dr);
     block_max(da, b.acc, ACC_DINF);
-    if (last_cta(b.counters + 4) && threadIdx.x == 0) ctrl_cg_dir(b.ctrl, b.acc);
+    if (last_cta(b.counters + 4) && threadIdx.x < 32) ctrl_cg_dir(b.ctrl, b.acc);
 }
 
 // per coordinate i < 2m: the direction (d, or -g after a restart) and the
@@ -277,9 +312,9 @@ k_cg_trial(int m, Grid gr, float x1, float y1, LoopBufs b) {
     b.v[i] = fminf(hi, fmaxf(lo, fmaf(scale, dir, b.u[i])));
 }
 
-// the step from the trial evaluation (one thread)
+// the step from the trial evaluation (one warp)
 __global__ void k_cg_alpha(double* ctrl, const double* acc) {
-    if (ctrl[C_DONE] != 0.0) return;
+    if (ctrl_f(ctrl)[F_DONE] != 0.0f) return;
     ctrl_cg_alpha(ctrl, acc);
 }
 
@@ -344,11 +379,10 @@ __global__ void k_place_init(int m, Grid gr, float x1, float y1, const float* __
     b.gprev[i] = 0.0f;
 }
 
-// gamma_0 from the overflow at the start (schedule mode).
+// gamma_0 from the overflow at the start (schedule mode; one warp).
 __global__ void k_gamma0(double* ctrl, const double* acc) {
-    double tau = acc_sum(acc, ACC_TAU) / ctrl[C_MOV_AREA];
-    ctrl[C_GAMMA] = gamma_schedule(tau, ctrl[C_WB]);
-    ctrl_mirror(ctrl);
+    ctrl_gamma_next(ctrl, acc);
+    if (threadIdx.x == 0) ctrl_take_gamma(ctrl);
 }
 
 static inline int nblk(long long m, int t) { return (int)((m + t - 1) / t); }
@@ -377,8 +411,13 @@ cudaError_t launch_loop_cells(Ctx& c, cudaStream_t s) {
     else
         k_loop_cells<false><<<nb, kCellThreads, 0, s>>>(c.grid, c.m_mov, b, c.E2, c.cell_rank,
                                                         nullptr, nullptr, c.gW2);
-    k_ctrl_lambda<<<1, 1, 0, s>>>(c.ctrl, c.acc);
-    c.launches += 2;
+    c.launches++;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_ctrl_lambda(Ctx& c, cudaStream_t s) {
+    k_ctrl_lambda<<<1, 64, 0, s>>>(c.ctrl, c.acc);
+    c.launches++;
     return cudaGetLastError();
 }
 
@@ -422,7 +461,7 @@ cudaError_t launch_cg_trial(Ctx& c, cudaStream_t s) {
 }
 
 cudaError_t launch_cg_alpha(Ctx& c, cudaStream_t s) {
-    k_cg_alpha<<<1, 1, 0, s>>>(c.ctrl, c.acc);
+    k_cg_alpha<<<1, 32, 0, s>>>(c.ctrl, c.acc);
     c.launches++;
     return cudaGetLastError();
 }
@@ -435,7 +474,7 @@ cudaError_t launch_cg_update(Ctx& c, cudaStream_t s) {
 }
 
 cudaError_t launch_gamma0(Ctx& c, cudaStream_t s) {
-    k_gamma0<<<1, 1, 0, s>>>(c.ctrl, c.acc);
+    k_gamma0<<<1, 32, 0, s>>>(c.ctrl, c.acc);
     c.launches++;
     return cudaGetLastError();
 }

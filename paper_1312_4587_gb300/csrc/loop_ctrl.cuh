@@ -3,6 +3,14 @@
 // updated by the last CTA of the kernel that produces their inputs (a CTA
 // learns it is last from an atomic ticket after a memory fence; nothing
 // waits, so no kernel can hang on it).
+//
+// The updates sit on the critical path of every iteration and the FP64 pipe
+// is narrow, so a warp reads the 32 stripes of a sum with one load per lane,
+// and what does not depend on an update's own input is formed beside it:
+// lambda_k (for k >= 1 from the HPWL change alone) and the momentum weight on
+// the wirelength stream, gamma_{k+1} by a second warp.  With one thread
+// walking the stripes, pow() and every scalar in line, the three updates took
+// 10 + 14 + 18 us of an iteration at 210K cells.
 #pragma once
 
 #include "fftpl_internal.cuh"
@@ -58,7 +66,12 @@ __host__ __device__ inline void ctrl_mirror(double* ctrl) {
     if (g > 0.0f) wa_scale(g, &f[F_INV_G], &f[F_L2G]);
 }
 constexpr int kRecFields = 8;
-constexpr int kCounters = 4;   // one ticket counter per loop kernel kind
+// Doubles after the control scalars that are not part of a saved state: one
+// ticket counter per loop kernel kind (32 bits each), then what one kernel of
+// an iteration leaves for the next.
+constexpr int kCounters = 8;
+enum { S_GAMMA_NEXT = C_COUNT + 4, S_SCALE_NEXT /* 1/gamma, log2(e)/gamma as floats */ };
+static_assert(S_SCALE_NEXT < C_COUNT + kCounters, "loop scratch too small");
 
 // After a block barrier (which orders every thread's earlier reductions
 // before thread 0's next operations), thread 0 fences at device scope and
@@ -83,98 +96,157 @@ __device__ __forceinline__ bool last_cta(unsigned int* counter) {
     return is_last;
 }
 
-// totals of the striped accumulators (read past L1)
+// Totals of the striped accumulators (read past L1), one stripe per lane;
+// called by a full warp, every lane gets the total.
 __device__ __forceinline__ double acc_sum(const double* acc, int q) {
-    double s = 0.0;
-    for (int k = 0; k < kAccStripes; ++k) s += __ldcg(acc + k * kAccStride + q);
+    static_assert(kAccStripes == 32, "one stripe per lane");
+    double s = __ldcg(acc + (threadIdx.x & 31) * kAccStride + q);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     return s;
 }
+// (non-negative values: ordered as their bit patterns)
 __device__ __forceinline__ double acc_max(const double* acc, int q) {
-    double s = 0.0;
-    for (int k = 0; k < kAccStripes; ++k) s = fmax(s, __ldcg(acc + k * kAccStride + q));
-    return s;
+    long long s = __double_as_longlong(__ldcg(acc + (threadIdx.x & 31) * kAccStride + q));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s = max(s, __shfl_xor_sync(0xffffffffu, s, o));
+    return __longlong_as_double(s);
 }
 
-// After the cell kernel: lambda_k.  lambda_0 = ||grad W~||_1 / ||grad N||_1
-// unless given; for k >= 1 lambda_k = mu_k lambda_{k-1} with
-// mu_k = 1.1^(-dW/dW_ref + 1) bounded to [0.75, 1.1], dW the HPWL change.
+// lambda_0 = ||grad W~||_1 / ||grad N||_1 unless given (a full warp).
+__device__ __forceinline__ double lambda_start(const double* acc) {
+    const double gn = acc_sum(acc, ACC_GN_L1), gw = acc_sum(acc, ACC_GW_L1);
+    return gn > 0.0 ? gw / gn : 1.0;
+}
+// whether the first iteration forms lambda_0 itself
+__device__ __forceinline__ bool lambda_from_norms(const double* ctrl) {
+    return ctrl_f(ctrl)[F_FIRST] != 0.0f && !(ctrl[C_LAMBDA0_OPT] > 0.0);
+}
+
+// After the wirelength kernels (one warp on their stream): lambda_k for
+// k >= 1, mu_k lambda_{k-1} with mu_k = 1.1^(-dW/dW_ref + 1) bounded to
+// [0.75, 1.1], dW the HPWL change (1.1^z as exp(z ln 1.1)); and the momentum
+// weight of iteration k, a_{k+1} = (1 + sqrt(1 + 4 a_k^2)) / 2,
+// beta_k = (a_k - 1) / a_{k+1}.
 __device__ __forceinline__ void ctrl_lambda(double* ctrl, const double* acc) {
-    int k = (int)ctrl[C_K];
-    double hp = acc_sum(acc, ACC_HPWL);
-    double lam = ctrl[C_LAMBDA];
-    if (k == 0 && ctrl[C_LAMBDA0_OPT] <= 0.0) {
-        double gn = acc_sum(acc, ACC_GN_L1), gw = acc_sum(acc, ACC_GW_L1);
-        lam = gn > 0.0 ? gw / gn : 1.0;
-    }
-    if (k >= 1) {
-        double mu = pow(1.1, -(hp - ctrl[C_HP_PREV]) / ctrl[C_DW_REF] + 1.0);
-        lam *= fmin(1.1, fmax(0.75, mu));
+    const double hp = acc_sum(acc, ACC_HPWL);
+    if ((threadIdx.x & 31) != 0) return;
+    float* f = ctrl_f(ctrl);
+    if (ctrl[C_K] >= 1.0) {
+        const double z = -(hp - ctrl[C_HP_PREV]) / ctrl[C_DW_REF] + 1.0;
+        const double mu = z >= 1.0 ? 1.1 : exp(z * 0.095310179804324860044);
+        const double lam = ctrl[C_LAMBDA] * fmin(1.1, fmax(0.75, mu));
+        ctrl[C_LAMBDA] = lam;
+        f[F_LAMBDA] = (float)lam;
     }
     ctrl[C_HP_PREV] = hp;
-    ctrl[C_LAMBDA] = lam;
-    ctrl_mirror(ctrl);
+}
+__device__ __forceinline__ void ctrl_momentum(double* ctrl) {
+    const double a = ctrl[C_A];
+    const double an = 0.5 * (1.0 + sqrt(1.0 + 4.0 * a * a)), beta = (a - 1.0) / an;
+    ctrl[C_A_NEXT] = an;
+    ctrl[C_BETA] = beta;
+    ctrl_f(ctrl)[F_BETA] = (float)beta;
 }
 
-// After the combined gradient: the step alpha_k and the momentum weight.
+// gamma = 8.0 w_b 10^((20/9)(tau - 0.1) - 1) (Section IV-A).
+__device__ __forceinline__ double gamma_schedule(double tau, double wb) {
+    return 8.0 * wb * exp10((20.0 / 9.0) * (tau - 0.1) - 1.0);
+}
+
+// gamma_{k+1} and its float32 factors into the loop scratch (a full warp; the
+// overflow of the evaluated point is known since the row pass).
+__device__ __forceinline__ void ctrl_gamma_next(double* ctrl, const double* acc) {
+    const double tau = acc_sum(acc, ACC_TAU) / ctrl[C_MOV_AREA];
+    if ((threadIdx.x & 31) != 0 || ctrl[C_GAMMA_FIXED] > 0.0) return;
+    const double g = gamma_schedule(tau, ctrl[C_WB]);
+    float* sc = reinterpret_cast<float*>(ctrl + S_SCALE_NEXT);
+    ctrl[S_GAMMA_NEXT] = g;
+    wa_scale((float)g, sc, sc + 1);
+}
+// gamma_{k+1} in force (one thread).
+__device__ __forceinline__ void ctrl_take_gamma(double* ctrl) {
+    if (ctrl[C_GAMMA_FIXED] > 0.0) return;
+    float* f = ctrl_f(ctrl);
+    const double g = ctrl[S_GAMMA_NEXT];
+    const float* sc = reinterpret_cast<const float*>(ctrl + S_SCALE_NEXT);
+    ctrl[C_GAMMA] = g;
+    if ((float)g > 0.0f) {
+        f[F_INV_G] = sc[0];
+        f[F_L2G] = sc[1];
+    }
+}
+
+// After the combined gradient (a full warp): the step alpha_k.
 // alpha_0 = alpha_max_0 / ||g||_inf; alpha_k = ||v_k - v_{k-1}|| / ||g_k - g_{k-1}||;
 // alpha_k ||g||_inf is then kept within [0.01 alpha_max_k, alpha_max_k].
 __device__ __forceinline__ void ctrl_alpha(double* ctrl, const double* acc) {
-    int k = (int)ctrl[C_K];
-    double ginf = acc_max(acc, ACC_GINF);
-    double alpha = ctrl[C_ALPHA], amax = ctrl[C_ALPHA_MAX];
-    if (k == 0) {
-        alpha = ginf > 0.0 ? ctrl[C_ALPHA_MAX0] / ginf : 0.0;
-    } else {
-        double dg2 = acc_sum(acc, ACC_DG2), dv2 = acc_sum(acc, ACC_DV2);
-        if (dg2 > 0.0) alpha = sqrt(dv2) / sqrt(dg2);
+    // the scalars' loads go out with the stripes'
+    double alpha = ctrl[C_ALPHA];
+    const double amax = ctrl[C_ALPHA_MAX], amax0 = ctrl[C_ALPHA_MAX0], k = ctrl[C_K];
+    const double ginf = acc_max(acc, ACC_GINF);
+    const double dg2 = acc_sum(acc, ACC_DG2), dv2 = acc_sum(acc, ACC_DV2);
+    if ((threadIdx.x & 31) != 0) return;
+    if (k == 0.0) {
+        alpha = ginf > 0.0 ? amax0 / ginf : 0.0;
+    } else if (dg2 > 0.0) {
+        alpha = sqrt(dv2) / sqrt(dg2);
     }
     if (ginf > 0.0) {
         if (alpha * ginf > amax) alpha = amax / ginf;
         if (alpha * ginf < 0.01 * amax) alpha = 0.01 * amax / ginf;
     }
-    double a = ctrl[C_A];
-    double an = 0.5 * (1.0 + sqrt(1.0 + 4.0 * a * a));
     ctrl[C_ALPHA] = alpha;
-    ctrl[C_A_NEXT] = an;
-    ctrl[C_BETA] = (a - 1.0) / an;
-    ctrl_mirror(ctrl);
+    ctrl_f(ctrl)[F_ALPHA] = (float)alpha;
 }
 
-// gamma = 8.0 w_b 10^((20/9)(tau - 0.1) - 1) (Section IV-A).
-__device__ __forceinline__ double gamma_schedule(double tau, double wb) {
-    return 8.0 * wb * pow(10.0, (20.0 / 9.0) * (tau - 0.1) - 1.0);
+// Counts iteration k done: k + 1 and the stop test (one thread).
+__device__ __forceinline__ void ctrl_advance(double* ctrl, int k, double tau) {
+    float* f = ctrl_f(ctrl);
+    ctrl[C_K] = (double)(k + 1);
+    f[F_FIRST] = 0.0f;
+    if (ctrl[C_STOP_ON_TAU] != 0.0 && tau <= ctrl[C_TAU_STOP]) {
+        ctrl[C_DONE] = 1.0;
+        f[F_DONE] = 1.0f;
+    }
 }
 
-// After the position update: record iteration k, then alpha_max_{k+1},
-// gamma_{k+1}, k+1 and the stop test tau <= tau_stop.  Adaptive restart
-// (the gradient test of O'Donoghue and Candes, 2015), one iteration late:
-// when g_k . (u_{k+1} - u_k) > 0 the momentum sequence starts over,
-// a_{k+1} = 1, so that the next momentum weight is 0.  alpha_max_{k+1} is
-// kept at or below the handle's ceiling (alpha_max_cap_bins bin widths).
+// After the position update (a full warp): record iteration k, then
+// alpha_max_{k+1}, gamma_{k+1}, k+1 and the stop test tau <= tau_stop.
+// Adaptive restart (the gradient test of O'Donoghue and Candes, 2015), one
+// iteration late: when g_k . (u_{k+1} - u_k) > 0 the momentum sequence starts
+// over, a_{k+1} = 1, so that the next momentum weight is 0.  alpha_max_{k+1}
+// is kept at or below the handle's ceiling (alpha_max_cap_bins bin widths).
 __device__ __forceinline__ void ctrl_record(double* ctrl, const double* acc, double* recs) {
-    int k = (int)ctrl[C_K];
-    double tau = acc_sum(acc, ACC_TAU) / ctrl[C_MOV_AREA];
-    double step_max = acc_max(acc, ACC_STEPMAX);
-    int slot = k - (int)ctrl[C_REC_BASE];
-    if (slot >= 0 && slot < (int)ctrl[C_REC_CAP]) {
+    // the scalars' loads go out with the stripes'
+    const double kd = ctrl[C_K], mov = ctrl[C_MOV_AREA], base = ctrl[C_REC_BASE],
+                 cap = ctrl[C_REC_CAP], half_ab = ctrl[C_HALF_AB], lam = ctrl[C_LAMBDA],
+                 gam = ctrl[C_GAMMA], alpha = ctrl[C_ALPHA], an = ctrl[C_A_NEXT],
+                 amax0 = ctrl[C_ALPHA_MAX0], acap = ctrl[C_ALPHA_CAP];
+    const double area = acc_sum(acc, ACC_TAU), step_max = acc_max(acc, ACC_STEPMAX);
+    const double W = acc_sum(acc, ACC_W), hp = acc_sum(acc, ACC_HPWL), N = acc_sum(acc, ACC_N);
+    const double gd = acc_sum(acc, ACC_GD);
+    if ((threadIdx.x & 31) != 0) return;
+    const int k = (int)kd;
+    const double tau = area / mov;
+    int slot = k - (int)base;
+    if (slot >= 0 && slot < (int)cap) {
         double* r = recs + (size_t)slot * kRecFields;
-        r[0] = acc_sum(acc, ACC_W);
-        r[1] = acc_sum(acc, ACC_HPWL);
-        r[2] = acc_sum(acc, ACC_N) * ctrl[C_HALF_AB];
+        r[0] = W;
+        r[1] = hp;
+        r[2] = N * half_ab;
         r[3] = tau;
-        r[4] = ctrl[C_LAMBDA];
-        r[5] = ctrl[C_GAMMA];
-        r[6] = ctrl[C_ALPHA];
+        r[4] = lam;
+        r[5] = gam;
+        r[6] = alpha;
         r[7] = step_max;
     }
-    ctrl[C_A] = acc_sum(acc, ACC_GD) > 0.0 ? 1.0 : ctrl[C_A_NEXT];
-    double amax = fmax(ctrl[C_ALPHA_MAX0], 2.0 * step_max);
-    if (ctrl[C_ALPHA_CAP] > 0.0) amax = fmin(amax, fmax(ctrl[C_ALPHA_CAP], ctrl[C_ALPHA_MAX0]));
+    ctrl[C_A] = gd > 0.0 ? 1.0 : an;
+    double amax = fmax(amax0, 2.0 * step_max);
+    if (acap > 0.0) amax = fmin(amax, fmax(acap, amax0));
     ctrl[C_ALPHA_MAX] = amax;
-    if (ctrl[C_GAMMA_FIXED] <= 0.0) ctrl[C_GAMMA] = gamma_schedule(tau, ctrl[C_WB]);
-    ctrl[C_K] = (double)(k + 1);
-    if (ctrl[C_STOP_ON_TAU] != 0.0 && tau <= ctrl[C_TAU_STOP]) ctrl[C_DONE] = 1.0;
-    ctrl_mirror(ctrl);
+    ctrl_take_gamma(ctrl);
+    ctrl_advance(ctrl, k, tau);
 }
 
 // ------------------------------------------------ conjugate-gradient loop
@@ -183,53 +255,67 @@ __device__ __forceinline__ void ctrl_record(double* ctrl, const double* acc, dou
 // cell move (direction scaled by 1/|d|_inf), one quadratic-fit line search
 // from f_k, the slope and one trial evaluation at a_max.
 
-// After g_k: beta_k (PR+), f_k and the values recorded for iteration k.
+// After g_k (a full warp): beta_k (PR+), f_k and the values recorded for
+// iteration k.
 __device__ __forceinline__ void ctrl_cg_g(double* ctrl, const double* acc) {
-    int k = (int)ctrl[C_K];
-    double gg = acc_sum(acc, ACC_DG2), ggp = acc_sum(acc, ACC_DV2);
-    double prev = ctrl[C_GG_PREV];
-    ctrl[C_BETA] = (k > 0 && prev > 0.0) ? fmax(0.0, (gg - ggp) / prev) : 0.0;
+    const double gg = acc_sum(acc, ACC_DG2), ggp = acc_sum(acc, ACC_DV2);
+    const double W = acc_sum(acc, ACC_W), hp = acc_sum(acc, ACC_HPWL);
+    const double N = acc_sum(acc, ACC_N) * ctrl[C_HALF_AB];
+    const double tau = acc_sum(acc, ACC_TAU) / ctrl[C_MOV_AREA];
+    if ((threadIdx.x & 31) != 0) return;
+    const double prev = ctrl[C_GG_PREV];
+    const double beta = (ctrl[C_K] > 0.0 && prev > 0.0) ? fmax(0.0, (gg - ggp) / prev) : 0.0;
+    ctrl[C_BETA] = beta;
+    ctrl_f(ctrl)[F_BETA] = (float)beta;
     ctrl[C_GG_PREV] = gg;
-    double W = acc_sum(acc, ACC_W), N = acc_sum(acc, ACC_N) * ctrl[C_HALF_AB];
     ctrl[C_FK] = W + ctrl[C_LAMBDA] * N;
     ctrl[C_W_K] = W;
-    ctrl[C_HP_K] = acc_sum(acc, ACC_HPWL);
+    ctrl[C_HP_K] = hp;
     ctrl[C_N_K] = N;
-    ctrl[C_TAU_K] = acc_sum(acc, ACC_TAU) / ctrl[C_MOV_AREA];
-    ctrl_mirror(ctrl);
+    ctrl[C_TAU_K] = tau;
 }
 
-// After d_k: restart to -g_k unless g_k . d_k < 0; |d|_inf and the slope.
+// After d_k (a full warp): restart to -g_k unless g_k . d_k < 0; |d|_inf and
+// the slope.
 __device__ __forceinline__ void ctrl_cg_dir(double* ctrl, const double* acc) {
     double gd = acc_sum(acc, ACC_GD), dinf = acc_max(acc, ACC_DINF);
-    bool restart = !(gd < 0.0);
+    const double ginf = acc_max(acc, ACC_GINF);
+    if ((threadIdx.x & 31) != 0) return;
+    float* f = ctrl_f(ctrl);
+    const bool restart = !(gd < 0.0);
     if (restart) {
-        dinf = acc_max(acc, ACC_GINF);
+        dinf = ginf;
         gd = -ctrl[C_GG_PREV];
     }
     ctrl[C_RESTART] = restart ? 1.0 : 0.0;
+    f[F_RESTART] = restart ? 1.0f : 0.0f;
     ctrl[C_DINF] = dinf;
     ctrl[C_SLOPE] = dinf > 0.0 ? gd / dinf : 0.0;
-    ctrl_mirror(ctrl);
+    f[F_SCALE_TRIAL] = dinf > 0.0 ? (float)(ctrl[C_ALPHA_MAX] / dinf) : 0.0f;
 }
 
-// After the trial evaluation at a_max: the step a_k from the parabola
-// through f_k (slope s) and f_t, kept in [0.01 a_max, a_max].
+// After the trial evaluation at a_max (a full warp): the step a_k from the
+// parabola through f_k (slope s) and f_t, kept in [0.01 a_max, a_max].
 __device__ __forceinline__ void ctrl_cg_alpha(double* ctrl, const double* acc) {
-    double amax = ctrl[C_ALPHA_MAX], alpha = 0.0;
-    if (ctrl[C_DINF] > 0.0) {
-        double ft = acc_sum(acc, ACC_W) + ctrl[C_LAMBDA] * acc_sum(acc, ACC_N) * ctrl[C_HALF_AB];
+    const double W = acc_sum(acc, ACC_W), N = acc_sum(acc, ACC_N);
+    if ((threadIdx.x & 31) != 0) return;
+    const double amax = ctrl[C_ALPHA_MAX], dinf = ctrl[C_DINF];
+    double alpha = 0.0;
+    if (dinf > 0.0) {
+        double ft = W + ctrl[C_LAMBDA] * N * ctrl[C_HALF_AB];
         double s = ctrl[C_SLOPE];
         double c = (ft - ctrl[C_FK] - s * amax) / (amax * amax);
         double as = c > 0.0 ? -s / (2.0 * c) : amax;
         alpha = fmin(amax, fmax(0.01 * amax, as));
     }
+    float* f = ctrl_f(ctrl);
     ctrl[C_ALPHA] = alpha;
-    ctrl_mirror(ctrl);
+    f[F_ALPHA] = (float)alpha;
+    f[F_SCALE_UPDATE] = dinf > 0.0 ? (float)(alpha / dinf) : 0.0f;
 }
 
-// After the position update: record iteration k, then a_max_{k+1} =
-// max(a_max_0, 2 a_k), gamma_{k+1}, k+1 and the stop test.
+// After the position update (one thread): record iteration k, then
+// a_max_{k+1} = max(a_max_0, 2 a_k), gamma_{k+1}, k+1 and the stop test.
 __device__ __forceinline__ void ctrl_record_cg(double* ctrl, double* recs) {
     int k = (int)ctrl[C_K];
     double tau = ctrl[C_TAU_K], alpha = ctrl[C_ALPHA];
@@ -246,10 +332,8 @@ __device__ __forceinline__ void ctrl_record_cg(double* ctrl, double* recs) {
         r[7] = alpha;
     }
     ctrl[C_ALPHA_MAX] = fmax(ctrl[C_ALPHA_MAX0], 2.0 * alpha);
-    if (ctrl[C_GAMMA_FIXED] <= 0.0) ctrl[C_GAMMA] = gamma_schedule(tau, ctrl[C_WB]);
-    ctrl[C_K] = (double)(k + 1);
-    if (ctrl[C_STOP_ON_TAU] != 0.0 && tau <= ctrl[C_TAU_STOP]) ctrl[C_DONE] = 1.0;
-    ctrl_mirror(ctrl);
+    ctrl_take_gamma(ctrl);
+    ctrl_advance(ctrl, k, tau);
 }
 
 }  // namespace fftpl
