@@ -30,6 +30,11 @@ namespace fftpl {
 
 // ------------------------------------------------------------------ sizes
 constexpr int kCellThreads = 256;
+// Blocks per SM of the cell kernels (field gather and pin sums): 24 warps of up
+// to 80 registers, room for four 32-byte loads in flight per thread and the
+// next cell's inputs.  k_cells at 2.2M cells under ncu with 2 / 3 / 4 blocks:
+// 48.6 / 39.2 / 45.1 us (4: spills).
+constexpr int kCellBlocks = 3;
 constexpr int kWaThreads = 256;
 // Nets of degree kBigMin..kBigMax go to the WA kernel with several lanes per
 // net (k_wa_grp, grp_lanes(d) lanes each, at most 4 pins per lane); the rest
@@ -69,47 +74,34 @@ static_assert(ACC_COUNT <= kAccStride, "accumulator stripe too small");
 // device error word bits
 enum { ERR_TIMEOUT = 1, ERR_BOUNDS = 2 };
 
-// Bin grid along both axes.  Edges e_k = x0 + k * wb are exact in float32
-// (checked at create), so comparisons against them decide indices exactly.
-// guard: see last_edge (1 = always take the exact comparisons).
+// Bin grid along both axes.  Edges e_k = x0 + k * wb, k <= n, are exact in
+// float32 (checked at create), so comparisons against them decide indices
+// exactly, and an edge formed as fma(k, wb, x0) or by adding wb to the one
+// before it is that same number.
 struct Grid {
     int n;
     float x0, y0, wb, hb, inv_wb, inv_hb;
-    float guard = 1.0f;
 };
 
 __device__ __forceinline__ float edge_at(float lo, float step, int k) {
     return __fadd_rn(lo, __fmul_rn((float)k, step));
 }
 
-// Largest k in [-1, n] with e_k <= t (strict: e_k < t).  The float estimate
-// q = (t - x0) * (1/w_b) is within one of the answer (its relative error is a
-// few 2^-24 and the quotient is at most n + 1 after clamping), so one
-// comparison against the exact edges in each direction settles the index.
-// Fast path: where 0 <= floor(q) < n and q lies at least `guard` bins from
-// both neighbouring integers, floor(q) is the answer without comparisons:
-// the edges are exact and q differs from (t - x0) / w_b by at most
-// n 2^-22 bins there, below guard = (n + 1) 2^-20 (q - floor(q) is exact).
+// Largest k in [-1, n] with e_k <= t (strict: e_k < t), limited to [LO, HI]
+// (-1 for NaN, limited alike).  The float estimate q = (t - x0) * (1/w_b) is
+// within one of the answer (its relative error is a few 2^-24 and the
+// quotient at most n + 1 after the limits), so one comparison against the
+// exact edge on each side settles the index.  No branches: a fast path for
+// estimates away from an edge, the comparisons otherwise, cost the cell
+// kernels more than the comparisons (a warp took both).
 template <bool STRICT>
-__device__ __forceinline__ int last_edge(float lo, float step, float inv, float guard, int n,
+__device__ __forceinline__ int last_edge(float lo, float step, float inv, float kmin, float kmax,
                                          float t) {
-    const float q = __fmul_rn(__fsub_rn(t, lo), inv);
-    float kf = floorf(q);
-    const float fr = q - kf;
-    if (kf >= 0.0f && kf < (float)n && fr >= guard && fr <= 1.0f - guard) return (int)kf;
-    int k;
-    if (!(kf >= -1.0f)) k = -1;          // also catches NaN
-    else if (kf > (float)n) k = n;
-    else k = (int)kf;
-    if (k < n) {
-        float e = edge_at(lo, step, k + 1);
-        if (STRICT ? (e < t) : (e <= t)) return k + 1;
-    }
-    if (k >= 0) {
-        float e = edge_at(lo, step, k);
-        if (!(STRICT ? (e < t) : (e <= t))) return k - 1;
-    }
-    return k;
+    float k = fminf(fmaxf(floorf(__fmul_rn(__fsub_rn(t, lo), inv)), kmin), kmax);
+    const float e0 = fmaf(k, step, lo), e1 = fmaf(k + 1.0f, step, lo);
+    const bool up = k < kmax && (STRICT ? e1 < t : e1 <= t);
+    const bool down = k > kmin && !(STRICT ? e0 < t : e0 <= t);
+    return (int)k + (up ? 1 : 0) - (down ? 1 : 0);
 }
 
 struct Span {
@@ -124,10 +116,11 @@ __device__ __forceinline__ Span cell_span(const Grid& g, float x, float y, float
     s.xh = __fadd_rn(x, hw);
     s.yl = __fsub_rn(y, hh);
     s.yh = __fadd_rn(y, hh);
-    s.ilo = max(last_edge<false>(g.x0, g.wb, g.inv_wb, g.guard, g.n, s.xl), 0);
-    s.ihi = min(last_edge<true>(g.x0, g.wb, g.inv_wb, g.guard, g.n, s.xh), g.n - 1);
-    s.jlo = max(last_edge<false>(g.y0, g.hb, g.inv_hb, g.guard, g.n, s.yl), 0);
-    s.jhi = min(last_edge<true>(g.y0, g.hb, g.inv_hb, g.guard, g.n, s.yh), g.n - 1);
+    const float n = (float)g.n;
+    s.ilo = last_edge<false>(g.x0, g.wb, g.inv_wb, 0.0f, n, s.xl);
+    s.ihi = last_edge<true>(g.x0, g.wb, g.inv_wb, -1.0f, n - 1.0f, s.xh);
+    s.jlo = last_edge<false>(g.y0, g.hb, g.inv_hb, 0.0f, n, s.yl);
+    s.jhi = last_edge<true>(g.y0, g.hb, g.inv_hb, -1.0f, n - 1.0f, s.yh);
     return s;
 }
 
@@ -138,68 +131,127 @@ __device__ __forceinline__ float ov_len(float lo, float step, int k, float a, fl
     return fmaxf(v, 0.0f);
 }
 
-// Overlap lengths of a span [lo, hi] along one axis: the end bins take the
-// generic formula; every bin strictly inside is covered whole, and
-// e_{k+1} - e_k is exactly the bin size in float32, so "step" is the same
-// value the generic formula gives there.
-struct AxisOv {
-    int lo, hi;
-    float first, last, step;
-};
-
-__device__ __forceinline__ AxisOv axis_ov(float e0, float step, int lo, int hi, float a, float b) {
-    AxisOv r;
-    r.lo = lo;
-    r.hi = hi;
-    r.step = step;
-    r.first = ov_len(e0, step, lo, a, b);
-    r.last = ov_len(e0, step, hi, a, b);
-    return r;
+// The same overlaps of consecutive bins: with c(e) = e limited to [a, b],
+// bin k's is c(e_{k+1}) - c(e_k) (both terms equal, so exactly 0, outside
+// the span; inside it the operands of ov_len).
+__device__ __forceinline__ float edge_in(float e, float a, float b) {
+    return fminf(fmaxf(e, a), b);
 }
 
-__device__ __forceinline__ float ov_at(const AxisOv& r, int k) {
-    return k == r.lo ? r.first : (k == r.hi ? r.last : r.step);
+// x overlaps of the aligned group of four bins 4 q .. 4 q + 3.
+__device__ __forceinline__ void quad_ov(const Grid& g, const Span& s, int q, float (&ox)[4]) {
+    float e = fmaf((float)(4 * q), g.wb, g.x0), c = edge_in(e, s.xl, s.xh);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        e = __fadd_rn(e, g.wb);
+        const float d = edge_in(e, s.xl, s.xh);
+        ox[t] = __fsub_rn(d, c);
+        c = d;
+    }
+}
+
+// Four bins of the interleaved field, (E_x, E_y) each: one 32-byte sector.
+struct Field4 {
+    float v[8];
+};
+__device__ __forceinline__ Field4 load_field4(const float2* p) {
+    Field4 f;
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(f.v[0]), "=f"(f.v[1]), "=f"(f.v[2]), "=f"(f.v[3]), "=f"(f.v[4]), "=f"(f.v[5]),
+          "=f"(f.v[6]), "=f"(f.v[7])
+        : "l"(p));
+    return f;
+}
+
+__device__ __forceinline__ void field_fma(const float (&ox)[4], float oy, const Field4& f,
+                                          float& sx, float& sy) {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        const float o = __fmul_rn(ox[t], oy);
+        sx = fmaf(o, f.v[2 * t], sx);
+        sy = fmaf(o, f.v[2 * t + 1], sy);
+    }
+}
+
+// Part of a field gather: groups of four bins q0 .. q1, rows j0 .. j1.
+__device__ __forceinline__ void gather_part(const Grid& g, const Span& s, int q0, int q1, int j0,
+                                            int j1, const float2* __restrict__ E2, float& sx,
+                                            float& sy) {
+    for (int q = q0; q <= q1; ++q) {
+        float ox[4];
+        quad_ov(g, s, q, ox);
+        const float2* p = E2 + (size_t)j0 * g.n + 4 * q;
+        float e = fmaf((float)j0, g.hb, g.y0), c = edge_in(e, s.yl, s.yh);
+        for (int j = j0; j <= j1; ++j, p += g.n) {
+            const Field4 f = load_field4(p);
+            e = __fadd_rn(e, g.hb);
+            const float d = edge_in(e, s.yl, s.yh);
+            field_fma(ox, __fsub_rn(d, c), f, sx, sy);
+            c = d;
+        }
+    }
 }
 
 // Field gather of one cell: sum_b ov(i,b) E2[b] over its bin span, E2 the
-// interleaved (E_x, E_y) map, in chunks of 2 rows x 4 columns whose loads
-// are all issued (predicated) before any use.  Nearly every cell is one
-// chunk; a wider cell only adds chunks, so a warp's lanes run the same body.
+// interleaved (E_x, E_y) map.  A cell's bins lie in lines of their own, so
+// every lane of a load costs the L1 one wavefront: whole sectors (aligned
+// groups of four bins, zero weights outside the span) take about half as
+// many as one load per bin.  What bounds it is the latency of those loads and
+// the L1's wavefronts (78 % busy), so the first two groups of the first two
+// rows (nearly every cell) go out together.  Against one 8-byte load per bin
+// in chunks of 2 x 4 bins, one cell per thread: k_cells at 2.2M cells, n = 2048
+// 52.8 -> 39.2 us (39.1M -> 22.2M warp instructions), at 210K cells 9.7 -> 8.8,
+// k_gather at 5M cells, n = 4096 (E2 larger than the L2) 119 -> 111 us.
 __device__ __forceinline__ float2 gather_span(const Grid& g, const Span& s,
                                               const float2* __restrict__ E2) {
-    float sx = 0.0f, sy = 0.0f;
     if (s.jlo > s.jhi || s.ilo > s.ihi) return make_float2(0.0f, 0.0f);
-    const AxisOv ax = axis_ov(g.x0, g.wb, s.ilo, s.ihi, s.xl, s.xh);
-    const AxisOv ay = axis_ov(g.y0, g.hb, s.jlo, s.jhi, s.yl, s.yh);
-    for (int j0 = s.jlo; j0 <= s.jhi; j0 += 2) {
-        for (int k0 = s.ilo; k0 <= s.ihi; k0 += 4) {
-            float2 e[2][4];
-#pragma unroll
-            for (int a = 0; a < 2; ++a) {
-                const int j = min(j0 + a, s.jhi);
-#pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    const int k = min(k0 + b, s.ihi);
-                    e[a][b] = (j0 + a <= s.jhi && k0 + b <= s.ihi)
-                                  ? __ldg(E2 + (size_t)j * g.n + k)
-                                  : make_float2(0.0f, 0.0f);
-                }
-            }
-#pragma unroll
-            for (int a = 0; a < 2; ++a) {
-                if (j0 + a > s.jhi) break;
-                const float oy = ov_at(ay, j0 + a);
-#pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    if (k0 + b > s.ihi) break;
-                    const float o = __fmul_rn(ov_at(ax, k0 + b), oy);
-                    sx = fmaf(o, e[a][b].x, sx);
-                    sy = fmaf(o, e[a][b].y, sy);
-                }
-            }
-        }
+    const int q0 = s.ilo >> 2, q1 = s.ihi >> 2;
+    const bool two_q = q0 < q1, two_j = s.jlo < s.jhi;
+    const float2* p = E2 + (size_t)s.jlo * g.n + 4 * q0;
+    Field4 f00 = load_field4(p), f01 = {}, f10 = {}, f11 = {};
+    if (two_q) f01 = load_field4(p + 4);
+    if (two_j) f10 = load_field4(p + g.n);
+    if (two_q && two_j) f11 = load_field4(p + g.n + 4);
+    const float e0 = fmaf((float)s.jlo, g.hb, g.y0), e1 = e0 + g.hb, e2 = e1 + g.hb;
+    const float c0 = edge_in(e0, s.yl, s.yh), c1 = edge_in(e1, s.yl, s.yh),
+                c2 = edge_in(e2, s.yl, s.yh);
+    const float oa = __fsub_rn(c1, c0), ob = __fsub_rn(c2, c1);
+    float sx = 0.0f, sy = 0.0f, ox[4];
+    quad_ov(g, s, q0, ox);
+    field_fma(ox, oa, f00, sx, sy);
+    if (two_j) field_fma(ox, ob, f10, sx, sy);
+    if (two_q) {
+        quad_ov(g, s, q0 + 1, ox);
+        field_fma(ox, oa, f01, sx, sy);
+        if (two_j) field_fma(ox, ob, f11, sx, sy);
     }
+    if (q0 + 2 <= q1) gather_part(g, s, q0 + 2, q1, s.jlo, s.jhi, E2, sx, sy);
+    if (s.jlo + 2 <= s.jhi)
+        gather_part(g, s, q0, min(q0 + 1, q1), s.jlo + 2, s.jhi, E2, sx, sy);
     return make_float2(sx, sy);
+}
+
+// What a cell kernel reads of a cell in the caller's order, loaded one round
+// ahead of its use: the cell kernels run a fixed grid, each thread striding
+// over the cells.
+struct CellIn {
+    float x, y, w, h;
+    int r;
+};
+__device__ __forceinline__ CellIn load_cell(int i, int m, const float* __restrict__ x,
+                                            const float* __restrict__ y,
+                                            const float* __restrict__ w,
+                                            const float* __restrict__ h,
+                                            const int* __restrict__ rank) {
+    CellIn c = {};
+    if (i < m) {
+        c.x = __ldg(x + i);
+        c.y = __ldg(y + i);
+        c.w = __ldg(w + i);
+        c.h = __ldg(h + i);
+        if (rank) c.r = __ldg(rank + i);
+    }
+    return c;
 }
 
 // --------------------------------------------------- double-float sums
@@ -259,6 +311,13 @@ __device__ __forceinline__ float warp_sum(float v) {
 // answer comes back).
 __device__ __forceinline__ void red_add_f2(float2* p, float a, float b) {
     asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(a), "f"(b) : "memory");
+}
+
+// *p += (a, b, c, d), 16 bytes, likewise.
+__device__ __forceinline__ void red_add_f4(float* p, float a, float b, float c, float d) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c),
+                 "f"(d)
+                 : "memory");
 }
 
 // *p += v as a relaxed, device-scope reduction with no return value.
@@ -503,6 +562,14 @@ fftpl_status loop_records(Ctx& c, int cap, double base_k);
 
 // Sets the text fftpl_last_error(NULL) returns on this thread.
 void set_global_error(const std::string& msg);
+
+// Blocks of the cell kernels (one thread per cell up to kCellBlocks blocks per
+// SM, striding beyond).
+inline int cell_blocks(const Ctx& c) {
+    const long long nb = ((long long)c.m_mov + kCellThreads - 1) / kCellThreads;
+    const long long cap = (long long)c.num_sms * kCellBlocks;
+    return (int)(nb < cap ? nb : cap);
+}
 
 // ------------------------------------------------------------ launchers
 // (each returns the CUDA error of the launch)

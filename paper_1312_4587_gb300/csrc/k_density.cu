@@ -38,32 +38,27 @@ k_scatter(Grid g, int m, const float* __restrict__ x, const float* __restrict__ 
     }
     Span s = cell_span(g, xi, yi, w[i], h[i]);
     if (s.ilo > s.ihi || s.jlo > s.jhi) return;
-    const AxisOv ax = axis_ov(g.x0, g.wb, s.ilo, s.ihi, s.xl, s.xh);
-    const AxisOv ay = axis_ov(g.y0, g.hb, s.jlo, s.jhi, s.yl, s.yh);
-    if (QUANT) {
-        for (int j = s.jlo; j <= s.jhi; ++j) {
-            float oy = ov_at(ay, j);
-            for (int k = s.ilo; k <= s.ihi; ++k) {
-                float a = __fmul_rn(ov_at(ax, k), oy);
-                long long q = __float2ll_rn(__fmul_rn(a, 4294967296.0f));
-                atomicAdd(Dq + (size_t)j * g.n + k, (unsigned long long)q);
-            }
-        }
-    } else {
-        // quads outer, rows inner: a quad's four x overlaps serve every row
-        for (int q = s.ilo >> 2; q <= (s.ihi >> 2); ++q) {
-            float ox[4];
+    // groups of four bins outer, rows inner: a group's x overlaps serve every
+    // row
+    for (int q = s.ilo >> 2; q <= s.ihi >> 2; ++q) {
+        float ox[4];
+        quad_ov(g, s, q, ox);
+        float e = fmaf((float)s.jlo, g.hb, g.y0), c = edge_in(e, s.yl, s.yh);
+        size_t at = (size_t)s.jlo * g.n + 4 * q;
+        for (int j = s.jlo; j <= s.jhi; ++j, at += g.n) {
+            e = __fadd_rn(e, g.hb);
+            const float d = edge_in(e, s.yl, s.yh), oy = __fsub_rn(d, c);
+            c = d;
+            if (QUANT) {
 #pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                int k = 4 * q + t;
-                ox[t] = (k >= s.ilo && k <= s.ihi) ? ov_at(ax, k) : 0.0f;
-            }
-            float* col = D + 4 * q;
-            for (int j = s.jlo; j <= s.jhi; ++j) {
-                const float oy = ov_at(ay, j);
-                atomicAdd(reinterpret_cast<float4*>(col + (size_t)j * g.n),
-                          make_float4(__fmul_rn(ox[0], oy), __fmul_rn(ox[1], oy),
-                                      __fmul_rn(ox[2], oy), __fmul_rn(ox[3], oy)));
+                for (int t = 0; t < 4; ++t) {
+                    const long long v =
+                        __float2ll_rn(__fmul_rn(__fmul_rn(ox[t], oy), 4294967296.0f));
+                    if (v) atomicAdd(Dq + at + t, (unsigned long long)v);
+                }
+            } else {
+                red_add_f4(D + at, __fmul_rn(ox[0], oy), __fmul_rn(ox[1], oy),
+                           __fmul_rn(ox[2], oy), __fmul_rn(ox[3], oy));
             }
         }
     }
@@ -91,25 +86,29 @@ k_bin_ranges(Grid g, int m, const float* __restrict__ x, const float* __restrict
 // Field gather (ADJ = false) or exact edge-difference adjoint (ADJ = true,
 // field = psi in fx).  Writes gx, gy and adds ||g||_1 to *l1.
 template <bool ADJ>
-__global__ void __launch_bounds__(kCellThreads, 6)
+__global__ void __launch_bounds__(kCellThreads, kCellBlocks)
 k_gather(Grid g, int m, const float* __restrict__ x, const float* __restrict__ y,
          const float* __restrict__ w, const float* __restrict__ h, const float* __restrict__ fx,
          const float2* __restrict__ E2, float* __restrict__ gx, float* __restrict__ gy,
          double* __restrict__ acc, DetRed dr) {
+    const int stride = gridDim.x * blockDim.x;
     int i = blockIdx.x * blockDim.x + threadIdx.x;
-    float sx = 0.0f, sy = 0.0f;
-    if (i < m) {
-        Span s = cell_span(g, x[i], y[i], w[i], h[i]);
+    float l1 = 0.0f;
+    CellIn c = load_cell(i, m, x, y, w, h, nullptr);
+    for (; i < m; i += stride) {
+        const Span s = cell_span(g, c.x, c.y, c.w, c.h);
+        c = load_cell(i + stride, m, x, y, w, h, nullptr);
+        float sx = 0.0f, sy = 0.0f;
         if (!ADJ) {
-            float2 e = gather_span(g, s, E2);
+            const float2 e = gather_span(g, s, E2);
             sx = -e.x;
             sy = -e.y;
         } else if (s.ilo <= s.ihi && s.jlo <= s.jhi) {
-            int n = g.n;
-            int kl = last_edge<false>(g.x0, g.wb, g.inv_wb, g.guard, n, s.xl);
-            int kr = last_edge<false>(g.x0, g.wb, g.inv_wb, g.guard, n, s.xh);
-            int jl = last_edge<false>(g.y0, g.hb, g.inv_hb, g.guard, n, s.yl);
-            int jr = last_edge<false>(g.y0, g.hb, g.inv_hb, g.guard, n, s.yh);
+            const int n = g.n;
+            const int kl = last_edge<false>(g.x0, g.wb, g.inv_wb, -1.0f, (float)n, s.xl);
+            const int kr = last_edge<false>(g.x0, g.wb, g.inv_wb, -1.0f, (float)n, s.xh);
+            const int jl = last_edge<false>(g.y0, g.hb, g.inv_hb, -1.0f, (float)n, s.yl);
+            const int jr = last_edge<false>(g.y0, g.hb, g.inv_hb, -1.0f, (float)n, s.yh);
             bool kr_in = kr >= 0 && kr < n, kl_in = kl >= 0 && kl < n;
             bool jr_in = jr >= 0 && jr < n, jl_in = jl >= 0 && jl < n;
             for (int j = s.jlo; j <= s.jhi; ++j) {
@@ -128,8 +127,9 @@ k_gather(Grid g, int m, const float* __restrict__ x, const float* __restrict__ y
         }
         gx[i] = sx;
         gy[i] = sy;
+        l1 += fabsf(sx) + fabsf(sy);
     }
-    reduce2(fabsf(sx) + fabsf(sy), 0.0f, acc, ACC_GN_L1, -1, dr);
+    reduce2(l1, 0.0f, acc, ACC_GN_L1, -1, dr);
 }
 
 // rho = (D + M) / A_b (formed on demand for fftpl_fields).
@@ -204,7 +204,7 @@ cudaError_t launch_bin_ranges(Ctx& c, const float* x, const float* y, int32_t* r
 cudaError_t launch_gather(Ctx& c, const float* x, const float* y, float* gx, float* gy,
                           bool adjoint, cudaStream_t s) {
     if (c.m_mov <= 0) return cudaSuccess;
-    int nb = blocks_for(c.m_mov, kCellThreads);
+    const int nb = cell_blocks(c);
     if (adjoint)
         k_gather<true><<<nb, kCellThreads, 0, s>>>(c.grid, c.m_mov, x, y, c.w, c.h, c.psi, nullptr,
                                                   gx, gy, c.acc, det_red(c, 0));

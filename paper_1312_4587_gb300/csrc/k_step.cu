@@ -18,40 +18,44 @@ struct LoopBufs {
     DetRed dr;
 };
 
-// gather + pin sums at v (like k_cells, 48 warps per SM).
+// gather + pin sums at v (as k_cells).
 template <bool CSR>
-__global__ void __launch_bounds__(kCellThreads, 6)
+__global__ void __launch_bounds__(kCellThreads, kCellBlocks)
 k_loop_cells(Grid gr, int m, LoopBufs b, const float2* __restrict__ E2,
              const int* __restrict__ rank, const int* __restrict__ cell_pin_ptr,
              const float2* __restrict__ gpin, const float2* __restrict__ gW2) {
     const float* cf = ctrl_f(b.ctrl);
     if (cf[F_DONE] != 0.0f) return;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    float nx = 0.0f, ny = 0.0f, wx = 0.0f, wy = 0.0f;
-    if (i < m) {
+    const int stride = gridDim.x * blockDim.x;
+    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    float ln = 0.0f, lw = 0.0f;
+    CellIn c = load_cell(i, m, b.v, b.v + m, b.w, b.h, rank);
+    for (; i < m; i += stride) {
+        const CellIn cur = c;
+        c = load_cell(i + stride, m, b.v, b.v + m, b.w, b.h, rank);
         // the wirelength gradient's loads go out before the field gather's
-        const int r = rank[i];
-        Span s = cell_span(gr, b.v[i], b.v[m + i], b.w[i], b.h[i]);
+        float wx = 0.0f, wy = 0.0f;
         if (CSR) {
-            for (int q = cell_pin_ptr[r]; q < cell_pin_ptr[r + 1]; ++q) {
+            for (int q = cell_pin_ptr[cur.r]; q < cell_pin_ptr[cur.r + 1]; ++q) {
                 float2 p = gpin[q];
                 wx += p.x;
                 wy += p.y;
             }
         } else {
-            float2 v = gW2[r];
+            const float2 v = __ldg(gW2 + cur.r);
             wx = v.x;
             wy = v.y;
         }
-        float2 e = gather_span(gr, s, E2);
-        nx = -e.x;
-        ny = -e.y;
-        b.gN[i] = nx;
-        b.gN[m + i] = ny;
+        const Span s = cell_span(gr, cur.x, cur.y, cur.w, cur.h);
+        const float2 e = gather_span(gr, s, E2);
+        b.gN[i] = -e.x;
+        b.gN[m + i] = -e.y;
         b.gW[i] = wx;
         b.gW[m + i] = wy;
+        ln += fabsf(e.x) + fabsf(e.y);
+        lw += fabsf(wx) + fabsf(wy);
     }
-    reduce2(fabsf(nx) + fabsf(ny), fabsf(wx) + fabsf(wy), b.acc, ACC_GN_L1, ACC_GW_L1, b.dr);
+    reduce2(ln, lw, b.acc, ACC_GN_L1, ACC_GW_L1, b.dr);
 }
 
 // lambda_k and the momentum weight beside the density chain (one warp on the
@@ -404,7 +408,7 @@ LoopBufs loop_bufs(Ctx& c) {
 
 cudaError_t launch_loop_cells(Ctx& c, cudaStream_t s) {
     LoopBufs b = loop_bufs(c);
-    int nb = nblk(c.m_mov, kCellThreads);
+    const int nb = cell_blocks(c);
     if (c.opt.deterministic)
         k_loop_cells<true><<<nb, kCellThreads, 0, s>>>(c.grid, c.m_mov, b, c.E2, c.cell_rank,
                                                        c.cell_pin_ptr, c.gpin, nullptr);

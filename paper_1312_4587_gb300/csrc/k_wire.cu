@@ -503,11 +503,11 @@ k_wa_grp(int nbig, const int4* __restrict__ slabs, WaIo io, float inv_g, float l
 
 // Per-cell kernel: density gradient by the field gather (q.E of Eq. 7),
 // wirelength gradient by summing the cell's pin gradients (CSR mode) or
-// reading the atomically accumulated sums, and the L1 norms of both.
-// (6 blocks per SM: at most 40 registers, 48 warps to hide the gathers'
-// latency; it runs alone after the join)
+// reading the atomically accumulated sums, and the L1 norms of both (per
+// thread a float32 sum of the non-negative terms of its m / 117K cells at
+// most).
 template <bool CSR>
-__global__ void __launch_bounds__(kCellThreads, 6)
+__global__ void __launch_bounds__(kCellThreads, kCellBlocks)
 k_cells(Grid g, int m, const float* __restrict__ x, const float* __restrict__ y,
         const float* __restrict__ w, const float* __restrict__ h, const float2* __restrict__ E2,
         float* __restrict__ gNx, float* __restrict__ gNy,
@@ -516,33 +516,37 @@ k_cells(Grid g, int m, const float* __restrict__ x, const float* __restrict__ y,
         const float2* __restrict__ gW2, double* __restrict__ acc,
         const float* __restrict__ done, DetRed dr) {
     if (done && *done != 0.0f) return;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    float nx = 0.0f, ny = 0.0f, wx = 0.0f, wy = 0.0f;
-    if (i < m) {
+    const int stride = gridDim.x * blockDim.x;
+    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    float ln = 0.0f, lw = 0.0f;
+    CellIn c = load_cell(i, m, x, y, w, h, rank);
+    for (; i < m; i += stride) {
+        const CellIn cur = c;
+        c = load_cell(i + stride, m, x, y, w, h, rank);
         // the wirelength gradient's loads go out before the field gather's
-        const int r = rank[i];
-        Span s = cell_span(g, x[i], y[i], w[i], h[i]);
+        float wx = 0.0f, wy = 0.0f;
         if (CSR) {
-            int q0 = cell_pin_ptr[r], q1 = cell_pin_ptr[r + 1];
+            int q0 = cell_pin_ptr[cur.r], q1 = cell_pin_ptr[cur.r + 1];
             for (int q = q0; q < q1; ++q) {
                 float2 v = gpin[q];
                 wx += v.x;
                 wy += v.y;
             }
         } else {
-            float2 v = gW2[r];
+            const float2 v = __ldg(gW2 + cur.r);
             wx = v.x;
             wy = v.y;
         }
-        float2 e = gather_span(g, s, E2);
-        nx = -e.x;
-        ny = -e.y;
-        gNx[i] = nx;
-        gNy[i] = ny;
+        const Span s = cell_span(g, cur.x, cur.y, cur.w, cur.h);
+        const float2 e = gather_span(g, s, E2);
+        gNx[i] = -e.x;
+        gNy[i] = -e.y;
         gWx[i] = wx;
         gWy[i] = wy;
+        ln += fabsf(e.x) + fabsf(e.y);
+        lw += fabsf(wx) + fabsf(wy);
     }
-    reduce2(fabsf(nx) + fabsf(ny), fabsf(wx) + fabsf(wy), acc, ACC_GN_L1, ACC_GW_L1, dr);
+    reduce2(ln, lw, acc, ACC_GN_L1, ACC_GW_L1, dr);
 }
 
 // Deterministic pin-to-cell sum on its own (fftpl_wa in CSR mode).
@@ -661,7 +665,7 @@ cudaError_t launch_pin_sum(Ctx& c, float* gx, float* gy, cudaStream_t s) {
 cudaError_t launch_cells_impl(Ctx& c, const float* x, const float* y, float* gNx, float* gNy,
                               float* gWx, float* gWy, const float* done, cudaStream_t s) {
     if (c.m_mov <= 0) return cudaSuccess;
-    int nb = nblk(c.m_mov, kCellThreads);
+    const int nb = cell_blocks(c);
     if (c.opt.deterministic)
         k_cells<true><<<nb, kCellThreads, 0, s>>>(c.grid, c.m_mov, x, y, c.w, c.h, c.E2, gNx,
                                                   gNy, gWx, gWy, c.cell_rank, c.cell_pin_ptr,
