@@ -2,11 +2,12 @@
 // the orchestration of one objective-gradient evaluation.
 //
 // One evaluation (Algorithm 1: f, density, FFT solve, gradient) runs as
-//   main stream: zero sums, zero D, scatter -> rows_fwd -> cols -> rows_inv
-//   side stream: (zero gW) -> WA                       (forked, concurrent)
+//   main stream: one memset (density map, sums, wirelength accumulator),
+//                scatter -> rows_fwd -> cols -> rows_inv
+//   side stream: WA                                (forked, concurrent)
 //   main stream: join -> cells (gather + pin sums + norms)
-// (with host outputs the WA branch writes grad W~ itself and the main
-// stream ends with the field gather before the join)
+// (with host outputs WA runs before the transforms and its gradient is
+// written beside them; the main stream ends with the field gather)
 // and, when use_graphs is set, is replayed from a captured CUDA graph.
 #include <math.h>
 #include <string.h>
@@ -317,6 +318,13 @@ cudaError_t launch_tau(Ctx& c, cudaStream_t s) {
     return c.tc ? launch_tc(c, 0, s) : launch_rows_fwd(c, s);
 }
 
+// Zeroes the sums and what the branches accumulate into, one memset.
+cudaError_t enqueue_zero(Ctx& c, bool dens, bool wa, cudaStream_t s) {
+    const size_t b = dens ? 0 : c.zero_density;
+    const size_t e = wa ? c.zero_bytes : c.zero_density + kAccDoubles * sizeof(double);
+    return cudaMemsetAsync(c.zero_block + b, 0, e - b, s);
+}
+
 // ---------------------------------------------------------------- evaluation
 // EV_HOST: the gradient arrays are pinned host memory written over the link
 enum { EV_DENSITY = 1, EV_WA = 2, EV_ADJOINT = 4, EV_NO_GATHER = 8, EV_HOST = 16 };
@@ -329,43 +337,56 @@ fftpl_status enqueue_eval(Ctx& c, const float* x, const float* y, float gamma, i
                           float* gNx, float* gNy, float* gWx, float* gWy,
                           float* stage = nullptr) {
     cudaStream_t s = c.stream;
-    size_t nn = (size_t)c.n * c.n;
-    CK(cudaMemsetAsync(c.acc, 0, kAccDoubles * sizeof(double), s));
     bool dens = (what & EV_DENSITY) != 0, wa = (what & EV_WA) != 0;
-    const bool grads = !(what & EV_NO_GATHER);
-    // with both branches the scatter also writes the WA kernel's positions,
-    // and the WA branch forks after it.  Device outputs: after the join one
-    // cell kernel writes both gradients (measured 18 % faster than a
-    // separate WA gradient pass beside the chain).  Host outputs (and the
-    // other combinations): the WA branch ends with its own gradient pass, so
-    // that its writes over the host link overlap the density chain (5 %
-    // faster end to end).
-    const bool pos_from_scatter = dens && wa;
+    const bool grads = !(what & EV_NO_GATHER), host = (what & EV_HOST) != 0;
     const bool fused = dens && wa && grads && !(what & (EV_ADJOINT | EV_HOST));
-    auto wa_branch = [&](bool interleave) -> fftpl_status {
-        CK(cudaEventRecord(c.ev_fork, s));
-        CK(cudaStreamWaitEvent(c.side, c.ev_fork, 0));
-        {
-            Stage st(c, 4, c.side);
-            if (!c.opt.deterministic)
-                CK(cudaMemsetAsync(c.gW2, 0, (size_t)c.m_mov * sizeof(float2), c.side));
-            CK(launch_wa_impl(c, x, y, gamma, nullptr, nullptr, interleave, c.side));
-            if (grads && !fused) CK(launch_pin_sum(c, gWx, gWy, c.side));
-        }
-        CK(cudaEventRecord(c.ev_join, c.side));
+    CK(enqueue_zero(c, dens, wa, s));
+    auto wa_kernel = [&](bool interleave, cudaStream_t q) -> fftpl_status {
+        Stage st(c, 4, q);
+        CK(launch_wa_impl(c, x, y, gamma, nullptr, nullptr, interleave, q));
         return FFTPL_OK;
     };
-    if (wa && !pos_from_scatter) TRY(wa_branch(true));
-    if (dens) {
-        {
-            Stage st(c, 0, s);
-            if (c.opt.deterministic) CK(cudaMemsetAsync(c.Dq, 0, nn * sizeof(long long), s));
-            else CK(cudaMemsetAsync(c.D, 0, nn * sizeof(float), s));
-            CK(launch_scatter_mov(c, x, y, pos_from_scatter, stage, s));
-        }
-        if (pos_from_scatter) TRY(wa_branch(false));
-        TRY(enqueue_solve(c, s));
+    auto fork = [&]() -> fftpl_status {
+        CK(cudaEventRecord(c.ev_fork, s));
+        CK(cudaStreamWaitEvent(c.side, c.ev_fork, 0));
+        return FFTPL_OK;
+    };
+    if (wa && !dens) {
+        // the wirelength alone: one chain on the main stream
+        TRY(wa_kernel(true, s));
+        if (grads) CK(launch_pin_sum(c, gWx, gWy, 0, s));
+        c.rho_valid = false;
+        c.split_valid = false;
+        c.fields_valid = false;
+        c.psi_valid = false;
+        return FFTPL_OK;
     }
+    {
+        // with both branches the scatter also writes the WA kernel's positions
+        Stage st(c, 0, s);
+        CK(launch_scatter_mov(c, x, y, wa, stage, s));
+    }
+    if (wa && host) {
+        // Host outputs: the link is what takes longest, so its first writes
+        // start as early as they can: the WA kernel with the GPU to itself
+        // (beside the transforms both branches' writes came at the end), its
+        // gradient pass on a few warps per SM (a full grid waiting for the
+        // link would keep the transforms' blocks out), the transforms and the
+        // gather beside it.
+        TRY(wa_kernel(false, s));
+        TRY(fork());
+        if (grads) CK(launch_pin_sum(c, gWx, gWy, 1, c.side));
+        CK(cudaEventRecord(c.ev_join, c.side));
+    } else if (wa) {
+        // the WA branch forks after the scatter; device outputs: after the
+        // join one cell kernel writes both gradients (a separate WA gradient
+        // pass beside the chain measured 18 % slower)
+        TRY(fork());
+        TRY(wa_kernel(false, c.side));
+        if (grads && !fused) CK(launch_pin_sum(c, gWx, gWy, 0, c.side));
+        CK(cudaEventRecord(c.ev_join, c.side));
+    }
+    TRY(enqueue_solve(c, s));
     const float* xs = stage ? stage : x;
     const float* ys = stage ? stage + c.m_mov : y;
     if (fused) {
@@ -373,7 +394,7 @@ fftpl_status enqueue_eval(Ctx& c, const float* x, const float* y, float gamma, i
         Stage st(c, 5, s);
         CK(launch_cells(c, xs, ys, gNx, gNy, gWx, gWy, s));
     } else {
-        if (dens && grads) {
+        if (grads) {
             if ((what & EV_ADJOINT) && !c.tc) CK(launch_rows_psi(c, s));
             Stage st(c, 5, s);
             CK(launch_gather(c, xs, ys, gNx, gNy, (what & EV_ADJOINT) != 0, s));
@@ -382,9 +403,9 @@ fftpl_status enqueue_eval(Ctx& c, const float* x, const float* y, float gamma, i
     }
     c.rho_valid = false;
     c.split_valid = false;
-    c.fields_valid = dens;
+    c.fields_valid = true;
     // the tensor-core solve writes psi; the adjoint gather formed it above
-    c.psi_valid = dens && (c.tc != nullptr || (what & EV_ADJOINT));
+    c.psi_valid = c.tc != nullptr || (what & EV_ADJOINT);
     return FFTPL_OK;
 }
 
@@ -415,9 +436,14 @@ void fill_report(const Ctx& c, const double* acc, fftpl_eval_report* rep) {
     rep->mov_area = c.mov_area;
 }
 
-fftpl_status read_report(Ctx& c, fftpl_eval_report* rep) {
-    CK(cudaMemcpyAsync(c.acc_host, c.acc, kAccDoubles * sizeof(double), cudaMemcpyDeviceToHost,
-                       c.stream));
+cudaError_t enqueue_report(Ctx& c) {
+    return cudaMemcpyAsync(c.acc_host, c.acc, kAccDoubles * sizeof(double), cudaMemcpyDeviceToHost,
+                           c.stream);
+}
+
+// enqueued: the sums are already on their way to the host mirror
+fftpl_status read_report(Ctx& c, fftpl_eval_report* rep, bool enqueued = false) {
+    if (!enqueued) CK(enqueue_report(c));
     CK(cudaStreamSynchronize(c.stream));
     if (rep) fill_report(c, c.acc_host, rep);
     return FFTPL_OK;
@@ -646,8 +672,8 @@ static fftpl_status build_slabs(Ctx& c, const fftpl_nets* nets, const fftpl_pins
         net_slot[e] = slabs[(size_t)(first_slab[d] + j / G)].x + (j % G) * L;
         net_lanes[e] = L;
     }
-    // the slabs of degree kBigMin..kBigMax first (k_wa_grp), the others
-    // after them in the same order (k_wa); the slot layout is unchanged
+    // the slabs of degree kBigMin..kBigMax first, the others
+    // after them in the same order ; the slot layout is unchanged
     auto is_big = [](const int4& sl) { return sl.y >= kBigMin && sl.y <= kBigMax; };
     std::stable_partition(slabs.begin(), slabs.end(), is_big);
     c.nbig = (int)std::count_if(slabs.begin(), slabs.end(), is_big);
@@ -762,19 +788,25 @@ static fftpl_status create_impl(Ctx& c, const fftpl_region* R, int32_t n, const 
     TRY(dalloc(c, &c.fix_x, c.m_fix));
     TRY(dalloc(c, &c.fix_y, c.m_fix));
     TRY(dalloc(c, &c.M, nn));
-    if (c.opt.deterministic) TRY(dalloc(c, &c.Dq, nn));
-    else TRY(dalloc(c, &c.D, nn));
+    c.zero_density = nn * (c.opt.deterministic ? sizeof(long long) : sizeof(float));
+    const size_t acc_bytes = kAccDoubles * sizeof(double);
+    c.zero_bytes = c.zero_density + acc_bytes +
+                   (c.opt.deterministic ? 0 : (size_t)c.m_mov * sizeof(float2));
+    TRY(dalloc(c, &c.zero_block, c.zero_bytes));
+    if (c.opt.deterministic) c.Dq = reinterpret_cast<long long*>(c.zero_block);
+    else c.D = reinterpret_cast<float*>(c.zero_block);
+    c.acc = reinterpret_cast<double*>(c.zero_block + c.zero_density);
+    if (!c.opt.deterministic)
+        c.gW2 = reinterpret_cast<float2*>(c.zero_block + c.zero_density + acc_bytes);
     TRY(dalloc(c, &c.T1, nn));
     TRY(dalloc(c, &c.PT, nn));
     TRY(dalloc(c, &c.RT, nn));
     spec_maps_init(c);
     TRY(dalloc(c, &c.psi, nn));
     TRY(dalloc(c, &c.E2, nn));
-    TRY(dalloc(c, &c.acc, kAccDoubles));
     TRY(dalloc(c, &c.err, 1));
     TRY(dalloc(c, &c.gN, 2 * (size_t)c.m_mov));
     TRY(dalloc(c, &c.gW, 2 * (size_t)c.m_mov));
-    TRY(dalloc(c, &c.gW2, (size_t)c.m_mov));
     TRY(dalloc(c, &c.pos2, (size_t)c.m_mov));
     if (c.opt.deterministic) {
         TRY(dalloc(c, &c.cell_pin_ptr, (size_t)c.m_mov + 1));
@@ -796,9 +828,7 @@ static fftpl_status create_impl(Ctx& c, const fftpl_region* R, int32_t n, const 
                                                                  (long long)(n / 128) * (n / 128)));
         if (c.opt.solve_path == FFTPL_SOLVE_TC_RADIX)
             cap0 = std::max<long long>(cap0, ((long long)(n / 2) * (n / 2 + 1) + 255) / 256);
-        long long cap1 = std::max<long long>(
-            ((long long)(c.nslabs - c.nbig) + kWaThreads / 32 - 1) / (kWaThreads / 32),
-            ((long long)c.nbig + kWaThreads / 32 - 1) / (kWaThreads / 32));
+        long long cap1 = (long long)wa_big_blocks(c) + wa_small_blocks(c);
         cap1 = std::max<long long>(cap1, ((long long)c.m_mov + kCellThreads - 1) / kCellThreads);
         c.det_cap[0] = (int)std::max<long long>(cap0, 1);
         c.det_cap[1] = (int)std::max<long long>(cap1, 1);
@@ -968,15 +998,19 @@ fftpl_status fftpl_wa(fftpl_t h, const float* x, const float* y, float gamma, do
 }
 
 // One full evaluation through the captured graph when use_graphs is set
-// (the graph is keyed by the buffers, gamma and the staging buffer).
+// (the graph is keyed by the buffers, gamma, the staging buffer and whether
+// it ends with the copy of the sums to the host); want: also enqueue that
+// copy.
 static fftpl_status eval_impl(Ctx& c, const float* x, const float* y, float gamma, float* gNx,
-                              float* gNy, float* gWx, float* gWy, float* stage) {
+                              float* gNy, float* gWx, float* gWy, float* stage, bool want) {
     // a staging buffer means x, y and the gradients are pinned host memory
     const int what = EV_DENSITY | EV_WA | (stage ? EV_HOST : 0);
     if (c.opt.use_graphs && !c.profiling) {
         float gk = gamma;
         const void* key[8] = {x, y, gNx, gNy, gWx, gWy, nullptr, stage};
+        const int32_t wk = want ? 1 : 0;
         memcpy(&key[6], &gk, sizeof(float));
+        memcpy((char*)&key[6] + sizeof(float), &wk, sizeof(wk));
         if (!c.eval_graph || memcmp(key, c.graph_key, sizeof(key)) != 0) {
             if (c.eval_graph) {
                 cudaGraphExecDestroy(c.eval_graph);
@@ -986,11 +1020,14 @@ static fftpl_status eval_impl(Ctx& c, const float* x, const float* y, float gamm
             CK(cudaStreamBeginCapture(c.stream, cudaStreamCaptureModeThreadLocal));
             int64_t before = c.launches;
             fftpl_status st = enqueue_eval(c, x, y, gamma, what, gNx, gNy, gWx, gWy, stage);
+            cudaError_t re = st == FFTPL_OK && want ? enqueue_report(c) : cudaSuccess;
             cudaError_t ee = cudaStreamEndCapture(c.stream, &g);
             if (st != FFTPL_OK) {
                 if (g) cudaGraphDestroy(g);
                 return st;
             }
+            if (re != cudaSuccess && g) cudaGraphDestroy(g);
+            CK(re);
             CK(ee);
             cudaError_t ie = cudaGraphInstantiate(&c.eval_graph, g, 0);
             cudaGraphDestroy(g);
@@ -1007,7 +1044,9 @@ static fftpl_status eval_impl(Ctx& c, const float* x, const float* y, float gamm
         c.psi_valid = c.tc != nullptr;
         return FFTPL_OK;
     }
-    return enqueue_eval(c, x, y, gamma, what, gNx, gNy, gWx, gWy, stage);
+    TRY(enqueue_eval(c, x, y, gamma, what, gNx, gNy, gWx, gWy, stage));
+    if (want) CK(enqueue_report(c));
+    return FFTPL_OK;
 }
 
 fftpl_status fftpl_eval(fftpl_t h, const float* x, const float* y, float gamma, float* gNx,
@@ -1019,8 +1058,8 @@ fftpl_status fftpl_eval(fftpl_t h, const float* x, const float* y, float gamma, 
     gNy = gNy ? gNy : scratch(c, 1);
     gWx = gWx ? gWx : scratch(c, 2);
     gWy = gWy ? gWy : scratch(c, 3);
-    TRY(eval_impl(c, x, y, gamma, gNx, gNy, gWx, gWy, nullptr));
-    if (rep) TRY(read_report(c, rep));
+    TRY(eval_impl(c, x, y, gamma, gNx, gNy, gWx, gWy, nullptr, rep != nullptr));
+    if (rep) TRY(read_report(c, rep, true));
     return FFTPL_OK;
 }
 
@@ -1060,17 +1099,18 @@ fftpl_status fftpl_eval_host(fftpl_t h, const float* x_host, const float* y_host
                    mapped_host(gWy_host)};
     if (m > 0 && xd && yd && gd[0] && gd[1] && gd[2] && gd[3]) {
         TRY(eval_impl(c, (const float*)xd, (const float*)yd, gamma, (float*)gd[0], (float*)gd[1],
-                      (float*)gd[2], (float*)gd[3], c.hx));
-        return read_report(c, rep);
+                      (float*)gd[2], (float*)gd[3], c.hx, true));
+        return read_report(c, rep, true);
     }
     CK(cudaMemcpyAsync(c.hx, x_host, m * sizeof(float), cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(c.hy, y_host, m * sizeof(float), cudaMemcpyHostToDevice, s));
-    TRY(eval_impl(c, c.hx, c.hy, gamma, c.hg, c.hg + m, c.hg + 2 * m, c.hg + 3 * m, nullptr));
+    TRY(eval_impl(c, c.hx, c.hy, gamma, c.hg, c.hg + m, c.hg + 2 * m, c.hg + 3 * m, nullptr,
+                  true));
     float* outs[4] = {gNx_host, gNy_host, gWx_host, gWy_host};
     for (int k = 0; k < 4; ++k)
         if (outs[k])
             CK(cudaMemcpyAsync(outs[k], c.hg + k * m, m * sizeof(float), cudaMemcpyDeviceToHost, s));
-    return read_report(c, rep);
+    return read_report(c, rep, true);
 }
 
 fftpl_status fftpl_report(fftpl_t h, fftpl_eval_report* rep) {
@@ -1171,10 +1211,7 @@ fftpl_status fftpl_place_init(fftpl_t h, const float* x0, const float* y0) {
     CK(launch_place_init(c, x0, y0, s));
     if (c.opt.gamma_fixed <= 0.0) {
         // gamma_0 from the overflow at the start
-        size_t nn = (size_t)c.n * c.n;
-        CK(cudaMemsetAsync(c.acc, 0, kAccDoubles * sizeof(double), s));
-        if (c.opt.deterministic) CK(cudaMemsetAsync(c.Dq, 0, nn * sizeof(long long), s));
-        else CK(cudaMemsetAsync(c.D, 0, nn * sizeof(float), s));
+        CK(enqueue_zero(c, true, false, s));
         CK(launch_scatter_mov(c, c.v, c.v + c.m_mov, false, nullptr, s));
         CK(launch_tau(c, s));
         CK(launch_gamma0(c, s));
@@ -1190,14 +1227,11 @@ extern "C++" {
 // `cells` also the per-cell gradients and lambda_k.
 static fftpl_status loop_eval(Ctx& c, bool cells) {
     cudaStream_t s = c.stream;
-    size_t nn = (size_t)c.n * c.n;
     const float* vx = c.v;
     const float* vy = c.v + c.m_mov;
-    CK(cudaMemsetAsync(c.acc, 0, kAccDoubles * sizeof(double), s));
+    CK(enqueue_zero(c, true, true, s));
     {
         Stage st(c, 0, s);
-        if (c.opt.deterministic) CK(cudaMemsetAsync(c.Dq, 0, nn * sizeof(long long), s));
-        else CK(cudaMemsetAsync(c.D, 0, nn * sizeof(float), s));
         CK(launch_scatter_mov(c, vx, vy, true, nullptr, s));
     }
     // the WA branch forks after the scatter, which wrote its positions
@@ -1205,8 +1239,6 @@ static fftpl_status loop_eval(Ctx& c, bool cells) {
     CK(cudaStreamWaitEvent(c.side, c.ev_fork, 0));
     {
         Stage st(c, 4, c.side);
-        if (!c.opt.deterministic)
-            CK(cudaMemsetAsync(c.gW2, 0, (size_t)c.m_mov * sizeof(float2), c.side));
         CK(launch_wa_impl(c, vx, vy, 1.0f, ctrl_f(c.ctrl) + F_INV_G, ctrl_f(c.ctrl) + F_DONE,
                           false, c.side));
         if (cells) CK(launch_ctrl_lambda(c, c.side));

@@ -36,9 +36,8 @@ constexpr int kCellThreads = 256;
 // 48.6 / 39.2 / 45.1 us (4: spills).
 constexpr int kCellBlocks = 3;
 constexpr int kWaThreads = 256;
-// Nets of degree kBigMin..kBigMax go to the WA kernel with several lanes per
-// net (k_wa_grp, grp_lanes(d) lanes each, at most 4 pins per lane); the rest
-// to k_wa (one lane per net).
+// Nets of degree kBigMin..kBigMax take several lanes per net in the WA kernel
+// (grp_lanes(d) lanes each, at most 4 pins per lane); the rest one lane.
 constexpr int kBigMin = 7;
 constexpr int kBigMax = 64;
 __host__ __device__ constexpr int grp_lanes(int d) {
@@ -356,11 +355,8 @@ struct DetRed {
     int cap;            // capacity in blocks
 };
 
-// add: the deterministic total is added to acc[q] instead of stored there
-// (for a second kernel on the same stream that reduces into the same
-// quantities after the first).
 __device__ __forceinline__ void reduce2(float a, float b, double* acc, int qa, int qb,
-                                        const DetRed& dr, bool add = false) {
+                                        const DetRed& dr) {
     if (!dr.part) {
         block_acc2(a, b, acc, qa, qb);
         return;
@@ -403,8 +399,8 @@ __device__ __forceinline__ void reduce2(float a, float b, double* acc, int qa, i
     if (threadIdx.x == 0) {
         double fa = 0.0, fb = 0.0;
         for (int k = 0; k < nw; ++k) { fa += s_a[k]; fb += s_b[k]; }
-        if (qa >= 0) acc[qa] = add ? acc[qa] + fa : fa;
-        if (qb >= 0) acc[qb] = add ? acc[qb] + fb : fb;
+        if (qa >= 0) acc[qa] = fa;
+        if (qb >= 0) acc[qb] = fb;
         __threadfence();
     }
 }
@@ -481,7 +477,7 @@ struct Ctx {
     int4* slabs = nullptr;      // {base slot, degree, net count, lanes per net (0: one
                                 // net per lane)}
     int nslabs = 0;
-    int nbig = 0;               // the first nbig slabs: degree kBigMin..kBigMax (k_wa_grp)
+    int nbig = 0;               // the first nbig slabs: degree kBigMin..kBigMax
     int num_sms = 1;            // of the handle's device
     int64_t slab_slots = 0;
     int32_t *pin_cell = nullptr, *pin_slot = nullptr, *cell_pin_ptr = nullptr;
@@ -498,6 +494,10 @@ struct Ctx {
     unsigned* det_ticket = nullptr;
     int det_cap[2] = {0, 0};
     double* acc = nullptr;
+    // what every evaluation starts from zero, in one block: the density map
+    // (D or Dq), the FP64 sums, the wirelength gradient accumulator
+    char* zero_block = nullptr;
+    size_t zero_density = 0, zero_bytes = 0;   // bytes of the map, of the block
     int* err = nullptr;
     double* acc_host = nullptr;   // pinned mirror
 
@@ -606,9 +606,12 @@ cudaError_t launch_wa(Ctx& c, const float* x, const float* y, float gamma, cudaS
 cudaError_t launch_wa_impl(Ctx& c, const float* x, const float* y, float gamma,
                            const float* scale_dev, const float* done, bool interleave,
                            cudaStream_t s);
-cudaError_t launch_pin_sum(Ctx& c, float* gx, float* gy, cudaStream_t s);
+cudaError_t launch_pin_sum(Ctx& c, float* gx, float* gy, int blocks_per_sm, cudaStream_t s);
 // 1 when the WA kernel runs slab pairs per warp (large instances)
 int wa_pairs(const Ctx& c);
+// blocks of the WA kernel: slabs of degree kBigMin..kBigMax, and the others
+int wa_big_blocks(const Ctx& c);
+int wa_small_blocks(const Ctx& c);
 
 // create-time netlist layout (k_setup.cu): label rounds for the internal
 // cell numbers (seeds every kSeedStride cells, kLabelRounds rounds, nets of

@@ -23,12 +23,12 @@ namespace fftpl {
 // base + 32 k + j: one warp per slab, one lane per net, every lane walks the
 // same d pins (no divergence), each pin-record read of the warp is one
 // contiguous access, and the cell-centre gathers of a slab touch nearby
-// lines (cells are numbered by regions of the netlist).  k_wa takes these
+// lines (cells are numbered by regions of the netlist)
 // (degree 2..6: the bulk of the nets, a body specialised for the degree,
 // pin coordinates in registers, two slabs per warp for degree 2..4 on large
 // instances; above kBigMax: runtime degree, coordinates staged in pxy).
-// k_wa_grp takes the slabs of degree kBigMin..kBigMax, several lanes per net
-// with shuffle reductions (see wa_group).
+// The slabs of degree kBigMin..kBigMax take several lanes per net with shuffle
+// reductions (see wa_group), in blocks of their own of the same launch.
 
 // (x, y) -> interleaved positions at each cell's internal number, so that
 // one 8-byte load (one sector) fetches a pin's cell centre and the pins of a
@@ -313,50 +313,6 @@ __device__ __forceinline__ void wa_slab(const WaIo& io, const int4& sl, int lane
     }
 }
 
-// pairs != 0: one warp per pair of consecutive slabs (2w, 2w+1); when both
-// have the same degree 2..4 (most nets) each lane runs its two nets with
-// their loads in flight together, otherwise the slabs go one after the
-// other.  pairs == 0: one warp per slab (small instances, where the GPU has
-// room for a warp per slab and latency matters more).
-template <bool CSR, bool LSE>
-__global__ void __launch_bounds__(kWaThreads, 4)
-k_wa(int nslabs, int pairs, const int4* __restrict__ slabs, WaIo io, float inv_g, float l2g,
-     const float* __restrict__ scale_dev, double* __restrict__ acc,
-     const float* __restrict__ done, DetRed dr) {
-    if (done && *done != 0.0f) return;
-    const int warp = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
-    const int lane = threadIdx.x & 31;
-    // 1/gamma and log2(e)/gamma: from the loop's control mirror, or computed
-    // on the host (exp(t / g) = exp2(t * log2(e) / g))
-    if (scale_dev) {
-        const float2 sc = *reinterpret_cast<const float2*>(scale_dev);
-        inv_g = sc.x;
-        l2g = sc.y;
-    }
-    const int4 zero = make_int4(0, 0, 0, 0);
-    float wsum = 0.0f, hsum = 0.0f;
-    if (!pairs) {
-        const int4 sl = warp < nslabs ? slabs[warp] : zero;
-        wa_slab<CSR, LSE>(io, sl, lane, l2g, inv_g, wsum, hsum);
-        reduce2(wsum, hsum, acc, ACC_W, ACC_HPWL, dr);
-        return;
-    }
-    const int4 sa = 2 * warp < nslabs ? slabs[2 * warp] : zero;
-    const int4 sb = 2 * warp + 1 < nslabs ? slabs[2 * warp + 1] : zero;
-    if (sa.y == sb.y && sa.y >= 2 && sa.y <= 4) {
-        const bool la = lane < sa.z, lb = lane < sb.z;
-        switch (sa.y) {
-            case 2: wa_pair<2, CSR, LSE>(io, sa.x + lane, la, sb.x + lane, lb, l2g, inv_g, wsum, hsum); break;
-            case 3: wa_pair<3, CSR, LSE>(io, sa.x + lane, la, sb.x + lane, lb, l2g, inv_g, wsum, hsum); break;
-            default: wa_pair<4, CSR, LSE>(io, sa.x + lane, la, sb.x + lane, lb, l2g, inv_g, wsum, hsum); break;
-        }
-    } else {
-        wa_slab<CSR, LSE>(io, sa, lane, l2g, inv_g, wsum, hsum);
-        wa_slab<CSR, LSE>(io, sb, lane, l2g, inv_g, wsum, hsum);
-    }
-    reduce2(wsum, hsum, acc, ACC_W, ACC_HPWL, dr);
-}
-
 // ------------------------------------------------ slabs of degree 7..64
 // L = grp_lanes(d) lanes per net (2 up to degree 8, 4 up to 16, 8 up to 32,
 // 16 up to 64), 32 / L nets per warp, R = ceil(d / L) <= 4 pins per lane: lane
@@ -465,15 +421,21 @@ __device__ __forceinline__ void wa_group(const WaIo& io, const int4& sl, int lan
     }
 }
 
-// One warp per slab of degree kBigMin..kBigMax.  Runs after k_wa on the same
-// stream and adds to its totals.
+// Blocks below nb_big: one warp per slab of degree kBigMin..kBigMax (the
+// first nbig slabs; several lanes per net).  The others: the nslabs - nbig
+// slabs of degree 2..6 and above kBigMax.  pairs != 0: one warp per pair of
+// consecutive slabs (2w, 2w+1); when both have the same degree 2..4 (most
+// nets) each lane runs its two nets with their loads in flight together,
+// otherwise the slabs go one after the other.  pairs == 0: one warp per slab
+// (small instances, where the GPU has room for a warp per slab and latency
+// matters more).  One launch for both kinds: as two, the second waited for
+// the first one's last blocks.
 template <bool CSR, bool LSE>
-__global__ void __launch_bounds__(kWaThreads)
-k_wa_grp(int nbig, const int4* __restrict__ slabs, WaIo io, float inv_g, float l2g,
-         const float* __restrict__ scale_dev, double* __restrict__ acc,
-         const float* __restrict__ done, DetRed dr, int* __restrict__ err) {
+__global__ void __launch_bounds__(kWaThreads, 4)
+k_wa(int nb_big, int nbig, int nslabs, int pairs, const int4* __restrict__ slabs, WaIo io,
+     float inv_g, float l2g, const float* __restrict__ scale_dev, double* __restrict__ acc,
+     const float* __restrict__ done, DetRed dr, int* __restrict__ err) {
     if (done && *done != 0.0f) return;
-    const int warp = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     // 1/gamma and log2(e)/gamma: from the loop's control mirror, or computed
     // on the host (exp(t / g) = exp2(t * log2(e) / g))
@@ -482,11 +444,14 @@ k_wa_grp(int nbig, const int4* __restrict__ slabs, WaIo io, float inv_g, float l
         inv_g = sc.x;
         l2g = sc.y;
     }
+    const int4 zero = make_int4(0, 0, 0, 0);
     float wsum = 0.0f, hsum = 0.0f;
-    if (warp < nbig) {
-        const int4 sl = slabs[warp];
+    if ((int)blockIdx.x < nb_big) {
+        const int warp = blockIdx.x * (kWaThreads / 32) + (threadIdx.x >> 5);
+        const int4 sl = warp < nbig ? slabs[warp] : zero;
         // (L, R) is the same for the whole warp: no divergence
-        switch (sl.w * 8 + (sl.y + sl.w - 1) / sl.w) {
+        switch (sl.w ? sl.w * 8 + (sl.y + sl.w - 1) / sl.w : 0) {
+            case 0: break;
             case 2 * 8 + 4: wa_group<2, 4, CSR, LSE>(io, sl, lane, l2g, inv_g, wsum, hsum); break;
             case 4 * 8 + 2: wa_group<4, 2, CSR, LSE>(io, sl, lane, l2g, inv_g, wsum, hsum); break;
             case 4 * 8 + 3: wa_group<4, 3, CSR, LSE>(io, sl, lane, l2g, inv_g, wsum, hsum); break;
@@ -497,8 +462,24 @@ k_wa_grp(int nbig, const int4* __restrict__ slabs, WaIo io, float inv_g, float l
             case 16 * 8 + 4: wa_group<16, 4, CSR, LSE>(io, sl, lane, l2g, inv_g, wsum, hsum); break;
             default: if (lane == 0) atomicOr(err, ERR_BOUNDS); break;   // no such layout
         }
+    } else {
+        const int warp = (blockIdx.x - nb_big) * (kWaThreads / 32) + (threadIdx.x >> 5);
+        const int ia = nbig + (pairs ? 2 * warp : warp), ib = ia + 1;
+        const int4 sa = ia < nslabs ? slabs[ia] : zero;
+        const int4 sb = pairs && ib < nslabs ? slabs[ib] : zero;
+        if (pairs && sa.y == sb.y && sa.y >= 2 && sa.y <= 4) {
+            const bool la = lane < sa.z, lb = lane < sb.z;
+            switch (sa.y) {
+                case 2: wa_pair<2, CSR, LSE>(io, sa.x + lane, la, sb.x + lane, lb, l2g, inv_g, wsum, hsum); break;
+                case 3: wa_pair<3, CSR, LSE>(io, sa.x + lane, la, sb.x + lane, lb, l2g, inv_g, wsum, hsum); break;
+                default: wa_pair<4, CSR, LSE>(io, sa.x + lane, la, sb.x + lane, lb, l2g, inv_g, wsum, hsum); break;
+            }
+        } else {
+            wa_slab<CSR, LSE>(io, sa, lane, l2g, inv_g, wsum, hsum);
+            if (pairs) wa_slab<CSR, LSE>(io, sb, lane, l2g, inv_g, wsum, hsum);
+        }
     }
-    reduce2(wsum, hsum, acc, ACC_W, ACC_HPWL, dr, true);
+    reduce2(wsum, hsum, acc, ACC_W, ACC_HPWL, dr);
 }
 
 // Per-cell kernel: density gradient by the field gather (q.E of Eq. 7),
@@ -554,10 +535,10 @@ __global__ void __launch_bounds__(kCellThreads)
 k_pin_sum(int m, const int* __restrict__ rank, const int* __restrict__ cell_pin_ptr,
           const float2* __restrict__ gpin, float* __restrict__ gx, float* __restrict__ gy,
           double* __restrict__ acc, DetRed dr) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    float wx = 0.0f, wy = 0.0f;
-    if (i < m) {
+    float l1 = 0.0f;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
         const int r = rank[i];
+        float wx = 0.0f, wy = 0.0f;
         for (int q = cell_pin_ptr[r]; q < cell_pin_ptr[r + 1]; ++q) {
             float2 v = gpin[q];
             wx += v.x;
@@ -565,23 +546,24 @@ k_pin_sum(int m, const int* __restrict__ rank, const int* __restrict__ cell_pin_
         }
         gx[i] = wx;
         gy[i] = wy;
+        l1 += fabsf(wx) + fabsf(wy);
     }
-    reduce2(fabsf(wx) + fabsf(wy), 0.0f, acc, ACC_GW_L1, -1, dr);
+    reduce2(l1, 0.0f, acc, ACC_GW_L1, -1, dr);
 }
 
 // Splits the interleaved atomic accumulator into gx, gy and adds ||g||_1.
 __global__ void __launch_bounds__(kCellThreads)
 k_split(int m, const int* __restrict__ rank, const float2* __restrict__ gW2,
         float* __restrict__ gx, float* __restrict__ gy, double* __restrict__ acc, DetRed dr) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    float v = 0.0f;
-    if (i < m) {
+    float l1 = 0.0f;
+#pragma unroll 2
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
         float2 g = gW2[rank[i]];
         gx[i] = g.x;
         gy[i] = g.y;
-        v = fabsf(g.x) + fabsf(g.y);
+        l1 += fabsf(g.x) + fabsf(g.y);
     }
-    reduce2(v, 0.0f, acc, ACC_GW_L1, -1, dr);
+    reduce2(l1, 0.0f, acc, ACC_GW_L1, -1, dr);
 }
 
 static inline int nblk(long long m, int t) { return (int)((m + t - 1) / t); }
@@ -590,6 +572,12 @@ static inline int nblk(long long m, int t) { return (int)((m + t - 1) / t); }
 // over (4 CTAs of 8 warps per SM); below that, one slab per warp.
 int wa_pairs(const Ctx& c) {
     return (c.nslabs - c.nbig) >= 2LL * c.num_sms * 4 * (kWaThreads / 32) ? 1 : 0;
+}
+
+int wa_big_blocks(const Ctx& c) { return nblk(c.nbig, kWaThreads / 32); }
+int wa_small_blocks(const Ctx& c) {
+    const int n = c.nslabs - c.nbig;
+    return nblk(wa_pairs(c) ? (n + 1) / 2 : n, kWaThreads / 32);
 }
 
 cudaError_t launch_wa_impl(Ctx& c, const float* x, const float* y, float gamma,
@@ -607,41 +595,20 @@ cudaError_t launch_wa_impl(Ctx& c, const float* x, const float* y, float gamma,
     const bool det = c.opt.deterministic != 0;
     float inv_g = 0.0f, l2g = 0.0f;
     if (!scale_dev) wa_scale(gamma, &inv_g, &l2g);
-    // k_wa: the slabs after the first nbig (degree 2..6 and above kBigMax);
-    // it stores the deterministic totals, k_wa_grp (next, same stream) adds
-    const int nsmall = c.nslabs - c.nbig;
-    if (nsmall > 0) {
-        const int wpb = kWaThreads / 32;
-        const int pairs = wa_pairs(c);
-        const int nb = std::max(1, nblk(pairs ? (nsmall + 1) / 2 : nsmall, wpb));
-        auto go = [&](auto kern) {
-            kern<<<nb, kWaThreads, 0, s>>>(nsmall, pairs, c.slabs + c.nbig, io, inv_g, l2g,
-                                           scale_dev, c.acc, done, det_red(c, 1));
-        };
-        if (det) {
-            if (lse) go(k_wa<true, true>);
-            else go(k_wa<true, false>);
-        } else {
-            if (lse) go(k_wa<false, true>);
-            else go(k_wa<false, false>);
-        }
-        c.launches++;
+    const int pairs = wa_pairs(c);
+    const int nb_big = wa_big_blocks(c), nb = nb_big + wa_small_blocks(c);
+    auto go = [&](auto kern) {
+        kern<<<nb, kWaThreads, 0, s>>>(nb_big, c.nbig, c.nslabs, pairs, c.slabs, io, inv_g, l2g,
+                                       scale_dev, c.acc, done, det_red(c, 1), c.err);
+    };
+    if (det) {
+        if (lse) go(k_wa<true, true>);
+        else go(k_wa<true, false>);
+    } else {
+        if (lse) go(k_wa<false, true>);
+        else go(k_wa<false, false>);
     }
-    if (c.nbig > 0) {
-        const int nb = nblk(c.nbig, kWaThreads / 32);
-        auto go = [&](auto kern) {
-            kern<<<nb, kWaThreads, 0, s>>>(c.nbig, c.slabs, io, inv_g, l2g, scale_dev, c.acc,
-                                           done, det_red(c, 1), c.err);
-        };
-        if (det) {
-            if (lse) go(k_wa_grp<true, true>);
-            else go(k_wa_grp<true, false>);
-        } else {
-            if (lse) go(k_wa_grp<false, true>);
-            else go(k_wa_grp<false, false>);
-        }
-        c.launches++;
-    }
+    c.launches++;
     return cudaGetLastError();
 }
 
@@ -649,15 +616,18 @@ cudaError_t launch_wa(Ctx& c, const float* x, const float* y, float gamma, cudaS
     return launch_wa_impl(c, x, y, gamma, nullptr, nullptr, true, s);
 }
 
-cudaError_t launch_pin_sum(Ctx& c, float* gx, float* gy, cudaStream_t s) {
+// blocks_per_sm > 0 bounds the grid (the threads then stride over the cells).
+cudaError_t launch_pin_sum(Ctx& c, float* gx, float* gy, int blocks_per_sm, cudaStream_t s) {
     if (c.m_mov <= 0) return cudaSuccess;
-    // region 1: this pass follows the WA kernels on their stream
+    int nb = nblk(c.m_mov, kCellThreads);
+    if (blocks_per_sm > 0) nb = std::min(nb, blocks_per_sm * c.num_sms);
+    // region 1: this pass follows the WA kernel on its stream
     if (c.opt.deterministic)
-        k_pin_sum<<<nblk(c.m_mov, kCellThreads), kCellThreads, 0, s>>>(
-            c.m_mov, c.cell_rank, c.cell_pin_ptr, c.gpin, gx, gy, c.acc, det_red(c, 1));
+        k_pin_sum<<<nb, kCellThreads, 0, s>>>(c.m_mov, c.cell_rank, c.cell_pin_ptr, c.gpin, gx, gy,
+                                              c.acc, det_red(c, 1));
     else
-        k_split<<<nblk(c.m_mov, kCellThreads), kCellThreads, 0, s>>>(
-            c.m_mov, c.cell_rank, c.gW2, gx, gy, c.acc, det_red(c, 1));
+        k_split<<<nb, kCellThreads, 0, s>>>(c.m_mov, c.cell_rank, c.gW2, gx, gy, c.acc,
+                                            det_red(c, 1));
     c.launches++;
     return cudaGetLastError();
 }
