@@ -354,7 +354,7 @@ fftpl_status enqueue_eval(Ctx& c, const float* x, const float* y, float gamma, i
     if (wa && !dens) {
         // the wirelength alone: one chain on the main stream
         TRY(wa_kernel(true, s));
-        if (grads) CK(launch_pin_sum(c, gWx, gWy, 0, s));
+        if (grads) CK(launch_pin_sum(c, gWx, gWy, false, s));
         c.rho_valid = false;
         c.split_valid = false;
         c.fields_valid = false;
@@ -370,12 +370,10 @@ fftpl_status enqueue_eval(Ctx& c, const float* x, const float* y, float gamma, i
         // Host outputs: the link is what takes longest, so its first writes
         // start as early as they can: the WA kernel with the GPU to itself
         // (beside the transforms both branches' writes came at the end), its
-        // gradient pass on a few warps per SM (a full grid waiting for the
-        // link would keep the transforms' blocks out), the transforms and the
-        // gather beside it.
+        // gradient pass on a few SMs, the transforms and the gather beside it.
         TRY(wa_kernel(false, s));
         TRY(fork());
-        if (grads) CK(launch_pin_sum(c, gWx, gWy, 1, c.side));
+        if (grads) CK(launch_pin_sum(c, gWx, gWy, true, c.side));
         CK(cudaEventRecord(c.ev_join, c.side));
     } else if (wa) {
         // the WA branch forks after the scatter; device outputs: after the
@@ -383,7 +381,7 @@ fftpl_status enqueue_eval(Ctx& c, const float* x, const float* y, float gamma, i
         // pass beside the chain measured 18 % slower)
         TRY(fork());
         TRY(wa_kernel(false, c.side));
-        if (grads && !fused) CK(launch_pin_sum(c, gWx, gWy, 0, c.side));
+        if (grads && !fused) CK(launch_pin_sum(c, gWx, gWy, false, c.side));
         CK(cudaEventRecord(c.ev_join, c.side));
     }
     TRY(enqueue_solve(c, s));

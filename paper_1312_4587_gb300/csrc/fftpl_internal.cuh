@@ -606,7 +606,7 @@ cudaError_t launch_wa(Ctx& c, const float* x, const float* y, float gamma, cudaS
 cudaError_t launch_wa_impl(Ctx& c, const float* x, const float* y, float gamma,
                            const float* scale_dev, const float* done, bool interleave,
                            cudaStream_t s);
-cudaError_t launch_pin_sum(Ctx& c, float* gx, float* gy, int blocks_per_sm, cudaStream_t s);
+cudaError_t launch_pin_sum(Ctx& c, float* gx, float* gy, bool few, cudaStream_t s);
 // 1 when the WA kernel runs slab pairs per warp (large instances)
 int wa_pairs(const Ctx& c);
 // blocks of the WA kernel: slabs of degree kBigMin..kBigMax, and the others

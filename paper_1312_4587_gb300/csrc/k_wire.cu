@@ -531,7 +531,7 @@ k_cells(Grid g, int m, const float* __restrict__ x, const float* __restrict__ y,
 }
 
 // Deterministic pin-to-cell sum on its own (fftpl_wa in CSR mode).
-__global__ void __launch_bounds__(kCellThreads)
+__global__ void __launch_bounds__(1024)
 k_pin_sum(int m, const int* __restrict__ rank, const int* __restrict__ cell_pin_ptr,
           const float2* __restrict__ gpin, float* __restrict__ gx, float* __restrict__ gy,
           double* __restrict__ acc, DetRed dr) {
@@ -551,17 +551,29 @@ k_pin_sum(int m, const int* __restrict__ rank, const int* __restrict__ cell_pin_
     reduce2(l1, 0.0f, acc, ACC_GW_L1, -1, dr);
 }
 
-// Splits the interleaved atomic accumulator into gx, gy and adds ||g||_1.
-__global__ void __launch_bounds__(kCellThreads)
+// Splits the interleaved atomic accumulator into gx, gy and adds ||g||_1 (four
+// cells of a thread in flight together on a bounded grid).
+__global__ void __launch_bounds__(1024)
 k_split(int m, const int* __restrict__ rank, const float2* __restrict__ gW2,
         float* __restrict__ gx, float* __restrict__ gy, double* __restrict__ acc, DetRed dr) {
+    const int stride = gridDim.x * blockDim.x;
     float l1 = 0.0f;
-#pragma unroll 2
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
-        float2 g = gW2[rank[i]];
-        gx[i] = g.x;
-        gy[i] = g.y;
-        l1 += fabsf(g.x) + fabsf(g.y);
+    for (int i0 = blockIdx.x * blockDim.x + threadIdx.x; i0 < m; i0 += 4 * stride) {
+        float2 g[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int i = i0 + k * stride;
+            g[k] = i < m ? __ldg(gW2 + __ldg(rank + i)) : make_float2(0.0f, 0.0f);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int i = i0 + k * stride;
+            if (i < m) {
+                gx[i] = g[k].x;
+                gy[i] = g[k].y;
+                l1 += fabsf(g[k].x) + fabsf(g[k].y);
+            }
+        }
     }
     reduce2(l1, 0.0f, acc, ACC_GW_L1, -1, dr);
 }
@@ -616,17 +628,23 @@ cudaError_t launch_wa(Ctx& c, const float* x, const float* y, float gamma, cudaS
     return launch_wa_impl(c, x, y, gamma, nullptr, nullptr, true, s);
 }
 
-// blocks_per_sm > 0 bounds the grid (the threads then stride over the cells).
-cudaError_t launch_pin_sum(Ctx& c, float* gx, float* gy, int blocks_per_sm, cudaStream_t s) {
+// few: kLinkBlocks large blocks, for writes over the host link beside other
+// kernels.  A block waiting for the link keeps registers from the column pass
+// (two blocks fill an SM), so the writes take as few SMs as keep the link busy:
+// evaluation of 2.2M cells with host buffers, 8 / 16 / 32 / 64 blocks of 1024
+// threads 458 / 384 / 378 / 371 us, one block of 256 on every SM 413.
+constexpr int kLinkBlocks = 64;
+cudaError_t launch_pin_sum(Ctx& c, float* gx, float* gy, bool few, cudaStream_t s) {
     if (c.m_mov <= 0) return cudaSuccess;
-    int nb = nblk(c.m_mov, kCellThreads);
-    if (blocks_per_sm > 0) nb = std::min(nb, blocks_per_sm * c.num_sms);
+    const int threads = few ? 1024 : kCellThreads;
+    int nb = nblk(c.m_mov, threads);
+    if (few) nb = std::min(nb, kLinkBlocks);
     // region 1: this pass follows the WA kernel on its stream
     if (c.opt.deterministic)
-        k_pin_sum<<<nb, kCellThreads, 0, s>>>(c.m_mov, c.cell_rank, c.cell_pin_ptr, c.gpin, gx, gy,
+        k_pin_sum<<<nb, threads, 0, s>>>(c.m_mov, c.cell_rank, c.cell_pin_ptr, c.gpin, gx, gy,
                                               c.acc, det_red(c, 1));
     else
-        k_split<<<nb, kCellThreads, 0, s>>>(c.m_mov, c.cell_rank, c.gW2, gx, gy, c.acc,
+        k_split<<<nb, threads, 0, s>>>(c.m_mov, c.cell_rank, c.gW2, gx, gy, c.acc,
                                             det_red(c, 1));
     c.launches++;
     return cudaGetLastError();
