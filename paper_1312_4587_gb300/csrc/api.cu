@@ -325,6 +325,16 @@ cudaError_t enqueue_zero(Ctx& c, bool dens, bool wa, cudaStream_t s) {
     return cudaMemsetAsync(c.zero_block + b, 0, e - b, s);
 }
 
+// Up to this many cells the kernels of both branches of an evaluation are
+// launched as programmatic chains (launch_chain).  A call with one branch
+// always takes them: density alone 24.7 -> 15.6 us (1,000 cells), 35.0 -> 28.3
+// (210K, n = 512), 131 -> 124 (2.2M, n = 2048); wirelength alone 15.5 -> 10.4,
+// 24.0 -> 20.1, 101 -> 97.  With two branches the waiting blocks of one keep
+// the other's out once the GPU is full: evaluation by graph 16.5 -> 14.4 us
+// (1,000), 22.7 -> 20.6 (34K), 34.9 -> 32.9 (210K), but 58.2 -> 60.0 (500K) and
+// 204 -> 211 (2.2M).
+constexpr int kChainCells = 256 * 1024;
+
 // ---------------------------------------------------------------- evaluation
 // EV_HOST: the gradient arrays are pinned host memory written over the link
 enum { EV_DENSITY = 1, EV_WA = 2, EV_ADJOINT = 4, EV_NO_GATHER = 8, EV_HOST = 16 };
@@ -341,6 +351,7 @@ fftpl_status enqueue_eval(Ctx& c, const float* x, const float* y, float gamma, i
     const bool grads = !(what & EV_NO_GATHER), host = (what & EV_HOST) != 0;
     const bool fused = dens && wa && grads && !(what & (EV_ADJOINT | EV_HOST));
     CK(enqueue_zero(c, dens, wa, s));
+    c.chain = !(dens && wa) || c.m_mov <= kChainCells;
     auto wa_kernel = [&](bool interleave, cudaStream_t q) -> fftpl_status {
         Stage st(c, 4, q);
         CK(launch_wa_impl(c, x, y, gamma, nullptr, nullptr, interleave, q));
@@ -975,6 +986,7 @@ fftpl_status fftpl_gather(fftpl_t h, const float* x, const float* y, int32_t mod
     if (c.m_mov > 0 && (!x || !y || !gx || !gy)) return set_err(c, FFTPL_EINVAL, "null argument");
     if (mode != 0 && mode != 1) return set_err(c, FFTPL_EINVAL, "mode must be 0 or 1");
     if (!c.fields_valid) return set_err(c, FFTPL_ESTATE, "no density evaluation yet");
+    c.chain = false;   // what precedes it on the stream is the caller's
     if (mode == 1) TRY(ensure_psi(c, c.stream));
     CK(launch_gather(c, x, y, gx, gy, mode == 1, c.stream));
     return FFTPL_OK;
@@ -1130,6 +1142,7 @@ fftpl_status fftpl_fields(fftpl_t h, const float** rho, const float** psi, const
         *rho = c.rho;
     }
     if (psi) {
+        c.chain = false;
         TRY(ensure_psi(c, c.stream));
         *psi = c.psi;
     }
@@ -1210,6 +1223,7 @@ fftpl_status fftpl_place_init(fftpl_t h, const float* x0, const float* y0) {
     if (c.opt.gamma_fixed <= 0.0) {
         // gamma_0 from the overflow at the start
         CK(enqueue_zero(c, true, false, s));
+        c.chain = true;
         CK(launch_scatter_mov(c, c.v, c.v + c.m_mov, false, nullptr, s));
         CK(launch_tau(c, s));
         CK(launch_gamma0(c, s));
@@ -1228,6 +1242,7 @@ static fftpl_status loop_eval(Ctx& c, bool cells) {
     const float* vx = c.v;
     const float* vy = c.v + c.m_mov;
     CK(enqueue_zero(c, true, true, s));
+    c.chain = c.m_mov <= kChainCells;
     {
         Stage st(c, 0, s);
         CK(launch_scatter_mov(c, vx, vy, true, nullptr, s));
@@ -1268,6 +1283,7 @@ fftpl_status fftpl::loop_enqueue(Ctx& c) {
         return FFTPL_OK;
     }
     Stage st(c, 6, s);
+    c.chain = true;   // one branch again
     CK(launch_loop_g(c, s));
     CK(launch_loop_update(c, s));
     return FFTPL_OK;

@@ -253,6 +253,36 @@ __device__ __forceinline__ CellIn load_cell(int i, int m, const float* __restric
     return c;
 }
 
+// ------------------------------------------- programmatic dependent launch
+// A kernel launched with launch_chain may start while the kernel before it in
+// the stream still runs, from the moment every block of that one has called
+// chain_trigger; what it reads of it comes after chain_wait, which returns
+// when that kernel has completed.  Every kernel of a chain calls both (chain_wait
+// first among its reads), so that its completion also means its
+// predecessors'.  Both are no-ops in a plain launch.
+__device__ __forceinline__ void chain_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void chain_trigger() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_chain(void (*kern)(P...), int blocks, int threads, size_t smem, cudaStream_t s,
+                         bool chain, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = chain ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 // --------------------------------------------------- double-float sums
 // An unevaluated sum hi + lo of two floats (error-free transformations:
 // Knuth's TwoSum and Dekker's Fast2Sum).  Used to keep the grid-wide FP64
@@ -479,6 +509,7 @@ struct Ctx {
     int nslabs = 0;
     int nbig = 0;               // the first nbig slabs: degree kBigMin..kBigMax
     int num_sms = 1;            // of the handle's device
+    bool chain = false;         // launch_chain for the kernels being enqueued
     int64_t slab_slots = 0;
     int32_t *pin_cell = nullptr, *pin_slot = nullptr, *cell_pin_ptr = nullptr;
     float *pin_dx = nullptr, *pin_dy = nullptr;

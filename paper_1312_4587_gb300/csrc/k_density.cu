@@ -28,6 +28,7 @@ k_scatter(Grid g, int m, const float* __restrict__ x, const float* __restrict__ 
           const float* __restrict__ w, const float* __restrict__ h, const int* __restrict__ rank,
           float2* __restrict__ pos, float* __restrict__ stage, float* __restrict__ D,
           unsigned long long* __restrict__ Dq) {
+    chain_trigger();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m) return;
     const float xi = x[i], yi = y[i];
@@ -94,6 +95,7 @@ k_gather(Grid g, int m, const float* __restrict__ x, const float* __restrict__ y
     const int stride = gridDim.x * blockDim.x;
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     float l1 = 0.0f;
+    chain_wait();
     CellIn c = load_cell(i, m, x, y, w, h, nullptr);
     for (; i < m; i += stride) {
         const Span s = cell_span(g, c.x, c.y, c.w, c.h);
@@ -204,15 +206,14 @@ cudaError_t launch_bin_ranges(Ctx& c, const float* x, const float* y, int32_t* r
 cudaError_t launch_gather(Ctx& c, const float* x, const float* y, float* gx, float* gy,
                           bool adjoint, cudaStream_t s) {
     if (c.m_mov <= 0) return cudaSuccess;
-    const int nb = cell_blocks(c);
-    if (adjoint)
-        k_gather<true><<<nb, kCellThreads, 0, s>>>(c.grid, c.m_mov, x, y, c.w, c.h, c.psi, nullptr,
-                                                  gx, gy, c.acc, det_red(c, 0));
-    else
-        k_gather<false><<<nb, kCellThreads, 0, s>>>(c.grid, c.m_mov, x, y, c.w, c.h, nullptr, c.E2,
-                                                   gx, gy, c.acc, det_red(c, 0));
+    auto go = [&](auto kern) {
+        return launch_chain(kern, cell_blocks(c), kCellThreads, 0, s, c.chain, c.grid, c.m_mov, x,
+                            y, c.w, c.h, c.psi, c.E2, gx, gy, c.acc, det_red(c, 0));
+    };
+    const cudaError_t e = adjoint ? go(k_gather<true>) : go(k_gather<false>);
     c.launches++;
-    return cudaGetLastError();
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_rho(Ctx& c, cudaStream_t s) {

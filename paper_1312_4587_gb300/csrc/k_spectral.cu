@@ -516,6 +516,8 @@ k_rows_fwd(const float* __restrict__ D, const long long* __restrict__ Dq,
     if (smem_addr(smem) & 127u) tma = 0;   // the TMA unit's source alignment
     int pa, pb;
     const int ta = lane_rev<LOGN, 2>(lt, &pa);
+    chain_wait();
+    chain_trigger();
     // per-thread sums of 2 E non-negative terms in float32
     float tau = 0.0f, charge = 0.0f;
     float2 v[1][E];
@@ -638,6 +640,8 @@ k_cols(const float* __restrict__ T1, float* __restrict__ PT, float* __restrict__
     int k;
     {
         float2 v[1][E];
+        chain_wait();
+        chain_trigger();
         const float4* row = reinterpret_cast<const float4*>(T1 + (size_t)(u0 / 2 + f) * (2 * N));
 #pragma unroll
         for (int q = 0; q < E / 2; ++q) {
@@ -757,6 +761,8 @@ k_rows_inv(const float* __restrict__ PT, const float* __restrict__ RT, float2* _
     const float2* pr = reinterpret_cast<const float2*>(PT) + (size_t)j * N + k;
     const float2* rr = reinterpret_cast<const float2*>(RT) + (size_t)j * N + k;
     const size_t row0 = (size_t)(2 * j) * N, row1 = row0 + N;
+    chain_wait();
+    chain_trigger();
     if (WHAT != INV_PSI) {
         float2 z[2][E];
         {
@@ -1110,33 +1116,32 @@ static cudaError_t launch_all_logn(Ctx& c, int which, cudaStream_t s) {
     const float pi_lx = (float)(M_PI / c.Lx), pi_ly = (float)(M_PI / c.Ly);
     const int tma = c.spec_tma ? 1 : 0;
     auto inv = [&](auto kern, int nv) {
-        kern<<<nb1, L1::T, L1::GB * L1::group_bytes(nv), s>>>(c.PT, c.RT, c.E2, c.psi, c.ex, c.ey,
-                                                              pi_lx);
+        return launch_chain(kern, nb1, L1::T, L1::GB * L1::group_bytes(nv), s, c.chain, c.PT, c.RT,
+                            c.E2, c.psi, c.ex, c.ey, pi_lx);
     };
+    cudaError_t e = cudaSuccess;
     switch (which) {
         case PASS_FWD: {
             const int smem = L2::GB * L2::group_bytes(1);
-            if (c.opt.deterministic)
-                k_rows_fwd<LOGN, true><<<nb2, L2::T, smem, s>>>(nullptr, c.Dq, c.M, inv_ab, cap,
-                                                                c.T1, c.acc, det_red(c, 0),
-                                                                c.map_t1, tma);
-            else
-                k_rows_fwd<LOGN, false><<<nb2, L2::T, smem, s>>>(c.D, nullptr, c.M, inv_ab, cap,
-                                                                 c.T1, c.acc, det_red(c, 0),
-                                                                 c.map_t1, tma);
+            auto fwd = [&](auto kern) {
+                return launch_chain(kern, nb2, L2::T, smem, s, c.chain, c.D, c.Dq, c.M, inv_ab,
+                                    cap, c.T1, c.acc, det_red(c, 0), c.map_t1, tma);
+            };
+            e = c.opt.deterministic ? fwd(k_rows_fwd<LOGN, true>) : fwd(k_rows_fwd<LOGN, false>);
             break;
         }
         case PASS_COLS:
-            k_cols<LOGN><<<nb2, L2::T, L2::GB * L2::group_bytes(2), s>>>(
-                c.T1, c.PT, c.RT, pi_lx, pi_ly, (float)c.opt.helmholtz_eps, c.acc, det_red(c, 0),
-                c.map_pt, c.map_rt, tma);
+            e = launch_chain(k_cols<LOGN>, nb2, L2::T, L2::GB * L2::group_bytes(2), s, c.chain,
+                             c.T1, c.PT, c.RT, pi_lx, pi_ly, (float)c.opt.helmholtz_eps, c.acc,
+                             det_red(c, 0), c.map_pt, c.map_rt, tma);
             break;
-        case PASS_FIELD: inv(k_rows_inv<LOGN, INV_FIELD>, 2); break;
-        case PASS_PSI: inv(k_rows_inv<LOGN, INV_PSI>, 1); break;
-        default: inv(k_rows_inv<LOGN, INV_MAPS>, 2); break;
+        case PASS_FIELD: e = inv(k_rows_inv<LOGN, INV_FIELD>, 2); break;
+        case PASS_PSI: e = inv(k_rows_inv<LOGN, INV_PSI>, 1); break;
+        default: e = inv(k_rows_inv<LOGN, INV_MAPS>, 2); break;
     }
     c.launches++;
-    return cudaGetLastError();
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
 }
 
 // Shared-memory opt-in for every kernel of one transform size (done at create,

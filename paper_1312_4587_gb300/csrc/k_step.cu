@@ -24,6 +24,7 @@ __global__ void __launch_bounds__(kCellThreads, kCellBlocks)
 k_loop_cells(Grid gr, int m, LoopBufs b, const float2* __restrict__ E2,
              const int* __restrict__ rank, const int* __restrict__ cell_pin_ptr,
              const float2* __restrict__ gpin, const float2* __restrict__ gW2) {
+    chain_trigger();
     const float* cf = ctrl_f(b.ctrl);
     if (cf[F_DONE] != 0.0f) return;
     const int stride = gridDim.x * blockDim.x;
@@ -100,6 +101,8 @@ constexpr int kVecBlocksPerSm = 6;
 
 // g = gW + lambda gN; sums for alpha_k; last CTA: alpha_k and gamma_{k+1}.
 __global__ void __launch_bounds__(kCellThreads, kVecBlocksPerSm) k_loop_g(int m2, LoopBufs b) {
+    chain_wait();
+    chain_trigger();
     const float* cf = ctrl_f(b.ctrl);
     if (cf[F_DONE] != 0.0f) return;
     const float lam = loop_lambda(b);
@@ -157,6 +160,7 @@ __global__ void __launch_bounds__(kCellThreads, kVecBlocksPerSm) k_loop_g(int m2
 // clamp keeps the cell inside the region.  Last CTA: record and advance.
 __global__ void __launch_bounds__(kCellThreads, kVecBlocksPerSm)
 k_loop_update(int m, Grid gr, float x1, float y1, LoopBufs b) {
+    chain_wait();
     const float* cf = ctrl_f(b.ctrl);
     if (cf[F_DONE] != 0.0f) return;
     const float alpha = cf[F_ALPHA], beta = cf[F_BETA];
@@ -426,16 +430,20 @@ cudaError_t launch_ctrl_lambda(Ctx& c, cudaStream_t s) {
 }
 
 cudaError_t launch_loop_g(Ctx& c, cudaStream_t s) {
-    k_loop_g<<<vec_blocks(c, 2LL * c.m_mov), kCellThreads, 0, s>>>(2 * c.m_mov, loop_bufs(c));
     c.launches++;
-    return cudaGetLastError();
+    const cudaError_t e = launch_chain(k_loop_g, vec_blocks(c, 2LL * c.m_mov), kCellThreads, 0, s,
+                                       c.chain, 2 * c.m_mov, loop_bufs(c));
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_loop_update(Ctx& c, cudaStream_t s) {
-    k_loop_update<<<vec_blocks(c, 2LL * c.m_mov), kCellThreads, 0, s>>>(
-        c.m_mov, c.grid, (float)c.x1, (float)c.y1, loop_bufs(c));
     c.launches++;
-    return cudaGetLastError();
+    const cudaError_t e = launch_chain(k_loop_update, vec_blocks(c, 2LL * c.m_mov), kCellThreads,
+                                       0, s, c.chain, c.m_mov, c.grid, (float)c.x1, (float)c.y1,
+                                       loop_bufs(c));
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_place_init(Ctx& c, const float* x0, const float* y0, cudaStream_t s) {

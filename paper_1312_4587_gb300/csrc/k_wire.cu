@@ -38,6 +38,7 @@ k_interleave(int m, const float* __restrict__ x, const float* __restrict__ y,
              const int* __restrict__ rank, float2* __restrict__ pos,
              const float* __restrict__ done) {
     if (done && *done != 0.0f) return;
+    chain_trigger();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < m) pos[rank[i]] = make_float2(x[i], y[i]);
 }
@@ -435,6 +436,8 @@ __global__ void __launch_bounds__(kWaThreads, 4)
 k_wa(int nb_big, int nbig, int nslabs, int pairs, const int4* __restrict__ slabs, WaIo io,
      float inv_g, float l2g, const float* __restrict__ scale_dev, double* __restrict__ acc,
      const float* __restrict__ done, DetRed dr, int* __restrict__ err) {
+    chain_wait();
+    chain_trigger();
     if (done && *done != 0.0f) return;
     const int lane = threadIdx.x & 31;
     // 1/gamma and log2(e)/gamma: from the loop's control mirror, or computed
@@ -536,6 +539,7 @@ k_pin_sum(int m, const int* __restrict__ rank, const int* __restrict__ cell_pin_
           const float2* __restrict__ gpin, float* __restrict__ gx, float* __restrict__ gy,
           double* __restrict__ acc, DetRed dr) {
     float l1 = 0.0f;
+    chain_wait();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
         const int r = rank[i];
         float wx = 0.0f, wy = 0.0f;
@@ -558,6 +562,7 @@ k_split(int m, const int* __restrict__ rank, const float2* __restrict__ gW2,
         float* __restrict__ gx, float* __restrict__ gy, double* __restrict__ acc, DetRed dr) {
     const int stride = gridDim.x * blockDim.x;
     float l1 = 0.0f;
+    chain_wait();
     for (int i0 = blockIdx.x * blockDim.x + threadIdx.x; i0 < m; i0 += 4 * stride) {
         float2 g[4];
 #pragma unroll
@@ -610,18 +615,19 @@ cudaError_t launch_wa_impl(Ctx& c, const float* x, const float* y, float gamma,
     const int pairs = wa_pairs(c);
     const int nb_big = wa_big_blocks(c), nb = nb_big + wa_small_blocks(c);
     auto go = [&](auto kern) {
-        kern<<<nb, kWaThreads, 0, s>>>(nb_big, c.nbig, c.nslabs, pairs, c.slabs, io, inv_g, l2g,
-                                       scale_dev, c.acc, done, det_red(c, 1), c.err);
+        return launch_chain(kern, nb, kWaThreads, 0, s, c.chain && interleave, nb_big, c.nbig,
+                            c.nslabs, pairs, c.slabs, io, inv_g, l2g, scale_dev, c.acc, done,
+                            det_red(c, 1), c.err);
     };
+    cudaError_t e = cudaSuccess;
     if (det) {
-        if (lse) go(k_wa<true, true>);
-        else go(k_wa<true, false>);
+        e = lse ? go(k_wa<true, true>) : go(k_wa<true, false>);
     } else {
-        if (lse) go(k_wa<false, true>);
-        else go(k_wa<false, false>);
+        e = lse ? go(k_wa<false, true>) : go(k_wa<false, false>);
     }
     c.launches++;
-    return cudaGetLastError();
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_wa(Ctx& c, const float* x, const float* y, float gamma, cudaStream_t s) {
@@ -639,15 +645,17 @@ cudaError_t launch_pin_sum(Ctx& c, float* gx, float* gy, bool few, cudaStream_t 
     const int threads = few ? 1024 : kCellThreads;
     int nb = nblk(c.m_mov, threads);
     if (few) nb = std::min(nb, kLinkBlocks);
+    cudaError_t e = cudaSuccess;
     // region 1: this pass follows the WA kernel on its stream
     if (c.opt.deterministic)
-        k_pin_sum<<<nb, threads, 0, s>>>(c.m_mov, c.cell_rank, c.cell_pin_ptr, c.gpin, gx, gy,
-                                              c.acc, det_red(c, 1));
+        e = launch_chain(k_pin_sum, nb, threads, 0, s, c.chain, c.m_mov, c.cell_rank,
+                         c.cell_pin_ptr, c.gpin, gx, gy, c.acc, det_red(c, 1));
     else
-        k_split<<<nb, threads, 0, s>>>(c.m_mov, c.cell_rank, c.gW2, gx, gy, c.acc,
-                                            det_red(c, 1));
+        e = launch_chain(k_split, nb, threads, 0, s, c.chain, c.m_mov, c.cell_rank, c.gW2, gx, gy,
+                         c.acc, det_red(c, 1));
     c.launches++;
-    return cudaGetLastError();
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_cells_impl(Ctx& c, const float* x, const float* y, float* gNx, float* gNy,

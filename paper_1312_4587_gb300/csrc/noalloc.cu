@@ -120,6 +120,11 @@ extern "C" fftpl_status fftpl_solve_noalloc(const float* rho, int32_t n, double 
     c.RT = reinterpret_cast<float*>(base + kOffRT);
     spec_maps_init(c);
     c.acc = reinterpret_cast<double*>(base + kOffAcc);
+    // programmatic launches: by graph 12.3 -> 10.3 us at n = 64, 14.4 -> 12.3 at
+    // 256, 14.4 either way at 512 (launched one by one 18.9 -> 15.4), but
+    // 24.6 -> 28.7 at 1024, where blocks that wait early end up unevenly
+    // spread over the SMs
+    c.chain = n <= 512;
     c.psi = psi;
     c.ex = ex;
     c.ey = ey;
