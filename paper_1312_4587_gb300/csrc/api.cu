@@ -87,10 +87,11 @@ cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s) {
     return cudaMallocFromPoolAsync(p, bytes, pool, s);
 }
 
-// The small pinned host mirror of a handle's FP64 sums, from a process-wide
-// arena (page-locked allocations and frees synchronise the device, so the
-// slots are recycled instead).
-constexpr size_t kHostSlot = kAccDoubles * sizeof(double);
+// The small pinned host mirror of the totals of a handle's FP64 sums, from a
+// process-wide arena (page-locked allocations and frees synchronise the
+// device, so the slots are recycled instead).
+constexpr size_t kHostSlot = 32 * sizeof(double);
+static_assert(kReportSums <= 32, "host slot too small");
 std::mutex g_host_mu;
 std::vector<double*> g_host_free;
 
@@ -99,7 +100,7 @@ cudaError_t host_slot(double** p) {
     if (g_host_free.empty()) {
         constexpr int kSlots = 256;
         char* block = nullptr;
-        cudaError_t e = cudaMallocHost((void**)&block, kSlots * kHostSlot);
+        cudaError_t e = cudaHostAlloc((void**)&block, kSlots * kHostSlot, cudaHostAllocMapped | cudaHostAllocPortable);
         if (e != cudaSuccess) return e;
         for (int k = kSlots - 1; k >= 0; --k)
             g_host_free.push_back(reinterpret_cast<double*>(block + k * kHostSlot));
@@ -427,32 +428,25 @@ fftpl_status ensure_psi(Ctx& c, cudaStream_t s) {
     return FFTPL_OK;
 }
 
-// total of one striped accumulator
-double acc_total(const double* acc, int q) {
-    double s = 0.0;
-    for (int k = 0; k < kAccStripes; ++k) s += acc[k * kAccStride + q];
-    return s;
-}
-
 void fill_report(const Ctx& c, const double* acc, fftpl_eval_report* rep) {
-    rep->N = 0.5 * c.Ab * acc_total(acc, ACC_N);
-    rep->W = acc_total(acc, ACC_W);
-    rep->hpwl = acc_total(acc, ACC_HPWL);
-    rep->tau = c.mov_area > 0 ? acc_total(acc, ACC_TAU) / c.mov_area : 0.0;
-    rep->gN_l1 = acc_total(acc, ACC_GN_L1);
-    rep->gW_l1 = acc_total(acc, ACC_GW_L1);
-    rep->charge = acc_total(acc, ACC_CHARGE);
+    rep->N = 0.5 * c.Ab * acc[ACC_N];
+    rep->W = acc[ACC_W];
+    rep->hpwl = acc[ACC_HPWL];
+    rep->tau = c.mov_area > 0 ? acc[ACC_TAU] / c.mov_area : 0.0;
+    rep->gN_l1 = acc[ACC_GN_L1];
+    rep->gW_l1 = acc[ACC_GW_L1];
+    rep->charge = acc[ACC_CHARGE];
     rep->mov_area = c.mov_area;
 }
 
-cudaError_t enqueue_report(Ctx& c) {
-    return cudaMemcpyAsync(c.acc_host, c.acc, kAccDoubles * sizeof(double), cudaMemcpyDeviceToHost,
-                           c.stream);
-}
+// What ends an evaluation on the main stream: a kernel, or the join with the
+// wirelength branch.
+enum { END_KERNEL = 1, END_JOIN = 0, END_ENQUEUED = -1 };
 
-// enqueued: the sums are already on their way to the host mirror
-fftpl_status read_report(Ctx& c, fftpl_eval_report* rep, bool enqueued = false) {
-    if (!enqueued) CK(enqueue_report(c));
+// end: what precedes on the stream, or END_ENQUEUED if the sums are already on
+// their way to the host
+fftpl_status read_report(Ctx& c, fftpl_eval_report* rep, int end) {
+    if (end != END_ENQUEUED) CK(launch_report(c, end == END_KERNEL, c.stream));
     CK(cudaStreamSynchronize(c.stream));
     if (rep) fill_report(c, c.acc_host, rep);
     return FFTPL_OK;
@@ -947,7 +941,7 @@ fftpl_status fftpl_density(fftpl_t h, const float* x, const float* y, double* N,
                      nullptr, nullptr));
     if (N) {
         fftpl_eval_report r;
-        TRY(read_report(c, &r));
+        TRY(read_report(c, &r, END_KERNEL));
         *N = r.N;
     }
     return FFTPL_OK;
@@ -961,7 +955,7 @@ fftpl_status fftpl_density_adjoint(fftpl_t h, const float* x, const float* y, do
                      gy ? gy : scratch(c, 1), nullptr, nullptr));
     if (N) {
         fftpl_eval_report r;
-        TRY(read_report(c, &r));
+        TRY(read_report(c, &r, END_KERNEL));
         *N = r.N;
     }
     return FFTPL_OK;
@@ -973,7 +967,7 @@ fftpl_status fftpl_energy(fftpl_t h, const float* x, const float* y, double* N) 
     TRY(enqueue_eval(c, x, y, 0.0f, EV_DENSITY | EV_NO_GATHER, nullptr, nullptr, nullptr, nullptr));
     if (N) {
         fftpl_eval_report r;
-        TRY(read_report(c, &r));
+        TRY(read_report(c, &r, END_KERNEL));
         *N = r.N;
     }
     return FFTPL_OK;
@@ -1001,7 +995,7 @@ fftpl_status fftpl_wa(fftpl_t h, const float* x, const float* y, float gamma, do
                      gy ? gy : scratch(c, 3)));
     if (W) {
         fftpl_eval_report r;
-        TRY(read_report(c, &r));
+        TRY(read_report(c, &r, END_KERNEL));
         *W = r.W;
     }
     return FFTPL_OK;
@@ -1030,7 +1024,8 @@ static fftpl_status eval_impl(Ctx& c, const float* x, const float* y, float gamm
             CK(cudaStreamBeginCapture(c.stream, cudaStreamCaptureModeThreadLocal));
             int64_t before = c.launches;
             fftpl_status st = enqueue_eval(c, x, y, gamma, what, gNx, gNy, gWx, gWy, stage);
-            cudaError_t re = st == FFTPL_OK && want ? enqueue_report(c) : cudaSuccess;
+            cudaError_t re = st == FFTPL_OK && want ? launch_report(c, !stage, c.stream)
+                                                    : cudaSuccess;
             cudaError_t ee = cudaStreamEndCapture(c.stream, &g);
             if (st != FFTPL_OK) {
                 if (g) cudaGraphDestroy(g);
@@ -1055,7 +1050,7 @@ static fftpl_status eval_impl(Ctx& c, const float* x, const float* y, float gamm
         return FFTPL_OK;
     }
     TRY(enqueue_eval(c, x, y, gamma, what, gNx, gNy, gWx, gWy, stage));
-    if (want) CK(enqueue_report(c));
+    if (want) CK(launch_report(c, !stage, c.stream));
     return FFTPL_OK;
 }
 
@@ -1069,7 +1064,7 @@ fftpl_status fftpl_eval(fftpl_t h, const float* x, const float* y, float gamma, 
     gWx = gWx ? gWx : scratch(c, 2);
     gWy = gWy ? gWy : scratch(c, 3);
     TRY(eval_impl(c, x, y, gamma, gNx, gNy, gWx, gWy, nullptr, rep != nullptr));
-    if (rep) TRY(read_report(c, rep, true));
+    if (rep) TRY(read_report(c, rep, END_ENQUEUED));
     return FFTPL_OK;
 }
 
@@ -1110,7 +1105,7 @@ fftpl_status fftpl_eval_host(fftpl_t h, const float* x_host, const float* y_host
     if (m > 0 && xd && yd && gd[0] && gd[1] && gd[2] && gd[3]) {
         TRY(eval_impl(c, (const float*)xd, (const float*)yd, gamma, (float*)gd[0], (float*)gd[1],
                       (float*)gd[2], (float*)gd[3], c.hx, true));
-        return read_report(c, rep, true);
+        return read_report(c, rep, END_ENQUEUED);
     }
     CK(cudaMemcpyAsync(c.hx, x_host, m * sizeof(float), cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(c.hy, y_host, m * sizeof(float), cudaMemcpyHostToDevice, s));
@@ -1120,12 +1115,12 @@ fftpl_status fftpl_eval_host(fftpl_t h, const float* x_host, const float* y_host
     for (int k = 0; k < 4; ++k)
         if (outs[k])
             CK(cudaMemcpyAsync(outs[k], c.hg + k * m, m * sizeof(float), cudaMemcpyDeviceToHost, s));
-    return read_report(c, rep, true);
+    return read_report(c, rep, END_ENQUEUED);
 }
 
 fftpl_status fftpl_report(fftpl_t h, fftpl_eval_report* rep) {
     if (!h || !rep) return FFTPL_EINVAL;
-    return read_report(*h, rep);
+    return read_report(*h, rep, END_JOIN);
 }
 
 fftpl_status fftpl_fields(fftpl_t h, const float** rho, const float** psi, const float** ex,
@@ -1179,10 +1174,9 @@ fftpl_status fftpl_bin_ranges(fftpl_t h, const float* x, const float* y, int32_t
     if (c.m_mov > 0 && (!x || !y || !ranges)) return set_err(c, FFTPL_EINVAL, "null argument");
     CK(cudaMemsetAsync(c.acc, 0, kAccDoubles * sizeof(double), c.stream));
     CK(launch_bin_ranges(c, x, y, ranges, c.stream));
-    CK(cudaMemcpyAsync(c.acc_host, c.acc, kAccDoubles * sizeof(double), cudaMemcpyDeviceToHost,
-                       c.stream));
+    CK(launch_report(c, true, c.stream));
     CK(cudaStreamSynchronize(c.stream));
-    if (pairs) *pairs = (int64_t)llround(acc_total(c.acc_host, ACC_CHARGE));
+    if (pairs) *pairs = (int64_t)llround(c.acc_host[ACC_CHARGE]);
     return FFTPL_OK;
 }
 

@@ -62,6 +62,9 @@ enum {
     ACC_COUNT
 };
 
+// the sums an evaluation reports: the first kReportSums quantities
+constexpr int kReportSums = ACC_CHARGE + 1;
+
 // The FP64 sums are striped: a block adds its total to stripe
 // (blockIdx & 31), one 128-byte line of kAccStride doubles per stripe, so no
 // single address takes every block's atomic; readers add the stripes.
@@ -530,7 +533,7 @@ struct Ctx {
     char* zero_block = nullptr;
     size_t zero_density = 0, zero_bytes = 0;   // bytes of the map, of the block
     int* err = nullptr;
-    double* acc_host = nullptr;   // pinned mirror
+    double* acc_host = nullptr;   // their totals in mapped host memory
 
     // placement loop state (2 m_mov each: x then y)
     float *u = nullptr, *v = nullptr, *vprev = nullptr, *g = nullptr, *gprev = nullptr;
@@ -693,6 +696,9 @@ cudaError_t launch_loop_g(Ctx& c, cudaStream_t s);
 cudaError_t launch_loop_update(Ctx& c, cudaStream_t s);
 cudaError_t launch_place_init(Ctx& c, const float* x0, const float* y0, cudaStream_t s);
 cudaError_t launch_gamma0(Ctx& c, cudaStream_t s);
+// totals of the reported sums into c.acc_host; chain: the last operation
+// enqueued on s is a kernel
+cudaError_t launch_report(Ctx& c, bool chain, cudaStream_t s);
 // conjugate-gradient loop (k_step.cu)
 cudaError_t launch_cg_g(Ctx& c, cudaStream_t s);
 cudaError_t launch_cg_dir(Ctx& c, cudaStream_t s);

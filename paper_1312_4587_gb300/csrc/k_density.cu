@@ -96,6 +96,7 @@ k_gather(Grid g, int m, const float* __restrict__ x, const float* __restrict__ y
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     float l1 = 0.0f;
     chain_wait();
+    chain_trigger();
     CellIn c = load_cell(i, m, x, y, w, h, nullptr);
     for (; i < m; i += stride) {
         const Span s = cell_span(g, c.x, c.y, c.w, c.h);

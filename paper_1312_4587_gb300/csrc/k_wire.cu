@@ -500,6 +500,7 @@ k_cells(Grid g, int m, const float* __restrict__ x, const float* __restrict__ y,
         const float2* __restrict__ gW2, double* __restrict__ acc,
         const float* __restrict__ done, DetRed dr) {
     if (done && *done != 0.0f) return;
+    chain_trigger();
     const int stride = gridDim.x * blockDim.x;
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     float ln = 0.0f, lw = 0.0f;
@@ -540,6 +541,7 @@ k_pin_sum(int m, const int* __restrict__ rank, const int* __restrict__ cell_pin_
           double* __restrict__ acc, DetRed dr) {
     float l1 = 0.0f;
     chain_wait();
+    chain_trigger();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
         const int r = rank[i];
         float wx = 0.0f, wy = 0.0f;
@@ -563,6 +565,7 @@ k_split(int m, const int* __restrict__ rank, const float2* __restrict__ gW2,
     const int stride = gridDim.x * blockDim.x;
     float l1 = 0.0f;
     chain_wait();
+    chain_trigger();
     for (int i0 = blockIdx.x * blockDim.x + threadIdx.x; i0 < m; i0 += 4 * stride) {
         float2 g[4];
 #pragma unroll
