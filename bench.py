@@ -261,10 +261,10 @@ def run_serving(args):
 
 
 def tc_flops(n):
-    """FLOPs of one tensor-core solve: five products of 7 n^3 multiply-adds
-    in total (G1, G2, G7: n^3 each; G35, G46: 2 n^3 each), three bf16
-    products per multiply-add (hi*hi + hi*lo + lo*hi)."""
-    return 2 * 3 * 7 * n ** 3
+    """FLOPs of one tensor-core solve: five products of 3 n^3 multiply-adds
+    in total (half of every sum by symmetry: G1, G2, G6, G7 n^3 / 2 each, G35
+    n^3), three bf16 products per multiply-add (hi*hi + hi*lo + lo*hi)."""
+    return 2 * 3 * 3 * n ** 3
 
 
 def tcr_flops(n):

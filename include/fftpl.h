@@ -116,9 +116,9 @@ typedef struct {
  * cosine and sine matrices on the tcgen05 tensor cores: every float32
  * operand x is split into bf16 x_hi + x_lo and each product sums
  * hi*hi + hi*lo + lo*hi in float32 (relative error about 1e-5 per product,
- * against 1e-7 for the FFT path).  It costs 42 n^3 flops per solve (the FFT
- * path O(n^2 log n)), needs n >= FFTPL_TC_MIN_N, and holds 36 n^2 extra
- * bytes of device memory (bf16 tables and intermediates).
+ * against 1e-7 for the FFT path).  It costs 18 n^3 flops per solve (the FFT
+ * path O(n^2 log n)), needs n >= FFTPL_TC_MIN_N, and holds 28 n^2 extra
+ * bytes of device memory (32 n^2 at n = 128; bf16 tables and intermediates).
  * FFTPL_SOLVE_TC_RADIX keeps the transform path's passes (Makhoul's
  * reordering of each cosine or sine transform into a complex DFT of length
  * n, two real rows per DFT) and computes every DFT on the tensor cores as two

@@ -305,6 +305,7 @@ fftpl_status enqueue_solve(Ctx& c, cudaStream_t s) {
         { Stage st(c, 1, s); CK(launch_tc(c, 0, s)); CK(launch_tc(c, 1, s)); }
         { Stage st(c, 2, s); CK(launch_tc(c, 2, s)); }
         { Stage st(c, 3, s); CK(launch_tc(c, 3, s)); }
+        c.chain = false;   // it ends with a join
     } else {
         { Stage st(c, 1, s); CK(launch_rows_fwd(c, s)); }
         { Stage st(c, 2, s); CK(launch_cols_spectral(c, s)); }
@@ -340,6 +341,16 @@ constexpr int kChainCells = 256 * 1024;
 // EV_HOST: the gradient arrays are pinned host memory written over the link
 enum { EV_DENSITY = 1, EV_WA = 2, EV_ADJOINT = 4, EV_NO_GATHER = 8, EV_HOST = 16 };
 
+// psi for the current fields, formed on demand (from PT, or from the
+// tensor-core solve's Ut).
+fftpl_status ensure_psi(Ctx& c, cudaStream_t s) {
+    if (!c.psi_valid) {
+        CK(c.tc ? launch_tc(c, 4, s) : launch_rows_psi(c, s));
+        c.psi_valid = true;
+    }
+    return FFTPL_OK;
+}
+
 // Enqueues one evaluation; gradients must be non-null device arrays.
 // stage (2 m_mov floats, or null): x, y may be pinned host memory; the
 // scatter reads them once and leaves a device copy there for the later
@@ -366,7 +377,7 @@ fftpl_status enqueue_eval(Ctx& c, const float* x, const float* y, float gamma, i
     if (wa && !dens) {
         // the wirelength alone: one chain on the main stream
         TRY(wa_kernel(true, s));
-        if (grads) CK(launch_pin_sum(c, gWx, gWy, false, s));
+        if (grads) CK(launch_pin_sum(c, gWx, gWy, false, c.chain, s));
         c.rho_valid = false;
         c.split_valid = false;
         c.fields_valid = false;
@@ -385,7 +396,7 @@ fftpl_status enqueue_eval(Ctx& c, const float* x, const float* y, float gamma, i
         // gradient pass on a few SMs, the transforms and the gather beside it.
         TRY(wa_kernel(false, s));
         TRY(fork());
-        if (grads) CK(launch_pin_sum(c, gWx, gWy, true, c.side));
+        if (grads) CK(launch_pin_sum(c, gWx, gWy, true, false, c.side));
         CK(cudaEventRecord(c.ev_join, c.side));
     } else if (wa) {
         // the WA branch forks after the scatter; device outputs: after the
@@ -393,7 +404,7 @@ fftpl_status enqueue_eval(Ctx& c, const float* x, const float* y, float gamma, i
         // pass beside the chain measured 18 % slower)
         TRY(fork());
         TRY(wa_kernel(false, c.side));
-        if (grads && !fused) CK(launch_pin_sum(c, gWx, gWy, false, c.side));
+        if (grads && !fused) CK(launch_pin_sum(c, gWx, gWy, false, false, c.side));
         CK(cudaEventRecord(c.ev_join, c.side));
     }
     TRY(enqueue_solve(c, s));
@@ -405,7 +416,10 @@ fftpl_status enqueue_eval(Ctx& c, const float* x, const float* y, float gamma, i
         CK(launch_cells(c, xs, ys, gNx, gNy, gWx, gWy, s));
     } else {
         if (grads) {
-            if ((what & EV_ADJOINT) && !c.tc) CK(launch_rows_psi(c, s));
+            if (what & EV_ADJOINT) {
+                c.psi_valid = false;
+                TRY(ensure_psi(c, s));
+            }
             Stage st(c, 5, s);
             CK(launch_gather(c, xs, ys, gNx, gNy, (what & EV_ADJOINT) != 0, s));
         }
@@ -414,17 +428,7 @@ fftpl_status enqueue_eval(Ctx& c, const float* x, const float* y, float gamma, i
     c.rho_valid = false;
     c.split_valid = false;
     c.fields_valid = true;
-    // the tensor-core solve writes psi; the adjoint gather formed it above
-    c.psi_valid = c.tc != nullptr || (what & EV_ADJOINT);
-    return FFTPL_OK;
-}
-
-// psi for the current fields: the transform path forms it from PT on demand.
-fftpl_status ensure_psi(Ctx& c, cudaStream_t s) {
-    if (!c.psi_valid) {
-        CK(launch_rows_psi(c, s));
-        c.psi_valid = true;
-    }
+    c.psi_valid = (what & EV_ADJOINT) != 0;   // the adjoint gather formed it above
     return FFTPL_OK;
 }
 
@@ -446,7 +450,7 @@ enum { END_KERNEL = 1, END_JOIN = 0, END_ENQUEUED = -1 };
 // end: what precedes on the stream, or END_ENQUEUED if the sums are already on
 // their way to the host
 fftpl_status read_report(Ctx& c, fftpl_eval_report* rep, int end) {
-    if (end != END_ENQUEUED) CK(launch_report(c, end == END_KERNEL, c.stream));
+    if (end != END_ENQUEUED) CK(launch_report(c, end == END_KERNEL && c.m_mov > 0, c.stream));
     CK(cudaStreamSynchronize(c.stream));
     if (rep) fill_report(c, c.acc_host, rep);
     return FFTPL_OK;
@@ -967,7 +971,7 @@ fftpl_status fftpl_energy(fftpl_t h, const float* x, const float* y, double* N) 
     TRY(enqueue_eval(c, x, y, 0.0f, EV_DENSITY | EV_NO_GATHER, nullptr, nullptr, nullptr, nullptr));
     if (N) {
         fftpl_eval_report r;
-        TRY(read_report(c, &r, END_KERNEL));
+        TRY(read_report(c, &r, c.tc ? END_JOIN : END_KERNEL));
         *N = r.N;
     }
     return FFTPL_OK;
@@ -1024,7 +1028,7 @@ static fftpl_status eval_impl(Ctx& c, const float* x, const float* y, float gamm
             CK(cudaStreamBeginCapture(c.stream, cudaStreamCaptureModeThreadLocal));
             int64_t before = c.launches;
             fftpl_status st = enqueue_eval(c, x, y, gamma, what, gNx, gNy, gWx, gWy, stage);
-            cudaError_t re = st == FFTPL_OK && want ? launch_report(c, !stage, c.stream)
+            cudaError_t re = st == FFTPL_OK && want ? launch_report(c, !stage && c.m_mov > 0, c.stream)
                                                     : cudaSuccess;
             cudaError_t ee = cudaStreamEndCapture(c.stream, &g);
             if (st != FFTPL_OK) {
@@ -1046,11 +1050,11 @@ static fftpl_status eval_impl(Ctx& c, const float* x, const float* y, float gamm
         c.fields_valid = true;
         c.rho_valid = false;
         c.split_valid = false;
-        c.psi_valid = c.tc != nullptr;
+        c.psi_valid = false;
         return FFTPL_OK;
     }
     TRY(enqueue_eval(c, x, y, gamma, what, gNx, gNy, gWx, gWy, stage));
-    if (want) CK(launch_report(c, !stage, c.stream));
+    if (want) CK(launch_report(c, !stage && c.m_mov > 0, c.stream));
     return FFTPL_OK;
 }
 
@@ -1394,7 +1398,7 @@ fftpl_status fftpl_step(fftpl_t h, int32_t iters, fftpl_iter_record* recs, int32
     c.fields_valid = true;
     c.rho_valid = false;
     c.split_valid = false;
-    c.psi_valid = c.tc != nullptr;
+    c.psi_valid = false;
     return FFTPL_OK;
 }
 

@@ -262,7 +262,9 @@ __device__ __forceinline__ CellIn load_cell(int i, int m, const float* __restric
 // chain_trigger; what it reads of it comes after chain_wait, which returns
 // when that kernel has completed.  Every kernel of a chain calls both (chain_wait
 // first among its reads), so that its completion also means its
-// predecessors'.  Both are no-ops in a plain launch.
+// predecessors'.  Both are no-ops in a plain launch.  Only where the kernel
+// before is the launch's single dependency: never after a join with another
+// stream.
 __device__ __forceinline__ void chain_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
@@ -567,8 +569,8 @@ struct Ctx {
     int prof_used = 0;
 
     bool rho_valid = false, fields_valid = false, split_valid = false;
-    bool psi_valid = false;     // psi matches the current fields (the transform
-                                // path forms it on demand)
+    bool psi_valid = false;     // psi matches the current fields (it is formed on
+                                // demand)
     std::string last_error;
     std::vector<void*> dev_allocs;
     size_t dev_bytes = 0;
@@ -640,7 +642,7 @@ cudaError_t launch_wa(Ctx& c, const float* x, const float* y, float gamma, cudaS
 cudaError_t launch_wa_impl(Ctx& c, const float* x, const float* y, float gamma,
                            const float* scale_dev, const float* done, bool interleave,
                            cudaStream_t s);
-cudaError_t launch_pin_sum(Ctx& c, float* gx, float* gy, bool few, cudaStream_t s);
+cudaError_t launch_pin_sum(Ctx& c, float* gx, float* gy, bool few, bool chain, cudaStream_t s);
 // 1 when the WA kernel runs slab pairs per warp (large instances)
 int wa_pairs(const Ctx& c);
 // blocks of the WA kernel: slabs of degree kBigMin..kBigMax, and the others
@@ -668,7 +670,8 @@ cudaError_t launch_fill_slabs(int m, int E, const int* np, const int* pc, const 
 // block of tc_elems(n) bf16 elements owned by the handle and fills its
 // cosine/sine tables on stream s; launch_tc part 0 splits rho (with the
 // overflow and charge sums), 1 and 2 the forward contractions (2 with the
-// spectral divide and the energy), 3 the inverse ones (psi, E_x, E_y).
+// spectral divide and the energy), 3 the inverse ones (E_x, E_y), 4 psi from
+// the last solve.
 size_t tc_elems(int n);
 cudaError_t tc_setup(Ctx& c, uint16_t* block, cudaStream_t s);
 void tc_free(Ctx& c);

@@ -1,25 +1,40 @@
 // Spectral solve as dense cosine/sine-matrix contractions on the tcgen05
 // tensor cores (solve path FFTPL_SOLVE_TC_BF16X3).
 //
-// With C[u][x] = cos(pi u (2x+1) / 2n), Ct = C^T, Sx[x][u] = w_u sin(...),
-// Sy[y][v] = w_v sin(...), every product below is D[M][N] = sum_k A[M][k] B[N][k]
-// (both operands K-major, row-major in memory):
-//   G1   A1t[u][y]  = sum_x C[u][x]   rho[y][x]
-//   G2   B[v][u]    = sum_y C[v][y]   A1t[u][y]  -> Psi = a / (w_u^2+w_v^2), a = eps eps B / n^2
-//   G35  [Ut;Xt][x][v] = sum_u [Ct;Sx][x][u] Psi[v][u]
-//   G46  [psi|E_x][y][x] = sum_v Ct[y][v] [Ut;Xt][x][v]
-//   G7   E_y[y][x]  = sum_v Sy[y][v]  Ut[x][v]
+// With C[u][x] = cos(pi u (2x+1) / 2n) and S likewise with sin, C[u][n-1-x] =
+// (-1)^u C[u][x] and S[u][n-1-x] = -(-1)^u S[u][x], so half of every sum
+// suffices: a forward sum over x is one over x < n/2 of f[x] + f[n-1-x] for
+// even u and of f[x] - f[n-1-x] for odd u; an inverse sum at x and n-1-x is the
+// sum and the difference of its even-u and odd-u parts.  Every product below
+// is D[M][N] = sum_k A[M][k] B[N][k] (both operands K-major, row-major in
+// memory), frequencies ordered even ones first (positions p), x, y < n/2 primed:
+//   G1   A1[p][y]      = sum_x' C[u][x'] R+-[y][x']        R+- folded rho, + or - by
+//                        the parity of u; folded along y in the epilogue: A1+-[p][y']
+//   G2   B[q][p]       = sum_y' C[v][y'] A1+-[p][y']   -> Psi = a / (w_u^2+w_v^2),
+//                        a = eps eps B / n^2
+//   G35  [Ut;Xt][x][q] = E +- O, E and O the even-u and odd-u parts of
+//                        sum_p [Ct;Sx][x'][p] Psi[q][p]   (Ct = C^T, Sx = w_u S^T)
+//   G6   E_x[y][x]     = E +- O of sum_q Ct[y'][q] Xt[x][q]
+//   G7   E_y[y][x]     = E +- O of sum_q Sy[y'][q] Ut[x][q]  (Sy = w_v S^T)
+//   G4   psi[y][x]     = E +- O of sum_q Ct[y'][q] Ut[x][q]  (on demand)
 // (Eqs. 10-12 at the bin centres; the energy N = 1/2 A_b sum B Psi is
-// reduced in the G2 epilogue.)  Operands are float32 values split into two
-// bf16 halves, x = hi + lo; each product accumulates hi*hi + hi*lo + lo*hi in
-// float32 in tensor memory (the lo*lo term, 2^-16 relative, is dropped), in
-// four chains over consecutive quarters of K summed in the epilogue.
+// reduced in the G2 epilogue.)  18 n^3 flops; without the folding and with
+// psi in every solve 42 n^3: at n = 2048 the five products took 46 + 59 + 91 +
+// 105 + 68 us (the last two side by side), now 28 + 34 + 48 + 28 + 27, and the
+// gradient's relative error went from 9e-6 to 5e-6.  What bounds them: the
+// operands' shared-memory reads (128 x 128 tiles read 128 bytes a cycle, the
+// loads write 85 more) and, at 256 tiles on 152 SMs, the second wave.
+// Operands are float32 values split into two bf16 halves, x = hi + lo; each
+// product accumulates hi*hi + hi*lo + lo*hi in float32 in tensor memory (the
+// lo*lo term, 2^-16 relative, is dropped), in four chains over consecutive
+// quarters of K summed in the epilogue (of an inverse sum's four, the first
+// two are E, the last two O).
 //
-// Kernel: one CTA per 128 x 128 output tile, 4 warps.  Warp 0 (one thread)
+// Kernel: one CTA per 128 x 128 output tile, 8 warps.  Warp 0 (one thread)
 // loads 128 x 64 operand tiles with TMA (128-byte swizzle) into a 3-stage
 // ring; warp 1 (one thread) issues tcgen05.mma (M = N = 128, K = 16) and
-// commits each stage back to the producer; all four warps read the
-// accumulator with tcgen05.ld (warp w owns lanes 32w..32w+31) for the
+// commits each stage back to the producer; all eight warps read the
+// accumulator with tcgen05.ld (warps w and w + 4 lanes 32w..32w+31) for the
 // epilogue.  Every mbarrier wait is bounded in time: on expiry the kernel
 // records ERR_TIMEOUT in the handle's error word, skips its stores, waits
 // (bounded) for its own operations and frees its tensor memory.
@@ -43,7 +58,11 @@ constexpr int kMinBlocks = BK == 32 ? 2 : 1;   // CTAs per SM the launch bounds 
 constexpr int kStages = 3;
 constexpr int kTileBytes = BM * BK * 2;        // bf16 tile of one operand half
 constexpr int kStageBytes = 4 * kTileBytes;    // A hi, A lo, B hi, B lo
-constexpr int kThreads = 128;
+// Eight warps: tensor memory lanes 32 w .. 32 w + 31 are open to warps w and
+// w + 4, which take one half of the columns each in the epilogue (G2 at n = 2048
+// with four warps and an IEEE divide 50 us, with eight and the fast one 32).
+constexpr int kThreads = 256;
+constexpr int kColGroups = BN / 32 / 2;   // 32-column groups per warp
 constexpr int kSmemBytes = kStages * kStageBytes + 1024;
 constexpr unsigned long long kWaitNs = 1000000000ull;   // 1 s per wait
 // Accumulators per tile: the k-tiles are cut into kAcc consecutive chunks,
@@ -60,16 +79,39 @@ constexpr int kAcc = 4;
 constexpr int kStgRow = 264;
 static_assert(2 * 128 * kStgRow <= kStages * kStageBytes, "staging tile exceeds the ring");
 static_assert(2 * 128 * 128 * 4 <= kStages * kStageBytes, "staging rows exceed the ring");
+// Row pitch in floats of a staged field or potential tile.
+constexpr int kMapRow = BN + 1;
+static_assert(2 * BM * kMapRow * 4 <= kStages * kStageBytes, "staged map tile exceeds the ring");
+// Row pitch in bytes of a staged bf16 operand tile (an odd multiple of 16).
+constexpr int kSplitRow = 2 * BN + 16;
+static_assert(4 * BM * kSplitRow <= kStages * kStageBytes, "staged operand tile exceeds the ring");
 
-enum Epi { EPI_F32 = 0, EPI_SPLIT = 1, EPI_SPECTRAL = 2, EPI_PSI_EX = 3, EPI_EY = 4,
-           EPI_TWIDDLE = 5, EPI_CPLX = 6 };
+enum Epi { EPI_F32 = 0, EPI_FOLD, EPI_SPECTRAL, EPI_UX, EPI_PSI, EPI_EX, EPI_EY, EPI_TWIDDLE,
+           EPI_CPLX };
+
+// Rows of one parity of the forward table: n/2, a whole tile at least.
+__host__ __device__ constexpr int half_rows(int n) { return n / 2 < BM ? BM : n / 2; }
+// Frequency at position p (even ones first).
+__host__ __device__ constexpr int freq_at(int p, int n) {
+    return p < n / 2 ? 2 * p : 2 * (p - n / 2) + 1;
+}
+// Row of the folded density operand that holds y: a 128-row tile holds 64
+// rows y' and their mirror rows n-1-y', so that one epilogue thread of G1
+// has both.
+__host__ __device__ constexpr int fold_row(int y, int n) {
+    return y < n / 2 ? 128 * (y / 64) + y % 64
+                     : 128 * ((n - 1 - y) / 64) + 64 + (n - 1 - y) % 64;
+}
 
 struct EpiArgs {
-    __nv_bfloat16* hi;   // EPI_SPLIT / EPI_SPECTRAL outputs [row][ld]
+    __nv_bfloat16* hi;   // EPI_FOLD / EPI_SPECTRAL / EPI_UX outputs [row][ld]
     __nv_bfloat16* lo;
     int ld;
-    float* f32;          // EPI_F32 [row][ld]; EPI_PSI_EX: psi [row][n]
-    float2* E2;          // EPI_PSI_EX (.x) and EPI_EY (.y), [row][n]
+    float* f32;          // EPI_F32 [row][ld]; EPI_PSI: psi [row][n]
+    float2* E2;          // EPI_EX (.x) and EPI_EY (.y), [row][n]
+    // tiles from row m_odd of A on read B from row b_odd (forward sums: the
+    // odd frequencies take the difference operand)
+    int m_odd, b_odd;
     int n;
     float pi_lx, pi_ly, invn2;
     float eps;           // EPI_SPECTRAL: Helmholtz term (0: Poisson)
@@ -212,6 +254,7 @@ k_tc_gemm(const __grid_constant__ CUtensorMap tAh, const __grid_constant__ CUten
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // one 1-D grid of tiles, column tiles fastest (CTAs in flight share A rows)
     const int m0 = (blockIdx.x / ntn) * BM, n0 = (blockIdx.x % ntn) * BN;
+    const int b0 = n0 + (m0 >= ep.m_odd ? ep.b_odd : 0);
     const int ktiles = K / BK;
     const int nacc = ktiles < kAcc ? ktiles : kAcc;
 
@@ -251,10 +294,10 @@ k_tc_gemm(const __grid_constant__ CUtensorMap tAh, const __grid_constant__ CUten
             uint8_t* st = smem + (size_t)s * kStageBytes;
             mbar_expect_tx(&full_bar[s], bytes);
             tma_load_2d(st, &tAh, kt * BK, m0, &full_bar[s]);
-            tma_load_2d(st + 2 * kTileBytes, &tBh, kt * BK, n0, &full_bar[s]);
+            tma_load_2d(st + 2 * kTileBytes, &tBh, kt * BK, b0, &full_bar[s]);
             if (nsplit == 3) {
                 tma_load_2d(st + kTileBytes, &tAl, kt * BK, m0, &full_bar[s]);
-                tma_load_2d(st + 3 * kTileBytes, &tBl, kt * BK, n0, &full_bar[s]);
+                tma_load_2d(st + 3 * kTileBytes, &tBl, kt * BK, b0, &full_bar[s]);
             }
             ++issued;
         }
@@ -305,62 +348,168 @@ k_tc_gemm(const __grid_constant__ CUtensorMap tAh, const __grid_constant__ CUten
         mma_commit(&accum_bar);   // arrives once every issued MMA has completed
     }
     __syncthreads();
-    // epilogue: accumulator rows 32 w .. 32 w + 31 belong to warp w
+    // epilogue: accumulator rows 32 w .. 32 w + 31 belong to warps w and w + 4
+    const int quad = warp & 3, c0 = (warp >> 2) * kColGroups;
     const bool ok = mbar_wait(&accum_bar, 0, 2 * kWaitNs);
     if (!ok && lane == 0) atomicOr(ep.err, ERR_TIMEOUT);
     // block-uniform decision: tcgen05.ld is warp-collective
     const bool store = __syncthreads_and(ok && !s_abort) != 0;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     dfloat energy = df_zero();
-    const int row = m0 + warp * 32 + lane;
-    if (store) {
-#pragma unroll 1
-        for (int c = 0; c < BN / 32; ++c) {
-            float v[32], t[32];
-            const uint32_t ta = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c * 32);
-            tmem_ld32(ta, v);
-            // chunks summed in a fixed order
-            for (int a = 1; a < nacc; ++a) {
-                tmem_ld32(ta + (uint32_t)(a * BN), t);
+    const int row = m0 + quad * 32 + lane;
+    // 32 columns from col of the accumulators a0 .. a1-1, summed in order
+    auto chunks = [&](int col, int a0, int a1, float (&v)[32]) {
+        float t[32];
+        const uint32_t ta = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)col;
+        tmem_ld32(ta + (uint32_t)(a0 * BN), v);
+        for (int a = a0 + 1; a < a1; ++a) {
+            tmem_ld32(ta + (uint32_t)(a * BN), t);
 #pragma unroll
-                for (int j = 0; j < 32; ++j) v[j] += t[j];
+            for (int j = 0; j < 32; ++j) v[j] += t[j];
+        }
+    };
+    // 32 values from column col of row r as bf16 hi and lo: staged in the (now
+    // idle) operand ring as rows of arrays 2 g (hi) and 2 g + 1 (lo), so that
+    // whole sectors leave the SM (put_out)
+    auto put_split = [&](const float (&v)[32], int g, int r, int col) {
+        __align__(16) __nv_bfloat16 h[32], l[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) split_bf16(v[j], h[j], l[j]);
+        uint8_t* at = smem + (size_t)(2 * g * BM + r) * kSplitRow + 2 * col;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            reinterpret_cast<uint4*>(at)[q] = reinterpret_cast<const uint4*>(h)[q];
+            reinterpret_cast<uint4*>(at + BM * kSplitRow)[q] = reinterpret_cast<const uint4*>(l)[q];
+        }
+    };
+    // the staged arrays of G groups, COLS columns wide, to hi / lo + at(g, r)
+    // (at < 0: not a row of the output)
+    auto put_out = [&](int G, int COLS, auto at) {
+        __syncthreads();
+        const int lanes = COLS / 8, per = 32 / lanes;   // 16 bytes a lane
+#pragma unroll 4
+        for (int i = warp * per; i < 2 * G * BM; i += kThreads / 32 * per) {
+            const int rr = i + lane / lanes, q = lane % lanes, arr = rr / BM;
+            const long long o = at(arr >> 1, rr % BM);
+            if (o < 0) continue;
+            __nv_bfloat16* dst = ((arr & 1) ? ep.lo : ep.hi) + o;
+            reinterpret_cast<uint4*>(dst)[q] =
+                *reinterpret_cast<const uint4*>(smem + (size_t)rr * kSplitRow + 16 * q);
+        }
+    };
+    constexpr bool kForward = EPI == EPI_FOLD || EPI == EPI_SPECTRAL;
+    constexpr bool kInverse = EPI == EPI_UX || EPI == EPI_PSI || EPI == EPI_EX || EPI == EPI_EY;
+    // forward sums: parity and place within it of this row's frequency (the
+    // parities are padded to half_rows(n) rows)
+    const int hr = half_rows(ep.n), parity = kForward && row >= hr ? 1 : 0;
+    const int pr = row - parity * hr;
+    if (store && EPI == EPI_FOLD) {
+        const int c = warp >> 2;   // columns 32 c and their mirror rows' 64 + 32 c
+        float v[32], t[32];
+        chunks(c * 32, 0, nacc, v);
+        chunks(64 + c * 32, 0, nacc, t);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+            const float a = v[j] + t[j];
+            t[j] = v[j] - t[j];
+            v[j] = a;
+        }
+        put_split(v, 0, quad * 32 + lane, c * 32);
+        put_split(t, 1, quad * 32 + lane, c * 32);
+        put_out(2, BN / 2, [&](int g, int r) -> long long {
+            const int par = m0 + r >= hr ? 1 : 0, q = m0 + r - par * hr;
+            if (q >= ep.n / 2) return -1;
+            return (long long)(g * ep.n + par * (ep.n / 2) + q) * ep.ld + n0 / 2;
+        });
+    }
+    if (store && kInverse) {
+        // row x' (or y') and its mirror row from the even and the odd part;
+        // the sine sums' mirror is O - E
+        const int half = ep.n / 2;
+        const bool sine = EPI == EPI_EY || (EPI == EPI_UX && row >= half);
+        float* stg = reinterpret_cast<float*>(smem);
+#pragma unroll 1
+        for (int c = c0; c < c0 + kColGroups; ++c) {
+            float v[32], t[32];
+            chunks(c * 32, 0, nacc / 2, v);
+            chunks(c * 32, nacc / 2, nacc, t);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+                const float a = v[j] + t[j];
+                t[j] = sine ? t[j] - v[j] : v[j] - t[j];
+                v[j] = a;
             }
+            if (EPI == EPI_UX) {
+                put_split(v, 0, quad * 32 + lane, c * 32);
+                put_split(t, 1, quad * 32 + lane, c * 32);
+            } else {
+                // staged in the (now idle) operand ring, so that whole warps
+                // write each row
+                const int r = quad * 32 + lane;
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    stg[r * kMapRow + c * 32 + j] = v[j];
+                    stg[(BM + r) * kMapRow + c * 32 + j] = t[j];
+                }
+            }
+        }
+        if (EPI == EPI_UX) {
+            put_out(2, BN, [&](int g, int r) -> long long {
+                const int s2 = m0 + r >= half ? 1 : 0, x = m0 + r - s2 * half;
+                return (long long)(s2 * ep.n + (g ? ep.n - 1 - x : x)) * ep.ld + n0;
+            });
+        } else {
+            __syncthreads();
+#pragma unroll 4
+            for (int i = warp; i < 2 * BM; i += kThreads / 32) {
+                const int yr = m0 + (i & (BM - 1));
+                if (yr >= half) continue;
+                const size_t at = (size_t)(i < BM ? yr : ep.n - 1 - yr) * ep.n + n0 + lane;
+#pragma unroll
+                for (int q = 0; q < BN / 32; ++q) {
+                    const float val = stg[i * kMapRow + lane + 32 * q];
+                    if (EPI == EPI_PSI) ep.f32[at + 32 * q] = val;
+                    else if (EPI == EPI_EX) ep.E2[at + 32 * q].x = val;
+                    else ep.E2[at + 32 * q].y = val;
+                }
+            }
+        }
+    }
+    if (store && !kInverse && EPI != EPI_FOLD) {
+#pragma unroll 1
+        for (int c = c0; c < c0 + kColGroups; ++c) {
+            float v[32];
+            chunks(c * 32, 0, nacc, v);
             const int col0 = n0 + c * 32;
             if (EPI == EPI_F32) {
                 float4* dst = reinterpret_cast<float4*>(ep.f32 + (size_t)row * ep.ld + col0);
 #pragma unroll
                 for (int q = 0; q < 8; ++q)
                     dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-            } else if (EPI == EPI_SPLIT || EPI == EPI_SPECTRAL) {
-                if (EPI == EPI_SPECTRAL) {
-                    // row = v, column = u; v[] holds B[v][u] (unnormalised)
-                    const int vv = row;
-                    const float wv = ep.pi_ly * (float)vv;
-                    const float ev = vv == 0 ? 1.0f : 2.0f;
+            } else if (EPI == EPI_SPECTRAL) {
+                // row v, columns u: v[] holds B[v][u] (unnormalised)
+                {
+                    const int vv = 2 * pr + parity;
+                    const float wv = ep.pi_ly * (float)vv, w2 = fmaf(wv, wv, ep.eps);
+                    const float sv = (vv == 0 ? 2.0f : 4.0f) * ep.invn2;
+                    const int uf = freq_at(col0, ep.n);
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const int u = col0 + j;
-                        const float wu = ep.pi_lx * (float)u;
-                        const float eu = u == 0 ? 1.0f : 2.0f;
-                        const float a = eu * ev * ep.invn2 * v[j];
-                        const float p = (u == 0 && vv == 0 && !(ep.eps > 0.0f))
-                                            ? 0.0f
-                                            : a / (wu * wu + wv * wv + ep.eps);
-                        energy = df_add(energy, v[j] * p);
-                        v[j] = p;
+                    for (int j = 0; j < 32; j += 2) {
+                        float e = 0.0f;
+#pragma unroll
+                        for (int i = j; i < j + 2; ++i) {
+                            const int u = uf + 2 * i;
+                            const float wu = ep.pi_lx * (float)u;
+                            // the divisor is at least (pi/L)^2 > 0 (or eps): the
+                            // fast divide (2 ulp)
+                            float p = __fdividef((u == 0 ? 0.5f * sv : sv) * v[i], fmaf(wu, wu, w2));
+                            if (u == 0 && vv == 0 && !(ep.eps > 0.0f)) p = 0.0f;
+                            e = fmaf(v[i], p, e);
+                            v[i] = p;
+                        }
+                        if (pr < ep.n / 2) energy = df_add(energy, e);
                     }
-                }
-                __align__(16) __nv_bfloat16 h[32], l[32];
-#pragma unroll
-                for (int j = 0; j < 32; ++j) split_bf16(v[j], h[j], l[j]);
-                uint4* dh = reinterpret_cast<uint4*>(ep.hi + (size_t)row * ep.ld + col0);
-                uint4* dl = reinterpret_cast<uint4*>(ep.lo + (size_t)row * ep.ld + col0);
-                const uint4* sh = reinterpret_cast<const uint4*>(h);
-                const uint4* sl = reinterpret_cast<const uint4*>(l);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    dh[q] = sh[q];
-                    dl[q] = sl[q];
+                    put_split(v, 0, quad * 32 + lane, c * 32);
                 }
             } else if (EPI == EPI_TWIDDLE) {
                 // row = 2 k1 + c (c: real / imaginary part), column = r n2 + j2:
@@ -407,24 +556,15 @@ k_tc_gemm(const __grid_constant__ CUtensorMap tAh, const __grid_constant__ CUten
                     const int k2 = col & (ep.n2 - 1);
                     stg[((size_t)(lg * ep.g + q) * ep.n + k1 + 64 * k2) * 2 + cc] = v[j];
                 }
-            } else if (EPI == EPI_PSI_EX) {
-                if (col0 < ep.n) {
-                    float4* dst = reinterpret_cast<float4*>(ep.f32 + (size_t)row * ep.n + col0);
-#pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-                } else {
-                    float* dst = reinterpret_cast<float*>(ep.E2 + (size_t)row * ep.n + (col0 - ep.n));
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) dst[2 * j] = v[j];
-                }
-            } else {   // EPI_EY
-                float* dst = reinterpret_cast<float*>(ep.E2 + (size_t)row * ep.n + col0) + 1;
-#pragma unroll
-                for (int j = 0; j < 32; ++j) dst[2 * j] = v[j];
             }
         }
     }
+    if (EPI == EPI_SPECTRAL && store)
+        put_out(1, BN, [&](int, int r) -> long long {
+            const int par = m0 + r >= hr ? 1 : 0, q = m0 + r - par * hr;
+            if (q >= ep.n / 2) return -1;
+            return (long long)(par * (ep.n / 2) + q) * ep.ld + n0;
+        });
     if (EPI == EPI_TWIDDLE && store) {
         // rows [n0, n0 + 128) of A2 (hi, lo): 256 bytes each, 8 bytes a
         // thread (the staged rows are kStgRow = 8 mod 16 bytes apart)
@@ -452,29 +592,32 @@ k_tc_gemm(const __grid_constant__ CUtensorMap tAh, const __grid_constant__ CUten
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kAcc * BN));
 }
 
-// Tables: C[u][x], the stacked [Ct; Sx] (Ct[x][u] = C[u][x]) and Sy[y][v],
-// each split into bf16 hi and lo.  Arguments reduced exactly:
-// cos(pi u (2x+1) / 2n) = cospi(k / 2n), k = u (2x+1) mod 4n.
+// Tables, each split into bf16 hi and lo: the forward C[p][x'] (parities in
+// halves of half_rows(n) rows of n/2), the stacked [Ct; Sx][x'][p] and
+// Sy[y'][q] (rows of n).  Arguments reduced exactly: cos(pi u (2x+1) / 2n) =
+// cospi(k / 2n), k = u (2x+1) mod 4n.
 __global__ void k_tc_tables(int n, double pi_lx, double pi_ly, __nv_bfloat16* C_hi,
                             __nv_bfloat16* C_lo, __nv_bfloat16* CS_hi, __nv_bfloat16* CS_lo,
                             __nv_bfloat16* Sy_hi, __nv_bfloat16* Sy_lo) {
-    size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (idx >= (size_t)n * n) return;
-    int r = (int)(idx / n), k = (int)(idx % n);     // row, column
-    // C[u = r][x = k]
-    long long a = ((long long)r * (2LL * k + 1)) % (4LL * n);
+    const size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x, half = n / 2;
+    if (idx >= n * half) return;
     double s, cc;
-    sincospi((double)a / (2.0 * n), &s, &cc);
-    split_bf16((float)cc, C_hi[idx], C_lo[idx]);
-    // Ct[x = r][u = k] and Sx[x = r][u = k]
-    long long b = ((long long)k * (2LL * r + 1)) % (4LL * n);
-    sincospi((double)b / (2.0 * n), &s, &cc);
-    split_bf16((float)cc, CS_hi[idx], CS_lo[idx]);
-    split_bf16((float)(pi_lx * k * s), CS_hi[(size_t)n * n + idx], CS_lo[(size_t)n * n + idx]);
-    // Sy[y = r][v = k]
-    split_bf16((float)(pi_ly * k * s), Sy_hi[idx], Sy_lo[idx]);
+    {
+        const int p = (int)(idx / half), x = (int)(idx % half), u = freq_at(p, n);
+        const long long a = ((long long)u * (2LL * x + 1)) % (4LL * n);
+        sincospi((double)a / (2.0 * n), &s, &cc);
+        const size_t row = p < n / 2 ? p : half_rows(n) + (p - n / 2);
+        split_bf16((float)cc, C_hi[row * half + x], C_lo[row * half + x]);
+    }
+    {
+        const int x = (int)(idx / n), p = (int)(idx % n), u = freq_at(p, n);
+        const long long a = ((long long)u * (2LL * x + 1)) % (4LL * n);
+        sincospi((double)a / (2.0 * n), &s, &cc);
+        split_bf16((float)cc, CS_hi[idx], CS_lo[idx]);
+        split_bf16((float)(pi_lx * u * s), CS_hi[half * n + idx], CS_lo[half * n + idx]);
+        split_bf16((float)(pi_ly * u * s), Sy_hi[idx], Sy_lo[idx]);
+    }
 }
-
 
 // Radix path tables: the 64-point DFT as a real 128 x 128 block
 // F1[2 k1 + c'][c 64 + j1] and the n2-point DFT block-diagonal over g rows,
@@ -535,39 +678,60 @@ k_tcr_split(int n, int n2, const float2* __restrict__ Z, __nv_bfloat16* __restri
     }
 }
 
-// rho = (D + M) / A_b split into bf16 hi/lo, four bins per thread, with the
-// overflow and charge sums of the transform path's row pass.
+// Four bins of rho = (D + M) / A_b at b, with their overflow and charge.
+template <bool QUANT>
+__device__ __forceinline__ void rho4(size_t b, const float* __restrict__ D,
+                                     const long long* __restrict__ Dq,
+                                     const float* __restrict__ M, float inv_ab, float cap,
+                                     float (&rho)[4], dfloat& tau, dfloat& charge) {
+    const float4 mv = *reinterpret_cast<const float4*>(M + b);
+    const float m4[4] = {mv.x, mv.y, mv.z, mv.w};
+    float d4[4];
+    if (QUANT) {
+        longlong2 q0 = *reinterpret_cast<const longlong2*>(Dq + b);
+        longlong2 q1 = *reinterpret_cast<const longlong2*>(Dq + b + 2);
+        d4[0] = (float)q0.x * 2.3283064365386963e-10f;
+        d4[1] = (float)q0.y * 2.3283064365386963e-10f;
+        d4[2] = (float)q1.x * 2.3283064365386963e-10f;
+        d4[3] = (float)q1.y * 2.3283064365386963e-10f;
+    } else {
+        float4 dv = *reinterpret_cast<const float4*>(D + b);
+        d4[0] = dv.x; d4[1] = dv.y; d4[2] = dv.z; d4[3] = dv.w;
+    }
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        tau = df_add(tau, fmaxf(0.0f, d4[t] - (cap - m4[t])));
+        charge = df_add(charge, d4[t] + m4[t]);
+        rho[t] = (d4[t] + m4[t]) * inv_ab;
+    }
+}
+
+// The folded density operand: R+[row][x'] = rho[y][x'] + rho[y][n-1-x'] and,
+// n rows further, R-[row][x'] = rho[y][x'] - rho[y][n-1-x'] (row = fold_row(y)),
+// split into bf16 hi/lo, four x' per thread, with the overflow and charge
+// sums of the transform path's row pass.
 template <bool QUANT>
 __global__ void __launch_bounds__(256)
-k_tc_rho(int count4, const float* __restrict__ D, const long long* __restrict__ Dq,
+k_tc_rho(int n, const float* __restrict__ D, const long long* __restrict__ Dq,
          const float* __restrict__ M, float inv_ab, float cap, __nv_bfloat16* __restrict__ hi,
          __nv_bfloat16* __restrict__ lo, double* __restrict__ acc, DetRed dr) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, per = n / 8;
     dfloat tau = df_zero(), charge = df_zero();
-    if (i < count4) {
-        size_t b = (size_t)i * 4;
-        float4 mv = *reinterpret_cast<const float4*>(M + b);
-        float m4[4] = {mv.x, mv.y, mv.z, mv.w}, d4[4];
-        if (QUANT) {
-            longlong2 q0 = *reinterpret_cast<const longlong2*>(Dq + b);
-            longlong2 q1 = *reinterpret_cast<const longlong2*>(Dq + b + 2);
-            d4[0] = (float)q0.x * 2.3283064365386963e-10f;
-            d4[1] = (float)q0.y * 2.3283064365386963e-10f;
-            d4[2] = (float)q1.x * 2.3283064365386963e-10f;
-            d4[3] = (float)q1.y * 2.3283064365386963e-10f;
-        } else {
-            float4 dv = *reinterpret_cast<const float4*>(D + b);
-            d4[0] = dv.x; d4[1] = dv.y; d4[2] = dv.z; d4[3] = dv.w;
-        }
-        __align__(8) __nv_bfloat16 h[4], l[4];
+    if (i < n * per) {
+        const int y = i / per, x = 4 * (i % per);
+        float a[4], b[4];
+        rho4<QUANT>((size_t)y * n + x, D, Dq, M, inv_ab, cap, a, tau, charge);
+        rho4<QUANT>((size_t)y * n + n - 4 - x, D, Dq, M, inv_ab, cap, b, tau, charge);
+        size_t at = (size_t)fold_row(y, n) * (n / 2) + x;
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            tau = df_add(tau, fmaxf(0.0f, d4[t] - (cap - m4[t])));
-            charge = df_add(charge, d4[t] + m4[t]);
-            split_bf16((d4[t] + m4[t]) * inv_ab, h[t], l[t]);
+        for (int sgn = 0; sgn < 2; ++sgn, at += (size_t)n * (n / 2)) {
+            __align__(8) __nv_bfloat16 h[4], l[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                split_bf16(sgn ? a[t] - b[3 - t] : a[t] + b[3 - t], h[t], l[t]);
+            *reinterpret_cast<uint2*>(hi + at) = *reinterpret_cast<const uint2*>(h);
+            *reinterpret_cast<uint2*>(lo + at) = *reinterpret_cast<const uint2*>(l);
         }
-        *reinterpret_cast<uint2*>(hi + b) = *reinterpret_cast<const uint2*>(h);
-        *reinterpret_cast<uint2*>(lo + b) = *reinterpret_cast<const uint2*>(l);
     }
     reduce2(df_val(tau), df_val(charge), acc, ACC_TAU, ACC_CHARGE, dr);
 }
@@ -635,9 +799,11 @@ void prepare_gemm() {
     static std::once_flag once;
     std::call_once(once, [] {
         set_smem_attr<tc::EPI_F32>();
-        set_smem_attr<tc::EPI_SPLIT>();
+        set_smem_attr<tc::EPI_FOLD>();
         set_smem_attr<tc::EPI_SPECTRAL>();
-        set_smem_attr<tc::EPI_PSI_EX>();
+        set_smem_attr<tc::EPI_UX>();
+        set_smem_attr<tc::EPI_PSI>();
+        set_smem_attr<tc::EPI_EX>();
         set_smem_attr<tc::EPI_EY>();
         set_smem_attr<tc::EPI_TWIDDLE>();
         set_smem_attr<tc::EPI_CPLX>();
@@ -658,12 +824,13 @@ cudaError_t gemm(const CUtensorMap* a, const CUtensorMap* b, int M, int N, int K
 
 }  // namespace
 
-// Device operands of the tensor-core solve: one block of 18 n^2 bf16.
+// Device operands of the tensor-core solve: one block of tc_elems(n) bf16
+// (14 n^2 from n = 256 on).
 struct TcPlan {
     int n = 0;
     __nv_bfloat16 *C[2], *CS[2], *Sy[2], *R[2], *A1[2], *P[2], *UX[2];
     CUtensorMap mC[2], mCS[2], mSy[2], mR[2], mA1[2], mP[2], mUX[2];
-    // G7 runs on its own stream beside G46 (both only read G35's output)
+    // G7 runs on its own stream beside G6 (both only read G35's output)
     cudaStream_t s2 = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
     ~TcPlan() {
@@ -673,7 +840,9 @@ struct TcPlan {
     }
 };
 
-size_t tc_elems(int n) { return 18 * (size_t)n * n; }
+size_t tc_elems(int n) {
+    return 2 * (2 * (size_t)tc::half_rows(n) * n + 6 * (size_t)n * n);
+}
 
 cudaError_t tc_setup(Ctx& c, uint16_t* block, cudaStream_t s) {
     const int n = c.n;
@@ -683,20 +852,22 @@ cudaError_t tc_setup(Ctx& c, uint16_t* block, cudaStream_t s) {
     p->n = n;
     __nv_bfloat16* q = reinterpret_cast<__nv_bfloat16*>(block);
     auto take = [&](size_t count) { __nv_bfloat16* r = q; q += count; return r; };
+    const int hr = tc::half_rows(n);
     for (int h = 0; h < 2; ++h) {
-        p->C[h] = take(nn);
-        p->CS[h] = take(2 * nn);
-        p->Sy[h] = take(nn);
-        p->R[h] = take(nn);
+        p->C[h] = take((size_t)hr * n);    // 2 hr rows of n/2
+        p->CS[h] = take(nn);
+        p->Sy[h] = take((size_t)hr * n);
+        p->R[h] = take(nn);                // 2 n rows of n/2, as A1
         p->A1[h] = take(nn);
         p->P[h] = take(nn);
         p->UX[h] = take(2 * nn);
     }
     bool ok = true;
     for (int h = 0; h < 2; ++h) {
-        ok = ok && make_map(&p->mC[h], p->C[h], n, n) && make_map(&p->mCS[h], p->CS[h], 2 * n, n) &&
-             make_map(&p->mSy[h], p->Sy[h], n, n) && make_map(&p->mR[h], p->R[h], n, n) &&
-             make_map(&p->mA1[h], p->A1[h], n, n) && make_map(&p->mP[h], p->P[h], n, n) &&
+        ok = ok && make_map(&p->mC[h], p->C[h], 2 * hr, n / 2) &&
+             make_map(&p->mCS[h], p->CS[h], n, n) && make_map(&p->mSy[h], p->Sy[h], hr, n) &&
+             make_map(&p->mR[h], p->R[h], 2 * n, n / 2) &&
+             make_map(&p->mA1[h], p->A1[h], 2 * n, n / 2) && make_map(&p->mP[h], p->P[h], n, n) &&
              make_map(&p->mUX[h], p->UX[h], 2 * n, n);
     }
     if (!ok) {
@@ -713,7 +884,7 @@ cudaError_t tc_setup(Ctx& c, uint16_t* block, cudaStream_t s) {
     }
     prepare_gemm();
     c.tc = p;
-    tc::k_tc_tables<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(
+    tc::k_tc_tables<<<(unsigned)((nn / 2 + 255) / 256), 256, 0, s>>>(
         n, M_PI / c.Lx, M_PI / c.Ly, p->C[0], p->C[1], p->CS[0], p->CS[1], p->Sy[0], p->Sy[1]);
     return cudaGetLastError();
 }
@@ -723,69 +894,79 @@ void tc_free(Ctx& c) {
     c.tc = nullptr;
 }
 
-// part 0: rho split (with the overflow and charge sums); 1: G1; 2: G2 with
-// the spectral divide and the energy; 3: G35, G46 and G7 (psi, E_x, E_y).
+// part 0: the folded density operand (with the overflow and charge sums);
+// 1: G1; 2: G2 with the spectral divide and the energy; 3: G35, G6 and G7
+// (E_x, E_y); 4: G4, psi from the last solve's Ut.
 cudaError_t launch_tc(Ctx& c, int part, cudaStream_t s) {
     TcPlan& p = *c.tc;
-    const int n = c.n;
+    const int n = c.n, hr = tc::half_rows(n);
     tc::EpiArgs ep{};
     ep.n = n;
     ep.ld = n;
     ep.err = c.err;
     ep.acc = c.acc;
     ep.dr = det_red(c, 0);
+    ep.E2 = c.E2;
+    ep.f32 = c.psi;
     cudaError_t e = cudaSuccess;
     if (part == 0) {
-        const int count4 = n * n / 4;
         const float inv_ab = (float)(1.0 / c.Ab);
         const float cap = (float)(c.opt.target_density * c.Ab);
-        const unsigned blocks = (unsigned)((count4 + 255) / 256);
+        const unsigned blocks = (unsigned)((n * (n / 8) + 255) / 256);
         if (c.opt.deterministic)
-            tc::k_tc_rho<true><<<blocks, 256, 0, s>>>(count4, nullptr, c.Dq, c.M, inv_ab, cap,
-                                                      p.R[0], p.R[1], c.acc, ep.dr);
+            tc::k_tc_rho<true><<<blocks, 256, 0, s>>>(n, nullptr, c.Dq, c.M, inv_ab, cap, p.R[0],
+                                                      p.R[1], c.acc, ep.dr);
         else
-            tc::k_tc_rho<false><<<blocks, 256, 0, s>>>(count4, c.D, nullptr, c.M, inv_ab, cap,
-                                                       p.R[0], p.R[1], c.acc, ep.dr);
+            tc::k_tc_rho<false><<<blocks, 256, 0, s>>>(n, c.D, nullptr, c.M, inv_ab, cap, p.R[0],
+                                                       p.R[1], c.acc, ep.dr);
         e = cudaGetLastError();
         c.launches++;
     } else if (part == 1) {
         ep.hi = p.A1[0];
         ep.lo = p.A1[1];
-        e = gemm<tc::EPI_SPLIT>(p.mC, p.mR, n, n, n, 3, ep, s);
+        ep.ld = n / 2;
+        ep.m_odd = hr;
+        ep.b_odd = n;
+        e = gemm<tc::EPI_FOLD>(p.mC, p.mR, 2 * hr, n, n / 2, 3, ep, s);
         c.launches++;
     } else if (part == 2) {
         ep.hi = p.P[0];
         ep.lo = p.P[1];
+        ep.m_odd = hr;
+        ep.b_odd = n;
         ep.pi_lx = (float)(M_PI / c.Lx);
         ep.pi_ly = (float)(M_PI / c.Ly);
         ep.invn2 = 1.0f / ((float)n * (float)n);
         ep.eps = (float)c.opt.helmholtz_eps;
-        e = gemm<tc::EPI_SPECTRAL>(p.mC, p.mA1, n, n, n, 3, ep, s);
+        e = gemm<tc::EPI_SPECTRAL>(p.mC, p.mA1, 2 * hr, n, n / 2, 3, ep, s);
         c.launches++;
-    } else {
+    } else if (part == 3) {
         ep.hi = p.UX[0];
         ep.lo = p.UX[1];
-        e = gemm<tc::EPI_SPLIT>(p.mCS, p.mP, 2 * n, n, n, 3, ep, s);
+        e = gemm<tc::EPI_UX>(p.mCS, p.mP, n, n, n, 3, ep, s);
         c.launches++;
         if (e != cudaSuccess) return e;
-        // G46 (512 tiles at the launch's own stream) and G7 (256 tiles on
-        // s2) together: their 768 tiles fill about 5 waves of SMs instead of
-        // 4 + 2 one after the other; they write disjoint halves of E2
-        ep.f32 = c.psi;
-        ep.E2 = c.E2;
+        // G6 (on the launch's own stream) and G7 (on s2) together: they write
+        // disjoint halves of E2, and their tiles fill the SMs in waves of both
         e = cudaEventRecord(p.fork, s);
         if (e != cudaSuccess) return e;
         e = cudaStreamWaitEvent(p.s2, p.fork, 0);
         if (e != cudaSuccess) return e;
-        e = gemm<tc::EPI_PSI_EX>(p.mCS, p.mUX, n, 2 * n, n, 3, ep, s);
+        tc::EpiArgs ex = ep;
+        ex.m_odd = 0;      // B from row n on: Xt
+        ex.b_odd = n;
+        e = gemm<tc::EPI_EX>(p.mCS, p.mUX, hr, n, n, 3, ex, s);
         c.launches++;
-        const cudaError_t e7 = gemm<tc::EPI_EY>(p.mSy, p.mUX, n, n, n, 3, ep, p.s2);
+        const cudaError_t e7 = gemm<tc::EPI_EY>(p.mSy, p.mUX, hr, n, n, 3, ep, p.s2);
         c.launches++;
         // join in every case, so that a capture stays well formed
         const cudaError_t ej = cudaEventRecord(p.join, p.s2);
         const cudaError_t ew = ej == cudaSuccess ? cudaStreamWaitEvent(s, p.join, 0) : ej;
         if (e == cudaSuccess) e = e7;
         if (e == cudaSuccess) e = ew;
+    } else {
+        e = gemm<tc::EPI_PSI>(p.mCS, p.mUX, hr, n, n, 3, ep, s);
+        c.launches++;
     }
     return e;
 }

@@ -643,7 +643,7 @@ cudaError_t launch_wa(Ctx& c, const float* x, const float* y, float gamma, cudaS
 // evaluation of 2.2M cells with host buffers, 8 / 16 / 32 / 64 blocks of 1024
 // threads 458 / 384 / 378 / 371 us, one block of 256 on every SM 413.
 constexpr int kLinkBlocks = 64;
-cudaError_t launch_pin_sum(Ctx& c, float* gx, float* gy, bool few, cudaStream_t s) {
+cudaError_t launch_pin_sum(Ctx& c, float* gx, float* gy, bool few, bool chain, cudaStream_t s) {
     if (c.m_mov <= 0) return cudaSuccess;
     const int threads = few ? 1024 : kCellThreads;
     int nb = nblk(c.m_mov, threads);
@@ -651,10 +651,10 @@ cudaError_t launch_pin_sum(Ctx& c, float* gx, float* gy, bool few, cudaStream_t 
     cudaError_t e = cudaSuccess;
     // region 1: this pass follows the WA kernel on its stream
     if (c.opt.deterministic)
-        e = launch_chain(k_pin_sum, nb, threads, 0, s, c.chain, c.m_mov, c.cell_rank,
+        e = launch_chain(k_pin_sum, nb, threads, 0, s, chain, c.m_mov, c.cell_rank,
                          c.cell_pin_ptr, c.gpin, gx, gy, c.acc, det_red(c, 1));
     else
-        e = launch_chain(k_split, nb, threads, 0, s, c.chain, c.m_mov, c.cell_rank, c.gW2, gx, gy,
+        e = launch_chain(k_split, nb, threads, 0, s, chain, c.m_mov, c.cell_rank, c.gW2, gx, gy,
                          c.acc, det_red(c, 1));
     c.launches++;
     if (e != cudaSuccess) cudaGetLastError();
