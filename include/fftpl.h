@@ -268,6 +268,14 @@ fftpl_status fftpl_energy(fftpl_t h, const float* x, const float* y, double* N);
 fftpl_status fftpl_gather(fftpl_t h, const float* x, const float* y, int32_t mode, float* gx,
                           float* gy);
 
+/* The same two without a word to the host, for a caller whose loss lives on
+ * the device.  fftpl_energy_device: fftpl_energy with N written to a device
+ * double; asynchronous.  fftpl_gather_scaled: fftpl_gather times *scale (a
+ * device double rounded to float32, read on the handle's stream; NULL: 1). */
+fftpl_status fftpl_energy_device(fftpl_t h, const float* x, const float* y, double* N);
+fftpl_status fftpl_gather_scaled(fftpl_t h, const float* x, const float* y, int32_t mode,
+                                 const double* scale, float* gx, float* gy);
+
 /* Weighted-average wirelength (Eq. 3) and its gradient; HPWL (Eq. 1) as a
  * by-product.  gx, gy device outputs (m_mov), may be NULL.  W host output:
  * non-NULL synchronises. */

@@ -6,6 +6,12 @@ the field-gather kernel (fftpl_gather, mode "gather": the q.E of Eq. 7) or
 the exact derivative of the binned energy (mode "adjoint"), scaled by the
 incoming gradient.  Positions are float32 CUDA tensors of the problem's
 movable cells.
+
+On the stream the handle is ordered with, neither direction waits for the
+device: the energy goes straight into the output tensor and the gather kernel
+reads the incoming gradient from the device.  (With a wait and a copy for the
+energy and two multiplications after the gather, forward and backward of 500K
+cells took 380 us of host time for 70 us of kernels.)
 """
 from __future__ import annotations
 
@@ -16,6 +22,21 @@ from . import fftpl as F
 _MODES = {"gather": 0, "adjoint": 1}
 
 
+def _same_stream(problem, device):
+    return torch.cuda.current_stream(device).cuda_stream == getattr(problem, "stream", None)
+
+
+def _plain_scalar(g):
+    """A float64 CUDA scalar with memory of its own (not, say, a batch of
+    gradients under vmap, which has no data pointer)."""
+    if g.dtype != torch.float64 or not g.is_cuda or g.dim() != 0:
+        return False
+    try:
+        return g.data_ptr() != 0
+    except RuntimeError:
+        return False
+
+
 class DensityEnergy(torch.autograd.Function):
     @staticmethod
     def forward(ctx, x, y, problem, mode="gather"):
@@ -23,13 +44,18 @@ class DensityEnergy(torch.autograd.Function):
             raise ValueError(f"mode must be one of {sorted(_MODES)}")
         x = x.detach().contiguous()
         y = y.detach().contiguous()
-        N = F.fftpl_energy(problem.h, x, y)
+        if _same_stream(problem, x.device):
+            N = torch.empty((), dtype=torch.float64, device=x.device)
+            F.fftpl_energy_device(problem.h, x, y, N)
+        else:
+            N = torch.tensor(F.fftpl_energy(problem.h, x, y), dtype=torch.float64,
+                             device=x.device)
         problem._energy_calls = getattr(problem, "_energy_calls", 0) + 1
         ctx.problem = problem
         ctx.mode = mode
         ctx.call = problem._energy_calls
         ctx.save_for_backward(x, y)
-        return torch.tensor(N, dtype=torch.float64, device=x.device)
+        return N
 
     @staticmethod
     def backward(ctx, grad_out):
@@ -41,6 +67,9 @@ class DensityEnergy(torch.autograd.Function):
             problem._energy_calls += 1
         gx = torch.empty_like(x)
         gy = torch.empty_like(y)
+        if _plain_scalar(grad_out) and _same_stream(problem, x.device):
+            F.fftpl_gather_scaled(problem.h, x, y, grad_out, gx, gy, _MODES[ctx.mode])
+            return gx, gy, None, None
         F.fftpl_gather(problem.h, x, y, gx, gy, _MODES[ctx.mode])
         s = grad_out.to(torch.float32)
         return gx * s, gy * s, None, None

@@ -421,7 +421,7 @@ fftpl_status enqueue_eval(Ctx& c, const float* x, const float* y, float gamma, i
                 TRY(ensure_psi(c, s));
             }
             Stage st(c, 5, s);
-            CK(launch_gather(c, xs, ys, gNx, gNy, (what & EV_ADJOINT) != 0, s));
+            CK(launch_gather(c, xs, ys, gNx, gNy, (what & EV_ADJOINT) != 0, nullptr, s));
         }
         if (wa) CK(cudaStreamWaitEvent(s, c.ev_join, 0));
     }
@@ -977,8 +977,22 @@ fftpl_status fftpl_energy(fftpl_t h, const float* x, const float* y, double* N) 
     return FFTPL_OK;
 }
 
+fftpl_status fftpl_energy_device(fftpl_t h, const float* x, const float* y, double* N) {
+    if (!h || (h->m_mov > 0 && (!x || !y))) return h ? set_err(*h, FFTPL_EINVAL, "null positions") : FFTPL_EINVAL;
+    Ctx& c = *h;
+    if (!N) return set_err(c, FFTPL_EINVAL, "null energy");
+    TRY(enqueue_eval(c, x, y, 0.0f, EV_DENSITY | EV_NO_GATHER, nullptr, nullptr, nullptr, nullptr));
+    CK(launch_energy_out(c, N, c.stream));
+    return FFTPL_OK;
+}
+
 fftpl_status fftpl_gather(fftpl_t h, const float* x, const float* y, int32_t mode, float* gx,
                           float* gy) {
+    return fftpl_gather_scaled(h, x, y, mode, nullptr, gx, gy);
+}
+
+fftpl_status fftpl_gather_scaled(fftpl_t h, const float* x, const float* y, int32_t mode,
+                                 const double* scale, float* gx, float* gy) {
     if (!h) return FFTPL_EINVAL;
     Ctx& c = *h;
     if (c.m_mov > 0 && (!x || !y || !gx || !gy)) return set_err(c, FFTPL_EINVAL, "null argument");
@@ -986,7 +1000,7 @@ fftpl_status fftpl_gather(fftpl_t h, const float* x, const float* y, int32_t mod
     if (!c.fields_valid) return set_err(c, FFTPL_ESTATE, "no density evaluation yet");
     c.chain = false;   // what precedes it on the stream is the caller's
     if (mode == 1) TRY(ensure_psi(c, c.stream));
-    CK(launch_gather(c, x, y, gx, gy, mode == 1, c.stream));
+    CK(launch_gather(c, x, y, gx, gy, mode == 1, scale, c.stream));
     return FFTPL_OK;
 }
 

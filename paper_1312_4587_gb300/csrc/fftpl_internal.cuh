@@ -635,8 +635,9 @@ bool make_map_f32(CUtensorMap* map, const float* base, int rows, int cols, int b
 cudaError_t launch_rho(Ctx& c, cudaStream_t s);
 cudaError_t launch_split_field(Ctx& c, cudaStream_t s);
 cudaError_t launch_q_to_f(const long long* q, float scale, float* out, int count, cudaStream_t s);
+// scale (device double or null): multiplies the gradient written
 cudaError_t launch_gather(Ctx& c, const float* x, const float* y, float* gx, float* gy,
-                          bool adjoint, cudaStream_t s);
+                          bool adjoint, const double* scale, cudaStream_t s);
 cudaError_t launch_wa(Ctx& c, const float* x, const float* y, float gamma, cudaStream_t s);
 // interleave = false: pos2 already written (by launch_scatter_mov)
 cudaError_t launch_wa_impl(Ctx& c, const float* x, const float* y, float gamma,
@@ -702,6 +703,8 @@ cudaError_t launch_gamma0(Ctx& c, cudaStream_t s);
 // totals of the reported sums into c.acc_host; chain: the last operation
 // enqueued on s is a kernel
 cudaError_t launch_report(Ctx& c, bool chain, cudaStream_t s);
+// N of the last solve to *out (device)
+cudaError_t launch_energy_out(Ctx& c, double* out, cudaStream_t s);
 // conjugate-gradient loop (k_step.cu)
 cudaError_t launch_cg_g(Ctx& c, cudaStream_t s);
 cudaError_t launch_cg_dir(Ctx& c, cudaStream_t s);

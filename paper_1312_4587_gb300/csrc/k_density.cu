@@ -85,18 +85,20 @@ k_bin_ranges(Grid g, int m, const float* __restrict__ x, const float* __restrict
 }
 
 // Field gather (ADJ = false) or exact edge-difference adjoint (ADJ = true,
-// field = psi in fx).  Writes gx, gy and adds ||g||_1 to *l1.
+// field = psi in fx).  Writes gx, gy, times *scale if given (rounded to
+// float32), and adds the unscaled ||g||_1 to the sums.
 template <bool ADJ>
 __global__ void __launch_bounds__(kCellThreads, kCellBlocks)
 k_gather(Grid g, int m, const float* __restrict__ x, const float* __restrict__ y,
          const float* __restrict__ w, const float* __restrict__ h, const float* __restrict__ fx,
          const float2* __restrict__ E2, float* __restrict__ gx, float* __restrict__ gy,
-         double* __restrict__ acc, DetRed dr) {
+         const double* __restrict__ scale, double* __restrict__ acc, DetRed dr) {
     const int stride = gridDim.x * blockDim.x;
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     float l1 = 0.0f;
     chain_wait();
     chain_trigger();
+    const float sc = scale ? (float)*scale : 1.0f;
     CellIn c = load_cell(i, m, x, y, w, h, nullptr);
     for (; i < m; i += stride) {
         const Span s = cell_span(g, c.x, c.y, c.w, c.h);
@@ -128,8 +130,8 @@ k_gather(Grid g, int m, const float* __restrict__ x, const float* __restrict__ y
                 sy = fmaf(ox, d, sy);
             }
         }
-        gx[i] = sx;
-        gy[i] = sy;
+        gx[i] = sc * sx;
+        gy[i] = sc * sy;
         l1 += fabsf(sx) + fabsf(sy);
     }
     reduce2(l1, 0.0f, acc, ACC_GN_L1, -1, dr);
@@ -205,11 +207,11 @@ cudaError_t launch_bin_ranges(Ctx& c, const float* x, const float* y, int32_t* r
 }
 
 cudaError_t launch_gather(Ctx& c, const float* x, const float* y, float* gx, float* gy,
-                          bool adjoint, cudaStream_t s) {
+                          bool adjoint, const double* scale, cudaStream_t s) {
     if (c.m_mov <= 0) return cudaSuccess;
     auto go = [&](auto kern) {
         return launch_chain(kern, cell_blocks(c), kCellThreads, 0, s, c.chain, c.grid, c.m_mov, x,
-                            y, c.w, c.h, c.psi, c.E2, gx, gy, c.acc, det_red(c, 0));
+                            y, c.w, c.h, c.psi, c.E2, gx, gy, scale, c.acc, det_red(c, 0));
     };
     const cudaError_t e = adjoint ? go(k_gather<true>) : go(k_gather<false>);
     c.launches++;

@@ -405,6 +405,14 @@ k_report(const double* __restrict__ acc, double* __restrict__ out) {
     if ((threadIdx.x & 31) == 0) out[q] = t;
 }
 
+// N of the last solve into device memory (one warp).
+__global__ void k_energy_out(const double* __restrict__ acc, double half_ab,
+                             double* __restrict__ out) {
+    chain_wait();
+    const double t = acc_sum(acc, ACC_N);
+    if (threadIdx.x == 0) *out = half_ab * t;
+}
+
 static inline int nblk(long long m, int t) { return (int)((m + t - 1) / t); }
 
 // blocks of a vector kernel over n coordinates (grid-stride)
@@ -501,6 +509,14 @@ cudaError_t launch_report(Ctx& c, bool chain, cudaStream_t s) {
     c.launches++;
     const cudaError_t e =
         launch_chain(k_report, 1, 32 * kReportSums, 0, s, chain, c.acc, c.acc_host);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
+
+cudaError_t launch_energy_out(Ctx& c, double* out, cudaStream_t s) {
+    c.launches++;
+    const cudaError_t e =
+        launch_chain(k_energy_out, 1, 32, 0, s, c.chain, c.acc, 0.5 * c.Ab, out);
     if (e != cudaSuccess) cudaGetLastError();
     return e;
 }

@@ -142,6 +142,8 @@ def lib():
             "fftpl_wa": (S, [_H, _P, _P, C.c_float, _P, _P, _P]),
             "fftpl_energy": (S, [_H, _P, _P, _P]),
             "fftpl_gather": (S, [_H, _P, _P, C.c_int32, _P, _P]),
+            "fftpl_energy_device": (S, [_H, _P, _P, _P]),
+            "fftpl_gather_scaled": (S, [_H, _P, _P, C.c_int32, _P, _P, _P]),
             "fftpl_eval": (S, [_H, _P, _P, C.c_float, _P, _P, _P, _P, _P]),
             "fftpl_eval_host": (S, [_H, _P, _P, C.c_float, _P, _P, _P, _P, _P]),
             "fftpl_report": (S, [_H, _P]),
@@ -228,6 +230,17 @@ def fftpl_default_options(**overrides):
     return o
 
 
+def _stream_id(stream):
+    """The given cudaStream_t, or torch's current one (0: none)."""
+    if stream is None:
+        try:
+            import torch
+            stream = torch.cuda.current_stream().cuda_stream if torch.cuda.is_available() else 0
+        except Exception:
+            stream = 0
+    return int(stream or 0)
+
+
 def fftpl_create(region, n, w, h, m_mov, fix_x, fix_y, net_ptr, pin_cell, pin_dx, pin_dy,
                  options=None, stream=None):
     """Creates a handle; host numpy arrays are deep-copied to the device."""
@@ -248,12 +261,7 @@ def fftpl_create(region, n, w, h, m_mov, fix_x, fix_y, net_ptr, pin_cell, pin_dx
                       _hptr(pin_dy, 0))
     if options is None:
         options = fftpl_default_options()
-    if stream is None:
-        try:
-            import torch
-            stream = torch.cuda.current_stream().cuda_stream if torch.cuda.is_available() else 0
-        except Exception:
-            stream = 0
+    stream = _stream_id(stream)
     out = C.c_void_p()
     st = lib().fftpl_create(C.byref(R), C.c_int32(int(n)), C.byref(cells), C.byref(nets),
                             C.byref(pins), C.byref(options), C.c_void_p(int(stream or 0)),
@@ -303,6 +311,17 @@ def fftpl_energy(h, x, y, sync=True):
 def fftpl_gather(h, x, y, gx, gy, mode=0):
     _check(lib().fftpl_gather(h, _dptr(x), _dptr(y), C.c_int32(int(mode)), _dptr(gx), _dptr(gy)),
            h)
+
+
+def fftpl_energy_device(h, x, y, N):
+    """N into a float64 CUDA scalar, without synchronising."""
+    _check(lib().fftpl_energy_device(h, _dptr(x), _dptr(y), _dptr(N)), h)
+
+
+def fftpl_gather_scaled(h, x, y, scale, gx, gy, mode=0):
+    """fftpl_gather times the float64 CUDA scalar scale."""
+    _check(lib().fftpl_gather_scaled(h, _dptr(x), _dptr(y), C.c_int32(int(mode)), _dptr(scale),
+                                     _dptr(gx), _dptr(gy)), h)
 
 
 def fftpl_wa(h, x, y, gamma, gx=None, gy=None, sync=True):
@@ -547,9 +566,11 @@ class Problem:
         self.n = int(inst.n)
         self.m = int(inst.m_mov)
         self.options = o
+        # the stream the handle is ordered with (0: the legacy default stream)
+        self.stream = _stream_id(stream)
         self.h = fftpl_create(inst.region, inst.n, inst.w, inst.h, inst.m_mov, inst.fix_x,
                               inst.fix_y, inst.net_ptr, inst.pin_cell, inst.pin_dx, inst.pin_dy,
-                              o, stream)
+                              o, self.stream)
 
     def close(self):
         if self.h:
