@@ -1266,7 +1266,6 @@ static fftpl_status loop_eval(Ctx& c, bool cells) {
         Stage st(c, 4, c.side);
         CK(launch_wa_impl(c, vx, vy, 1.0f, ctrl_f(c.ctrl) + F_INV_G, ctrl_f(c.ctrl) + F_DONE,
                           false, c.side));
-        if (cells) CK(launch_ctrl_lambda(c, c.side));
     }
     CK(cudaEventRecord(c.ev_join, c.side));
     TRY(enqueue_solve(c, s));

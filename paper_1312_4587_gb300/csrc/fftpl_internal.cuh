@@ -694,8 +694,6 @@ cudaError_t launch_cells(Ctx& c, const float* x, const float* y, float* gNx, flo
                          float* gWx, float* gWy, cudaStream_t s);
 // placement loop
 cudaError_t launch_loop_cells(Ctx& c, cudaStream_t s);
-// lambda_k and the momentum weight, after the wirelength kernels on s
-cudaError_t launch_ctrl_lambda(Ctx& c, cudaStream_t s);
 cudaError_t launch_loop_g(Ctx& c, cudaStream_t s);
 cudaError_t launch_loop_update(Ctx& c, cudaStream_t s);
 cudaError_t launch_place_init(Ctx& c, const float* x0, const float* y0, cudaStream_t s);

@@ -18,7 +18,10 @@ struct LoopBufs {
     DetRed dr;
 };
 
-// gather + pin sums at v (as k_cells).
+// gather + pin sums at v (as k_cells).  The last block forms lambda_k and the
+// momentum weight instead (as a kernel of its own at the end of the
+// wirelength branch, the longer one up to 210K cells, they took 3.4 us of its
+// critical path); lambda_0 waits for the gradient norms (loop_lambda).
 template <bool CSR>
 __global__ void __launch_bounds__(kCellThreads, kCellBlocks)
 k_loop_cells(Grid gr, int m, LoopBufs b, const float2* __restrict__ E2,
@@ -27,9 +30,14 @@ k_loop_cells(Grid gr, int m, LoopBufs b, const float2* __restrict__ E2,
     chain_trigger();
     const float* cf = ctrl_f(b.ctrl);
     if (cf[F_DONE] != 0.0f) return;
-    const int stride = gridDim.x * blockDim.x;
+    const int stride = (gridDim.x - 1) * blockDim.x;
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     float ln = 0.0f, lw = 0.0f;
+    if (blockIdx.x == gridDim.x - 1) {
+        if (threadIdx.x < 32) ctrl_lambda(b.ctrl, b.acc);
+        else if (threadIdx.x == 32) ctrl_momentum(b.ctrl);
+        i = m;
+    }
     CellIn c = load_cell(i, m, b.v, b.v + m, b.w, b.h, rank);
     for (; i < m; i += stride) {
         const CellIn cur = c;
@@ -59,15 +67,6 @@ k_loop_cells(Grid gr, int m, LoopBufs b, const float2* __restrict__ E2,
     reduce2(ln, lw, b.acc, ACC_GN_L1, ACC_GW_L1, b.dr);
 }
 
-// lambda_k and the momentum weight beside the density chain (one warp on the
-// wirelength stream, after its kernels); lambda_0 waits for the gradient
-// norms (loop_lambda).
-__global__ void k_ctrl_lambda(double* ctrl, const double* acc) {
-    if (ctrl_f(ctrl)[F_DONE] != 0.0f) return;
-    if (threadIdx.x < 32) ctrl_lambda(ctrl, acc);
-    else if (threadIdx.x == 32) ctrl_momentum(ctrl);
-}
-
 // lambda for the combined gradient: from the control scalars, in the first
 // iteration (unless given) from the gradients' norms, which the first warp of
 // every block forms for the block (FP64 by every warp took the first iteration
@@ -88,6 +87,47 @@ __device__ __forceinline__ void store_lambda(const LoopBufs& b) {
     if (threadIdx.x != 0) return;
     b.ctrl[C_LAMBDA] = lam;
     ctrl_f(b.ctrl)[F_LAMBDA] = (float)lam;
+}
+
+// Sums a and b (float32, non-negative or collapsed double-float partials) and
+// the maximum mx of a block into the sums: warps by shuffles, the block's warp
+// totals by its first warp, one atomic each per block (per warp, 912 blocks send
+// 22K atomics to 32 lines; iteration at 500K cells, with lambda in the cell
+// kernel, 86.6 -> 83.4 us).  qb, qm < 0: none.
+__device__ __forceinline__ void block_reduce(float a, float b, float mx, double* acc, int qa,
+                                             int qb, int qm, const DetRed& dr) {
+    if (dr.part) {
+        reduce2(a, b, acc, qa, qb, dr);
+        if (qm >= 0) block_max(mx, acc, qm);
+        return;
+    }
+    __shared__ float s[3][kCellThreads / 32];
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    a = warp_sum(a);
+    b = warp_sum(b);
+    mx = warp_max(mx);
+    if (l == 0) {
+        s[0][w] = a;
+        s[1][w] = b;
+        s[2][w] = mx;
+    }
+    __syncthreads();
+    if (w != 0) return;
+    a = l < kCellThreads / 32 ? s[0][l] : 0.0f;
+    b = l < kCellThreads / 32 ? s[1][l] : 0.0f;
+    mx = l < kCellThreads / 32 ? s[2][l] : 0.0f;
+    double da = (double)a, db = (double)b;
+#pragma unroll
+    for (int o = kCellThreads / 64; o > 0; o >>= 1) {
+        da += __shfl_xor_sync(0xffffffffu, da, o);
+        db += __shfl_xor_sync(0xffffffffu, db, o);
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
+    if (l != 0) return;
+    double* st = acc_stripe(acc, 0);
+    red_add_f64(st + qa, da);
+    if (qb >= 0) red_add_f64(st + qb, db);
+    if (qm >= 0) atomic_max_nonneg(st + qm, (double)mx);
 }
 
 // The vector kernels of the loop (2m coordinates) run on a fixed grid of
@@ -145,8 +185,7 @@ __global__ void __launch_bounds__(kCellThreads, kVecBlocksPerSm) k_loop_g(int m2
             }
         }
     }
-    reduce2(df_val(dg), df_val(dv), b.acc, ACC_DG2, ACC_DV2, b.dr);
-    block_max(gi, b.acc, ACC_GINF);
+    block_reduce(df_val(dg), df_val(dv), gi, b.acc, ACC_DG2, ACC_DV2, ACC_GINF, b.dr);
     if (!last_cta(b.counters + 1)) return;
     if (threadIdx.x < 32) {
         store_lambda(b);
@@ -201,8 +240,7 @@ k_loop_update(int m, Grid gr, float x1, float y1, LoopBufs b) {
             }
         }
     }
-    block_max(step, b.acc, ACC_STEPMAX);
-    reduce2(df_val(uphill), 0.0f, b.acc, ACC_GD, -1, b.dr);
+    block_reduce(df_val(uphill), 0.0f, step, b.acc, ACC_GD, -1, ACC_STEPMAX, b.dr);
     if (last_cta(b.counters + 2) && threadIdx.x < 32) ctrl_record(b.ctrl, b.acc, b.recs);
 }
 
@@ -246,8 +284,7 @@ __global__ void __launch_bounds__(kCellThreads, kVecBlocksPerSm) k_cg_g(int m2, 
             }
         }
     }
-    reduce2(df_val(sq), df_val(gp), b.acc, ACC_DG2, ACC_DV2, b.dr);
-    block_max(gi, b.acc, ACC_GINF);
+    block_reduce(df_val(sq), df_val(gp), gi, b.acc, ACC_DG2, ACC_DV2, ACC_GINF, b.dr);
     if (!last_cta(b.counters + 3)) return;
     if (threadIdx.x < 32) {
         store_lambda(b);
@@ -290,8 +327,7 @@ __global__ void __launch_bounds__(kCellThreads, kVecBlocksPerSm) k_cg_dir(int m2
             }
         }
     }
-    reduce2(df_val(gd), 0.0f, b.acc, ACC_GD, -1, b.dr);
-    block_max(da, b.acc, ACC_DINF);
+    block_reduce(df_val(gd), 0.0f, da, b.acc, ACC_GD, -1, ACC_DINF, b.dr);
     if (last_cta(b.counters + 4) && threadIdx.x < 32) ctrl_cg_dir(b.ctrl, b.acc);
 }
 
@@ -415,9 +451,11 @@ __global__ void k_energy_out(const double* __restrict__ acc, double half_ab,
 
 static inline int nblk(long long m, int t) { return (int)((m + t - 1) / t); }
 
-// blocks of a vector kernel over n coordinates (grid-stride)
+// blocks of a vector kernel over n coordinates (grid-stride): two coordinates a
+// thread (iteration at 210K cells with 1 / 2 / 4 / 8: 51.5 / 51.3 / 53.2 / 53.4 us)
+// up to the fixed grid
 static inline int vec_blocks(const Ctx& c, long long n) {
-    return std::max(1, std::min(nblk(n, kCellThreads), c.num_sms * kVecBlocksPerSm));
+    return std::max(1, std::min(nblk(n, 2 * kCellThreads), c.num_sms * kVecBlocksPerSm));
 }
 
 LoopBufs loop_bufs(Ctx& c) {
@@ -432,19 +470,13 @@ LoopBufs loop_bufs(Ctx& c) {
 
 cudaError_t launch_loop_cells(Ctx& c, cudaStream_t s) {
     LoopBufs b = loop_bufs(c);
-    const int nb = cell_blocks(c);
+    const int nb = cell_blocks(c) + 1;
     if (c.opt.deterministic)
         k_loop_cells<true><<<nb, kCellThreads, 0, s>>>(c.grid, c.m_mov, b, c.E2, c.cell_rank,
                                                        c.cell_pin_ptr, c.gpin, nullptr);
     else
         k_loop_cells<false><<<nb, kCellThreads, 0, s>>>(c.grid, c.m_mov, b, c.E2, c.cell_rank,
                                                         nullptr, nullptr, c.gW2);
-    c.launches++;
-    return cudaGetLastError();
-}
-
-cudaError_t launch_ctrl_lambda(Ctx& c, cudaStream_t s) {
-    k_ctrl_lambda<<<1, 64, 0, s>>>(c.ctrl, c.acc);
     c.launches++;
     return cudaGetLastError();
 }

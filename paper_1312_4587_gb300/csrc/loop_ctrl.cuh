@@ -7,8 +7,8 @@
 // The updates sit on the critical path of every iteration and the FP64 pipe
 // is narrow, so a warp reads the 32 stripes of a sum with one load per lane,
 // and what does not depend on an update's own input is formed beside it:
-// lambda_k (for k >= 1 from the HPWL change alone) and the momentum weight on
-// the wirelength stream, gamma_{k+1} by a second warp.  With one thread
+// lambda_k (for k >= 1 from the HPWL change alone) and the momentum weight by
+// one block of the cell kernel, gamma_{k+1} by a second warp.  With one thread
 // walking the stripes, pow() and every scalar in line, the three updates took
 // 10 + 14 + 18 us of an iteration at 210K cells.
 #pragma once
@@ -123,8 +123,7 @@ __device__ __forceinline__ bool lambda_from_norms(const double* ctrl) {
     return ctrl_f(ctrl)[F_FIRST] != 0.0f && !(ctrl[C_LAMBDA0_OPT] > 0.0);
 }
 
-// After the wirelength kernels (one warp on their stream): lambda_k for
-// k >= 1, mu_k lambda_{k-1} with mu_k = 1.1^(-dW/dW_ref + 1) bounded to
+// After the wirelength kernel (one warp): lambda_k for k >= 1, mu_k lambda_{k-1} with mu_k = 1.1^(-dW/dW_ref + 1) bounded to
 // [0.75, 1.1], dW the HPWL change (1.1^z as exp(z ln 1.1)); and the momentum
 // weight of iteration k, a_{k+1} = (1 + sqrt(1 + 4 a_k^2)) / 2,
 // beta_k = (a_k - 1) / a_{k+1}.
