@@ -14,6 +14,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <chrono>
 #include <cstdio>
 #include <mutex>
 #include <string>
@@ -91,7 +92,7 @@ cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s) {
 // process-wide arena (page-locked allocations and frees synchronise the
 // device, so the slots are recycled instead).
 constexpr size_t kHostSlot = 32 * sizeof(double);
-static_assert(kReportSums <= 32, "host slot too small");
+static_assert(kReportSums <= kReportFlag && kReportFlag < 32, "host slot too small");
 std::mutex g_host_mu;
 std::vector<double*> g_host_free;
 
@@ -107,6 +108,7 @@ cudaError_t host_slot(double** p) {
     }
     *p = g_host_free.back();
     g_host_free.pop_back();
+    memset(*p, 0, kHostSlot);
     return cudaSuccess;
 }
 
@@ -445,13 +447,28 @@ void fill_report(const Ctx& c, const double* acc, fftpl_eval_report* rep) {
 
 // What ends an evaluation on the main stream: a kernel, or the join with the
 // wirelength branch.
-enum { END_KERNEL = 1, END_JOIN = 0, END_ENQUEUED = -1 };
+enum { END_KERNEL = 1, END_JOIN = 0 };
 
-// end: what precedes on the stream, or END_ENQUEUED if the sums are already on
-// their way to the host
-fftpl_status read_report(Ctx& c, fftpl_eval_report* rep, int end) {
-    if (end != END_ENQUEUED) CK(launch_report(c, end == END_KERNEL && c.m_mov > 0, c.stream));
+// Waits for the last report enqueued, the last operation on the stream: the
+// host looks for its number in the mirror for as long as a short call takes,
+// then waits for the stream (which also tells of errors).  Seen 2.4 us before
+// a stream synchronisation returns.
+fftpl_status wait_report(Ctx& c) {
+    const unsigned* flag = reinterpret_cast<const unsigned*>(c.acc_host + kReportFlag);
+    const auto t0 = std::chrono::steady_clock::now();
+    for (;;) {
+        for (int k = 0; k < 64; ++k)
+            if (__atomic_load_n(flag, __ATOMIC_ACQUIRE) == c.reports) return FFTPL_OK;
+        if (std::chrono::steady_clock::now() - t0 > std::chrono::microseconds(500)) break;
+    }
     CK(cudaStreamSynchronize(c.stream));
+    c.reports = *flag;   // in step again after a call that failed
+    return FFTPL_OK;
+}
+
+fftpl_status read_report(Ctx& c, fftpl_eval_report* rep, int end) {
+    CK(launch_report(c, end == END_KERNEL && c.m_mov > 0, c.stream));
+    TRY(wait_report(c));
     if (rep) fill_report(c, c.acc_host, rep);
     return FFTPL_OK;
 }
@@ -811,7 +828,8 @@ static fftpl_status create_impl(Ctx& c, const fftpl_region* R, int32_t n, const 
     spec_maps_init(c);
     TRY(dalloc(c, &c.psi, nn));
     TRY(dalloc(c, &c.E2, nn));
-    TRY(dalloc(c, &c.err, 1));
+    TRY(dalloc(c, &c.err, 2));
+    c.report_count = reinterpret_cast<unsigned*>(c.err + 1);
     TRY(dalloc(c, &c.gN, 2 * (size_t)c.m_mov));
     TRY(dalloc(c, &c.gW, 2 * (size_t)c.m_mov));
     TRY(dalloc(c, &c.pos2, (size_t)c.m_mov));
@@ -856,7 +874,7 @@ static fftpl_status create_impl(Ctx& c, const fftpl_region* R, int32_t n, const 
         if (e == cudaSuccess) e = e2;
         CK(e);
     }
-    CK(cudaMemsetAsync(c.err, 0, sizeof(int), s));
+    CK(cudaMemsetAsync(c.err, 0, 2 * sizeof(int), s));
     prepare_spectral(c.logn);
     if (c.opt.solve_path == FFTPL_SOLVE_TC_BF16X3) {
         uint16_t* block = nullptr;
@@ -1033,6 +1051,7 @@ static fftpl_status eval_impl(Ctx& c, const float* x, const float* y, float gamm
         const int32_t wk = want ? 1 : 0;
         memcpy(&key[6], &gk, sizeof(float));
         memcpy((char*)&key[6] + sizeof(float), &wk, sizeof(wk));
+        const unsigned reports = c.reports;
         if (!c.eval_graph || memcmp(key, c.graph_key, sizeof(key)) != 0) {
             if (c.eval_graph) {
                 cudaGraphExecDestroy(c.eval_graph);
@@ -1045,6 +1064,7 @@ static fftpl_status eval_impl(Ctx& c, const float* x, const float* y, float gamm
             cudaError_t re = st == FFTPL_OK && want ? launch_report(c, !stage && c.m_mov > 0, c.stream)
                                                     : cudaSuccess;
             cudaError_t ee = cudaStreamEndCapture(c.stream, &g);
+            c.reports = reports;
             if (st != FFTPL_OK) {
                 if (g) cudaGraphDestroy(g);
                 return st;
@@ -1059,7 +1079,9 @@ static fftpl_status eval_impl(Ctx& c, const float* x, const float* y, float gamm
             c.graph_nkernels = c.launches - before;
             c.launches = before;  // counted at replay
         }
+        c.reports = reports;   // a captured report has not run yet
         CK(cudaGraphLaunch(c.eval_graph, c.stream));
+        if (want) c.reports++;
         c.launches += c.graph_nkernels;
         c.fields_valid = true;
         c.rho_valid = false;
@@ -1082,7 +1104,10 @@ fftpl_status fftpl_eval(fftpl_t h, const float* x, const float* y, float gamma, 
     gWx = gWx ? gWx : scratch(c, 2);
     gWy = gWy ? gWy : scratch(c, 3);
     TRY(eval_impl(c, x, y, gamma, gNx, gNy, gWx, gWy, nullptr, rep != nullptr));
-    if (rep) TRY(read_report(c, rep, END_ENQUEUED));
+    if (rep) {
+        TRY(wait_report(c));
+        fill_report(c, c.acc_host, rep);
+    }
     return FFTPL_OK;
 }
 
@@ -1123,7 +1148,10 @@ fftpl_status fftpl_eval_host(fftpl_t h, const float* x_host, const float* y_host
     if (m > 0 && xd && yd && gd[0] && gd[1] && gd[2] && gd[3]) {
         TRY(eval_impl(c, (const float*)xd, (const float*)yd, gamma, (float*)gd[0], (float*)gd[1],
                       (float*)gd[2], (float*)gd[3], c.hx, true));
-        return read_report(c, rep, END_ENQUEUED);
+        // the gradients in host memory are complete when the stream is
+        CK(cudaStreamSynchronize(s));
+        if (rep) fill_report(c, c.acc_host, rep);
+        return FFTPL_OK;
     }
     CK(cudaMemcpyAsync(c.hx, x_host, m * sizeof(float), cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(c.hy, y_host, m * sizeof(float), cudaMemcpyHostToDevice, s));
@@ -1133,7 +1161,9 @@ fftpl_status fftpl_eval_host(fftpl_t h, const float* x_host, const float* y_host
     for (int k = 0; k < 4; ++k)
         if (outs[k])
             CK(cudaMemcpyAsync(outs[k], c.hg + k * m, m * sizeof(float), cudaMemcpyDeviceToHost, s));
-    return read_report(c, rep, END_ENQUEUED);
+    CK(cudaStreamSynchronize(s));
+    if (rep) fill_report(c, c.acc_host, rep);
+    return FFTPL_OK;
 }
 
 fftpl_status fftpl_report(fftpl_t h, fftpl_eval_report* rep) {
@@ -1193,7 +1223,7 @@ fftpl_status fftpl_bin_ranges(fftpl_t h, const float* x, const float* y, int32_t
     CK(cudaMemsetAsync(c.acc, 0, kAccDoubles * sizeof(double), c.stream));
     CK(launch_bin_ranges(c, x, y, ranges, c.stream));
     CK(launch_report(c, true, c.stream));
-    CK(cudaStreamSynchronize(c.stream));
+    TRY(wait_report(c));
     if (pairs) *pairs = (int64_t)llround(c.acc_host[ACC_CHARGE]);
     return FFTPL_OK;
 }

@@ -64,6 +64,8 @@ enum {
 
 // the sums an evaluation reports: the first kReportSums quantities
 constexpr int kReportSums = ACC_CHARGE + 1;
+// where the host mirror holds the number of the report it is from
+constexpr int kReportFlag = 31;
 
 // The FP64 sums are striped: a block adds its total to stripe
 // (blockIdx & 31), one 128-byte line of kAccStride doubles per stripe, so no
@@ -553,6 +555,8 @@ struct Ctx {
     size_t zero_density = 0, zero_bytes = 0;   // bytes of the map, of the block
     int* err = nullptr;
     double* acc_host = nullptr;   // their totals in mapped host memory
+    unsigned* report_count = nullptr;   // reports made, on the device
+    unsigned reports = 0;               // reports enqueued
 
     // placement loop state (2 m_mov each: x then y)
     float *u = nullptr, *v = nullptr, *vprev = nullptr, *g = nullptr, *gprev = nullptr;
@@ -715,8 +719,8 @@ cudaError_t launch_loop_g(Ctx& c, cudaStream_t s);
 cudaError_t launch_loop_update(Ctx& c, cudaStream_t s);
 cudaError_t launch_place_init(Ctx& c, const float* x0, const float* y0, cudaStream_t s);
 cudaError_t launch_gamma0(Ctx& c, cudaStream_t s);
-// totals of the reported sums into c.acc_host; chain: the last operation
-// enqueued on s is a kernel
+// totals of the reported sums into c.acc_host (counted in c.reports); chain:
+// the last operation enqueued on s is a kernel
 cudaError_t launch_report(Ctx& c, bool chain, cudaStream_t s);
 // N of the last solve to *out (device)
 cudaError_t launch_energy_out(Ctx& c, double* out, cudaStream_t s);

@@ -434,11 +434,19 @@ __global__ void k_gamma0(double* ctrl, const double* acc) {
 // than a plain synchronisation (210K cells; 4.6 at 1,000); this kernel,
 // resident before its predecessor ends, 0.9 (1.3).
 __global__ void __launch_bounds__(32 * kReportSums)
-k_report(const double* __restrict__ acc, double* __restrict__ out) {
+k_report(const double* __restrict__ acc, double* __restrict__ out, unsigned* __restrict__ count) {
     chain_wait();
     const int q = threadIdx.x >> 5;
     const double t = acc_sum(acc, q);
     if ((threadIdx.x & 31) == 0) out[q] = t;
+    // then the number of this report, for a host that looks for it
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const unsigned c = *count + 1u;
+        *count = c;
+        __threadfence_system();
+        *reinterpret_cast<volatile unsigned*>(out + kReportFlag) = c;
+    }
 }
 
 // N of the last solve into device memory (one warp).
@@ -540,8 +548,9 @@ cudaError_t launch_cg_update(Ctx& c, cudaStream_t s) {
 cudaError_t launch_report(Ctx& c, bool chain, cudaStream_t s) {
     c.launches++;
     const cudaError_t e =
-        launch_chain(k_report, 1, 32 * kReportSums, 0, s, chain, c.acc, c.acc_host);
+        launch_chain(k_report, 1, 32 * kReportSums, 0, s, chain, c.acc, c.acc_host, c.report_count);
     if (e != cudaSuccess) cudaGetLastError();
+    else c.reports++;
     return e;
 }
 
