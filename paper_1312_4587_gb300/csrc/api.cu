@@ -866,8 +866,7 @@ static fftpl_status create_impl(Ctx& c, const fftpl_region* R, int32_t n, const 
         long long* q = nullptr;
         CK(pool_alloc((void**)&q, nn * sizeof(long long), s));
         cudaError_t e = cudaMemsetAsync(q, 0, nn * sizeof(long long), s);
-        if (e == cudaSuccess && c.m_fix > 0)
-            e = launch_scatter(c, c.fix_x, c.fix_y, c.w + c.m_mov, c.h + c.m_mov, c.m_fix, nullptr, q, s);
+        if (e == cudaSuccess) e = launch_scatter_fixed(c, q, s);
         if (e == cudaSuccess) e = launch_q_to_f(q, (float)c.opt.target_density, c.M, (int)nn, s);
         cudaFreeAsync(q, s);
         cudaError_t e2 = cudaStreamSynchronize(s);

@@ -631,8 +631,8 @@ inline int cell_blocks(const Ctx& c) {
 // ------------------------------------------------------------ launchers
 // (each returns the CUDA error of the launch)
 void prepare_spectral(int logn);
-cudaError_t launch_scatter(Ctx& c, const float* x, const float* y, const float* w,
-                           const float* h, int m, float* D, long long* Dq, cudaStream_t s);
+// fixed cells into Dq (int64 units of 2^-32), at create
+cudaError_t launch_scatter_fixed(Ctx& c, long long* Dq, cudaStream_t s);
 // movable cells into the handle's D / Dq; write_pos: also the interleaved
 // centres pos2 (by internal cell number) for the WA kernel; stage (2 m_mov
 // floats or null): also a device copy of (x, y)

@@ -65,6 +65,27 @@ k_scatter(Grid g, int m, const float* __restrict__ x, const float* __restrict__ 
     }
 }
 
+// The fixed cells' overlap areas in units of 2^-32 (as the deterministic
+// scatter), a block per cell: a macro covers hundreds of bins a side (150
+// macros on 2048 x 2048 bins, a thread each, took 369 us of a handle's
+// creation).
+__global__ void __launch_bounds__(128)
+k_scatter_fixed(Grid g, const float* __restrict__ x, const float* __restrict__ y,
+                const float* __restrict__ w, const float* __restrict__ h,
+                unsigned long long* __restrict__ Dq) {
+    const int i = blockIdx.x;
+    const Span s = cell_span(g, x[i], y[i], w[i], h[i]);
+    if (s.ilo > s.ihi || s.jlo > s.jhi) return;
+    const int nx = s.ihi - s.ilo + 1, nb = nx * (s.jhi - s.jlo + 1);
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) {
+        const int j = s.jlo + b / nx, k = s.ilo + b % nx;
+        const float a = __fmul_rn(ov_len(g.x0, g.wb, k, s.xl, s.xh),
+                                  ov_len(g.y0, g.hb, j, s.yl, s.yh));
+        const long long q = __float2ll_rn(__fmul_rn(a, 4294967296.0f));
+        atomicAdd(Dq + (size_t)j * g.n + k, (unsigned long long)q);
+    }
+}
+
 __global__ void __launch_bounds__(kCellThreads)
 k_bin_ranges(Grid g, int m, const float* __restrict__ x, const float* __restrict__ y,
              const float* __restrict__ w, const float* __restrict__ h, int4* __restrict__ out,
@@ -165,17 +186,11 @@ __global__ void k_q_to_f(const long long* __restrict__ q, float scale, float* __
 
 static inline int blocks_for(long long m, int t) { return (int)((m + t - 1) / t); }
 
-cudaError_t launch_scatter(Ctx& c, const float* x, const float* y, const float* w, const float* h,
-                           int m, float* D, long long* Dq, cudaStream_t s) {
-    if (m <= 0) return cudaSuccess;
-    int nb = blocks_for(m, kCellThreads);
-    if (Dq)
-        k_scatter<true><<<nb, kCellThreads, 0, s>>>(c.grid, m, x, y, w, h, nullptr, nullptr,
-                                                   nullptr, nullptr,
-                                                   reinterpret_cast<unsigned long long*>(Dq));
-    else
-        k_scatter<false><<<nb, kCellThreads, 0, s>>>(c.grid, m, x, y, w, h, nullptr, nullptr,
-                                                    nullptr, D, nullptr);
+cudaError_t launch_scatter_fixed(Ctx& c, long long* Dq, cudaStream_t s) {
+    if (c.m_fix <= 0) return cudaSuccess;
+    k_scatter_fixed<<<c.m_fix, 128, 0, s>>>(c.grid, c.fix_x, c.fix_y, c.w + c.m_mov,
+                                            c.h + c.m_mov,
+                                            reinterpret_cast<unsigned long long*>(Dq));
     c.launches++;
     return cudaGetLastError();
 }

@@ -16,11 +16,12 @@ namespace fftpl {
 
 constexpr int kIntMax = 0x7fffffff;
 
-__global__ void k_lp_init(int m, int stride, int* __restrict__ lab, int* __restrict__ dist) {
+__global__ void k_lp_init(int m, int stride, int* __restrict__ lab, int* __restrict__ next,
+                          int* __restrict__ dist) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m) return;
     bool seed = (i % stride) == 0;
-    lab[i] = seed ? i : kIntMax;
+    lab[i] = next[i] = seed ? i : kIntMax;
     dist[i] = seed ? 0 : kIntMax;
 }
 
@@ -38,7 +39,8 @@ __global__ void k_lp_net(int E, const int* __restrict__ np, const int* __restric
     netlab[e] = v;
 }
 
-// next[c] = min(next[c], netlab[e]) for every movable cell c of net e
+// next[c] = min(next[c], netlab[e]) for every movable cell c of net e (next
+// starts a round equal to lab: k_lp_step leaves them so)
 __global__ void k_lp_cell(int E, const int* __restrict__ np, const int* __restrict__ pc, int m,
                           const int* __restrict__ netlab, int* __restrict__ next) {
     int e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -118,12 +120,10 @@ static inline unsigned nb(long long n) { return (unsigned)((n + 255) / 256); }
 cudaError_t launch_label_rounds(int m, int E, const int* np, const int* pc, int* lab, int* next,
                                 int* dist, int* netlab, cudaStream_t s) {
     if (m <= 0) return cudaSuccess;
-    k_lp_init<<<nb(m), 256, 0, s>>>(m, kSeedStride, lab, dist);
+    k_lp_init<<<nb(m), 256, 0, s>>>(m, kSeedStride, lab, next, dist);
     // no nets: every cell keeps its seed label (or none) at distance 0 / unset
     for (int r = 0; r < (E > 0 ? kLabelRounds : 0); ++r) {
         k_lp_net<<<nb(E), 256, 0, s>>>(E, np, pc, m, kRankMaxDegree, lab, netlab);
-        cudaError_t e = cudaMemcpyAsync(next, lab, (size_t)m * sizeof(int), cudaMemcpyDeviceToDevice, s);
-        if (e != cudaSuccess) return e;
         k_lp_cell<<<nb(E), 256, 0, s>>>(E, np, pc, m, netlab, next);
         k_lp_step<<<nb(m), 256, 0, s>>>(m, r, lab, next, dist);
     }
