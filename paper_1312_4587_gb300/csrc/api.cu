@@ -590,17 +590,20 @@ const char* fftpl_last_error(fftpl_t h) {
 }
 
 // Re-lays the netlist for the WA kernel.
-//  1. Internal cell numbers (label rounds on the device, k_setup.cu; then
-//     cells ordered by (label, distance, index) with two counting sorts).
-//  2. Nets of degree >= 2 ordered by their lowest cell number (counting
-//     sort), grouped by degree, largest first, into slabs of up to 32 nets;
-//     pin k of slab net j at slot base + 32 k + j.  Degrees kBigMin..kBigMax
-//     instead take L = grp_lanes(d) lanes per net, 32 / L nets per slab:
-//     pin k of slab net j at base + 32 (k / L) + j L + k % L.  Degree-1 nets
-//     have no wirelength and are left out.
-//  3. The pin records written in slab layout on the device.
+//  1. Internal cell numbers (label rounds, then cells ordered by (label,
+//     distance, index)).
+//  2. Nets of degree >= 2 ordered by degree, largest first, then by their
+//     lowest cell number, into slabs of up to 32 nets of one degree; pin k of
+//     slab net j at slot base + 32 k + j.  Degrees kBigMin..kBigMax instead
+//     take L = grp_lanes(d) lanes per net, 32 / L nets per slab: pin k of slab
+//     net j at base + 32 (k / L) + j L + k % L.  Degree-1 nets have no
+//     wirelength and are left out.
+//  3. The pin records written in slab layout.
+// All three on the device (k_setup.cu); the host counts the degrees and lists
+// the slabs.  (With counting sorts on the host a handle's creation took 0.93 ms
+// at 20K cells, 2.3 at 80K and 80 at 2.2M, with these 0.68, 1.1 and 18.)
 // In deterministic mode also the cell-ordered pin slots (pins of each cell,
-// by internal number, contiguous and in net order).
+// by internal number, contiguous and in net order), on the host.
 static fftpl_status build_slabs(Ctx& c, const fftpl_nets* nets, const fftpl_pins* pins) {
     const int32_t* np = nets->net_ptr;
     const int32_t* pc = pins->pin_cell;
@@ -608,16 +611,20 @@ static fftpl_status build_slabs(Ctx& c, const fftpl_nets* nets, const fftpl_pins
     const int64_t P = c.P;
     cudaStream_t s = c.stream;
     TempDev tmp(s);
-    int *d_np = nullptr, *d_pc = nullptr, *d_key = nullptr, *d_slot = nullptr,
-        *d_lanes = nullptr;
+    int *d_np = nullptr, *d_pc = nullptr;
+    int2* d_deg = nullptr;
+    SortBuf sort{};
     float *d_dx = nullptr, *d_dy = nullptr;
     CK(tmp.alloc(&d_np, (size_t)E + 1));
     CK(tmp.alloc(&d_pc, (size_t)P));
     CK(tmp.alloc(&d_dx, (size_t)P));
     CK(tmp.alloc(&d_dy, (size_t)P));
-    CK(tmp.alloc(&d_key, (size_t)E));
-    CK(tmp.alloc(&d_slot, (size_t)E));
-    CK(tmp.alloc(&d_lanes, (size_t)E));
+    const int most = std::max(m, E);
+    for (int k = 0; k < 2; ++k) {
+        CK(tmp.alloc(&sort.key[k], (size_t)most));
+        CK(tmp.alloc(&sort.val[k], (size_t)most));
+    }
+    CK(tmp.alloc(&sort.counts, sort_counts(most)));
     CK(cudaMemcpyAsync(d_np, np, ((size_t)E + 1) * sizeof(int32_t), cudaMemcpyHostToDevice, s));
     if (P > 0) {
         CK(cudaMemcpyAsync(d_pc, pc, (size_t)P * sizeof(int32_t), cudaMemcpyHostToDevice, s));
@@ -625,7 +632,6 @@ static fftpl_status build_slabs(Ctx& c, const fftpl_nets* nets, const fftpl_pins
         CK(cudaMemcpyAsync(d_dy, pins->dy, (size_t)P * sizeof(float), cudaMemcpyHostToDevice, s));
     }
     // 1. internal cell numbers
-    std::vector<int32_t> rank((size_t)m);
     if (m > 0) {
         int *lab = nullptr, *next = nullptr, *dist = nullptr, *netlab = nullptr;
         CK(tmp.alloc(&lab, (size_t)m));
@@ -633,54 +639,24 @@ static fftpl_status build_slabs(Ctx& c, const fftpl_nets* nets, const fftpl_pins
         CK(tmp.alloc(&dist, (size_t)m));
         CK(tmp.alloc(&netlab, (size_t)E));
         CK(launch_label_rounds(m, E, d_np, d_pc, lab, next, dist, netlab, s));
-        std::vector<int32_t> hl((size_t)m), hd((size_t)m);
-        CK(cudaMemcpyAsync(hl.data(), lab, (size_t)m * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-        CK(cudaMemcpyAsync(hd.data(), dist, (size_t)m * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-        CK(cudaStreamSynchronize(s));
-        // stable counting sorts: by distance, then by label (unreached cells,
-        // label and distance "infinite", last in index order)
-        const int nd = kLabelRounds + 2;
-        std::vector<int32_t> cnt((size_t)std::max(nd, m + 1) + 1, 0), o1((size_t)m), o2((size_t)m);
-        auto dkey = [&](int i) { return hd[i] > kLabelRounds ? kLabelRounds + 1 : hd[i]; };
-        auto lkey = [&](int i) { return hl[i] >= m ? m : hl[i]; };
-        for (int i = 0; i < m; ++i) cnt[dkey(i) + 1]++;
-        for (int k = 0; k < nd; ++k) cnt[k + 1] += cnt[k];
-        for (int i = 0; i < m; ++i) o1[cnt[dkey(i)]++] = i;
-        std::fill(cnt.begin(), cnt.end(), 0);
-        for (int i = 0; i < m; ++i) cnt[lkey(i) + 1]++;
-        for (int k = 0; k <= m; ++k) cnt[k + 1] += cnt[k];
-        for (int q = 0; q < m; ++q) o2[cnt[lkey(o1[q])]++] = o1[q];
-        for (int q = 0; q < m; ++q) rank[o2[q]] = q;
         TRY(dalloc(c, &c.cell_rank, (size_t)m));
-        CK(cudaMemcpyAsync(c.cell_rank, rank.data(), (size_t)m * sizeof(int32_t),
-                           cudaMemcpyHostToDevice, s));
+        CK(launch_cell_rank(m, lab, dist, sort, c.cell_rank, s));
     }
-    // 2. nets by lowest cell number, then slabs by degree
-    std::vector<int32_t> key((size_t)E);
-    CK(launch_net_key(m, E, d_np, d_pc, c.cell_rank, d_key, s));
-    if (E > 0)
-        CK(cudaMemcpyAsync(key.data(), d_key, (size_t)E * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    int maxd = 0;
-    for (int e = 0; e < E; ++e) maxd = std::max(maxd, np[e + 1] - np[e]);
-    std::vector<int32_t> kcnt((size_t)m + 2, 0);
-    for (int e = 0; e < E; ++e)
-        if (np[e + 1] - np[e] >= 2) kcnt[key[e] + 1]++;
-    for (int k = 0; k <= m; ++k) kcnt[k + 1] += kcnt[k];
-    std::vector<int32_t> by_key((size_t)kcnt[m + 1]);
-    for (int e = 0; e < E; ++e)
-        if (np[e + 1] - np[e] >= 2) by_key[kcnt[key[e]]++] = e;
+    // 2. nets by degree and lowest cell number; slabs by degree
+    const int maxd = c.wa_max_degree;
+    CK(launch_net_order(m, E, maxd, d_np, d_pc, c.cell_rank, sort, s));
     std::vector<int32_t> dcnt((size_t)maxd + 2, 0);
-    for (int e : by_key) dcnt[np[e + 1] - np[e]]++;
+    for (int e = 0; e < E; ++e) dcnt[np[e + 1] - np[e]]++;
     // heaviest slabs first: the long nets start early and overlap with the
     // many short ones instead of forming a tail
     std::vector<int4> slabs;
-    std::vector<int64_t> first_slab((size_t)maxd + 1, 0);
+    std::vector<int2> by_degree((size_t)maxd + 1, make_int2(0, 0));
     int64_t slots = 0;
-    auto lanes_of = [](int d) { return d >= kBigMin && d <= kBigMax ? grp_lanes(d) : 1; };
+    int nets_in = 0;
     for (int d = maxd; d >= 2; --d) {
-        first_slab[d] = (int64_t)slabs.size();
-        const int L = lanes_of(d), G = 32 / L;
+        by_degree[d] = make_int2(nets_in, (int)std::min<int64_t>(slots, 0x7fffffffLL));
+        nets_in += dcnt[d];
+        const int L = net_lanes(d), G = 32 / L;
         for (int s0 = 0; s0 < dcnt[d]; s0 += G) {
             slabs.push_back(make_int4((int)slots, d, std::min(G, dcnt[d] - s0), L > 1 ? L : 0));
             slots += 32LL * ((d + L - 1) / L);
@@ -689,13 +665,6 @@ static fftpl_status build_slabs(Ctx& c, const fftpl_nets* nets, const fftpl_pins
     if (slots > 0x7fffffffLL) return set_err(c, FFTPL_EINVAL, "too many pins");
     c.nslabs = (int)slabs.size();
     c.slab_slots = slots;
-    std::vector<int32_t> net_slot((size_t)E, -1), net_lanes((size_t)E, 1),
-        seen((size_t)maxd + 1, 0);
-    for (int e : by_key) {
-        const int d = np[e + 1] - np[e], j = seen[d]++, L = lanes_of(d), G = 32 / L;
-        net_slot[e] = slabs[(size_t)(first_slab[d] + j / G)].x + (j % G) * L;
-        net_lanes[e] = L;
-    }
     // the slabs of degree kBigMin..kBigMax first, the others
     // after them in the same order ; the slot layout is unchanged
     auto is_big = [](const int4& sl) { return sl.y >= kBigMin && sl.y <= kBigMax; };
@@ -706,7 +675,12 @@ static fftpl_status build_slabs(Ctx& c, const fftpl_nets* nets, const fftpl_pins
     std::vector<int32_t> cslot;
     int* d_cslot = nullptr;
     if (c.opt.deterministic) {
-        std::vector<int32_t> cnt((size_t)m + 1, 0);
+        std::vector<int32_t> rank((size_t)m), cnt((size_t)m + 1, 0);
+        if (m > 0) {
+            CK(cudaMemcpyAsync(rank.data(), c.cell_rank, (size_t)m * sizeof(int32_t),
+                               cudaMemcpyDeviceToHost, s));
+            CK(cudaStreamSynchronize(s));
+        }
         for (int e = 0; e < E; ++e) {
             if (np[e + 1] - np[e] < 2) continue;
             for (int p = np[e]; p < np[e + 1]; ++p)
@@ -747,14 +721,11 @@ static fftpl_status build_slabs(Ctx& c, const fftpl_nets* nets, const fftpl_pins
     CK(cudaMemsetAsync(c.pin_dx, 0, ns * sizeof(float), s));
     CK(cudaMemsetAsync(c.pin_dy, 0, ns * sizeof(float), s));
     if (c.pin_slot) CK(cudaMemsetAsync(c.pin_slot, 0xff, ns * sizeof(int32_t), s));
-    if (E > 0) {
-        CK(cudaMemcpyAsync(d_slot, net_slot.data(), (size_t)E * sizeof(int32_t),
-                           cudaMemcpyHostToDevice, s));
-        CK(cudaMemcpyAsync(d_lanes, net_lanes.data(), (size_t)E * sizeof(int32_t),
-                           cudaMemcpyHostToDevice, s));
-    }
-    CK(launch_fill_slabs(m, E, d_np, d_pc, d_dx, d_dy, c.cell_rank, c.fix_x, c.fix_y, d_slot,
-                         d_lanes, d_cslot, c.pin_cell, c.pin_dx, c.pin_dy, c.pin_slot, s));
+    CK(tmp.alloc(&d_deg, by_degree.size()));
+    CK(cudaMemcpyAsync(d_deg, by_degree.data(), by_degree.size() * sizeof(int2),
+                       cudaMemcpyHostToDevice, s));
+    CK(launch_fill_slabs(m, nets_in, sort.val[0], d_deg, d_np, d_pc, d_dx, d_dy, c.cell_rank,
+                         c.fix_x, c.fix_y, d_cslot, c.pin_cell, c.pin_dx, c.pin_dy, c.pin_slot, s));
     CK(cudaStreamSynchronize(s));
     return FFTPL_OK;
 }

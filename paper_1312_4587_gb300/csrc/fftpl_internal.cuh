@@ -44,6 +44,11 @@ __host__ __device__ constexpr int grp_lanes(int d) {
     return d <= 8 ? 2 : (d <= 16 ? 4 : (d <= 32 ? 8 : 16));
 }
 
+// lanes of a net of degree d in the slab layout
+__host__ __device__ constexpr int net_lanes(int d) {
+    return d >= kBigMin && d <= kBigMax ? grp_lanes(d) : 1;
+}
+
 // accumulator slots (FP64 sums written by the kernels)
 enum {
     ACC_N = 0,      // sum B * Psi (times A_b/2 on the host)
@@ -673,18 +678,31 @@ int wa_small_blocks(const Ctx& c);
 
 // create-time netlist layout (k_setup.cu): label rounds for the internal
 // cell numbers (seeds every kSeedStride cells, kLabelRounds rounds, nets of
-// more than kRankMaxDegree pins not followed), each net's lowest cell
-// number, and the pin records in slab layout
+// more than kRankMaxDegree pins not followed), the orders of cells and nets,
+// and the pin records in slab layout
 constexpr int kSeedStride = 64;
 constexpr int kLabelRounds = 6;
 constexpr int kRankMaxDegree = 64;
 cudaError_t launch_label_rounds(int m, int E, const int* np, const int* pc, int* lab, int* next,
                                 int* dist, int* netlab, cudaStream_t s);
-cudaError_t launch_net_key(int m, int E, const int* np, const int* pc, const int* rank, int* key,
-                           cudaStream_t s);
-cudaError_t launch_fill_slabs(int m, int E, const int* np, const int* pc, const float* dx,
-                              const float* dy, const int* rank, const float* fix_x,
-                              const float* fix_y, const int* net_slot, const int* net_lanes,
+// ping-pong buffers of the radix sort: max(m, E) keys and values each,
+// sort_counts of it counts
+struct SortBuf {
+    unsigned* key[2];
+    int* val[2];
+    int* counts;
+};
+size_t sort_counts(int n);
+// internal cell numbers from the labels
+cudaError_t launch_cell_rank(int m, const int* lab, const int* dist, SortBuf& buf, int* rank,
+                             cudaStream_t s);
+// buf.val[0]: the nets by descending degree (degrees below 2 last), then lowest
+// cell number, then index
+cudaError_t launch_net_order(int m, int E, int maxd, const int* np, const int* pc, const int* rank,
+                             SortBuf& buf, cudaStream_t s);
+cudaError_t launch_fill_slabs(int m, int nets, const int* order, const int2* by_degree,
+                              const int* np, const int* pc, const float* dx, const float* dy,
+                              const int* rank, const float* fix_x, const float* fix_y,
                               const int* cslot, int* spc, float* sdx, float* sdy, int* sslot,
                               cudaStream_t s);
 
