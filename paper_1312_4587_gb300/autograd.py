@@ -28,7 +28,10 @@ def _same_stream(problem, device):
 
 def _plain_scalar(g):
     """A float64 CUDA scalar with memory of its own (not, say, a batch of
-    gradients under vmap, which has no data pointer)."""
+    gradients under vmap, which has no data pointer) that no graph is being
+    recorded for (create_graph: the product with it is differentiable)."""
+    if torch.is_grad_enabled() and g.requires_grad:
+        return False
     if g.dtype != torch.float64 or not g.is_cuda or g.dim() != 0:
         return False
     try:

@@ -1,5 +1,6 @@
 """density_energy where its device-side path may not be taken: on another
-stream than the handle's, and with a batch of incoming gradients.  The handle
+stream than the handle's, with a batch of incoming gradients, and where the
+gradient is itself differentiated by the incoming one.  The handle
 is deterministic, so every way has to give the same bits."""
 import numpy as np
 import pytest
@@ -64,3 +65,24 @@ def test_batched_gradients(F):
         for k in range(3):
             hx, hy = torch.autograd.grad(N, (x, y), grad_outputs=w[k], retain_graph=True)
             assert torch.equal(gx[k], hx) and torch.equal(gy[k], hy)
+
+
+def test_gradient_differentiable_by_the_incoming_one(F):
+    # d/dw sum(w dN/dx) = sum(dN/dx)
+    import torch
+    from paper_1312_4587_gb300.autograd import density_energy
+    inst = synth.make_instance("medium")
+    x = torch.from_numpy(inst.x).cuda().requires_grad_(True)
+    y = torch.from_numpy(inst.y).cuda()
+    w = torch.tensor(0.3, dtype=torch.float64, device="cuda", requires_grad=True)
+    with F.Problem(inst, deterministic=1) as p:
+        N = density_energy(x, y, p)
+        gx, = torch.autograd.grad(N, x, grad_outputs=w, create_graph=True)
+        one, = torch.autograd.grad(N, x, retain_graph=True)
+        plain, = torch.autograd.grad(N, x, grad_outputs=w.detach())
+        assert torch.equal(gx, plain)
+        v = one.sign()
+        dw, = torch.autograd.grad((gx * v).sum(), w)
+        ref = one.double().abs().sum().item()
+        # a float32 sum of m terms
+        assert abs(dw.item() - ref) <= 2.0 ** -24 * x.numel() * ref
