@@ -50,19 +50,18 @@ def stage_bytes(m, n, P, E):
 STAGE_IDS = {"scatter": 0, "rows_fwd": 1, "cols": 2, "rows_inv": 3, "wa": 4, "cells": 5}
 
 # DRAM traffic per stage launch on the 2.2M-cell instance, dram__bytes_read.sum
-# + dram__bytes_write.sum of the stage's kernels from one ncu --set full
+# + dram__bytes_write.sum of the stage's kernels from one ncu
 # capture of this script (its summary is kept under profiles/), valid only
 # while the kernel
 # source it was taken from is unchanged: key = first 16 hex digits of the
 # SHA-256 of the kernel file followed by fftpl_internal.cuh.
 STAGE_TRAFFIC = {
-    "scatter": ("k_density.cu", "fd2949651050cefb", 50778624 + 627968),
-    "rows_fwd": ("k_spectral.cu", "a85e897b6059aa28", 33647616 + 16384),
-    "cols": ("k_spectral.cu", "a85e897b6059aa28", 17206528 + 331520),
-    "rows_inv": ("k_spectral.cu", "a85e897b6059aa28", 33614080 + 526336),
-    # k_wa and k_wa_grp
-    "wa": ("k_wire.cu", "a06baad7461894fc", 103047680 + 4505856 + 70472448 + 968704),
-    "cells": ("k_wire.cu", "a06baad7461894fc", 76424960 + 14908672),
+    "scatter": ("k_density.cu", "9c3e14b604172bd7", 50747136 + 1101824),
+    "rows_fwd": ("k_spectral.cu", "83c53d6aa0bbad29", 33621760 + 25088),
+    "cols": ("k_spectral.cu", "83c53d6aa0bbad29", 16872192 + 9472),
+    "rows_inv": ("k_spectral.cu", "83c53d6aa0bbad29", 33615104 + 302336),
+    "wa": ("k_wire.cu", "9c6f67605701cf9e", 139707136 + 4197376),
+    "cells": ("k_wire.cu", "9c6f67605701cf9e", 76204032 + 13038848),
 }
 
 
