@@ -101,7 +101,8 @@ cudaError_t host_slot(double** p) {
     if (g_host_free.empty()) {
         constexpr int kSlots = 256;
         char* block = nullptr;
-        cudaError_t e = cudaHostAlloc((void**)&block, kSlots * kHostSlot, cudaHostAllocMapped | cudaHostAllocPortable);
+        cudaError_t e = cudaHostAlloc((void**)&block, kSlots * kHostSlot,
+                                      cudaHostAllocMapped | cudaHostAllocPortable);
         if (e != cudaSuccess) return e;
         for (int k = kSlots - 1; k >= 0; --k)
             g_host_free.push_back(reinterpret_cast<double*>(block + k * kHostSlot));
@@ -665,8 +666,8 @@ static fftpl_status build_slabs(Ctx& c, const fftpl_nets* nets, const fftpl_pins
     if (slots > 0x7fffffffLL) return set_err(c, FFTPL_EINVAL, "too many pins");
     c.nslabs = (int)slabs.size();
     c.slab_slots = slots;
-    // the slabs of degree kBigMin..kBigMax first, the others
-    // after them in the same order ; the slot layout is unchanged
+    // the slabs of degree kBigMin..kBigMax first, the others after them in the
+    // same order; the slot layout is unchanged
     auto is_big = [](const int4& sl) { return sl.y >= kBigMin && sl.y <= kBigMax; };
     std::stable_partition(slabs.begin(), slabs.end(), is_big);
     c.nbig = (int)std::count_if(slabs.begin(), slabs.end(), is_big);
