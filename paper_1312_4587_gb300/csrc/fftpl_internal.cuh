@@ -159,16 +159,18 @@ __device__ __forceinline__ void quad_ov(const Grid& g, const Span& s, int q, flo
     }
 }
 
-// Four bins of the interleaved field, (E_x, E_y) each: one 32-byte sector.
+// Four bins of the interleaved field, (E_x, E_y) each: one 32-byte sector (a
+// coherent load behind chain_wait, as ld_dep).
 struct Field4 {
     float v[8];
 };
 __device__ __forceinline__ Field4 load_field4(const float2* p) {
     Field4 f;
-    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=f"(f.v[0]), "=f"(f.v[1]), "=f"(f.v[2]), "=f"(f.v[3]), "=f"(f.v[4]), "=f"(f.v[5]),
-          "=f"(f.v[6]), "=f"(f.v[7])
-        : "l"(p));
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(f.v[0]), "=f"(f.v[1]), "=f"(f.v[2]), "=f"(f.v[3]), "=f"(f.v[4]),
+                   "=f"(f.v[5]), "=f"(f.v[6]), "=f"(f.v[7])
+                 : "l"(p)
+                 : "memory");
     return f;
 }
 
@@ -277,6 +279,33 @@ __device__ __forceinline__ void chain_wait() {
 }
 __device__ __forceinline__ void chain_trigger() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+// What the kernel before in a chain writes is read with these: coherent (the
+// read-only path, ld.global.nc and __ldg, is for data that no one writes while
+// the kernel lives, and a kernel of a chain lives while its predecessor still
+// writes) and volatile (no compiler moves them above chain_wait).
+__device__ __forceinline__ float ld_dep(const float* p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ float2 ld_dep(const float2* p) {
+    float2 v;
+    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ float4 ld_dep(const float4* p) {
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "l"(p)
+                 : "memory");
+    return v;
+}
+__device__ __forceinline__ longlong2 ld_dep(const longlong2* p) {
+    longlong2 v;
+    asm volatile("ld.global.v2.s64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
+    return v;
 }
 
 template <typename... P, typename... A>

@@ -111,8 +111,8 @@ k_bin_ranges(Grid g, int m, const float* __restrict__ x, const float* __restrict
 template <bool ADJ>
 __global__ void __launch_bounds__(kCellThreads, kCellBlocks)
 k_gather(Grid g, int m, const float* __restrict__ x, const float* __restrict__ y,
-         const float* __restrict__ w, const float* __restrict__ h, const float* __restrict__ fx,
-         const float2* __restrict__ E2, float* __restrict__ gx, float* __restrict__ gy,
+         const float* __restrict__ w, const float* __restrict__ h, const float* fx,
+         const float2* E2, float* __restrict__ gx, float* __restrict__ gy,
          const double* __restrict__ scale, double* __restrict__ acc, DetRed dr) {
     const int stride = gridDim.x * blockDim.x;
     int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -140,14 +140,14 @@ k_gather(Grid g, int m, const float* __restrict__ x, const float* __restrict__ y
             for (int j = s.jlo; j <= s.jhi; ++j) {
                 float oy = ov_len(g.y0, g.hb, j, s.yl, s.yh);
                 const float* r = fx + (size_t)j * n;
-                float d = (kr_in ? __ldg(r + kr) : 0.0f) - (kl_in ? __ldg(r + kl) : 0.0f);
+                float d = (kr_in ? ld_dep(r + kr) : 0.0f) - (kl_in ? ld_dep(r + kl) : 0.0f);
                 sx = fmaf(oy, d, sx);
             }
             const float* rt = fx + (size_t)(jr_in ? jr : 0) * n;
             const float* rb = fx + (size_t)(jl_in ? jl : 0) * n;
             for (int k = s.ilo; k <= s.ihi; ++k) {
                 float ox = ov_len(g.x0, g.wb, k, s.xl, s.xh);
-                float d = (jr_in ? __ldg(rt + k) : 0.0f) - (jl_in ? __ldg(rb + k) : 0.0f);
+                float d = (jr_in ? ld_dep(rt + k) : 0.0f) - (jl_in ? ld_dep(rb + k) : 0.0f);
                 sy = fmaf(ox, d, sy);
             }
         }

@@ -38,6 +38,8 @@
 // (bound by the shared-memory pipe at 22 % warps active), launch times under
 // ncu, cold caches: n = 2048 rows_fwd 19.9 -> 15.2, cols 39.3 -> 24.5,
 // rows_inv 26.6 -> 15.8 us; n = 4096 96 -> 58, 187 -> 99, 111 -> 52 us.
+#include <type_traits>
+
 #include "fftpl_internal.cuh"
 
 namespace fftpl {
@@ -501,7 +503,7 @@ __device__ __forceinline__ void store_tile(const float4* tile, float* dst, const
 // Group: 4 rows y0 .. y0+3 of rho (2 per complex FFT) -> T1[u/2][y0..y0+3].
 template <int LOGN, bool QUANT>
 __global__ void __launch_bounds__(Lay<LOGN, 2>::T, spec_blocks(LOGN, Lay<LOGN, 2>::T))
-k_rows_fwd(const float* __restrict__ D, const long long* __restrict__ Dq,
+k_rows_fwd(const float* D, const long long* Dq,
            const float* __restrict__ M, float inv_ab, float cap, float* __restrict__ T1,
            double* __restrict__ acc, DetRed dr, const __grid_constant__ CUtensorMap mT1, int tma) {
     using L = Lay<LOGN, 2>;
@@ -521,27 +523,32 @@ k_rows_fwd(const float* __restrict__ D, const long long* __restrict__ Dq,
     // per-thread sums of 2 E non-negative terms in float32
     float tau = 0.0f, charge = 0.0f;
     float2 v[1][E];
+    // all of D's loads first
+    const size_t b = (size_t)(y0 + 2 * f) * N + 2 * ta;
+    typename std::conditional<QUANT, longlong2, float2>::type dd[2][E / 2];
 #pragma unroll
     for (int q = 0; q < E / 2; ++q) {
-        // samples 2p and 2p+1 of both rows: elements p and N-1-p
-        const int p = ta + Q * q;
-        const size_t b0 = (size_t)(y0 + 2 * f) * N + 2 * p, b1 = b0 + N;
+        const size_t b0 = b + 2 * Q * q;
+        if constexpr (QUANT) {
+            dd[0][q] = ld_dep(reinterpret_cast<const longlong2*>(Dq + b0));
+            dd[1][q] = ld_dep(reinterpret_cast<const longlong2*>(Dq + b0 + N));
+        } else {
+            dd[0][q] = ld_dep(reinterpret_cast<const float2*>(D + b0));
+            dd[1][q] = ld_dep(reinterpret_cast<const float2*>(D + b0 + N));
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < E / 2; ++q) {
+        // samples 2p and 2p+1 of both rows, p = ta + Q q: elements p and N-1-p
+        const size_t b0 = b + 2 * Q * q, b1 = b0 + N;
         float d[4], mm[4];
         const float2 m0 = __ldg(reinterpret_cast<const float2*>(M + b0));
         const float2 m1 = __ldg(reinterpret_cast<const float2*>(M + b1));
         mm[0] = m0.x; mm[1] = m0.y; mm[2] = m1.x; mm[3] = m1.y;
-        if (QUANT) {
-            const longlong2 q0 = __ldg(reinterpret_cast<const longlong2*>(Dq + b0));
-            const longlong2 q1 = __ldg(reinterpret_cast<const longlong2*>(Dq + b1));
-            d[0] = (float)q0.x * 2.3283064365386963e-10f;
-            d[1] = (float)q0.y * 2.3283064365386963e-10f;
-            d[2] = (float)q1.x * 2.3283064365386963e-10f;
-            d[3] = (float)q1.y * 2.3283064365386963e-10f;
-        } else {
-            const float2 v0 = __ldg(reinterpret_cast<const float2*>(D + b0));
-            const float2 v1 = __ldg(reinterpret_cast<const float2*>(D + b1));
-            d[0] = v0.x; d[1] = v0.y; d[2] = v1.x; d[3] = v1.y;
-        }
+        d[0] = (float)dd[0][q].x; d[1] = (float)dd[0][q].y;
+        d[2] = (float)dd[1][q].x; d[3] = (float)dd[1][q].y;
+        if (QUANT)
+            for (int t = 0; t < 4; ++t) d[t] *= 2.3283064365386963e-10f;
         float rv[4];
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
@@ -620,7 +627,7 @@ __device__ __forceinline__ void spectral_elem(float2 zu, float2 zn, float2 p, fl
 // begin with, so the spectrum never leaves the registers.
 template <int LOGN>
 __global__ void __launch_bounds__(Lay<LOGN, 2>::T, spec_blocks(LOGN, Lay<LOGN, 2>::T))
-k_cols(const float* __restrict__ T1, float* __restrict__ PT, float* __restrict__ RT, float pi_lx,
+k_cols(const float* T1, float* __restrict__ PT, float* __restrict__ RT, float pi_lx,
        float pi_ly, float eps, double* __restrict__ acc, DetRed dr,
        const __grid_constant__ CUtensorMap mPT, const __grid_constant__ CUtensorMap mRT, int tma) {
     using L = Lay<LOGN, 2>;
@@ -645,7 +652,7 @@ k_cols(const float* __restrict__ T1, float* __restrict__ PT, float* __restrict__
         const float4* row = reinterpret_cast<const float4*>(T1 + (size_t)(u0 / 2 + f) * (2 * N));
 #pragma unroll
         for (int q = 0; q < E / 2; ++q) {
-            const float4 a = __ldg(row + ta + Q * q);   // samples 2p, 2p+1 of both rows
+            const float4 a = ld_dep(row + ta + Q * q);   // samples 2p, 2p+1 of both rows
             v[0][q] = make_float2(a.x, a.y);
             v[0][E - 1 - q] = make_float2(a.z, a.w);
         }
@@ -744,7 +751,7 @@ enum { INV_FIELD, INV_PSI, INV_MAPS };
 // by Parseval).
 template <int LOGN, int WHAT>
 __global__ void __launch_bounds__(Lay<LOGN, 1>::T, spec_blocks(LOGN, Lay<LOGN, 1>::T))
-k_rows_inv(const float* __restrict__ PT, const float* __restrict__ RT, float2* __restrict__ E2,
+k_rows_inv(const float* PT, const float* RT, float2* __restrict__ E2,
            float* __restrict__ psi, float* __restrict__ ex, float* __restrict__ ey, float pi_lx) {
     using L = Lay<LOGN, 1>;
     constexpr int N = L::N, Q = L::Q, E = L::E;
@@ -769,8 +776,8 @@ k_rows_inv(const float* __restrict__ PT, const float* __restrict__ RT, float2* _
             float2 c[E], e[E];
 #pragma unroll
             for (int q = 0; q < E; ++q) {
-                c[q] = __ldg(pr + Q * q);
-                e[q] = __ldg(rr + Q * q);
+                c[q] = ld_dep(pr + Q * q);
+                e[q] = ld_dep(rr + Q * q);
             }
             pack_rows<LOGN, true>(c, z[0], k, pb, pi_lx);
             pack_rows<LOGN, false>(e, z[1], k, pb, pi_lx);
@@ -798,7 +805,7 @@ k_rows_inv(const float* __restrict__ PT, const float* __restrict__ RT, float2* _
         {
             float2 c[E];
 #pragma unroll
-            for (int q = 0; q < E; ++q) c[q] = __ldg(pr + Q * q);
+            for (int q = 0; q < E; ++q) c[q] = ld_dep(pr + Q * q);
             pack_rows<LOGN, false>(c, z[0], k, pb, pi_lx);
         }
         if (WHAT == INV_MAPS) group_sync<LOGN, 1>();   // the field's exchange has been read

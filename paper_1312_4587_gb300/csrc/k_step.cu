@@ -150,8 +150,7 @@ __global__ void __launch_bounds__(kCellThreads, kVecBlocksPerSm) k_loop_g(int m2
     dfloat dg = df_zero(), dv = df_zero();
     float gi = 0.0f;
     const int stride = gridDim.x * blockDim.x;
-    const float* __restrict__ GN = b.gN;
-    const float* __restrict__ GW = b.gW;
+    // (the kernel before this one writes gN and gW, the iteration before the rest)
     const float* __restrict__ GP = b.gprev;
     const float* __restrict__ V = b.v;
     const float* __restrict__ VP = b.vprev;
@@ -161,8 +160,8 @@ __global__ void __launch_bounds__(kCellThreads, kVecBlocksPerSm) k_loop_g(int m2
         for (int k = 0; k < 4; ++k) {
             const int i = i0 + k * stride;
             if (i < m2) {
-                gn[k] = GN[i];
-                gw[k] = GW[i];
+                gn[k] = ld_dep(b.gN + i);
+                gw[k] = ld_dep(b.gW + i);
                 if (!first) {
                     gp[k] = GP[i];
                     v[k] = V[i];
@@ -207,7 +206,6 @@ k_loop_update(int m, Grid gr, float x1, float y1, LoopBufs b) {
     dfloat uphill = df_zero();
     const int stride = gridDim.x * blockDim.x, n2 = 2 * m;
     const float* __restrict__ V = b.v;
-    const float* __restrict__ G = b.g;
     const float* __restrict__ U = b.u;
     for (int i0 = blockIdx.x * blockDim.x + threadIdx.x; i0 < n2; i0 += 4 * stride) {
         float vv[4], gg[4], uu[4], hw[4];
@@ -218,7 +216,7 @@ k_loop_update(int m, Grid gr, float x1, float y1, LoopBufs b) {
                 const bool isx = i < m;
                 hw[k] = isx ? b.w[i] : b.h[i - m];
                 vv[k] = V[i];
-                gg[k] = G[i];
+                gg[k] = ld_dep(b.g + i);
                 uu[k] = U[i];
             }
         }
@@ -434,7 +432,7 @@ __global__ void k_gamma0(double* ctrl, const double* acc) {
 // than a plain synchronisation (210K cells; 4.6 at 1,000); this kernel,
 // resident before its predecessor ends, 0.9 (1.3).
 __global__ void __launch_bounds__(32 * kReportSums)
-k_report(const double* __restrict__ acc, double* __restrict__ out, unsigned* __restrict__ count) {
+k_report(const double* acc, double* __restrict__ out, unsigned* __restrict__ count) {
     chain_wait();
     const int q = threadIdx.x >> 5;
     const double t = acc_sum(acc, q);
@@ -450,7 +448,7 @@ k_report(const double* __restrict__ acc, double* __restrict__ out, unsigned* __r
 }
 
 // N of the last solve into device memory (one warp).
-__global__ void k_energy_out(const double* __restrict__ acc, double half_ab,
+__global__ void k_energy_out(const double* acc, double half_ab,
                              double* __restrict__ out) {
     chain_wait();
     const double t = acc_sum(acc, ACC_N);

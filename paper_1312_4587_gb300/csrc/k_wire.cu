@@ -537,7 +537,7 @@ k_cells(Grid g, int m, const float* __restrict__ x, const float* __restrict__ y,
 // Deterministic pin-to-cell sum on its own (fftpl_wa in CSR mode).
 __global__ void __launch_bounds__(1024)
 k_pin_sum(int m, const int* __restrict__ rank, const int* __restrict__ cell_pin_ptr,
-          const float2* __restrict__ gpin, float* __restrict__ gx, float* __restrict__ gy,
+          const float2* gpin, float* __restrict__ gx, float* __restrict__ gy,
           double* __restrict__ acc, DetRed dr) {
     float l1 = 0.0f;
     chain_wait();
@@ -546,7 +546,7 @@ k_pin_sum(int m, const int* __restrict__ rank, const int* __restrict__ cell_pin_
         const int r = rank[i];
         float wx = 0.0f, wy = 0.0f;
         for (int q = cell_pin_ptr[r]; q < cell_pin_ptr[r + 1]; ++q) {
-            float2 v = gpin[q];
+            float2 v = ld_dep(gpin + q);
             wx += v.x;
             wy += v.y;
         }
@@ -560,7 +560,7 @@ k_pin_sum(int m, const int* __restrict__ rank, const int* __restrict__ cell_pin_
 // Splits the interleaved atomic accumulator into gx, gy and adds ||g||_1 (four
 // cells of a thread in flight together on a bounded grid).
 __global__ void __launch_bounds__(1024)
-k_split(int m, const int* __restrict__ rank, const float2* __restrict__ gW2,
+k_split(int m, const int* __restrict__ rank, const float2* gW2,
         float* __restrict__ gx, float* __restrict__ gy, double* __restrict__ acc, DetRed dr) {
     const int stride = gridDim.x * blockDim.x;
     float l1 = 0.0f;
@@ -571,7 +571,7 @@ k_split(int m, const int* __restrict__ rank, const float2* __restrict__ gW2,
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int i = i0 + k * stride;
-            g[k] = i < m ? __ldg(gW2 + __ldg(rank + i)) : make_float2(0.0f, 0.0f);
+            g[k] = i < m ? ld_dep(gW2 + __ldg(rank + i)) : make_float2(0.0f, 0.0f);
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
