@@ -276,6 +276,14 @@ fftpl_status fftpl_energy_device(fftpl_t h, const float* x, const float* y, doub
 fftpl_status fftpl_gather_scaled(fftpl_t h, const float* x, const float* y, int32_t mode,
                                  const double* scale, float* gx, float* gy);
 
+/* Order between the handle and another stream (a cudaStream_t; NULL: the
+ * legacy default stream) whose tensors a call takes or gives; neither waits on
+ * the host.  fftpl_order_after: what the handle enqueues from now on follows
+ * what is on the stream now.  fftpl_order_before: what is enqueued on the
+ * stream from now on follows what the handle has enqueued. */
+fftpl_status fftpl_order_after(fftpl_t h, void* stream);
+fftpl_status fftpl_order_before(fftpl_t h, void* stream);
+
 /* Weighted-average wirelength (Eq. 3) and its gradient; HPWL (Eq. 1) as a
  * by-product.  gx, gy device outputs (m_mov), may be NULL.  W host output:
  * non-NULL synchronises. */

@@ -7,11 +7,14 @@ the exact derivative of the binned energy (mode "adjoint"), scaled by the
 incoming gradient.  Positions are float32 CUDA tensors of the problem's
 movable cells.
 
-On the stream the handle is ordered with, neither direction waits for the
-device: the energy goes straight into the output tensor and the gather kernel
-reads the incoming gradient from the device.  (With a wait and a copy for the
-energy and two multiplications after the gather, forward and backward of 500K
-cells took 380 us of host time for 70 us of kernels.)
+On a stream other than the handle's, the handle's work is ordered after what
+that stream holds (the positions, the incoming gradient, the memory of the
+outputs) and that stream after the handle's work.  On the handle's own stream
+neither direction waits for the device: the energy goes straight into the
+output tensor and the gather kernel reads the incoming gradient from the
+device.  (With a wait and a copy for the energy and two multiplications after
+the gather, forward and backward of 500K cells took 380 us of host time for
+70 us of kernels.)
 """
 from __future__ import annotations
 
@@ -22,8 +25,10 @@ from . import fftpl as F
 _MODES = {"gather": 0, "adjoint": 1}
 
 
-def _same_stream(problem, device):
-    return torch.cuda.current_stream(device).cuda_stream == getattr(problem, "stream", None)
+def _other_stream(problem, device):
+    """The current stream if the handle is not ordered with it, else None."""
+    cur = torch.cuda.current_stream(device).cuda_stream
+    return None if cur == getattr(problem, "stream", None) else cur
 
 
 def _plain_scalar(g):
@@ -47,10 +52,12 @@ class DensityEnergy(torch.autograd.Function):
             raise ValueError(f"mode must be one of {sorted(_MODES)}")
         x = x.detach().contiguous()
         y = y.detach().contiguous()
-        if _same_stream(problem, x.device):
+        other = _other_stream(problem, x.device)
+        if other is None:
             N = torch.empty((), dtype=torch.float64, device=x.device)
             F.fftpl_energy_device(problem.h, x, y, N)
         else:
+            F.fftpl_order_after(problem.h, other)
             N = torch.tensor(F.fftpl_energy(problem.h, x, y), dtype=torch.float64,
                              device=x.device)
         problem._energy_calls = getattr(problem, "_energy_calls", 0) + 1
@@ -64,16 +71,21 @@ class DensityEnergy(torch.autograd.Function):
     def backward(ctx, grad_out):
         x, y = ctx.saved_tensors
         problem = ctx.problem
+        gx = torch.empty_like(x)
+        gy = torch.empty_like(y)
+        other = _other_stream(problem, x.device)
+        if other is not None:
+            F.fftpl_order_after(problem.h, other)
         if problem._energy_calls != ctx.call:
             # the handle's maps belong to a later evaluation: recompute them
             F.fftpl_energy(problem.h, x, y, sync=False)
             problem._energy_calls += 1
-        gx = torch.empty_like(x)
-        gy = torch.empty_like(y)
-        if _plain_scalar(grad_out) and _same_stream(problem, x.device):
+        if other is None and _plain_scalar(grad_out):
             F.fftpl_gather_scaled(problem.h, x, y, grad_out, gx, gy, _MODES[ctx.mode])
             return gx, gy, None, None
         F.fftpl_gather(problem.h, x, y, gx, gy, _MODES[ctx.mode])
+        if other is not None:
+            F.fftpl_order_before(problem.h, other)
         s = grad_out.to(torch.float32)
         return gx * s, gy * s, None, None
 

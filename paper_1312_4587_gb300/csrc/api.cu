@@ -993,6 +993,21 @@ fftpl_status fftpl_gather_scaled(fftpl_t h, const float* x, const float* y, int3
     return FFTPL_OK;
 }
 
+// (ev_fork is free between calls: a wait takes the record before it)
+static fftpl_status order_streams(Ctx& c, cudaStream_t first, cudaStream_t then) {
+    CK(cudaEventRecord(c.ev_fork, first));
+    CK(cudaStreamWaitEvent(then, c.ev_fork, 0));
+    return FFTPL_OK;
+}
+
+fftpl_status fftpl_order_after(fftpl_t h, void* stream) {
+    return h ? order_streams(*h, (cudaStream_t)stream, h->stream) : FFTPL_EINVAL;
+}
+
+fftpl_status fftpl_order_before(fftpl_t h, void* stream) {
+    return h ? order_streams(*h, h->stream, (cudaStream_t)stream) : FFTPL_EINVAL;
+}
+
 fftpl_status fftpl_wa(fftpl_t h, const float* x, const float* y, float gamma, double* W,
                       float* gx, float* gy) {
     if (!h || (h->m_mov > 0 && (!x || !y))) return h ? set_err(*h, FFTPL_EINVAL, "null positions") : FFTPL_EINVAL;

@@ -142,6 +142,8 @@ def lib():
             "fftpl_wa": (S, [_H, _P, _P, C.c_float, _P, _P, _P]),
             "fftpl_energy": (S, [_H, _P, _P, _P]),
             "fftpl_gather": (S, [_H, _P, _P, C.c_int32, _P, _P]),
+            "fftpl_order_after": (S, [_H, _P]),
+            "fftpl_order_before": (S, [_H, _P]),
             "fftpl_energy_device": (S, [_H, _P, _P, _P]),
             "fftpl_gather_scaled": (S, [_H, _P, _P, C.c_int32, _P, _P, _P]),
             "fftpl_eval": (S, [_H, _P, _P, C.c_float, _P, _P, _P, _P, _P]),
@@ -311,6 +313,16 @@ def fftpl_energy(h, x, y, sync=True):
 def fftpl_gather(h, x, y, gx, gy, mode=0):
     _check(lib().fftpl_gather(h, _dptr(x), _dptr(y), C.c_int32(int(mode)), _dptr(gx), _dptr(gy)),
            h)
+
+
+def fftpl_order_after(h, stream):
+    """The handle's later work follows what is on the cudaStream_t now."""
+    _check(lib().fftpl_order_after(h, C.c_void_p(int(stream or 0))), h)
+
+
+def fftpl_order_before(h, stream):
+    """Later work on the cudaStream_t follows what the handle has enqueued."""
+    _check(lib().fftpl_order_before(h, C.c_void_p(int(stream or 0))), h)
 
 
 def fftpl_energy_device(h, x, y, N):
