@@ -19,6 +19,7 @@ the gather, forward and backward of 500K cells took 380 us of host time for
 from __future__ import annotations
 
 import torch
+from torch.autograd import forward_ad
 
 from . import fftpl as F
 
@@ -34,15 +35,18 @@ def _other_stream(problem, device):
 def _plain_scalar(g):
     """A float64 CUDA scalar with memory of its own (not, say, a batch of
     gradients under vmap, which has no data pointer) that no graph is being
-    recorded for (create_graph: the product with it is differentiable)."""
+    recorded for (create_graph: the product with it is differentiable) and that
+    carries no forward-mode tangent (the product carries it on)."""
     if torch.is_grad_enabled() and g.requires_grad:
         return False
     if g.dtype != torch.float64 or not g.is_cuda or g.dim() != 0:
         return False
     try:
-        return g.data_ptr() != 0
+        if g.data_ptr() == 0:
+            return False
     except RuntimeError:
         return False
+    return forward_ad.unpack_dual(g).tangent is None
 
 
 class DensityEnergy(torch.autograd.Function):
