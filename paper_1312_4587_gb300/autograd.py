@@ -36,7 +36,8 @@ def _plain_scalar(g):
     """A float64 CUDA scalar with memory of its own (not, say, a batch of
     gradients under vmap, which has no data pointer) that no graph is being
     recorded for (create_graph: the product with it is differentiable) and that
-    carries no forward-mode tangent (the product carries it on)."""
+    carries no forward-mode tangent (the product carries it on); its memory
+    holds the value itself, not the negative a view may stand for."""
     if torch.is_grad_enabled() and g.requires_grad:
         return False
     if g.dtype != torch.float64 or not g.is_cuda or g.dim() != 0:
@@ -46,7 +47,7 @@ def _plain_scalar(g):
             return False
     except RuntimeError:
         return False
-    return forward_ad.unpack_dual(g).tangent is None
+    return not g.is_neg() and forward_ad.unpack_dual(g).tangent is None
 
 
 class DensityEnergy(torch.autograd.Function):

@@ -1,5 +1,6 @@
 """Incoming gradients that the device-side gather cannot take as they lie in
-memory: one that carries a forward-mode tangent."""
+memory: one that carries a forward-mode tangent, one whose memory holds its
+negative."""
 import pytest
 
 import synth
@@ -36,3 +37,21 @@ def test_forward_mode_tangent_of_the_incoming_gradient(case):
                 assert torch.equal(u.primal, r)
                 assert u.tangent is not None
                 assert torch.equal(u.tangent, d)
+
+
+def test_incoming_gradient_with_the_negative_bit(case):
+    # the imaginary part of a conjugate is a view that stands for the negative
+    # of what lies in memory
+    import torch
+    from paper_1312_4587_gb300 import fftpl as F
+    from paper_1312_4587_gb300.autograd import density_energy
+    inst, x, y = case
+    w = torch.tensor([0.5, 0.3], dtype=torch.float64, device="cuda")
+    neg = torch.view_as_complex(w).conj().imag
+    assert neg.is_neg() and neg.item() == -0.3
+    with F.Problem(inst, deterministic=1) as p:
+        N = density_energy(x, y, p)
+        got = torch.autograd.grad(N, (x, y), grad_outputs=neg, retain_graph=True)
+        ref = torch.autograd.grad(N, (x, y), grad_outputs=neg.clone().resolve_neg())
+        for g, r in zip(got, ref):
+            assert torch.equal(g, r)
