@@ -535,7 +535,7 @@ k_cells(Grid g, int m, const float* __restrict__ x, const float* __restrict__ y,
 }
 
 // Deterministic pin-to-cell sum on its own (fftpl_wa in CSR mode).
-__global__ void __launch_bounds__(1024)
+__global__ void __launch_bounds__(kCellThreads)
 k_pin_sum(int m, const int* __restrict__ rank, const int* __restrict__ cell_pin_ptr,
           const float2* gpin, float* __restrict__ gx, float* __restrict__ gy,
           double* __restrict__ acc, DetRed dr) {
@@ -642,15 +642,19 @@ cudaError_t launch_wa(Ctx& c, const float* x, const float* y, float gamma, cudaS
 // (two blocks fill an SM), so the writes take as few SMs as keep the link busy:
 // evaluation of 2.2M cells with host buffers, 8 / 16 / 32 / 64 blocks of 1024
 // threads 458 / 384 / 378 / 371 us, one block of 256 on every SM 413.
+// Deterministic mode takes the cell kernel's grid and blocks instead, whose
+// order of summation it then shares: an evaluation reports the same norm
+// whether its buffers are pinned or not.
 constexpr int kLinkBlocks = 64;
 cudaError_t launch_pin_sum(Ctx& c, float* gx, float* gy, bool few, bool chain, cudaStream_t s) {
     if (c.m_mov <= 0) return cudaSuccess;
-    const int threads = few ? 1024 : kCellThreads;
+    const bool det = c.opt.deterministic != 0;
+    const int threads = few && !det ? 1024 : kCellThreads;
     int nb = nblk(c.m_mov, threads);
-    if (few) nb = std::min(nb, kLinkBlocks);
+    if (few) nb = det ? cell_blocks(c) : std::min(nb, kLinkBlocks);
     cudaError_t e = cudaSuccess;
     // region 1: this pass follows the WA kernel on its stream
-    if (c.opt.deterministic)
+    if (det)
         e = launch_chain(k_pin_sum, nb, threads, 0, s, chain, c.m_mov, c.cell_rank,
                          c.cell_pin_ptr, c.gpin, gx, gy, c.acc, det_red(c, 1));
     else
