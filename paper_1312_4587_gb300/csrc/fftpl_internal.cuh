@@ -405,7 +405,9 @@ __device__ __forceinline__ void red_add_f64(double* p, double v) {
 
 // Sums of non-negative per-thread values a and b over each warp (a float32
 // tree: relative error at most 5 units in the last place for non-negative
-// terms); lane 0 adds each nonzero warp total in FP64 to the stripe of
+// terms, besides what the caller's own sums over a thread's items lost: kernels
+// whose threads take a number of items that grows with the instance keep them
+// as double-float pairs); lane 0 adds each nonzero warp total in FP64 to the stripe of
 // quantity qa / qb (qb < 0: none) chosen by the warp's global index.  No
 // block-wide barrier, and the atomics spread over 32 lines.
 __device__ __forceinline__ void block_acc2(float a, float b, double* acc, int qa, int qb) {

@@ -116,7 +116,7 @@ k_gather(Grid g, int m, const float* __restrict__ x, const float* __restrict__ y
          const double* __restrict__ scale, double* __restrict__ acc, DetRed dr) {
     const int stride = gridDim.x * blockDim.x;
     int i = blockIdx.x * blockDim.x + threadIdx.x;
-    float l1 = 0.0f;
+    dfloat l1 = df_zero();
     chain_wait();
     chain_trigger();
     const float sc = scale ? (float)*scale : 1.0f;
@@ -153,9 +153,9 @@ k_gather(Grid g, int m, const float* __restrict__ x, const float* __restrict__ y
         }
         gx[i] = sc * sx;
         gy[i] = sc * sy;
-        l1 += fabsf(sx) + fabsf(sy);
+        l1 = df_add(l1, fabsf(sx) + fabsf(sy));
     }
-    reduce2(l1, 0.0f, acc, ACC_GN_L1, -1, dr);
+    reduce2(df_val(l1), 0.0f, acc, ACC_GN_L1, -1, dr);
 }
 
 // rho = (D + M) / A_b (formed on demand for fftpl_fields).

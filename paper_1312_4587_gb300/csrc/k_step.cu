@@ -32,7 +32,7 @@ k_loop_cells(Grid gr, int m, LoopBufs b, const float2* __restrict__ E2,
     if (cf[F_DONE] != 0.0f) return;
     const int stride = (gridDim.x - 1) * blockDim.x;
     int i = blockIdx.x * blockDim.x + threadIdx.x;
-    float ln = 0.0f, lw = 0.0f;
+    dfloat ln = df_zero(), lw = df_zero();
     if (blockIdx.x == gridDim.x - 1) {
         if (threadIdx.x < 32) ctrl_lambda(b.ctrl, b.acc);
         else if (threadIdx.x == 32) ctrl_momentum(b.ctrl);
@@ -61,10 +61,10 @@ k_loop_cells(Grid gr, int m, LoopBufs b, const float2* __restrict__ E2,
         b.gN[m + i] = -e.y;
         b.gW[i] = wx;
         b.gW[m + i] = wy;
-        ln += fabsf(e.x) + fabsf(e.y);
-        lw += fabsf(wx) + fabsf(wy);
+        ln = df_add(ln, fabsf(e.x) + fabsf(e.y));
+        lw = df_add(lw, fabsf(wx) + fabsf(wy));
     }
-    reduce2(ln, lw, b.acc, ACC_GN_L1, ACC_GW_L1, b.dr);
+    reduce2(df_val(ln), df_val(lw), b.acc, ACC_GN_L1, ACC_GW_L1, b.dr);
 }
 
 // lambda for the combined gradient: from the control scalars, in the first

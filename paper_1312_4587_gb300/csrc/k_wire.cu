@@ -487,9 +487,9 @@ k_wa(int nb_big, int nbig, int nslabs, int pairs, const int4* __restrict__ slabs
 
 // Per-cell kernel: density gradient by the field gather (q.E of Eq. 7),
 // wirelength gradient by summing the cell's pin gradients (CSR mode) or
-// reading the atomically accumulated sums, and the L1 norms of both (per
-// thread a float32 sum of the non-negative terms of its m / 117K cells at
-// most).
+// reading the atomically accumulated sums, and the L1 norms of both (a
+// double-float sum over the cells of a thread, however many the grid leaves
+// it).
 template <bool CSR>
 __global__ void __launch_bounds__(kCellThreads, kCellBlocks)
 k_cells(Grid g, int m, const float* __restrict__ x, const float* __restrict__ y,
@@ -503,7 +503,7 @@ k_cells(Grid g, int m, const float* __restrict__ x, const float* __restrict__ y,
     chain_trigger();
     const int stride = gridDim.x * blockDim.x;
     int i = blockIdx.x * blockDim.x + threadIdx.x;
-    float ln = 0.0f, lw = 0.0f;
+    dfloat ln = df_zero(), lw = df_zero();
     CellIn c = load_cell(i, m, x, y, w, h, rank);
     for (; i < m; i += stride) {
         const CellIn cur = c;
@@ -528,10 +528,10 @@ k_cells(Grid g, int m, const float* __restrict__ x, const float* __restrict__ y,
         gNy[i] = -e.y;
         gWx[i] = wx;
         gWy[i] = wy;
-        ln += fabsf(e.x) + fabsf(e.y);
-        lw += fabsf(wx) + fabsf(wy);
+        ln = df_add(ln, fabsf(e.x) + fabsf(e.y));
+        lw = df_add(lw, fabsf(wx) + fabsf(wy));
     }
-    reduce2(ln, lw, acc, ACC_GN_L1, ACC_GW_L1, dr);
+    reduce2(df_val(ln), df_val(lw), acc, ACC_GN_L1, ACC_GW_L1, dr);
 }
 
 // Deterministic pin-to-cell sum on its own (fftpl_wa in CSR mode).
@@ -539,7 +539,7 @@ __global__ void __launch_bounds__(kCellThreads)
 k_pin_sum(int m, const int* __restrict__ rank, const int* __restrict__ cell_pin_ptr,
           const float2* gpin, float* __restrict__ gx, float* __restrict__ gy,
           double* __restrict__ acc, DetRed dr) {
-    float l1 = 0.0f;
+    dfloat l1 = df_zero();
     chain_wait();
     chain_trigger();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
@@ -552,9 +552,9 @@ k_pin_sum(int m, const int* __restrict__ rank, const int* __restrict__ cell_pin_
         }
         gx[i] = wx;
         gy[i] = wy;
-        l1 += fabsf(wx) + fabsf(wy);
+        l1 = df_add(l1, fabsf(wx) + fabsf(wy));
     }
-    reduce2(l1, 0.0f, acc, ACC_GW_L1, -1, dr);
+    reduce2(df_val(l1), 0.0f, acc, ACC_GW_L1, -1, dr);
 }
 
 // Splits the interleaved atomic accumulator into gx, gy and adds ||g||_1 (four
@@ -563,7 +563,7 @@ __global__ void __launch_bounds__(1024)
 k_split(int m, const int* __restrict__ rank, const float2* gW2,
         float* __restrict__ gx, float* __restrict__ gy, double* __restrict__ acc, DetRed dr) {
     const int stride = gridDim.x * blockDim.x;
-    float l1 = 0.0f;
+    dfloat l1 = df_zero();
     chain_wait();
     chain_trigger();
     for (int i0 = blockIdx.x * blockDim.x + threadIdx.x; i0 < m; i0 += 4 * stride) {
@@ -579,11 +579,11 @@ k_split(int m, const int* __restrict__ rank, const float2* gW2,
             if (i < m) {
                 gx[i] = g[k].x;
                 gy[i] = g[k].y;
-                l1 += fabsf(g[k].x) + fabsf(g[k].y);
+                l1 = df_add(l1, fabsf(g[k].x) + fabsf(g[k].y));
             }
         }
     }
-    reduce2(l1, 0.0f, acc, ACC_GW_L1, -1, dr);
+    reduce2(df_val(l1), 0.0f, acc, ACC_GW_L1, -1, dr);
 }
 
 static inline int nblk(long long m, int t) { return (int)((m + t - 1) / t); }
