@@ -614,8 +614,9 @@ __device__ __forceinline__ void spectral_elem(float2 zu, float2 zn, float2 p, fl
         nb = 0.0f;
     }
     // B Psi: Psi = 2 ct but at v = 0 (ct = Psi); B is half of ba
-    const float e = fmaf(ba, ca, bb * cb);
-    *energy = df_add(*energy, v0 ? 0.5f * e : e);
+    const float ea = ba * ca, eb = bb * cb;
+    sum2_add(*energy, v0 ? 0.5f * ea : ea);
+    sum2_add(*energy, v0 ? 0.5f * eb : eb);
     *zp = pack_inv(ca, na, cb, nb, p);
     *zr = pack_inv(wn * na, wv * ca, wn * nb, wv * cb, p);
 }
