@@ -173,7 +173,8 @@ void free_ctx(fftpl_ctx* c) {
     if (!c) return;
     if (c->stream) cudaStreamSynchronize(c->stream);
     if (c->side) cudaStreamSynchronize(c->side);
-    if (c->eval_graph) cudaGraphExecDestroy(c->eval_graph);
+    for (auto& g : c->eval_graph)
+        if (g.exec) cudaGraphExecDestroy(g.exec);
     if (c->loop_graph) cudaGraphExecDestroy(c->loop_graph);
     for (void* p : c->dev_allocs) cudaFreeAsync(p, c->stream);
     if (!c->dev_allocs.empty() && c->stream) cudaStreamSynchronize(c->stream);
@@ -554,9 +555,9 @@ fftpl_status fftpl_debug_transpose_stores(fftpl_t h, int32_t tma) {
     Ctx& c = *h;
     if (tma && !c.spec_maps_ok) return set_err(c, FFTPL_ESTATE, "tensor maps not available");
     CK(cudaStreamSynchronize(c.stream));
-    if (c.eval_graph) {
-        cudaGraphExecDestroy(c.eval_graph);
-        c.eval_graph = nullptr;
+    for (auto& g : c.eval_graph) {
+        if (g.exec) cudaGraphExecDestroy(g.exec);
+        g.exec = nullptr;
     }
     if (c.loop_graph) {
         cudaGraphExecDestroy(c.loop_graph);
@@ -1024,9 +1025,8 @@ fftpl_status fftpl_wa(fftpl_t h, const float* x, const float* y, float gamma, do
 }
 
 // One full evaluation through the captured graph when use_graphs is set
-// (the graph is keyed by the buffers, gamma, the staging buffer and whether
-// it ends with the copy of the sums to the host); want: also enqueue that
-// copy.
+// (keyed by the buffers, gamma and the staging buffer); want: the report of the
+// sums to the host at the end, in a graph of its own.
 static fftpl_status eval_impl(Ctx& c, const float* x, const float* y, float gamma, float* gNx,
                               float* gNy, float* gWx, float* gWy, float* stage, bool want) {
     // a staging buffer means x, y and the gradients are pinned host memory
@@ -1034,14 +1034,13 @@ static fftpl_status eval_impl(Ctx& c, const float* x, const float* y, float gamm
     if (c.opt.use_graphs && !c.profiling) {
         float gk = gamma;
         const void* key[8] = {x, y, gNx, gNy, gWx, gWy, nullptr, stage};
-        const int32_t wk = want ? 1 : 0;
         memcpy(&key[6], &gk, sizeof(float));
-        memcpy((char*)&key[6] + sizeof(float), &wk, sizeof(wk));
+        auto& eg = c.eval_graph[want ? 1 : 0];
         const unsigned reports = c.reports;
-        if (!c.eval_graph || memcmp(key, c.graph_key, sizeof(key)) != 0) {
-            if (c.eval_graph) {
-                cudaGraphExecDestroy(c.eval_graph);
-                c.eval_graph = nullptr;
+        if (!eg.exec || memcmp(key, eg.key, sizeof(key)) != 0) {
+            if (eg.exec) {
+                cudaGraphExecDestroy(eg.exec);
+                eg.exec = nullptr;
             }
             cudaGraph_t g = nullptr;
             CK(cudaStreamBeginCapture(c.stream, cudaStreamCaptureModeThreadLocal));
@@ -1058,17 +1057,17 @@ static fftpl_status eval_impl(Ctx& c, const float* x, const float* y, float gamm
             if (re != cudaSuccess && g) cudaGraphDestroy(g);
             CK(re);
             CK(ee);
-            cudaError_t ie = cudaGraphInstantiate(&c.eval_graph, g, 0);
+            cudaError_t ie = cudaGraphInstantiate(&eg.exec, g, 0);
             cudaGraphDestroy(g);
             CK(ie);
-            memcpy(c.graph_key, key, sizeof(key));
-            c.graph_nkernels = c.launches - before;
+            memcpy(eg.key, key, sizeof(key));
+            eg.nkernels = c.launches - before;
             c.launches = before;  // counted at replay
         }
         c.reports = reports;   // a captured report has not run yet
-        CK(cudaGraphLaunch(c.eval_graph, c.stream));
+        CK(cudaGraphLaunch(eg.exec, c.stream));
         if (want) c.reports++;
-        c.launches += c.graph_nkernels;
+        c.launches += eg.nkernels;
         c.fields_valid = true;
         c.rho_valid = false;
         c.split_valid = false;
