@@ -316,7 +316,9 @@ fftpl_status fftpl_report(fftpl_t h, fftpl_eval_report* rep);
 
 /* Borrowed device views of the maps of the last density evaluation: bin
  * density rho, potential psi (Eq. 11), field E_x, E_y (Eq. 12).  Any pointer
- * may be NULL.  rho is formed on demand. */
+ * may be NULL.  The maps are formed on demand; after a call that the caller
+ * captured into a graph of its own, on every call, since the handle does not
+ * see that graph's replays. */
 fftpl_status fftpl_fields(fftpl_t h, const float** rho, const float** psi,
                           const float** ex, const float** ey);
 

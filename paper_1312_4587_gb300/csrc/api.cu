@@ -345,10 +345,19 @@ constexpr int kChainCells = 256 * 1024;
 // EV_HOST: the gradient arrays are pinned host memory written over the link
 enum { EV_DENSITY = 1, EV_WA = 2, EV_ADJOINT = 4, EV_NO_GATHER = 8, EV_HOST = 16 };
 
+// Notes a call made while the caller captures the handle's stream.
+void note_capture(Ctx& c) {
+    if (c.replayed || c.own_capture) return;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c.stream, &st) != cudaSuccess) cudaGetLastError();
+    else c.replayed = st != cudaStreamCaptureStatusNone;
+}
+
 // psi for the current fields, formed on demand (from PT, or from the
 // tensor-core solve's Ut).
 fftpl_status ensure_psi(Ctx& c, cudaStream_t s) {
-    if (!c.psi_valid) {
+    note_capture(c);
+    if (!c.psi_valid || c.replayed) {
         CK(c.tc ? launch_tc(c, 4, s) : launch_rows_psi(c, s));
         c.psi_valid = true;
     }
@@ -366,6 +375,7 @@ fftpl_status enqueue_eval(Ctx& c, const float* x, const float* y, float gamma, i
     bool dens = (what & EV_DENSITY) != 0, wa = (what & EV_WA) != 0;
     const bool grads = !(what & EV_NO_GATHER), host = (what & EV_HOST) != 0;
     const bool fused = dens && wa && grads && !(what & (EV_ADJOINT | EV_HOST));
+    note_capture(c);
     CK(enqueue_zero(c, dens, wa, s));
     c.chain = !(dens && wa) || c.m_mov <= kChainCells;
     auto wa_kernel = [&](bool interleave, cudaStream_t q) -> fftpl_status {
@@ -1045,7 +1055,9 @@ static fftpl_status eval_impl(Ctx& c, const float* x, const float* y, float gamm
             cudaGraph_t g = nullptr;
             CK(cudaStreamBeginCapture(c.stream, cudaStreamCaptureModeThreadLocal));
             int64_t before = c.launches;
+            c.own_capture = true;
             fftpl_status st = enqueue_eval(c, x, y, gamma, what, gNx, gNy, gWx, gWy, stage);
+            c.own_capture = false;
             cudaError_t re = st == FFTPL_OK && want ? launch_report(c, !stage && c.m_mov > 0, c.stream)
                                                     : cudaSuccess;
             cudaError_t ee = cudaStreamEndCapture(c.stream, &g);
@@ -1163,7 +1175,7 @@ fftpl_status fftpl_fields(fftpl_t h, const float** rho, const float** psi, const
     if (!c.fields_valid) return set_err(c, FFTPL_ESTATE, "no density evaluation yet");
     if (rho) {
         if (!c.rho) TRY(dalloc(c, &c.rho, (size_t)c.n * c.n));
-        if (!c.rho_valid) {
+        if (!c.rho_valid || c.replayed) {
             CK(launch_rho(c, c.stream));
             c.rho_valid = true;
         }
@@ -1179,7 +1191,7 @@ fftpl_status fftpl_fields(fftpl_t h, const float** rho, const float** psi, const
             TRY(dalloc(c, &c.ex, (size_t)c.n * c.n));
             TRY(dalloc(c, &c.ey, (size_t)c.n * c.n));
         }
-        if (!c.split_valid) {
+        if (!c.split_valid || c.replayed) {
             CK(launch_split_field(c, c.stream));
             c.split_valid = true;
         }

@@ -643,6 +643,10 @@ struct Ctx {
     bool rho_valid = false, fields_valid = false, split_valid = false;
     bool psi_valid = false;     // psi matches the current fields (it is formed on
                                 // demand)
+    bool own_capture = false;   // eval_impl is capturing
+    bool replayed = false;      // a call went into a caller's own capture, whose
+                                // replays the handle does not see: no map formed
+                                // on demand counts as current from then on
     std::string last_error;
     std::vector<void*> dev_allocs;
     size_t dev_bytes = 0;
