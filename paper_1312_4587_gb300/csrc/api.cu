@@ -6,8 +6,9 @@
 //                scatter -> rows_fwd -> cols -> rows_inv
 //   side stream: WA                                (forked, concurrent)
 //   main stream: join -> cells (gather + pin sums + norms)
-// (with host outputs WA runs before the transforms and its gradient is
-// written beside them; the main stream ends with the field gather)
+// (with host outputs the WA branch ends with its own gradient pass and the main
+// stream with the field gather; for many cells WA runs before the transforms
+// and only its gradient is written beside them)
 // and, when use_graphs is set, is replayed from a captured CUDA graph.
 #include <math.h>
 #include <string.h>
@@ -341,6 +342,15 @@ cudaError_t enqueue_zero(Ctx& c, bool dens, bool wa, cudaStream_t s) {
 // 204 -> 211 (2.2M).
 constexpr int kChainCells = 256 * 1024;
 
+// Up to this many cells an evaluation with host outputs runs the wirelength
+// kernel beside the transforms, above it before them: 31.1 us beside and 36.1
+// before (1,000 cells, pinned buffers, by graph), 38.5 and 43.5 (34K), 49.5 and
+// 51.3 (110K), 61.8 and 67.7 (210K), but 110.7 and 106.6 (500K), 183.9 and 181.5
+// (1M), 381 and 366 (2.2M).  Deterministic mode, whose passes are bound by the
+// device rather than by the link, always beside: 76 and 87 (210K), 140 and 160
+// (500K), 506 and 547 (2.2M).
+constexpr int kHostBesideCells = 256 * 1024;
+
 // ---------------------------------------------------------------- evaluation
 // EV_HOST: the gradient arrays are pinned host memory written over the link
 enum { EV_DENSITY = 1, EV_WA = 2, EV_ADJOINT = 4, EV_NO_GATHER = 8, EV_HOST = 16 };
@@ -403,7 +413,7 @@ fftpl_status enqueue_eval(Ctx& c, const float* x, const float* y, float gamma, i
         Stage st(c, 0, s);
         CK(launch_scatter_mov(c, x, y, wa, stage, s));
     }
-    if (wa && host) {
+    if (wa && host && c.m_mov > kHostBesideCells && !c.opt.deterministic) {
         // Host outputs: the link is what takes longest, so its first writes
         // start as early as they can: the WA kernel with the GPU to itself
         // (beside the transforms both branches' writes came at the end), its
@@ -418,7 +428,7 @@ fftpl_status enqueue_eval(Ctx& c, const float* x, const float* y, float gamma, i
         // pass beside the chain measured 18 % slower)
         TRY(fork());
         TRY(wa_kernel(false, c.side));
-        if (grads && !fused) CK(launch_pin_sum(c, gWx, gWy, false, false, c.side));
+        if (grads && !fused) CK(launch_pin_sum(c, gWx, gWy, host, false, c.side));
         CK(cudaEventRecord(c.ev_join, c.side));
     }
     TRY(enqueue_solve(c, s));
