@@ -7,6 +7,8 @@
 // scatter weights.  Adjoint: the exact derivative of the binned energy,
 // sum over rows of the row overlap times (psi at the right-edge bin - psi at
 // the left-edge bin), and likewise in y.
+#include <algorithm>
+
 #include "fftpl_internal.cuh"
 
 namespace fftpl {
@@ -66,23 +68,51 @@ k_scatter(Grid g, int m, const float* __restrict__ x, const float* __restrict__ 
 }
 
 // The fixed cells' overlap areas in units of 2^-32 (as the deterministic
-// scatter), a block per cell: a macro covers hundreds of bins a side (150
+// scatter).  A macro covers hundreds of bins a side and takes a block (150
 // macros on 2048 x 2048 bins, a thread each, took 369 us of a handle's
-// creation).
-__global__ void __launch_bounds__(128)
-k_scatter_fixed(Grid g, const float* __restrict__ x, const float* __restrict__ y,
-                const float* __restrict__ w, const float* __restrict__ h,
-                unsigned long long* __restrict__ Dq) {
-    const int i = blockIdx.x;
-    const Span s = cell_span(g, x[i], y[i], w[i], h[i]);
-    if (s.ilo > s.ihi || s.jlo > s.jhi) return;
+// creation); a pad of a few bins takes a thread (creation with 400K fixed cells
+// of 2 x 2 bins 1276 us with a block each, 1075 so; 1.5M 4086 and 3333).  At most
+// kFixedBlocks blocks per SM: a thread of block b looks at cell b + gridDim.x t,
+// t = its index and 128 further on in each round, so that macros listed side by
+// side fall to different blocks.
+constexpr int kFixedThreads = 128, kFixedBlocks = 16, kFixedSmall = 16;
+
+__device__ __forceinline__ void add_fixed(const Grid& g, const Span& s, int first, int step,
+                                          unsigned long long* Dq) {
     const int nx = s.ihi - s.ilo + 1, nb = nx * (s.jhi - s.jlo + 1);
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) {
+    for (int b = first; b < nb; b += step) {
         const int j = s.jlo + b / nx, k = s.ilo + b % nx;
         const float a = __fmul_rn(ov_len(g.x0, g.wb, k, s.xl, s.xh),
                                   ov_len(g.y0, g.hb, j, s.yl, s.yh));
         const long long q = __float2ll_rn(__fmul_rn(a, 4294967296.0f));
         atomicAdd(Dq + (size_t)j * g.n + k, (unsigned long long)q);
+    }
+}
+
+__global__ void __launch_bounds__(kFixedThreads)
+k_scatter_fixed(Grid g, int m, const float* __restrict__ x, const float* __restrict__ y,
+                const float* __restrict__ w, const float* __restrict__ h,
+                unsigned long long* __restrict__ Dq) {
+    __shared__ int big[kFixedThreads], nbig;
+    for (int c0 = blockIdx.x; c0 < m; c0 += gridDim.x * kFixedThreads) {
+        if (threadIdx.x == 0) nbig = 0;
+        __syncthreads();
+        const int i = c0 + gridDim.x * threadIdx.x;
+        if (i < m) {
+            const Span s = cell_span(g, x[i], y[i], w[i], h[i]);
+            if (s.ilo <= s.ihi && s.jlo <= s.jhi) {
+                if ((s.ihi - s.ilo + 1) * (s.jhi - s.jlo + 1) <= kFixedSmall)
+                    add_fixed(g, s, 0, 1, Dq);
+                else
+                    big[atomicAdd(&nbig, 1)] = i;
+            }
+        }
+        __syncthreads();
+        for (int q = 0; q < nbig; ++q) {
+            const int k = big[q];
+            add_fixed(g, cell_span(g, x[k], y[k], w[k], h[k]), threadIdx.x, kFixedThreads, Dq);
+        }
+        __syncthreads();
     }
 }
 
@@ -188,9 +218,9 @@ static inline int blocks_for(long long m, int t) { return (int)((m + t - 1) / t)
 
 cudaError_t launch_scatter_fixed(Ctx& c, long long* Dq, cudaStream_t s) {
     if (c.m_fix <= 0) return cudaSuccess;
-    k_scatter_fixed<<<c.m_fix, 128, 0, s>>>(c.grid, c.fix_x, c.fix_y, c.w + c.m_mov,
-                                            c.h + c.m_mov,
-                                            reinterpret_cast<unsigned long long*>(Dq));
+    k_scatter_fixed<<<std::min(c.m_fix, kFixedBlocks * c.num_sms), kFixedThreads, 0, s>>>(
+        c.grid, c.m_fix, c.fix_x, c.fix_y, c.w + c.m_mov, c.h + c.m_mov,
+        reinterpret_cast<unsigned long long*>(Dq));
     c.launches++;
     return cudaGetLastError();
 }
