@@ -527,6 +527,12 @@ fftpl_status fftpl_debug_tc_gemm(const void* a_hi, const void* a_lo, const void*
  * for and the tensor maps are not available. */
 fftpl_status fftpl_debug_transpose_stores(fftpl_t h, int32_t tma);
 
+/* What creation laid out, into host memory: the internal number of each movable
+ * cell (m_mov) and, by pin slot, its cell's internal number (-1: fixed cell or
+ * padding).  *slots: in, the room of pin_cell; out, the number of slots.  Either
+ * array may be NULL.  Synchronises the handle's stream. */
+fftpl_status fftpl_debug_layout(fftpl_t h, int32_t* cell_rank, int32_t* pin_cell, int64_t* slots);
+
 #ifdef __cplusplus
 }
 #endif

@@ -570,6 +570,21 @@ fftpl_status fftpl_fillers(const fftpl_region* R, const fftpl_cells* cells,
 
 void fftpl_debug_fail_alloc_after(int32_t k) { g_fail_after.store(k > 0 ? k : 0); }
 
+fftpl_status fftpl_debug_layout(fftpl_t h, int32_t* cell_rank, int32_t* pin_cell, int64_t* slots) {
+    if (!h || !slots) return FFTPL_EINVAL;
+    Ctx& c = *h;
+    if (pin_cell && *slots < c.slab_slots) return set_err(c, FFTPL_EINVAL, "too few slots");
+    if (cell_rank && c.m_mov > 0)
+        CK(cudaMemcpyAsync(cell_rank, c.cell_rank, (size_t)c.m_mov * sizeof(int32_t),
+                           cudaMemcpyDeviceToHost, c.stream));
+    if (pin_cell && c.slab_slots > 0)
+        CK(cudaMemcpyAsync(pin_cell, c.pin_cell, (size_t)c.slab_slots * sizeof(int32_t),
+                           cudaMemcpyDeviceToHost, c.stream));
+    *slots = c.slab_slots;
+    CK(cudaStreamSynchronize(c.stream));
+    return FFTPL_OK;
+}
+
 fftpl_status fftpl_debug_transpose_stores(fftpl_t h, int32_t tma) {
     if (!h) return FFTPL_EINVAL;
     Ctx& c = *h;

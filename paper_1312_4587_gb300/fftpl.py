@@ -161,6 +161,7 @@ def lib():
             "fftpl_stage_times": (S, [_H, _P, _P, C.c_int32]),
             "fftpl_launch_count": (C.c_int64, [_H]),
             "fftpl_debug_fail_alloc_after": (None, [C.c_int32]),
+            "fftpl_debug_layout": (S, [_H, _P, _P, _P]),
             "fftpl_debug_transpose_stores": (S, [_H, C.c_int32]),
             "fftpl_fillers": (S, [_P, _P, C.c_double, _P, _P, _P]),
             "fftpl_debug_tc_gemm": (S, [_P, _P, _P, _P, C.c_int32, C.c_int32, C.c_int32, _P,
@@ -543,6 +544,17 @@ def fftpl_fillers(region, w, h, m_mov, fix_x=None, fix_y=None, target_density=1.
 
 def fftpl_debug_fail_alloc_after(k):
     lib().fftpl_debug_fail_alloc_after(C.c_int32(int(k)))
+
+
+def fftpl_debug_layout(h, m):
+    """(internal number of each of the m movable cells, internal cell number by
+    pin slot), numpy int32."""
+    slots = C.c_int64(0)
+    _check(lib().fftpl_debug_layout(h, None, None, C.byref(slots)), h)
+    rank = np.empty(m, np.int32)
+    pins = np.empty(slots.value, np.int32)
+    _check(lib().fftpl_debug_layout(h, _hptr(rank, 0), _hptr(pins, 0), C.byref(slots)), h)
+    return rank, pins
 
 
 def fftpl_debug_transpose_stores(h, tma):
