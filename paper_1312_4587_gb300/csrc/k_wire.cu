@@ -608,6 +608,8 @@ cudaError_t launch_wa_impl(Ctx& c, const float* x, const float* y, float gamma,
         k_interleave<<<nblk(c.m_mov, 256), 256, 0, s>>>(c.m_mov, x, y, c.cell_rank, c.pos2,
                                                          done);
         c.launches++;
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
     }
     const WaIo io{c.pin_cell, c.pin_dx, c.pin_dy, c.pos2, c.pxy,
                   c.opt.deterministic ? nullptr : c.gW2, c.pin_slot, c.gpin};
