@@ -358,17 +358,6 @@ __device__ __forceinline__ void sum2_add(dfloat& a, float b) {
     a.hi = s;
 }
 
-__device__ __forceinline__ dfloat warp_df_sum(dfloat v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        dfloat w;
-        w.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
-        w.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
-        v = df_add(v, w);
-    }
-    return v;
-}
-
 __device__ __forceinline__ double* acc_stripe(double* acc, int q) {
     return acc + (blockIdx.x & (kAccStripes - 1)) * kAccStride + q;
 }
@@ -526,9 +515,6 @@ __device__ __forceinline__ void block_max(float v, double* acc, int q) {
 // ------------------------------------------------------------ complex
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-__device__ __forceinline__ float2 cmulc(float2 a, float2 b) {  // a * conj(b)
-    return make_float2(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
 }
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
@@ -714,7 +700,6 @@ cudaError_t launch_q_to_f(const long long* q, float scale, float* out, int count
 // scale (device double or null): multiplies the gradient written
 cudaError_t launch_gather(Ctx& c, const float* x, const float* y, float* gx, float* gy,
                           bool adjoint, const double* scale, cudaStream_t s);
-cudaError_t launch_wa(Ctx& c, const float* x, const float* y, float gamma, cudaStream_t s);
 // interleave = false: pos2 already written (by launch_scatter_mov)
 cudaError_t launch_wa_impl(Ctx& c, const float* x, const float* y, float gamma,
                            const float* scale_dev, const float* done, bool interleave,

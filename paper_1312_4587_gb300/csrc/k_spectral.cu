@@ -478,8 +478,6 @@ __device__ __forceinline__ float2 pack_inv(float c1u, float c1nu, float c2u, flo
     return make_float2(re * ph.x + im * ph.y, im * ph.x - re * ph.y);
 }
 
-// Position of sample x in Makhoul's reordering.
-__device__ __forceinline__ int mk_pos(int x, int N) { return (x & 1) ? (N - 1 - (x >> 1)) : (x >> 1); }
 // Sample of the natural order held at position k of the reordering.
 __device__ __forceinline__ int mk_src(int y, int N) { return (y & 1) ? (N - 1 - (y >> 1)) : (y >> 1); }
 

@@ -35,9 +35,7 @@ namespace fftpl {
 // slab read nearby sectors.
 __global__ void __launch_bounds__(256)
 k_interleave(int m, const float* __restrict__ x, const float* __restrict__ y,
-             const int* __restrict__ rank, float2* __restrict__ pos,
-             const float* __restrict__ done) {
-    if (done && *done != 0.0f) return;
+             const int* __restrict__ rank, float2* __restrict__ pos) {
     chain_trigger();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < m) pos[rank[i]] = make_float2(x[i], y[i]);
@@ -237,7 +235,7 @@ __device__ __forceinline__ void wa_pair(const WaIo& io, int base_a, bool live_a,
     if (live_b) wa_core<D, CSR, LSE>(bx, by, base_b, io, l2g, inv_g, wsum, hsum);
 }
 
-// Runtime degree d (slabs of degree > 6): the first pass stores the pin
+// Runtime degree d (slabs of degree above kBigMax): the first pass stores the pin
 // coordinates in the pins' own slots of pxy, the later passes re-read them.
 template <bool CSR, bool LSE>
 __device__ __forceinline__ void wa_net_any(const WaIo& io, int base, int d, float l2g,
@@ -497,9 +495,7 @@ k_cells(Grid g, int m, const float* __restrict__ x, const float* __restrict__ y,
         float* __restrict__ gNx, float* __restrict__ gNy,
         float* __restrict__ gWx, float* __restrict__ gWy, const int* __restrict__ rank,
         const int* __restrict__ cell_pin_ptr, const float2* __restrict__ gpin,
-        const float2* __restrict__ gW2, double* __restrict__ acc,
-        const float* __restrict__ done, DetRed dr) {
-    if (done && *done != 0.0f) return;
+        const float2* __restrict__ gW2, double* __restrict__ acc, DetRed dr) {
     chain_trigger();
     const int stride = gridDim.x * blockDim.x;
     int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -605,8 +601,7 @@ cudaError_t launch_wa_impl(Ctx& c, const float* x, const float* y, float gamma,
                            cudaStream_t s) {
     if (c.nslabs <= 0) return cudaSuccess;
     if (c.m_mov > 0 && interleave) {
-        k_interleave<<<nblk(c.m_mov, 256), 256, 0, s>>>(c.m_mov, x, y, c.cell_rank, c.pos2,
-                                                         done);
+        k_interleave<<<nblk(c.m_mov, 256), 256, 0, s>>>(c.m_mov, x, y, c.cell_rank, c.pos2);
         c.launches++;
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -633,10 +628,6 @@ cudaError_t launch_wa_impl(Ctx& c, const float* x, const float* y, float gamma,
     c.launches++;
     if (e != cudaSuccess) cudaGetLastError();
     return e;
-}
-
-cudaError_t launch_wa(Ctx& c, const float* x, const float* y, float gamma, cudaStream_t s) {
-    return launch_wa_impl(c, x, y, gamma, nullptr, nullptr, true, s);
 }
 
 // few: kLinkBlocks large blocks, for writes over the host link beside other
@@ -667,27 +658,20 @@ cudaError_t launch_pin_sum(Ctx& c, float* gx, float* gy, bool few, bool chain, c
     return e;
 }
 
-cudaError_t launch_cells_impl(Ctx& c, const float* x, const float* y, float* gNx, float* gNy,
-                              float* gWx, float* gWy, const float* done, cudaStream_t s) {
+cudaError_t launch_cells(Ctx& c, const float* x, const float* y, float* gNx, float* gNy,
+                         float* gWx, float* gWy, cudaStream_t s) {
     if (c.m_mov <= 0) return cudaSuccess;
     const int nb = cell_blocks(c);
     if (c.opt.deterministic)
         k_cells<true><<<nb, kCellThreads, 0, s>>>(c.grid, c.m_mov, x, y, c.w, c.h, c.E2, gNx,
                                                   gNy, gWx, gWy, c.cell_rank, c.cell_pin_ptr,
-                                                  c.gpin, nullptr,
-                                                  c.acc, done, det_red(c, 0));
+                                                  c.gpin, nullptr, c.acc, det_red(c, 0));
     else
         k_cells<false><<<nb, kCellThreads, 0, s>>>(c.grid, c.m_mov, x, y, c.w, c.h, c.E2,
                                                    gNx, gNy, gWx, gWy, c.cell_rank, nullptr,
-                                                   nullptr, c.gW2,
-                                                   c.acc, done, det_red(c, 0));
+                                                   nullptr, c.gW2, c.acc, det_red(c, 0));
     c.launches++;
     return cudaGetLastError();
-}
-
-cudaError_t launch_cells(Ctx& c, const float* x, const float* y, float* gNx, float* gNy,
-                         float* gWx, float* gWy, cudaStream_t s) {
-    return launch_cells_impl(c, x, y, gNx, gNy, gWx, gWy, nullptr, s);
 }
 
 }  // namespace fftpl
