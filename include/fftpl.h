@@ -45,6 +45,8 @@
  * and, where it says so, synchronises it.  With NULL the handle creates a
  * blocking stream of its own, which the legacy default stream orders with
  * implicitly.  A handle is not thread-safe; use one handle per host thread.
+ * A call that returns scalars polls host memory for them for up to 500 us, a
+ * core's time, before it waits on the stream.
  *
  * Errors: every call returns fftpl_status and never throws.  FFTPL_EINVAL
  * comes from host-side validation before any device work is queued.  The

@@ -336,7 +336,11 @@ cudaError_t enqueue_zero(Ctx& c, bool dens, bool wa, cudaStream_t s) {
 // launched as programmatic chains (launch_chain).  A call with one branch
 // always takes them: density alone 24.7 -> 15.6 us (1,000 cells), 35.0 -> 28.3
 // (210K, n = 512), 131 -> 124 (2.2M, n = 2048); wirelength alone 15.5 -> 10.4,
-// 24.0 -> 20.1, 101 -> 97.  With two branches the waiting blocks of one keep
+// 24.0 -> 20.1, 101 -> 97; density, called back to back, at every grid, n = 1024
+// included (where the three passes of a solve alone lose, see noalloc.cu): 39.7 ->
+// 32.5 us (20K cells, n = 256), 51.8 -> 48.7 (70K, 1024), 62.7 -> 60.1 (500K,
+// 1024), 72 -> 68 (1M, 1024), 100 -> 91 (500K, 2048), 326 -> 319 (2M, 4096), 438
+// either way (5M, 4096).  With two branches the waiting blocks of one keep
 // the other's out once the GPU is full: evaluation by graph 16.5 -> 14.4 us
 // (1,000), 22.7 -> 20.6 (34K), 34.9 -> 32.9 (210K), but 58.2 -> 60.0 (500K) and
 // 204 -> 211 (2.2M).
@@ -472,9 +476,9 @@ void fill_report(const Ctx& c, const double* acc, fftpl_eval_report* rep) {
 enum { END_KERNEL = 1, END_JOIN = 0 };
 
 // Waits for the last report enqueued, the last operation on the stream: the
-// host looks for its number in the mirror for as long as a short call takes,
-// then waits for the stream (which also tells of errors).  Seen 2.4 us before
-// a stream synchronisation returns.
+// host looks for its number in the mirror, on a core of its own, for as long as
+// a short call takes, then waits for the stream (which also tells of errors).
+// Seen 2.4 us before a stream synchronisation returns.
 fftpl_status wait_report(Ctx& c) {
     const unsigned* flag = reinterpret_cast<const unsigned*>(c.acc_host + kReportFlag);
     const auto t0 = std::chrono::steady_clock::now();
