@@ -56,12 +56,12 @@ STAGE_IDS = {"scatter": 0, "rows_fwd": 1, "cols": 2, "rows_inv": 3, "wa": 4, "ce
 # source it was taken from is unchanged: key = first 16 hex digits of the
 # SHA-256 of the kernel file followed by fftpl_internal.cuh.
 STAGE_TRAFFIC = {
-    "scatter": ("k_density.cu", "9c3e14b604172bd7", 50747136 + 1101824),
-    "rows_fwd": ("k_spectral.cu", "83c53d6aa0bbad29", 33621760 + 25088),
-    "cols": ("k_spectral.cu", "83c53d6aa0bbad29", 16872192 + 9472),
-    "rows_inv": ("k_spectral.cu", "83c53d6aa0bbad29", 33615104 + 302336),
-    "wa": ("k_wire.cu", "9c6f67605701cf9e", 139707136 + 4197376),
-    "cells": ("k_wire.cu", "9c6f67605701cf9e", 76204032 + 13038848),
+    "scatter": ("k_density.cu", "82559d45d5283669", 50750720 + 976384),
+    "rows_fwd": ("k_spectral.cu", "e6b2ddb80b0cca59", 33622528 + 48640),
+    "cols": ("k_spectral.cu", "e6b2ddb80b0cca59", 16872960 + 20224),
+    "rows_inv": ("k_spectral.cu", "e6b2ddb80b0cca59", 33615104 + 321024),
+    "wa": ("k_wire.cu", "cc44c7f35cf5bc76", 139702784 + 4531712),
+    "cells": ("k_wire.cu", "cc44c7f35cf5bc76", 76207616 + 13415680),
 }
 
 

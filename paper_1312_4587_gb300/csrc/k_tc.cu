@@ -20,7 +20,7 @@
 // (Eqs. 10-12 at the bin centres; the energy N = 1/2 A_b sum B Psi is
 // reduced in the G2 epilogue.)  18 n^3 flops; without the folding and with
 // psi in every solve 42 n^3: at n = 2048 the five products took 46 + 59 + 91 +
-// 105 + 68 us (the last two side by side), now 28 + 34 + 48 + 28 + 27, and the
+// 105 + 68 us (the last two side by side), now 29 + 37 + 49 + 28 + 28, and the
 // gradient's relative error went from 9e-6 to 5e-6.  What bounds them: the
 // operands' shared-memory reads (128 x 128 tiles read 128 bytes a cycle, the
 // loads write 85 more) and, at 256 tiles on 152 SMs, the second wave.
